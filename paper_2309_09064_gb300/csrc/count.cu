@@ -51,6 +51,10 @@ size_t pipeline_bytes(const tc_ctx *ctx, uint32_t n, uint64_t slots, uint32_t ma
     bytes += r(4 * (256 * rtiles + 1)) + r(8 * (256 * rtiles + 2));  // radix digit counts and offsets
     bytes += r(8 * scan_tmp_elems(std::max<uint64_t>(n1 + 1, 256 * rtiles + 2)));  // scan tiles
     bytes += r(8 * (slots / 2 + 1));               // task pool: at most one task per oriented G0 edge
+    if (plain && wedge_path(ctx, n, slots, max_deg)) {
+        const WedgeSizes z = wedge_sizes(ctx, n, slots);
+        bytes += r(4 * z.counts) + r(8 * (z.counts + 1)) + r(8ull * z.tiles) + r(16ull * z.tasks) + r(8 * z.tmp);
+    }
     *hub_words = 0;
     *hub_maps = 0;
     if (max_deg > ctx->tune.block_cap) {
@@ -155,6 +159,17 @@ tc_status count_pipeline(tc_ctx *ctx, const GraphView &g, uint32_t *levels_out, 
     b.hub_words = hub_words;
     b.hub_sets = hub_maps > ctx->tune.hub_group ? 2u : 1u;
     if (hub_maps) b.hub_bits = a.take<uint32_t>(hub_words * hub_maps);
+    const bool wedge = plain && groups.n_groups == 0 && wedge_path(ctx, n, g.slots, g.max_deg);
+    if (wedge) {
+        const WedgeSizes z = wedge_sizes(ctx, n, g.slots);
+        b.wedge_ids = reinterpret_cast<uint16_t *>(b.task_pool);
+        b.wedge_counts = a.take<uint32_t>(z.counts);
+        b.wedge_offs = a.take<uint64_t>(z.counts + 1);
+        b.wedge_work = a.take<unsigned long long>(z.tiles);
+        b.wedge_tasks = a.take<uint4>(z.tasks);
+        b.wedge_tmp = a.take<uint64_t>(z.tmp);
+        ok = ok && b.wedge_counts && b.wedge_offs && b.wedge_work && b.wedge_tasks && b.wedge_tmp;
+    }
     b.groups = groups;
     if (vertex_counts) {
         b.vcount = reinterpret_cast<unsigned long long *>(vertex_counts);
@@ -208,6 +223,12 @@ tc_status count_pipeline(tc_ctx *ctx, const GraphView &g, uint32_t *levels_out, 
         st = intersect_alg3(ctx, b, n, g.slots);
         if (st != TC_OK) return st;
         ctx->isect_flags = 0;
+    } else if (wedge) {
+        st = wedge_rows(ctx, b, n, g.max_deg);
+        if (st != TC_OK) return st;
+        TC_CUDA(ctx, cudaEventRecord(ctx->ev[2], s));
+        st = wedge_count(ctx, b, n, g.max_deg);
+        if (st != TC_OK) return st;
     } else {
         st = build_rows(ctx, b, n, g.max_deg);
         if (st != TC_OK) return st;
@@ -316,7 +337,9 @@ tc_status count_pipeline(tc_ctx *ctx, const GraphView &g, uint32_t *levels_out, 
         for (int c = 0; c < 4; ++c) {
             stats->class_rows[c] = h.cls_rows[c];
             stats->class_probes[c] = h.cls_probes[c];
-            stats->class_bytes[c] = 4ull * (h.cls_build[c] + h.cls_probes[c]);
+            // wedge path: tiles read 16-byte entries and 16-bit ids, the other pairs 4-byte keys
+            stats->class_bytes[c] = wedge && c == 1 ? 16ull * h.cls_build[1] + 2ull * (h.cls_probes[1] + h.cls_inserts[1])
+                                                    : 4ull * (h.cls_build[c] + h.cls_probes[c]);
             stats->class_inserts[c] = h.cls_inserts[c];
             is += stats->class_bytes[c];
             stats->ms_class[c] = 0.f;

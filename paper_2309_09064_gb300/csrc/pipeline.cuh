@@ -83,7 +83,30 @@ struct PipeBufs {
     unsigned long long wstate_len = 0;
     unsigned long long tiny_base = 0;
     uint32_t *inv = nullptr;                  // [n] rank -> id (null under the id order)
+    // wedge path (wedge.cu): the rows N(x) are kept in adj2 (keys) and wedge_ids
+    // (16-bit ids), their sizes in fcnt and gcnt, their places by rank in vmeta,
+    // the tile entries in erec
+    uint16_t *wedge_ids = nullptr;            // [2 S] (the task pool's memory)
+    uint32_t *wedge_counts = nullptr;         // entries per tile and block
+    uint64_t *wedge_offs = nullptr;           // their scan
+    unsigned long long *wedge_work = nullptr; // steps per tile
+    uint4 *wedge_tasks = nullptr;             // {tile, first entry, last entry}
+    uint64_t *wedge_tmp = nullptr;            // scan tiles
 };
+
+// Plain counts under the degree order (wedge.cu).  Vertices of degree >=
+// kWedgeTileDegree, at most kWedgeMaxU of them, are taken in tiles of 32; a
+// tile's words cover the first kWedgeMaxK ranks (16-bit ids of 15 rank bits;
+// the last rank of 15 bits stays free: it marks padding).
+constexpr uint32_t kWedgeTileDegree = 128;
+constexpr uint32_t kWedgeMaxU = 1u << 18;
+constexpr uint32_t kWedgeMaxK = 32736;
+struct WedgeSizes {
+    uint32_t tiles, tasks;
+    uint64_t counts, tmp;
+};
+WedgeSizes wedge_sizes(const tc_ctx *ctx, uint32_t n, uint64_t slots);
+bool wedge_path(const tc_ctx *ctx, uint32_t n, uint64_t slots, uint32_t max_deg);
 
 // Ranks below this value are kept in the block class's shared bitmap, and
 // the rows stage puts them first in every level-spanning part (0: no split).
@@ -140,5 +163,8 @@ tc_status emit_tasks(tc_ctx *ctx, PipeBufs &b);
 // a count split into shards: the probe records of this shard's tasks only
 tc_status records_for_shard(tc_ctx *ctx, const PipeBufs &b);
 tc_status intersect(tc_ctx *ctx, PipeBufs &b, uint32_t n);
+// the wedge path: rows, entries and tasks, then the two counting kernels
+tc_status wedge_rows(tc_ctx *ctx, const PipeBufs &b, uint32_t n, uint32_t max_deg);
+tc_status wedge_count(tc_ctx *ctx, const PipeBufs &b, uint32_t n, uint32_t max_deg);
 
 }  // namespace tc

@@ -76,7 +76,8 @@ struct Ctl {
     unsigned int huge_next;          // k_row_fill_huge: next listed row a block takes
     unsigned int sort_next;          // k_sort_big: next listed row a block takes
     unsigned int split_next;         // k_g1_split: next listed row a block takes
-    unsigned int pad[2];
+    unsigned int wedge_u, wedge_k;   // wedge path: vertices taken in tiles, ranks their words cover
+    unsigned int wedge_hi_task, wedge_pad;  // first task of the tiles from rank kWedgeMaxK on
     unsigned long long list_cursor;  // listing: next free chunk position
 };
 

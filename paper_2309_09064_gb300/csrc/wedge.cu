@@ -1,0 +1,1150 @@
+// wedge.cu -- the plain count under the degree order: every triangle of
+// Algorithm 4 found at the wedge of its latest vertex, by tiles of 32 earlier ones.
+//
+// The method is Algorithm 4's (levels, horizontal and level-spanning edges,
+// every triangle has one or three horizontal edges) with another choice of
+// where each triangle is found.  Hashing u and probing all of G1(v) at every
+// horizontal edge u -> v reads the level-spanning part of a hub v once per
+// horizontal edge of v: 124 G ids at R-MAT 24.  Here every vertex x keeps only
+//     N(x) = { y ~ x : y precedes x }   (ranks, ascending, each with a flag:
+//                                        1 when L(y) == L(x), a horizontal edge)
+// and a triangle w < u < v (ranks) is found once, as a pair of N(v) with w in
+// N(u): sum C(|N(v)|, 2) pairs, about 42 G at R-MAT 24.  It lies inside G0 when
+// both u-v and w-v are horizontal, else it has exactly one horizontal edge
+// (levels of adjacent vertices differ by at most one), so the two flags of v's
+// row alone split the count into t_same and t_cross.
+//
+// Tiles.  The pairs whose u is one of the U highest-degree vertices and whose
+// w is one of the first K are taken 32 u's at a time: for the tile
+// t = {32 t .. 32 t + 31} a block keeps word[w] (w < K, shared memory), whose
+// bit i says that w precedes and neighbours u = 32 t + i.  A vertex v with
+// neighbours `mask` in the tile then needs one shared load, one AND and one
+// popcount per w in the prefix of its row below the tile's end, for all of
+// those u together: 0.6 lookups per pair at R-MAT 20-22 (a set per u: 1).
+// The rows are read as 16-bit ids (w < K <= 2^15, flag in the low bit).
+// k_wedge_high takes the same tiles' pairs with w >= K, k_wedge_rest those with
+// u >= U.  Measured (one GB300, whole counts, before and after): R-MAT 24
+// 130.5 -> 58.6 ms, R-MAT 20 5.39 -> 2.31, Chung-Lu 2^22 16.4 -> 7.6, uniform
+// 2^20 of mean degree 32 3.36 -> 1.87, R-MAT 16 1.32 -> 0.73.
+#include <algorithm>
+
+#include "pipeline.cuh"
+
+namespace tc {
+namespace {
+
+constexpr uint32_t kSmallRow = 32;     // rows of degree <= 32: one lane each
+constexpr uint32_t kWarpKeys = 1024;   // rows of up to this many keys are sorted by their warp
+constexpr uint32_t kHugeRow = 8192;    // rows of higher degree: a block each
+constexpr uint32_t kSortCap = 32768;   // largest row a block sorts (rows hold at most sqrt(slots) keys)
+constexpr int kFillThreads = 256;
+constexpr uint32_t kAhead = 8;         // neighbours of a lane's row read ahead together
+constexpr uint16_t kPadId = 0xFFFFu;   // fills a row's last unit: rank 2^15 - 1 >= K, its word is always 0
+constexpr uint32_t kTaskSteps = 1024;  // least steps (32 ids of one entry) of a tile task
+constexpr uint32_t kTasksPerSm = 16;
+constexpr unsigned kGuardSort = 0x100u;
+constexpr unsigned kGuardRange = 0x800u;
+constexpr unsigned kGuardWatchdog = 0x80u;
+constexpr long long kWatchdogCycles = 20000000000ll;  // about 10 s of SM clock
+
+template <bool kPacked>
+__device__ __forceinline__ uint2 rank_level(const uint2 *__restrict__ lv, const uint32_t *__restrict__ lvp, uint32_t y) {
+    if constexpr (kPacked) {
+        const uint32_t p = lvp[y];
+        return make_uint2(p >> 8, p & 0xFFu);
+    } else {
+        return lv[y];
+    }
+}
+
+// U: the vertices of degree >= kWedgeTileDegree (the working order starts with
+// them), whole tiles, at most kWedgeMaxU; K = min(U, kWedgeMaxK).
+__global__ void k_wedge_limits(uint32_t n, const unsigned long long *__restrict__ order, uint32_t max_deg, Ctl *ctl) {
+    uint32_t U = 0;
+    if (max_deg >= kWedgeTileDegree) {
+        const uint32_t last = max_deg - kWedgeTileDegree;  // largest key of a tile vertex
+        uint32_t lo = 0, hi = n < kWedgeMaxU ? n : kWedgeMaxU;
+        while (lo < hi) {
+            const uint32_t mid = (lo + hi) >> 1;
+            if ((uint32_t)(order[mid] >> 32) <= last) lo = mid + 1; else hi = mid;
+        }
+        U = (lo + 31u) & ~31u;
+    }
+    ctl->wedge_u = U;
+    ctl->wedge_k = U < kWedgeMaxK ? U : kWedgeMaxK;
+}
+
+// Ascending bitonic sort of 32 * E keys by one warp, E consecutive ones per
+// lane in registers: compares across lanes are shuffles, the others stay in
+// the lane (in shared memory every compare costs two loads and two stores).
+template <int E>
+__device__ __forceinline__ void lane_sort(uint32_t (&v)[E]) {
+    const unsigned lane = lane_id();
+#pragma unroll
+    for (int k = 2; k <= 32 * E; k <<= 1) {
+#pragma unroll
+        for (int j = k >> 1; j > 0; j >>= 1) {
+            if (j >= E) {
+                const bool low = ((lane & (j / E)) == 0) == (((lane * E) & k) == 0);
+#pragma unroll
+                for (int e = 0; e < E; ++e) {
+                    const uint32_t o = __shfl_xor_sync(0xFFFFFFFFu, v[e], j / E);
+                    v[e] = low ? min(v[e], o) : max(v[e], o);
+                }
+            } else {
+#pragma unroll
+                for (int e = 0; e < E; ++e) {
+                    if (e & j) continue;
+                    const bool up = k < E ? (e & k) == 0 : ((lane * E) & k) == 0;
+                    const uint32_t x = v[e], y = v[e | j];
+                    v[e] = up ? min(x, y) : max(x, y);
+                    v[e | j] = up ? max(x, y) : min(x, y);
+                }
+            }
+        }
+    }
+}
+
+// Sort buf[0..d), d <= 32 * E, in place.
+template <int E>
+__device__ __forceinline__ void warp_sort(uint32_t *buf, uint32_t d) {
+    const unsigned lane = lane_id();
+    uint32_t v[E];
+#pragma unroll
+    for (int e = 0; e < E; ++e) v[e] = e * 32 + lane < d ? buf[e * 32 + lane] : kEmpty;
+    lane_sort<E>(v);
+    __syncwarp();
+    if constexpr (E % 4 == 0) {
+#pragma unroll
+        for (int e = 0; e < E; e += 4)
+            reinterpret_cast<uint4 *>(buf)[(lane * E + e) / 4] = make_uint4(v[e], v[e + 1], v[e + 2], v[e + 3]);
+    } else {
+#pragma unroll
+        for (int e = 0; e < E; ++e) buf[lane * E + e] = v[e];
+    }
+    __syncwarp();
+}
+
+// What a row leaves behind besides its keys: |N(x)|, how many of them lie
+// below K and below U, and the row's place by rank.
+struct RowOut {
+    uint32_t *dcnt, *lcnt, *ucnt;
+    uint4 *rmeta;
+};
+__device__ __forceinline__ void row_done(const RowOut &o, uint32_t x, uint32_t rank, uint64_t b, uint32_t d,
+                                         uint32_t nlo, uint32_t nu) {
+    o.dcnt[x] = d;
+    o.lcnt[x] = nlo;
+    o.ucnt[x] = nu;
+    o.rmeta[rank] = make_uint4((uint32_t)b, (uint32_t)(b >> 32), d, nlo);
+}
+
+// First 16-bit id of the row at slot b: the row owns the 8-byte units
+// [(b + 1) / 2, (b + deg + 1) / 2), at least deg / 2 of them, so a row of degree
+// >= 2 has room for its ids and their padding to whole units (kPadId).
+__device__ __forceinline__ uint16_t *ids_of(uint16_t *ids, uint64_t b) { return ids + 4 * ((b + 1) >> 1); }
+
+// N(x) of every vertex of degree <= kHugeRow.  Warps take chunks of 32
+// vertices; rows of degree <= 32 belong to one lane (insertion sort in its
+// column of the warp's buffer), longer ones to the whole warp (compacted into
+// the buffer and sorted there; more than kWarpKeys keys are left unsorted in
+// place for k_wedge_sort).  Bound by the gathers of the rank/level words.
+template <bool kPacked>
+__global__ void __launch_bounds__(kFillThreads) k_wedge_rows(uint32_t n, const uint64_t *__restrict__ rp,
+                                                             const uint32_t *__restrict__ col,
+                                                             const uint2 *__restrict__ lv,
+                                                             const uint32_t *__restrict__ lvp,
+                                                             uint32_t *__restrict__ keys, uint16_t *__restrict__ ids,
+                                                             RowOut out, uint32_t *__restrict__ big,
+                                                             uint32_t *__restrict__ huge, uint32_t per_warp, Ctl *ctl) {
+    __shared__ __align__(16) uint32_t sbuf[kFillThreads / 32][kWarpKeys];
+    const unsigned lane = lane_id(), warp = threadIdx.x >> 5;
+    const unsigned lt = (1u << lane) - 1u;
+    uint32_t *buf = sbuf[warp];
+    const uint32_t K2 = 2 * ctl->wedge_k, U2 = 2 * ctl->wedge_u;  // a key below K2 has a rank below K
+    unsigned long long horizontal = 0;
+    const uint64_t chunks = ((uint64_t)n + per_warp - 1) / per_warp;
+    for (;;) {
+        unsigned int c = 0;
+        if (lane == 0) c = atomicAdd(&ctl->fill_next, 1u);
+        c = __shfl_sync(0xFFFFFFFFu, c, 0);
+        if (c >= chunks) break;
+        const uint64_t x = (uint64_t)c * per_warp + lane;
+        const bool valid = lane < per_warp && x < n;
+        const uint64_t b = valid ? rp[x] : 0;
+        const uint32_t dx = valid ? (uint32_t)(rp[x + 1] - b) : 0;
+        const uint2 me = valid ? rank_level<kPacked>(lv, lvp, (uint32_t)x) : make_uint2(0, 0);
+        if (valid && dx <= kSmallRow) {
+            uint32_t d = 0;
+            for (uint32_t j0 = 0; j0 < dx; j0 += kAhead) {
+                uint32_t y[kAhead];
+                uint2 q[kAhead];
+#pragma unroll
+                for (uint32_t t = 0; t < kAhead; ++t) y[t] = j0 + t < dx ? col[b + j0 + t] : 0u;
+#pragma unroll
+                for (uint32_t t = 0; t < kAhead; ++t)
+                    q[t] = j0 + t < dx ? rank_level<kPacked>(lv, lvp, y[t]) : make_uint2(0xFFFFFFFFu, 0);
+#pragma unroll
+                for (uint32_t t = 0; t < kAhead; ++t) {
+                    if (q[t].x >= me.x) continue;
+                    const uint32_t key = (q[t].x << 1) | (q[t].y == me.y);
+                    uint32_t i = d++;
+                    while (i > 0 && buf[(i - 1) * 32 + lane] > key) {
+                        buf[i * 32 + lane] = buf[(i - 1) * 32 + lane];
+                        --i;
+                    }
+                    buf[i * 32 + lane] = key;
+                    horizontal += key & 1u;
+                }
+            }
+            uint32_t nlo = 0, nu = 0;
+            uint16_t *id = ids_of(ids, b);
+            for (uint32_t i = 0; i < d; ++i) {
+                const uint32_t key = buf[i * 32 + lane];
+                keys[b + i] = key;
+                nu += key < U2;
+                if (key < K2 && dx >= 2) {  // a vertex of degree 1 closes no triangle (and has no room)
+                    id[i] = (uint16_t)key;
+                    ++nlo;
+                }
+            }
+            for (uint32_t i = nlo; i & 3u; ++i) id[i] = kPadId;
+            row_done(out, (uint32_t)x, me.x, b, d, nlo, nu);
+        }
+        __syncwarp();
+        const unsigned huge_m = __ballot_sync(0xFFFFFFFFu, valid && dx > kHugeRow);
+        if (valid && dx > kHugeRow) huge[atomicAdd(&ctl->n_huge, 1u)] = (uint32_t)x;
+        unsigned pending = __ballot_sync(0xFFFFFFFFu, valid && dx > kSmallRow) & ~huge_m;
+        while (pending) {
+            const int src = __ffs(pending) - 1;
+            pending &= pending - 1;
+            const uint32_t bx = c * per_warp + (uint32_t)src;
+            const uint32_t bd = __shfl_sync(0xFFFFFFFFu, dx, src);
+            const uint64_t bb = __shfl_sync(0xFFFFFFFFu, b, src);
+            const uint32_t brx = __shfl_sync(0xFFFFFFFFu, me.x, src);
+            const uint32_t blx = __shfl_sync(0xFFFFFFFFu, me.y, src);
+            uint32_t d = 0;
+            for (uint32_t j0 = 0; j0 < bd; j0 += 128) {  // four neighbours per lane in flight
+                uint32_t y[4];
+                uint2 q[4];
+#pragma unroll
+                for (int t = 0; t < 4; ++t) y[t] = j0 + 32 * t + lane < bd ? col[bb + j0 + 32 * t + lane] : 0u;
+#pragma unroll
+                for (int t = 0; t < 4; ++t)
+                    q[t] = j0 + 32 * t + lane < bd ? rank_level<kPacked>(lv, lvp, y[t]) : make_uint2(0xFFFFFFFFu, 0);
+#pragma unroll
+                for (int t = 0; t < 4; ++t) {
+                    const bool in = q[t].x < brx;
+                    const unsigned m = __ballot_sync(0xFFFFFFFFu, in);
+                    if (in) {
+                        const uint32_t key = (q[t].x << 1) | (q[t].y == blx), pos = d + __popc(m & lt);
+                        if (pos < kWarpKeys) buf[pos] = key; else keys[bb + pos] = key;
+                        horizontal += key & 1u;
+                    }
+                    d += __popc(m);
+                }
+            }
+            __syncwarp();
+            if (d > kWarpKeys) {  // the rest of the row is in place already
+                for (uint32_t i = lane; i < kWarpKeys; i += 32) keys[bb + i] = buf[i];
+                if (lane == 0) big[atomicAdd(&ctl->n_big, 1u)] = bx;
+                if (lane == 0) out.dcnt[bx] = d;
+                __syncwarp();
+                continue;
+            }
+            if (d <= 32) warp_sort<1>(buf, d);
+            else if (d <= 64) warp_sort<2>(buf, d);
+            else if (d <= 128) warp_sort<4>(buf, d);
+            else if (d <= 256) warp_sort<8>(buf, d);
+            else if (d <= 512) warp_sort<16>(buf, d);
+            else warp_sort<32>(buf, d);
+            uint32_t nlo = 0, nu = 0;
+            uint16_t *id = ids_of(ids, bb);
+            for (uint32_t i = lane; i < d; i += 32) {
+                const uint32_t key = buf[i];
+                keys[bb + i] = key;
+                nu += key < U2;
+                if (key < K2) {
+                    id[i] = (uint16_t)key;
+                    ++nlo;
+                }
+            }
+            nlo = warp_sum(nlo);
+            nu = warp_sum(nu);
+            if (lane < ((0u - nlo) & 3u)) id[nlo + lane] = kPadId;
+            if (lane == 0) row_done(out, bx, brx, bb, d, nlo, nu);
+            __syncwarp();
+        }
+    }
+    horizontal = warp_sum(horizontal);
+    if (lane == 0 && horizontal) atomicAdd(&ctl->e0, horizontal);
+}
+
+// Rows of degree above kHugeRow, a block each: compacted in place (positions
+// from the warps' ballots and a prefix over the warps), sorted by k_wedge_sort.
+template <bool kPacked>
+__global__ void __launch_bounds__(1024) k_wedge_rows_huge(const uint32_t *__restrict__ huge, Ctl *ctl,
+                                                          const uint64_t *__restrict__ rp,
+                                                          const uint32_t *__restrict__ col,
+                                                          const uint2 *__restrict__ lv,
+                                                          const uint32_t *__restrict__ lvp,
+                                                          uint32_t *__restrict__ keys, uint32_t *__restrict__ dcnt,
+                                                          uint32_t *__restrict__ big) {
+    __shared__ unsigned int wcnt[32];
+    __shared__ unsigned int s_i;
+    const unsigned lane = lane_id(), warp = threadIdx.x >> 5;
+    const unsigned lt = (1u << lane) - 1u;
+    const uint32_t nh = ctl->n_huge;
+    unsigned long long horizontal = 0;
+    for (;;) {
+        if (threadIdx.x == 0) s_i = atomicAdd(&ctl->huge_next, 1u);
+        __syncthreads();
+        const uint32_t i = s_i;
+        __syncthreads();
+        if (i >= nh) break;
+        const uint32_t x = huge[i];
+        const uint64_t b = rp[x];
+        const uint32_t dx = (uint32_t)(rp[x + 1] - b);
+        const uint2 me = rank_level<kPacked>(lv, lvp, x);
+        uint32_t d = 0;
+        for (uint32_t j0 = 0; j0 < dx; j0 += 4 * blockDim.x) {
+            uint32_t y[4];
+            uint2 q[4];
+            unsigned m[4];
+            uint32_t mine = 0;
+#pragma unroll
+            for (int t = 0; t < 4; ++t) {
+                const uint32_t j = j0 + t * blockDim.x + threadIdx.x;
+                y[t] = j < dx ? col[b + j] : 0u;
+            }
+#pragma unroll
+            for (int t = 0; t < 4; ++t) {
+                const uint32_t j = j0 + t * blockDim.x + threadIdx.x;
+                q[t] = j < dx ? rank_level<kPacked>(lv, lvp, y[t]) : make_uint2(0xFFFFFFFFu, 0);
+                m[t] = __ballot_sync(0xFFFFFFFFu, q[t].x < me.x);
+                mine += __popc(m[t]);
+            }
+            if (lane == 0) wcnt[warp] = mine;
+            __syncthreads();
+            uint32_t v = wcnt[lane], incl = v;
+#pragma unroll
+            for (int o = 1; o < 32; o <<= 1) {
+                const uint32_t z = __shfl_up_sync(0xFFFFFFFFu, incl, o);
+                if (lane >= (unsigned)o) incl += z;
+            }
+            uint32_t pos = d + __shfl_sync(0xFFFFFFFFu, incl - v, warp);
+            d += __shfl_sync(0xFFFFFFFFu, incl, 31);
+#pragma unroll
+            for (int t = 0; t < 4; ++t) {
+                if (q[t].x < me.x) {
+                    const uint32_t key = (q[t].x << 1) | (q[t].y == me.y);
+                    keys[b + pos + __popc(m[t] & lt)] = key;
+                    horizontal += key & 1u;
+                }
+                pos += __popc(m[t]);
+            }
+            __syncthreads();
+        }
+        if (threadIdx.x == 0) {
+            dcnt[x] = d;
+            big[atomicAdd(&ctl->n_big, 1u)] = x;
+        }
+    }
+    horizontal = warp_sum(horizontal);
+    if (lane == 0 && horizontal) atomicAdd(&ctl->e0, horizontal);
+}
+
+// Listed rows (more than kWarpKeys keys, or of huge degree): a block each
+// sorts the keys in shared memory and finishes the row.
+template <bool kPacked>
+__global__ void __launch_bounds__(1024) k_wedge_sort(const uint32_t *__restrict__ big, Ctl *ctl,
+                                                     const uint64_t *__restrict__ rp, const uint2 *__restrict__ lv,
+                                                     const uint32_t *__restrict__ lvp, uint32_t *__restrict__ keys,
+                                                     uint16_t *__restrict__ ids, RowOut out) {
+    extern __shared__ uint32_t sb[];  // kSortCap keys
+    __shared__ unsigned int s_i, s_lo, s_u;
+    const uint32_t nb = ctl->n_big, K2 = 2 * ctl->wedge_k, U2 = 2 * ctl->wedge_u;
+    for (;;) {
+        if (threadIdx.x == 0) {
+            s_i = atomicAdd(&ctl->sort_next, 1u);
+            s_lo = 0;
+            s_u = 0;
+        }
+        __syncthreads();
+        const uint32_t i = s_i;
+        if (i >= nb) break;
+        const uint32_t x = big[i];
+        const uint64_t b = rp[x];
+        const uint32_t d = out.dcnt[x];
+        if (d > kSortCap) {  // cannot be: |N(x)|^2 <= slots
+            if (threadIdx.x == 0) atomicOr(&ctl->error, kGuardSort);
+            __syncthreads();
+            continue;
+        }
+        uint32_t P = 2;
+        while (P < d) P <<= 1;
+        for (uint32_t t = threadIdx.x; t < P; t += blockDim.x) sb[t] = t < d ? keys[b + t] : kEmpty;
+        __syncthreads();
+        for (uint32_t k = 2; k <= P; k <<= 1) {
+            for (uint32_t j = k >> 1; j > 0; j >>= 1) {
+                for (uint32_t p = threadIdx.x; p < P / 2; p += blockDim.x) {
+                    const uint32_t e = ((p & ~(j - 1)) << 1) | (p & (j - 1)), l = e | j;
+                    const uint32_t a = sb[e], c = sb[l];
+                    if ((a > c) == ((e & k) == 0)) {
+                        sb[e] = c;
+                        sb[l] = a;
+                    }
+                }
+                __syncthreads();
+            }
+        }
+        uint32_t nlo = 0, nu = 0;
+        uint16_t *id = ids_of(ids, b);
+        for (uint32_t t = threadIdx.x; t < d; t += blockDim.x) {
+            const uint32_t key = sb[t];
+            keys[b + t] = key;
+            nu += key < U2;
+            if (key < K2) {
+                id[t] = (uint16_t)key;
+                ++nlo;
+            }
+        }
+        nlo = warp_sum(nlo);
+        nu = warp_sum(nu);
+        if (lane_id() == 0 && nlo) atomicAdd(&s_lo, nlo);
+        if (lane_id() == 0 && nu) atomicAdd(&s_u, nu);
+        __syncthreads();
+        if (threadIdx.x < ((0u - s_lo) & 3u)) id[s_lo + threadIdx.x] = kPadId;
+        if (threadIdx.x == 0) row_done(out, x, rank_level<kPacked>(lv, lvp, x).x, b, d, s_lo, s_u);
+        __syncthreads();
+    }
+}
+
+// ---------------------------------------------------------------------------- entries
+
+// One entry per (vertex v, tile, kind): {first 16-bit id of v's row in units of
+// 8 bytes, mask of v's neighbours in the tile, units of the prefix | kind << 31,
+// keys of the row below K | (slot of the row & 1) << 15 | high keys << 16}.
+// kind 1: v's edges to the mask's vertices are horizontal.  The prefix holds
+// every w of N(v) below K and not above the mask's last vertex, the high keys
+// those from K on.
+// Two launches make them tile by tile: kScatter = false counts every block's
+// entries per tile, kScatter = true writes them at the scanned offsets; a
+// block takes the same rows (a contiguous range) in both.  A warp flattens the keys of 32 rows, one per lane and step;
+// the last of the consecutive lanes of one row and tile makes their entries
+// (a tile that straddles two steps gets entries from both).
+template <bool kScatter>
+__global__ void __launch_bounds__(1024) k_wedge_entries(uint32_t n, uint64_t slots, const uint64_t *__restrict__ rp,
+                                                        const uint32_t *__restrict__ keys,
+                                                        const uint32_t *__restrict__ dcnt,
+                                                        const uint32_t *__restrict__ lcnt,
+                                                        uint32_t *__restrict__ counts,
+                                                        const unsigned long long *__restrict__ offs,
+                                                        unsigned long long *__restrict__ work,
+                                                        uint4 *__restrict__ entries, uint64_t cap, uint32_t tiles_cap,
+                                                        Ctl *ctl) {
+    extern __shared__ uint32_t sm[];  // tiles_cap counts or cursors, then (counting) tiles_cap steps
+    __shared__ uint32_t s_row[2], s_next;
+    const unsigned lane = lane_id();
+    const uint32_t U = ctl->wedge_u;
+    const uint32_t tiles = U >> 5, nb = gridDim.x;
+    if (tiles == 0) return;
+    if (tiles > tiles_cap) {
+        if (threadIdx.x == 0) atomicOr(&ctl->error, kGuardRange);
+        return;
+    }
+    if (threadIdx.x < 2) {  // rows are shared out by slots + rows (a long run of empty rows is spread too)
+        const uint64_t at = (slots + n) * (blockIdx.x + threadIdx.x) / nb;
+        uint32_t lo = 0, hi = n;
+        while (lo < hi) {
+            const uint32_t mid = lo + ((hi - lo) >> 1);
+            if (rp[mid] + mid < at) lo = mid + 1; else hi = mid;
+        }
+        s_row[threadIdx.x] = blockIdx.x + threadIdx.x == nb ? n : lo;
+    }
+    if (threadIdx.x == 0) s_next = 0;
+    for (uint32_t t = threadIdx.x; t < tiles; t += blockDim.x) {
+        sm[t] = kScatter ? (uint32_t)offs[(uint64_t)t * nb + blockIdx.x] : 0u;
+        if (!kScatter) sm[tiles_cap + t] = 0u;
+    }
+    __syncthreads();
+    const uint32_t row_lo = s_row[0], row_hi = s_row[1];
+    unsigned long long probes = 0;
+    for (;;) {
+        uint32_t g = 0;
+        if (lane == 0) g = atomicAdd(&s_next, 32u);
+        g = __shfl_sync(0xFFFFFFFFu, g, 0);
+        if (row_lo + g >= row_hi || g >= row_hi - row_lo) break;
+        const uint32_t x = row_lo + g + lane;
+        uint32_t d = 0, nlo = 0;
+        uint64_t b = 0;
+        if (x < row_hi) {
+            d = dcnt[x];
+            nlo = lcnt[x];
+            if (d < 2) d = 0;
+            else b = rp[x];
+        }
+        uint32_t incl = d;
+#pragma unroll
+        for (int o = 1; o < 32; o <<= 1) {
+            const uint32_t y = __shfl_up_sync(0xFFFFFFFFu, incl, o);
+            if (lane >= (unsigned)o) incl += y;
+        }
+        const uint32_t total = __shfl_sync(0xFFFFFFFFu, incl, 31);
+        for (uint32_t e0 = 0; e0 < total; e0 += 32) {
+            const uint32_t e = e0 + lane;
+            uint32_t r = 0;  // the row of flat position e: the first whose inclusive count passes it
+#pragma unroll
+            for (int o = 16; o > 0; o >>= 1)
+                if (__shfl_sync(0xFFFFFFFFu, incl, r + o - 1) <= e) r += o;
+            r = r > 31u ? 31u : r;
+            const uint32_t dr = __shfl_sync(0xFFFFFFFFu, d, r);
+            const uint32_t pos = e - (__shfl_sync(0xFFFFFFFFu, incl, r) - dr);
+            const uint64_t br = __shfl_sync(0xFFFFFFFFu, b, r);
+            const uint32_t lr = __shfl_sync(0xFFFFFFFFu, nlo, r);
+            uint32_t rank = 0xFFFFFFFFu, kind = 0;
+            if (e < total) {
+                const uint32_t key = keys[br + pos];
+                rank = key >> 1;
+                kind = key & 1u;
+            }
+            const bool in = rank < U;
+            const uint32_t tile = rank >> 5;
+            // segments of consecutive lanes of the same row and tile
+            const uint32_t seg = in ? (tile << 5) | r : 0xFFFFFFFFu;
+            const uint32_t left = __shfl_up_sync(0xFFFFFFFFu, seg, 1);
+            const unsigned heads = __ballot_sync(0xFFFFFFFFu, lane == 0 || left != seg);
+            const int start = 31 - __clz(heads & (0xFFFFFFFFu >> (31u - lane)));
+            uint32_t hor = in && kind ? 1u << (rank & 31u) : 0u, ver = in && !kind ? 1u << (rank & 31u) : 0u;
+#pragma unroll
+            for (int o = 1; o < 32; o <<= 1) {
+                const uint32_t h = __shfl_up_sync(0xFFFFFFFFu, hor, o), v = __shfl_up_sync(0xFFFFFFFFu, ver, o);
+                if ((int)lane - o >= start) {
+                    hor |= h;
+                    ver |= v;
+                }
+            }
+            const bool tail = lane == 31 || ((heads >> (lane + 1)) & 1u);
+            // a first key alone has no earlier one to pair with
+            if (in && tail && pos >= 1) {  // so the prefix or the high keys hold a pair
+                const uint32_t len = pos + 1 < lr ? pos + 1 : lr;
+                uint32_t high = pos + 1 > lr ? pos + 1 - lr : 0u;
+                if (high == 1) high = 0;  // the mask's vertex alone
+                const uint32_t parts = (hor != 0) + (ver != 0);
+                if constexpr (kScatter) {
+                    const uint32_t at = atomicAdd(&sm[tile], parts);
+                    const uint32_t id8 = (uint32_t)((br + 1) >> 1), units = (len + 3) / 4;
+                    const uint32_t place = lr | (uint32_t)(br & 1u) << 15 | high << 16;
+                    if ((uint64_t)at + parts > cap) {
+                        atomicOr(&ctl->error, kGuardRange);
+                    } else {
+                        if (hor) entries[at] = make_uint4(id8, hor, units | 0x80000000u, place);
+                        if (ver) entries[at + (hor != 0)] = make_uint4(id8, ver, units, place);
+                    }
+                } else {
+                    atomicAdd(&sm[tile], parts);
+                    atomicAdd(&sm[tiles_cap + tile], parts * ((len + 31) / 32 + (high + 15) / 16));
+                    probes += (unsigned long long)parts * (len + high);
+                }
+            }
+        }
+    }
+    if constexpr (!kScatter) {
+        probes = warp_sum(probes);
+        if (lane == 0 && probes) {
+            atomicAdd(&ctl->probes, probes);
+            atomicAdd(&ctl->cls_probes[1], probes);
+        }
+        __syncthreads();
+        for (uint32_t t = threadIdx.x; t < tiles; t += blockDim.x) {
+            counts[(uint64_t)t * nb + blockIdx.x] = sm[t];
+            if (sm[tiles_cap + t]) atomicAdd(&work[t], (unsigned long long)sm[tiles_cap + t]);
+        }
+    }
+}
+
+// Tile tasks: equal slices of a tile's entries, of about the same number of
+// steps everywhere (one block; at most task_cap of them).
+__global__ void __launch_bounds__(1024) k_wedge_plan(const unsigned long long *__restrict__ offs, uint32_t nb,
+                                                     const unsigned long long *__restrict__ work, uint32_t num_sms,
+                                                     uint4 *__restrict__ tasks, uint32_t task_cap, Ctl *ctl) {
+    __shared__ unsigned long long s_sum[32];
+    __shared__ unsigned int s_warp[32], s_base;
+    const unsigned lane = lane_id(), warp = threadIdx.x >> 5;
+    const uint32_t tiles = ctl->wedge_u >> 5;
+    if (tiles == 0) return;
+    unsigned long long sum = 0;
+    for (uint32_t t = threadIdx.x; t < tiles; t += blockDim.x) sum += work[t];
+    sum = warp_sum(sum);
+    if (lane == 0) s_sum[warp] = sum;
+    if (threadIdx.x == 0) s_base = 0;
+    __syncthreads();
+    sum = warp_sum(s_sum[lane]);
+    unsigned long long target = sum / ((unsigned long long)num_sms * kTasksPerSm) + 1;
+    if (target < kTaskSteps) target = kTaskSteps;
+    for (uint32_t t0 = 0; t0 < tiles; t0 += blockDim.x) {
+        const uint32_t t = t0 + threadIdx.x;
+        unsigned long long lo = 0, ent = 0, nt = 0;
+        if (t < tiles) {
+            lo = offs[(uint64_t)t * nb];
+            ent = offs[(uint64_t)(t + 1) * nb] - lo;
+            nt = (work[t] + target - 1) / target;
+            if (nt > ent) nt = ent;
+        }
+        uint32_t incl = (uint32_t)nt;
+#pragma unroll
+        for (int o = 1; o < 32; o <<= 1) {
+            const uint32_t y = __shfl_up_sync(0xFFFFFFFFu, incl, o);
+            if (lane >= (unsigned)o) incl += y;
+        }
+        if (lane == 31) s_warp[warp] = incl;
+        __syncthreads();
+        uint32_t before = s_base + incl - (uint32_t)nt;
+        for (unsigned w = 0; w < warp; ++w) before += s_warp[w];
+        if (t == kWedgeMaxK / 32) ctl->wedge_hi_task = before;
+        for (uint32_t i = 0; i < (uint32_t)nt; ++i) {
+            if (before + i >= task_cap) {
+                atomicOr(&ctl->error, kGuardRange);
+                break;
+            }
+            tasks[before + i] = make_uint4(t, (uint32_t)(lo + ent * i / nt), (uint32_t)(lo + ent * (i + 1) / nt), 0u);
+        }
+        __syncthreads();
+        if (threadIdx.x == blockDim.x - 1) s_base = before + (uint32_t)nt;
+        __syncthreads();
+    }
+    if (threadIdx.x == 0) {
+        ctl->n_tasks[1] = s_base;
+        ctl->cls_rows[1] = s_base;
+        ctl->cls_build[1] = offs[(uint64_t)tiles * nb];  // entries
+    }
+}
+
+// ---------------------------------------------------------------------------- tiles
+
+constexpr uint32_t kTileThreads = 1024;
+constexpr uint32_t kTileWords = 32768;
+constexpr size_t kTileSmem = 4ull * kTileWords + (kTileThreads / 32) * 32 * sizeof(uint4);
+
+__device__ __forceinline__ uint32_t lds(uint32_t addr) {
+    uint32_t v;
+    asm volatile("ld.shared.u32 %0, [%1];" : "=r"(v) : "r"(addr));
+    return v;
+}
+
+// The 32 entries a warp holds and the steps (`per` units each) of its walk: the
+// steps of all entries are shared out evenly over the warp's eight groups of
+// four lanes, so short and long rows keep every lane busy.
+struct Walk {
+    uint32_t i, left, iters;  // the group's entry, its steps, the steps of the longest group
+    uint32_t skip;            // steps of entry i that belong to the groups before
+};
+__device__ __forceinline__ Walk share_steps(uint32_t steps) {
+    const unsigned lane = lane_id();
+    uint32_t incl = steps;
+#pragma unroll
+    for (int o = 1; o < 32; o <<= 1) {
+        const uint32_t y = __shfl_up_sync(0xFFFFFFFFu, incl, o);
+        if (lane >= (unsigned)o) incl += y;
+    }
+    const uint32_t total = __shfl_sync(0xFFFFFFFFu, incl, 31);
+    Walk w;
+    w.iters = (total + 7) / 8;
+    const uint32_t c = min((lane >> 2) * w.iters, total);
+    w.left = min(w.iters, total - c);
+    w.i = 0;  // the entry of step c: the first whose inclusive count passes it
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1)
+        if (__shfl_sync(0xFFFFFFFFu, incl, w.i + o - 1) <= c) w.i += o;
+    w.skip = c - __shfl_sync(0xFFFFFFFFu, incl - steps, w.i);
+    return w;
+}
+
+__device__ __forceinline__ uint4 next_tile_task(Ctl *ctl, int counter, uint32_t first, uint32_t n_tasks,
+                                                const uint4 *__restrict__ tasks, uint4 *s_task, long long t_start) {
+    __syncthreads();
+    if (threadIdx.x == 0) {
+        const uint32_t k = first + atomicAdd(&ctl->task_next[counter], 1u);
+        uint4 t = make_uint4(0xFFFFFFFFu, 0, 0, 0);
+        if (clock64() - t_start > kWatchdogCycles) atomicOr(&ctl->error, kGuardWatchdog);
+        else if (k < n_tasks) t = tasks[k];
+        *s_task = t;
+    }
+    __syncthreads();
+    return *s_task;
+}
+
+// One block per SM; a task is a slice of one tile's entries.  Each warp takes
+// 32 entries at a time, four lanes walk a row's prefix 32 ids (64 bytes) a
+// step; the next step's ids are loaded before the current ones are looked up.
+// Units past the prefix are kPadId; ids of the prefix's last unit past the
+// mask's last vertex read words that are 0.  Bound by issue and by the bank
+// conflicts of the lookups (3.6 wavefronts per 32).
+__global__ void __launch_bounds__(kTileThreads, 1) k_wedge_tiles(uint32_t n, const uint4 *__restrict__ tasks,
+                                                                 const uint4 *__restrict__ entries,
+                                                                 const uint16_t *__restrict__ ids,
+                                                                 const uint4 *__restrict__ rmeta, Ctl *ctl) {
+    extern __shared__ __align__(16) uint32_t word[];
+    __shared__ uint4 s_task;
+    const unsigned lane = lane_id(), warp = threadIdx.x >> 5;
+    const uint32_t sub = lane & 3u;
+    uint4 *ent = reinterpret_cast<uint4 *>(word + kTileWords) + warp * 32;
+    const uint32_t wbase = (uint32_t)__cvta_generic_to_shared(word);
+    const uint32_t n_tasks = (uint32_t)ctl->n_tasks[1];
+    const uint2 *id8 = reinterpret_cast<const uint2 *>(ids);
+    unsigned long long same = 0, cross = 0, inserts = 0;
+    uint32_t tile = 0xFFFFFFFFu;
+    const long long t_start = clock64();
+    for (uint32_t i = threadIdx.x; i < kTileWords / 4; i += kTileThreads)
+        reinterpret_cast<uint4 *>(word)[i] = make_uint4(0, 0, 0, 0);
+    uint32_t dirty = 0;  // words [0, dirty) may be set
+    for (;;) {
+        const uint4 task = next_tile_task(ctl, 1, 0, n_tasks, tasks, &s_task, t_start);
+        if (task.x == 0xFFFFFFFFu) break;
+        if (task.x != tile) {
+            tile = task.x;
+            for (uint32_t i = threadIdx.x; i < dirty / 4; i += kTileThreads)
+                reinterpret_cast<uint4 *>(word)[i] = make_uint4(0, 0, 0, 0);
+            dirty = 32 * (tile + 1) < kTileWords ? 32 * (tile + 1) : kTileWords;
+            __syncthreads();
+            const uint32_t u = 32 * tile + warp;  // one row per warp
+            if (u < n) {
+                const uint4 m = rmeta[u];
+                const uint16_t *id = ids + 4 * (((((uint64_t)m.y << 32) | m.x) + 1) >> 1);
+                for (uint32_t i = lane; i < m.w; i += 32) atomicOr(&word[id[i] >> 1], 1u << warp);
+                if (lane == 0) inserts += m.w;
+            }
+            __syncthreads();
+        }
+        uint32_t tot = 0, sam = 0;
+        for (uint32_t base = task.y + warp * 32; base < task.z; base += kTileThreads) {
+            uint4 en = make_uint4(0, 0, 0, 0);
+            if (base + lane < task.z) en = entries[base + lane];
+            __syncwarp();
+            ent[lane] = en;
+            __syncwarp();
+            Walk w = share_steps(((en.z & 0x7FFFFFFFu) + 7) >> 3);
+            uint4 cur = ent[w.i];
+            uint32_t at = cur.x + sub + 8 * w.skip;                            // this lane's first unit
+            int rem = (int)(cur.z & 0x7FFFFFFFu) - (int)(8 * w.skip + sub);    // units from there on
+            const uint2 pad = make_uint2(0xFFFFFFFFu, 0xFFFFFFFFu);
+            uint2 a = pad, b = pad, a1, b1;
+            uint32_t mv = 0, kl = 0, mv1, kl1;
+            auto fetch = [&](uint2 &x, uint2 &y, uint32_t &mm, uint32_t &kk) {
+                x = pad;
+                y = pad;
+                if (w.left) {
+                    --w.left;
+                    while (rem + (int)sub <= 0) {  // entries may have no units (high keys only)
+                        w.i = (w.i + 1) & 31u;
+                        cur = ent[w.i];
+                        at = cur.x + sub;
+                        rem = (int)(cur.z & 0x7FFFFFFFu) - (int)sub;
+                    }
+                    if (rem > 0) x = __ldg(id8 + at);
+                    if (rem > 4) y = __ldg(id8 + at + 4);
+                    at += 8;
+                    rem -= 8;
+                }
+                mm = cur.y;
+                kk = cur.z >> 31;
+            };
+            auto look = [&](uint32_t x, uint32_t mm, uint32_t kk) {
+                const uint32_t w0 = lds(wbase + ((x << 1) & 0x1FFFCu)), w1 = lds(wbase + ((x >> 15) & 0x1FFFCu));
+                const uint32_t p0 = __popc(w0 & mm), p1 = __popc(w1 & mm);
+                tot += p0 + p1;
+                if (x & kk) sam += p0;
+                if (x & (kk << 16)) sam += p1;
+            };
+            fetch(a, b, mv, kl);
+            for (uint32_t k = 0; k < w.iters; ++k) {
+                fetch(a1, b1, mv1, kl1);
+                look(a.x, mv, kl);
+                look(a.y, mv, kl);
+                look(b.x, mv, kl);
+                look(b.y, mv, kl);
+                a = a1;
+                b = b1;
+                mv = mv1;
+                kl = kl1;
+            }
+        }
+        same += sam;
+        cross += tot - sam;
+    }
+    same = warp_sum(same);
+    cross = warp_sum(cross);
+    inserts = warp_sum(inserts);
+    if (lane == 0) {
+        if (same) atomicAdd(&ctl->t_same, same);
+        if (cross) atomicAdd(&ctl->t_cross, cross);
+        if (inserts) atomicAdd(&ctl->cls_inserts[1], inserts);
+    }
+}
+
+// The high keys (w >= K) of the tiles from rank K on, where a tile's vertices
+// have few of them: the tile's words sit in a hash table (linear probing,
+// 8192 slots of {rank, word}, at most about half full; a tile with more high
+// keys is taken in several rounds, each with the keys of one hash class), and
+// four lanes walk the high keys of an entry's row 16 a step.
+constexpr uint32_t kHighThreads = 512;
+constexpr uint32_t kHighSlots = 8192, kHighShift = 19, kHighKeys = 4096;
+constexpr size_t kHighSmem = 8ull * kHighSlots + (kHighThreads / 32) * 32 * sizeof(uint4);
+constexpr unsigned kGuardInsert = 0x10u;
+
+__global__ void __launch_bounds__(kHighThreads, 3) k_wedge_high(uint32_t n, const uint4 *__restrict__ tasks,
+                                                                const uint4 *__restrict__ entries,
+                                                                const uint32_t *__restrict__ keys,
+                                                                const uint4 *__restrict__ rmeta, Ctl *ctl) {
+    extern __shared__ __align__(16) uint32_t word[];
+    uint2 *table = reinterpret_cast<uint2 *>(word);
+    __shared__ uint4 s_task;
+    __shared__ uint32_t s_items;
+    const unsigned lane = lane_id(), warp = threadIdx.x >> 5;
+    const uint32_t sub = lane & 3u;
+    uint4 *ent = reinterpret_cast<uint4 *>(word + 2 * kHighSlots) + warp * 32;
+    const uint32_t n_tasks = (uint32_t)ctl->n_tasks[1];
+    if (ctl->wedge_u <= kWedgeMaxK) return;
+    const uint32_t first_task = ctl->wedge_hi_task;
+    unsigned long long same = 0, cross = 0, inserts = 0;
+    uint32_t tile = 0xFFFFFFFFu, rounds = 1;
+    const long long t_start = clock64();
+    for (;;) {
+        const uint4 task = next_tile_task(ctl, 2, first_task, n_tasks, tasks, &s_task, t_start);
+        if (task.x == 0xFFFFFFFFu) break;
+        const bool fresh = task.x != tile || rounds > 1;
+        if (fresh) {
+            tile = task.x;
+            if (threadIdx.x == 0) s_items = 0;
+            __syncthreads();
+            if (threadIdx.x < 32 && 32 * tile + lane < n) {
+                const uint4 m = rmeta[32 * tile + lane];
+                if (m.z > m.w) atomicAdd(&s_items, m.z - m.w);
+            }
+            __syncthreads();
+            rounds = (s_items + kHighKeys - 1) / kHighKeys;
+            if (threadIdx.x == 0) inserts += s_items;
+        }
+        for (uint32_t round = 0; round < rounds; ++round) {
+            if (fresh) {
+                for (uint32_t i = threadIdx.x; i < kHighSlots; i += kHighThreads) table[i] = make_uint2(kEmpty, 0u);
+                __syncthreads();
+                for (uint32_t r = warp; r < 32; r += kHighThreads / 32) {
+                    if (32 * tile + r >= n) break;
+                    const uint4 m = rmeta[32 * tile + r];
+                    const uint32_t *nu = keys + (((uint64_t)m.y << 32) | m.x);
+                    for (uint32_t p = m.w + lane; p < m.z; p += 32) {
+                        const uint32_t w = nu[p] >> 1, h = w * 0x9E3779B1u;
+                        if (rounds > 1 && (h & 0xFFFFu) % rounds != round) continue;
+                        uint32_t s = h >> kHighShift, tries = 0;
+                        for (; tries < kHighSlots; ++tries) {
+                            const uint32_t old = atomicCAS(&table[s].x, kEmpty, w);
+                            if (old == kEmpty || old == w) {
+                                atomicOr(&table[s].y, 1u << r);
+                                break;
+                            }
+                            s = (s + 1) & (kHighSlots - 1);
+                        }
+                        if (tries == kHighSlots) atomicOr(&ctl->error, kGuardInsert);
+                    }
+                }
+                __syncthreads();
+            }
+            uint32_t tot = 0, sam = 0;
+            for (uint32_t base = task.y + warp * 32; base < task.z; base += kHighThreads) {
+                uint4 en = make_uint4(0, 0, 0, 0);
+                if (base + lane < task.z) en = entries[base + lane];
+                __syncwarp();
+                ent[lane] = en;
+                __syncwarp();
+                Walk w = share_steps(((en.w >> 16) + 15) >> 4);
+                while (w.left) {  // entries without high keys have no steps
+                    const uint4 cur = ent[w.i];
+                    const uint32_t cnt = cur.w >> 16;
+                    if (16 * w.skip >= cnt) {
+                        w.i = (w.i + 1) & 31u;
+                        w.skip = 0;
+                        continue;
+                    }
+                    --w.left;
+                    const uint32_t *row = keys + (2 * (uint64_t)cur.x - ((cur.w >> 15) & 1u) + (cur.w & 0x7FFFu));
+                    uint32_t key[4];
+#pragma unroll
+                    for (int t = 0; t < 4; ++t) {
+                        const uint32_t p = 16 * w.skip + sub + 4 * t;
+                        key[t] = p < cnt ? __ldg(row + p) : 0u;  // rank 0 is below K: never in the table
+                    }
+                    ++w.skip;
+#pragma unroll
+                    for (int t = 0; t < 4; ++t) {
+                        const uint32_t r = key[t] >> 1;
+                        uint32_t s = (r * 0x9E3779B1u) >> kHighShift;
+                        uint2 e = table[s];
+                        for (uint32_t tries = 0; e.x != r && e.x != kEmpty && tries < kHighSlots; ++tries) {
+                            s = (s + 1) & (kHighSlots - 1);
+                            e = table[s];
+                        }
+                        if (e.x == r) {
+                            const uint32_t p = __popc(e.y & cur.y);
+                            tot += p;
+                            if (key[t] & (cur.z >> 31)) sam += p;
+                        }
+                    }
+                }
+                __syncwarp();
+            }
+            same += sam;
+            cross += tot - sam;
+            if (rounds > 1) __syncthreads();  // the table is cleared next
+        }
+    }
+    same = warp_sum(same);
+    cross = warp_sum(cross);
+    inserts = warp_sum(inserts);
+    if (lane == 0) {
+        if (same) atomicAdd(&ctl->t_same, same);
+        if (cross) atomicAdd(&ctl->t_cross, cross);
+        if (inserts) atomicAdd(&ctl->cls_inserts[1], inserts);
+    }
+}
+
+// ---------------------------------------------------------------------------- the other pairs
+
+constexpr int kRestThreads = 256;
+constexpr uint32_t kRestTiny = 8;           // rows of up to this many keys: one lane each
+constexpr uint32_t kFilterBits = 1u << 14;  // per warp
+
+// Position of `rank` among the ascending keys a[lo..hi): the key's value, or kEmpty.
+__device__ __forceinline__ uint32_t find_key(const uint32_t *__restrict__ a, uint32_t lo, uint32_t hi, uint32_t rank) {
+    while (lo < hi) {
+        const uint32_t mid = (lo + hi) >> 1, k = a[mid];
+        if ((k >> 1) == rank) return k;
+        if ((k >> 1) < rank) lo = mid + 1; else hi = mid;
+    }
+    return kEmpty;
+}
+
+// The pairs w < u of N(v) with u >= U, which no tile takes.  A row of at most
+// kRestTiny keys: one lane tries its pairs, each by a search of w in N(u).  A
+// longer one: its warp sets a filter bit per key of N(v), eight lanes a time
+// walk N(u) and search N(v) for the keys that pass the filter.
+__global__ void __launch_bounds__(kRestThreads) k_wedge_rest(uint32_t n, const uint64_t *__restrict__ rp,
+                                                             const uint32_t *__restrict__ keys,
+                                                             const uint32_t *__restrict__ dcnt,
+                                                             const uint32_t *__restrict__ ucnt,
+                                                             const uint4 *__restrict__ rmeta, Ctl *ctl) {
+    __shared__ uint32_t sfilter[kRestThreads / 32][kFilterBits / 32];
+    const unsigned lane = lane_id(), warp = threadIdx.x >> 5;
+    const uint32_t sub = lane & 7u, group = lane >> 3;
+    uint32_t *filter = sfilter[warp];
+    for (uint32_t i = lane; i < kFilterBits / 32; i += 32) filter[i] = 0;
+    __syncwarp();
+    unsigned long long same = 0, cross = 0, probes = 0;
+    uint32_t done = 0;
+    const uint64_t chunks = ((uint64_t)n + 31) / 32;
+    const long long t_start = clock64();
+    for (;;) {
+        unsigned int c = 0;
+        if (lane == 0) {
+            c = atomicAdd(&ctl->task_next[0], 1u);
+            if (clock64() - t_start > kWatchdogCycles) {
+                atomicOr(&ctl->error, kGuardWatchdog);
+                c = 0xFFFFFFFFu;
+            }
+        }
+        c = __shfl_sync(0xFFFFFFFFu, c, 0);
+        if (c >= chunks) break;
+        const uint64_t x = (uint64_t)c * 32 + lane;
+        uint32_t d = 0, nu = 0;  // keys, and those below U
+        uint64_t b = 0;
+        if (x < n) {
+            d = dcnt[x];
+            nu = ucnt[x];
+            if (d < 2 || d == nu) d = 0;
+            else b = rp[x];
+        }
+        if (d && d <= kRestTiny) {
+            const uint32_t *row = keys + b;
+            for (uint32_t j = nu > 1 ? nu : 1; j < d; ++j) {
+                const uint32_t ku = row[j];
+                const uint4 m = rmeta[ku >> 1];
+                if (m.z == 0) continue;
+                const uint32_t *nb = keys + (((uint64_t)m.y << 32) | m.x);
+                for (uint32_t i = 0; i < j; ++i) {
+                    const uint32_t kw = row[i];
+                    if (find_key(nb, 0, m.z, kw >> 1) != kEmpty) {
+                        if (ku & kw & 1u) ++same; else ++cross;
+                    }
+                }
+                probes += j;
+            }
+            ++done;
+        }
+        unsigned pending = __ballot_sync(0xFFFFFFFFu, d > kRestTiny);
+        while (pending) {
+            const int src = __ffs(pending) - 1;
+            pending &= pending - 1;
+            const uint32_t vd = __shfl_sync(0xFFFFFFFFu, d, src), vu = __shfl_sync(0xFFFFFFFFu, nu, src);
+            const uint64_t vb = __shfl_sync(0xFFFFFFFFu, b, src);
+            const uint32_t *row = keys + vb;
+            for (uint32_t i = lane; i < vd; i += 32) {
+                const uint32_t h = (row[i] >> 1) & (kFilterBits - 1);
+                atomicOr(&filter[h >> 5], 1u << (h & 31u));
+            }
+            __syncwarp();
+            for (uint32_t j = (vu > 1 ? vu : 1) + group; j < vd; j += 4) {
+                const uint32_t ku = row[j];
+                const uint4 m = rmeta[ku >> 1];
+                const uint32_t *nb = keys + (((uint64_t)m.y << 32) | m.x);
+                if (sub == 0) probes += m.z;
+                for (uint32_t p = sub; p < m.z; p += 32) {
+                    uint32_t w[4];
+#pragma unroll
+                    for (int t = 0; t < 4; ++t) w[t] = p + 8 * t < m.z ? nb[p + 8 * t] >> 1 : kEmpty;
+#pragma unroll
+                    for (int t = 0; t < 4; ++t) {
+                        const uint32_t h = w[t] & (kFilterBits - 1);
+                        if (w[t] != kEmpty && ((filter[h >> 5] >> (h & 31u)) & 1u)) {
+                            const uint32_t kw = find_key(row, 0, j, w[t]);
+                            if (kw != kEmpty) {
+                                if (ku & kw & 1u) ++same; else ++cross;
+                            }
+                        }
+                    }
+                }
+            }
+            __syncwarp();
+            for (uint32_t i = lane; i < vd; i += 32) filter[((row[i] >> 1) & (kFilterBits - 1)) >> 5] = 0;
+            __syncwarp();
+            if (lane == 0) ++done;
+        }
+    }
+    same = warp_sum(same);
+    cross = warp_sum(cross);
+    probes = warp_sum(probes);
+    const unsigned long long rows = warp_sum((unsigned long long)done);
+    if (lane == 0) {
+        if (same) atomicAdd(&ctl->t_same, same);
+        if (cross) atomicAdd(&ctl->t_cross, cross);
+        if (probes) {
+            atomicAdd(&ctl->probes, probes);
+            atomicAdd(&ctl->cls_probes[0], probes);
+        }
+        if (rows) atomicAdd(&ctl->cls_rows[0], rows);
+    }
+}
+
+unsigned grid_for(uint64_t work, unsigned threads, unsigned cap) {
+    uint64_t b = (work + threads - 1) / threads;
+    if (b < 1) b = 1;
+    if (b > cap) b = cap;
+    return (unsigned)b;
+}
+
+uint32_t tiles_cap(uint32_t n) { return std::min(kWedgeMaxU, n) / 32 + 1; }
+
+// Blocks of the entry kernels: a row range each.
+uint32_t entry_blocks(const tc_ctx *ctx, uint64_t slots) {
+    return (uint32_t)std::min<uint64_t>(2ull * ctx->num_sms, slots / 4096 + 1);
+}
+
+uint32_t tasks_cap(const tc_ctx *ctx, uint32_t n) { return tiles_cap(n) + (uint32_t)ctx->num_sms * kTasksPerSm + 1; }
+
+}  // namespace
+
+WedgeSizes wedge_sizes(const tc_ctx *ctx, uint32_t n, uint64_t slots) {
+    WedgeSizes z;
+    z.tiles = tiles_cap(n);
+    z.counts = (uint64_t)z.tiles * entry_blocks(ctx, slots);
+    z.tasks = tasks_cap(ctx, n);
+    z.tmp = scan_tmp_elems(z.counts + 1);
+    return z;
+}
+
+bool wedge_path(const tc_ctx *ctx, uint32_t n, uint64_t slots, uint32_t max_deg) {
+    const Tuning &t = ctx->tune, def;
+    // the class knobs choose among the kernels of isect.cu: any of them set away from its default means these
+    const bool classes = t.warp_cap != def.warp_cap || t.block_cap != def.block_cap || t.tiny_cap != def.tiny_cap ||
+                         t.table_kind != def.table_kind || t.flat_cap != def.flat_cap ||
+                         t.block_bits_log2 != def.block_bits_log2;
+    return !classes && ctx->opt.order == TC_ORDER_DEGREE && ctx->nshards == 1 && max_deg > 0 && n < (1u << 31) &&
+           slots <= (uint64_t)kSortCap * kSortCap;
+}
+
+tc_status wedge_rows(tc_ctx *ctx, const PipeBufs &b, uint32_t n, uint32_t max_deg) {
+    cudaStream_t s = ctx->stream;
+    const unsigned cap = (unsigned)ctx->num_sms * 16u;
+    uint16_t *ids = b.wedge_ids;
+    uint32_t launches = 2;
+    const RowOut out{b.fcnt, b.gcnt, b.glo, b.vmeta};
+    // warps of small graphs take fewer vertices each, so that long rows spread over the GPU
+    const uint32_t per_warp = n >= (1u << 20) ? 32u : n >= (1u << 18) ? 16u : 8u;
+    k_wedge_limits<<<1, 1, 0, s>>>(n, b.order, max_deg, ctx->d_ctl);
+    auto rows = b.lvp ? k_wedge_rows<true> : k_wedge_rows<false>;
+    rows<<<grid_for((uint64_t)n * (32 / per_warp), kFillThreads, cap), kFillThreads, 0, s>>>(
+        n, b.rp, b.col, b.lv, b.lvp, b.adj2, ids, out, b.big, b.huge, per_warp, ctx->d_ctl);
+    if (max_deg > kHugeRow) {
+        auto huge = b.lvp ? k_wedge_rows_huge<true> : k_wedge_rows_huge<false>;
+        huge<<<(unsigned)ctx->num_sms, 1024, 0, s>>>(b.huge, ctx->d_ctl, b.rp, b.col, b.lv, b.lvp, b.adj2, b.fcnt,
+                                                     b.big);
+        ++launches;
+    }
+    if (max_deg > kWarpKeys) {
+        auto sort = b.lvp ? k_wedge_sort<true> : k_wedge_sort<false>;
+        const int smem = (int)(4 * kSortCap);
+        TC_CUDA(ctx, cudaFuncSetAttribute(sort, cudaFuncAttributeMaxDynamicSharedMemorySize, smem));
+        sort<<<(unsigned)ctx->num_sms, 1024, smem, s>>>(b.big, ctx->d_ctl, b.rp, b.lv, b.lvp, b.adj2, ids, out);
+        ++launches;
+    }
+    if (max_deg >= kWedgeTileDegree) {
+        const uint32_t nb = entry_blocks(ctx, b.slots), tiles = tiles_cap(n);
+        const uint64_t cells = (uint64_t)tiles * nb;
+        TC_CUDA(ctx, cudaMemsetAsync(b.wedge_counts, 0, 4 * cells, s));
+        TC_CUDA(ctx, cudaMemsetAsync(b.wedge_work, 0, 8ull * tiles, s));
+        const int smem = (int)(8 * tiles);
+        TC_CUDA(ctx, cudaFuncSetAttribute(k_wedge_entries<false>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem));
+        TC_CUDA(ctx, cudaFuncSetAttribute(k_wedge_entries<true>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem));
+        auto *offs = reinterpret_cast<unsigned long long *>(b.wedge_offs);
+        k_wedge_entries<false><<<nb, 1024, smem, s>>>(n, b.slots, b.rp, b.adj2, b.fcnt, b.gcnt, b.wedge_counts, offs,
+                                                      b.wedge_work, b.erec, b.erec_cap, tiles, ctx->d_ctl);
+        launches += 3 + scan_u32_to_u64(b.wedge_counts, b.wedge_offs, cells, b.wedge_tmp, s);
+        k_wedge_entries<true><<<nb, 1024, smem, s>>>(n, b.slots, b.rp, b.adj2, b.fcnt, b.gcnt, b.wedge_counts, offs,
+                                                     b.wedge_work, b.erec, b.erec_cap, tiles, ctx->d_ctl);
+        k_wedge_plan<<<1, 1024, 0, s>>>(offs, nb, b.wedge_work, (uint32_t)ctx->num_sms, b.wedge_tasks,
+                                        tasks_cap(ctx, n), ctx->d_ctl);
+    }
+    note_launch(ctx, launches);
+    TC_CUDA(ctx, cudaGetLastError());
+    return TC_OK;
+}
+
+tc_status wedge_count(tc_ctx *ctx, const PipeBufs &b, uint32_t n, uint32_t max_deg) {
+    cudaStream_t s = ctx->stream;
+    const bool tiles = max_deg >= kWedgeTileDegree;
+    TC_CUDA(ctx, cudaEventRecord(ctx->ev[4], s));
+    int per_sm = 0;
+    TC_CUDA(ctx, cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k_wedge_rest, kRestThreads, 0));
+    const uint64_t blocks = ((uint64_t)n + 32 * (kRestThreads / 32) - 1) / (32 * (kRestThreads / 32));
+    const uint64_t resident = (uint64_t)ctx->num_sms * std::max(per_sm, 1);
+    k_wedge_rest<<<(unsigned)std::min(blocks, resident), kRestThreads, 0, s>>>(n, b.rp, b.adj2, b.fcnt, b.glo,
+                                                                               b.vmeta, ctx->d_ctl);
+    TC_CUDA(ctx, cudaEventRecord(ctx->ev[5], s));
+    if (tiles) {
+        TC_CUDA(ctx, cudaFuncSetAttribute(k_wedge_tiles, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kTileSmem));
+        k_wedge_tiles<<<(unsigned)ctx->num_sms, kTileThreads, kTileSmem, s>>>(n, b.wedge_tasks, b.erec, b.wedge_ids,
+                                                                             b.vmeta, ctx->d_ctl);
+        if (n > kWedgeMaxK) {
+            TC_CUDA(ctx, cudaFuncSetAttribute(k_wedge_high, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kHighSmem));
+            k_wedge_high<<<(unsigned)ctx->num_sms * 3u, kHighThreads, kHighSmem, s>>>(n, b.wedge_tasks, b.erec, b.adj2,
+                                                                                     b.vmeta, ctx->d_ctl);
+            note_launch(ctx);
+        }
+    }
+    TC_CUDA(ctx, cudaEventRecord(ctx->ev[6], s));
+    ctx->isect_flags = tiles ? 3u : 1u;
+    note_launch(ctx, tiles ? 2 : 1);
+    TC_CUDA(ctx, cudaGetLastError());
+    return TC_OK;
+}
+
+}  // namespace tc
