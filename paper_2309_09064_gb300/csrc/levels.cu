@@ -12,7 +12,10 @@
 //      multi-source BFS from those roots levels them.
 // BFS distances are unique given the roots, so L matches the serial
 // algorithm exactly whatever the thread schedule.
+#include <cooperative_groups.h>
+
 #include <algorithm>
+#include <type_traits>
 
 #include "pipeline.cuh"
 
@@ -66,21 +69,6 @@ __global__ void k_init(uint32_t n, const uint64_t *__restrict__ rp, uint32_t *__
             atomicAdd(&ctl->components, s_iso);
         }
     }
-}
-
-// Seed the BFS with the globally first non-isolated vertex (if any).
-__global__ void k_seed(const uint32_t *__restrict__ deg, uint32_t *__restrict__ L, uint32_t *__restrict__ q,
-                       Ctl *ctl, int cur) {
-    unsigned long long key = ctl->root_key;
-    if (key == ~0ull) return;
-    uint32_t r = (uint32_t)(key & 0xFFFFFFFFull);
-    L[r] = 0;
-    q[0] = r;
-    ctl->fr_count[cur] = 1;
-    ctl->fr_edges[cur] = deg[r];
-    ctl->visited += 1;
-    ctl->visited_edges += deg[r];
-    ctl->components += 1;
 }
 
 __global__ void k_gather_deg(const uint32_t *__restrict__ q, uint32_t count, const uint32_t *__restrict__ deg,
@@ -287,7 +275,7 @@ __global__ void k_count_roots(Ctl *ctl, int cur) {
 __global__ void k_reset_next(Ctl *ctl, int nxt) {
     ctl->fr_count[nxt] = 0;
     ctl->fr_edges[nxt] = 0;
-    ctl->bar_count = 0;  // a persistent launch may follow: its barriers count from zero
+    ctl->bfs_spill = 0;
 }
 
 __global__ void k_after_level(Ctl *ctl, int nxt, uint32_t level) {
@@ -296,13 +284,12 @@ __global__ void k_after_level(Ctl *ctl, int nxt, uint32_t level) {
     if (ctl->fr_count[nxt]) ctl->max_level = level + 1 > ctl->max_level ? level + 1 : ctl->max_level;
 }
 
-// Grid-wide barrier for the persistent BFS (all blocks are co-resident: the
-// kernel is launched cooperatively).  The arrival counter only grows within
-// a launch (the host zeroes it before each launch): barrier k of the launch
-// is passed once the counter reaches (k + 1) x nblocks, so an arriving block
-// adds one and waits for that count, with no generation word to reset.  A
-// wait gives up after `timeout_cycles` of clock time, raises the error flag
-// and returns false, so the kernel ends and the host reads TC_ERR_TIMEOUT.
+// Grid-wide barrier with a bounded wait (all blocks are co-resident: the
+// kernel is launched cooperatively); tc_selftest_barrier drives it.  Barrier k
+// of a launch is passed once the arrival counter, zero before the launch,
+// reaches (k + 1) x nblocks.  A wait gives up after `timeout_cycles` of clock
+// time, raises the error flag and returns false, so the kernel ends and the
+// host reads TC_ERR_TIMEOUT.
 __device__ __forceinline__ bool grid_barrier(Ctl *ctl, unsigned nblocks, unsigned k, long long timeout_cycles) {
     __shared__ int s_ok;
     __syncthreads();
@@ -328,130 +315,359 @@ __device__ __forceinline__ bool grid_barrier(Ctl *ctl, unsigned nblocks, unsigne
     return s_ok != 0;
 }
 
-// Persistent top-down BFS for small frontiers (high-diameter graphs): one
-// launch runs level after level, one grid barrier per level, until the
-// frontier is empty or leaves [min_f, max_f] x [0, max_e], or its mean
-// degree passes max_avg (a high-degree vertex would hold up the one warp
-// that expands it; the edge-balanced kernel spreads it over the GPU); then
-// the host takes over again.  A frontier vertex of degree <= 32 is expanded
-// by a group of G lanes (G = the threads the grid has per frontier vertex,
-// a power of two up to 32; one thread when the frontier is large); larger
-// rows by the whole warp, one at a time.  Counter slots rotate mod 3 (level L reads
-// slot s, writes s+1, and s+2 is cleared for level L+1); queues alternate.
-__global__ void __launch_bounds__(512) k_bfs_persist(uint32_t *__restrict__ q0, uint32_t *__restrict__ q1,
-                                                     const uint64_t *__restrict__ rp,
-                                                     const uint32_t *__restrict__ col,
-                                                     const uint32_t *__restrict__ deg, uint32_t *L, Ctl *ctl,
-                                                     uint32_t slot, uint32_t queue, uint32_t level, uint32_t max_f,
-                                                     unsigned long long max_e, uint32_t min_f, uint32_t max_avg) {
-    const unsigned lane = lane_id();
-    const unsigned gwarp = (blockIdx.x * blockDim.x + threadIdx.x) >> 5;
-    const unsigned nwarps = (gridDim.x * blockDim.x) >> 5;
-    volatile unsigned *vcount = ctl->fr_count;
-    volatile unsigned long long *vedges = ctl->fr_edges;
-    // levels this launch adds (written once at the end by block 0, thread 0)
-    unsigned int add_visited = 0;
-    unsigned long long add_edges = 0;
-    uint32_t start_level = level;
-    unsigned bar_k = 0;  // barriers passed in this launch
-    for (;;) {
-        const uint32_t fcount = vcount[slot];
-        const unsigned long long fedges = vedges[slot];
-        if (fcount == 0 || fcount > max_f || fedges > max_e || fcount < min_f ||
-            fedges > (unsigned long long)fcount * max_avg)
-            break;
-        const uint32_t s1 = slot == 2 ? 0 : slot + 1, s2 = s1 == 2 ? 0 : s1 + 1;
-        if (blockIdx.x == 0 && threadIdx.x == 0) {
-            ctl->fr_count[s2] = 0;
-            ctl->fr_edges[s2] = 0;
-        }
-        const uint32_t *q = queue ? q1 : q0;
-        uint32_t *qn = queue ? q0 : q1;
-        unsigned long long edges = 0;
-        const uint32_t nthreads = nwarps * 32u, gtid = gwarp * 32u + lane;
-        // Lanes per frontier vertex: as many as the grid has to spare (a power
-        // of two up to 32), so that the neighbours of a small frontier are
-        // visited in parallel rather than one after another by one thread.
-        uint32_t G = 1;
-        while (G < 32 && (unsigned long long)fcount * (G * 2) <= nthreads) G <<= 1;
-        const uint32_t sub = lane & (G - 1), ngroups = nthreads / G, vt = gtid / G;
-        for (uint32_t r0 = 0; r0 < fcount; r0 += ngroups) {
-            const uint32_t i = r0 + vt;
-            const bool valid = i < fcount;
-            const uint32_t v = valid ? q[i] : 0u;
-            const uint64_t b = valid ? rp[v] : 0, e = valid ? rp[v + 1] : 0;
-            const bool small = e - b <= 32;
-            if (G == 1) {
-                if (small) {
-                    for (uint64_t j = b; j < e; ++j) {
-                        const uint32_t w = col[j];
-                        if (L[w] == kUnvisited && atomicCAS(&L[w], kUnvisited, level + 1) == kUnvisited) {
-                            qn[atomicAdd(&ctl->fr_count[s1], 1u)] = w;
-                            edges += deg[w];
-                        }
-                    }
-                }
-            } else {  // the G lanes of a group take their vertex's neighbours in turn
-                const uint32_t d = valid && small ? (uint32_t)(e - b) : 0u;
-                const uint32_t kmax = __reduce_max_sync(0xFFFFFFFFu, (d + G - 1) / G);
-                for (uint32_t k = 0; k < kmax; ++k) {
-                    const uint32_t j = k * G + sub;
-                    bool claim = false;
-                    uint32_t w = 0, dw = 0;
-                    if (j < d) {
-                        w = col[b + j];
-                        dw = deg[w];  // read beside L[w], not after the claim
-                        claim = L[w] == kUnvisited && atomicCAS(&L[w], kUnvisited, level + 1) == kUnvisited;
-                    }
-                    const uint32_t pos = warp_append(claim, &ctl->fr_count[s1]);
-                    if (claim) {
-                        qn[pos] = w;
-                        edges += dw;
-                    }
-                }
-            }
-            unsigned big = __ballot_sync(0xFFFFFFFFu, valid && !small && sub == 0);
-            while (big) {
-                const int src = __ffs(big) - 1;
-                big &= big - 1;
-                const uint64_t bb = __shfl_sync(0xFFFFFFFFu, b, src), be = __shfl_sync(0xFFFFFFFFu, e, src);
-                for (uint64_t j0 = bb; j0 < be; j0 += 32) {
-                    const uint64_t j = j0 + lane;
-                    bool claim = false;
-                    uint32_t w = 0;
-                    if (j < be) {
-                        w = col[j];
-                        claim = L[w] == kUnvisited && atomicCAS(&L[w], kUnvisited, level + 1) == kUnvisited;
-                    }
-                    const uint32_t pos = warp_append(claim, &ctl->fr_count[s1]);
-                    if (claim) {
-                        qn[pos] = w;
-                        edges += deg[w];
-                    }
-                }
-            }
-        }
-        edges = warp_sum(edges);
-        if (lane == 0 && edges) atomicAdd(&ctl->fr_edges[s1], edges);
-        if (!grid_barrier(ctl, gridDim.x, bar_k++, 4000000000ll)) return;  // ~2 s at 2 GHz
-        if (blockIdx.x == 0 && threadIdx.x == 0) {
-            add_visited += vcount[s1];
-            add_edges += vedges[s1];
-        }
-        slot = s1;
-        queue ^= 1u;
-        ++level;
+// Levels of small frontiers (high-diameter graphs, and whole small graphs): one
+// thread-block cluster runs level after level with a hardware cluster barrier
+// each.  The frontier lives in shared memory as a queue of edge slots: a
+// claimed vertex puts the slots of its row into its block's queue, so in the
+// next level every thread takes one edge and no lane waits for a longer row.  A
+// level's dependent chain is col -> L -> claim (with the row's place and degree
+// read beside it) -> queue -> barrier; a 4096 x 4096 grid (4746 levels of about
+// 3500 vertices) took 5.7 us a level with a grid-wide barrier over 64 blocks and
+// a queue in global memory, 4.8 with queues of vertices here.
+// Claimed vertices stay with their block, except in the first levels and every
+// 16th one, when they are spread over the cluster by their ids.
+// A vertex of degree above kHubDeg is expanded by the whole cluster (its edges
+// strided over all blocks).  The kernel ends when a frontier was empty or had
+// more than max_f vertices or max_e edges, or (the `stop` flag, set in every
+// block before the barrier, so that all leave at the same level) when a vertex
+// of degree above max_d is claimed or a queue overflows; the frontier left is
+// written back to q0.  With `whole` it goes on with the first vertex of the next
+// component, up to kMaxRoots of them.
+// Where ids follow the geometry (grids, road networks) the lines ahead of and
+// behind a claimed vertex's are the next levels': they are asked into L2.
+constexpr uint32_t kClusterThreads = 1024;  // 32 warps: wkey below counts on it
+constexpr uint32_t kQueueCap = 4096;   // frontier vertices a block keeps (past it: a list in global memory)
+constexpr uint32_t kEdgeBytes = 48 * 1024;  // room for the edge slots of one frontier
+constexpr uint32_t kHubDeg = 256;
+constexpr uint32_t kHubCap = 256;      // hubs per level expanded by the whole cluster
+constexpr uint32_t kMaxRoots = 32;
+constexpr uint32_t kSpreadFirst = 3;
+constexpr uint32_t kLaneRow = 8;
+
+// Slot: an edge's place in col (32 bits where they are enough).
+template <class Slot>
+struct BfsShared {
+    static constexpr uint32_t kEdgeCap = kEdgeBytes / sizeof(Slot);
+    static constexpr Slot kNoEdge = ~(Slot)0;
+    Slot qe[2][kEdgeCap];
+    uint64_t hb[2][kHubCap];
+    uint32_t qv[2][kQueueCap], hd[2][kHubCap];
+    unsigned int cnt[3], edges[3];  // vertices and edge slots queued, by level mod 3
+    unsigned int hubs[3], ticket[3], stop[3], total[2], heavy[2];
+    unsigned long long wkey[32];  // smallest key of an unvisited vertex each warp saw
+};
+
+struct BfsArgs {
+    uint32_t n;
+    uint32_t *q0, *q1, *spill;
+    const uint64_t *rp;
+    const uint32_t *col, *deg;
+    uint32_t *L;
+    Ctl *ctl;
+    uint32_t fcount, queue, level;  // the frontier to start from (seed: the first vertex of the working order)
+    uint32_t seed, order, max_f, max_e, max_d, whole;
+};
+
+template <class Slot>
+__global__ void __launch_bounds__(kClusterThreads, 1) k_bfs_cluster(const BfsArgs g) {
+    namespace cg = cooperative_groups;
+    using Shared = BfsShared<Slot>;
+    extern __shared__ __align__(16) unsigned char smem_raw[];
+    Shared &S = *reinterpret_cast<Shared *>(smem_raw);
+    __shared__ uint32_t s_base;
+    cg::cluster_group cl = cg::this_cluster();
+    const unsigned lane = lane_id(), warp = threadIdx.x >> 5;
+    const uint32_t C = cl.num_blocks(), me = cl.block_rank();
+    const uint32_t hshift = 32u - (31u - __clz(C));
+    uint32_t *L = g.L;
+    if (threadIdx.x < 3) {
+        S.cnt[threadIdx.x] = S.edges[threadIdx.x] = 0;
+        S.hubs[threadIdx.x] = S.ticket[threadIdx.x] = S.stop[threadIdx.x] = 0;
     }
-    if (blockIdx.x == 0 && threadIdx.x == 0) {
-        ctl->p_slot = slot;
-        ctl->p_queue = queue;
-        ctl->p_level = level;
-        ctl->visited += add_visited;
-        ctl->visited_edges += add_edges;
-        // the last level that received vertices: the final frontier's level if it is
-        // non-empty, else the one before
-        const uint32_t last = vcount[slot] ? level : level - 1;
-        if (level > start_level && last > ctl->max_level) ctl->max_level = last;
+    if (threadIdx.x < 2) S.total[threadIdx.x] = S.heavy[threadIdx.x] = 0;
+    uint32_t visited = g.ctl->visited;  // before this kernel adds any (read before the first barrier)
+    const unsigned long long root_key = g.ctl->root_key;
+    cl.sync();
+
+    auto stop_all = [&](uint32_t s) {
+        for (uint32_t r = 0; r < C; ++r) cl.map_shared_rank(&S, r)->stop[s] = 1;
+    };
+    // a hub goes to every block's list; false: no room left, its edges are queued like any other's
+    auto push_hub = [&](uint64_t b, uint32_t d, uint32_t s, uint32_t p) {
+        const uint32_t h = atomicAdd(&cl.map_shared_rank(&S, 0)->ticket[s], 1u);
+        if (h >= kHubCap) return false;
+        for (uint32_t r = 0; r < C; ++r) {
+            Shared *R = cl.map_shared_rank(&S, r);
+            R->hb[p][h] = b;
+            R->hd[p][h] = d;
+            atomicAdd(&R->hubs[s], 1u);
+        }
+        return true;
+    };
+    // vertex v (row start b, degree d) at place `at` of block T's queue, its `e` edge slots from `first` on
+    // (false: they did not fit, v went to the spill list)
+    auto store = [&](Shared *T, uint32_t v, uint64_t b, uint32_t e, uint32_t at, uint32_t first, uint32_t p) {
+        const bool fits = at < kQueueCap && first + e <= Shared::kEdgeCap;
+        if (at < kQueueCap) T->qv[p][at] = fits ? v : kUnvisited;
+        for (uint32_t k = first; k < first + e && k < Shared::kEdgeCap; ++k)
+            T->qe[p][k] = fits ? (Slot)(b + (k - first)) : Shared::kNoEdge;
+        if (!fits) g.spill[atomicAdd(&g.ctl->bfs_spill, 1u)] = v;
+        return fits;
+    };
+    // by one lane, into the block v's id hashes to
+    auto push_spread = [&](uint32_t v, uint64_t b, uint32_t d, uint32_t s, uint32_t p) {
+        const uint32_t e = d > kHubDeg && push_hub(b, d, s, p) ? 0u : d;
+        Shared *T = cl.map_shared_rank(&S, (v * 0x9E3779B1u) >> hshift);
+        const uint32_t at = atomicAdd(&T->cnt[s], 1u), first = atomicAdd(&T->edges[s], e);
+        if (!store(T, v, b, e, at, first, p) || d > g.max_d) stop_all(s);
+    };
+    // Ask L2 for the lines of L, rp, deg and col 32 vertices either side of v (a DRAM
+    // access per level and array otherwise), once per line.
+    const uint64_t slots = g.rp[g.n];
+    auto ask = [](const void *q) { asm volatile("prefetch.global.L2 [%0];" ::"l"(q)); };
+    auto ask_ahead = [&](uint32_t v, uint64_t b) {
+        if ((v & 3u) == 0) {
+            if (b + 64 < slots) ask(g.col + b + 64);
+            if (b >= 64) ask(g.col + b - 64);
+        }
+        if ((v & 15u) == 0) {
+            if (v + 32 < g.n) {
+                ask(g.rp + v + 32);
+                ask(g.deg + v + 32);
+                ask(L + v + 32);
+            }
+            if (v >= 32) {
+                ask(g.rp + v - 32);
+                ask(g.deg + v - 32);
+                ask(L + v - 32);
+            }
+        }
+    };
+
+    uint32_t cs = 0, p = 0, level = g.level, roots = 0, top = 0;
+    if (g.seed) {
+        if (root_key != ~0ull) {
+            const uint32_t r = (uint32_t)(root_key & 0xFFFFFFFFull);
+            if (me == 0 && threadIdx.x == 0) {
+                L[r] = 0;
+                push_spread(r, g.rp[r], g.deg[r], 0, 0);
+            }
+            ++roots;
+            ++visited;
+        }
+    } else {
+        const uint32_t *q = g.queue ? g.q1 : g.q0;
+        for (uint32_t i = threadIdx.x; i < g.fcount; i += kClusterThreads) {
+            const uint32_t v = q[i];
+            // every block reads the whole queue and takes its own vertices
+            if ((v * 0x9E3779B1u) >> hshift == me) push_spread(v, g.rp[v], g.deg[v], 0, 0);
+        }
+    }
+    unsigned long long claimed = 0;  // degrees of the vertices claimed by this thread
+    uint32_t added = 0;              // vertices of the finished frontiers claimed here (uniform)
+    bool first = true;
+    cl.sync();
+    for (;;) {
+        if (S.stop[cs]) break;
+        const uint32_t ns = cs == 2 ? 0 : cs + 1, os = ns == 2 ? 0 : ns + 1, np = p ^ 1u;
+        const uint32_t ne = min(S.edges[cs], Shared::kEdgeCap), nh = min(S.hubs[cs], kHubCap);
+        if (threadIdx.x == 0) {  // the slot of the level before: nobody reads it any more
+            S.cnt[os] = S.edges[os] = 0;
+            S.hubs[os] = S.ticket[os] = S.stop[os] = 0;
+        }
+        const bool spread = level < kSpreadFirst || (level & 15u) == 0;
+        // every lane of a warp: claim vertex w if it is unvisited, queue the claimed ones
+        auto claim = [&](uint32_t w, bool valid) {
+            const bool open = valid && __ldcg(L + w) == kUnvisited;
+            uint64_t b = 0;
+            uint32_t d = 0;
+            bool got = false;
+            if (open) {  // the row's place and degree beside the claim, not after it
+                b = g.rp[w];
+                d = g.deg[w];
+                got = atomicCAS(&L[w], kUnvisited, level + 1) == kUnvisited;
+            }
+            const unsigned m = __ballot_sync(0xFFFFFFFFu, got);
+            if (m == 0) return;
+            if (got) {
+                claimed += d;
+                ask_ahead(w, b);
+            }
+            bool remote = false;
+            uint32_t e = got ? d : 0u;
+            if (e > kHubDeg && push_hub(b, d, ns, np)) {
+                e = 0;
+                remote = true;
+            }
+            // places in the queues: the claiming block's, or the one the id hashes to
+            uint32_t owner = me, at = 0, first_edge = 0;
+            if (spread) {
+                owner = (w * 0x9E3779B1u) >> hshift;
+                if (got) {
+                    Shared *T = cl.map_shared_rank(&S, owner);
+                    at = atomicAdd(&T->cnt[ns], 1u);
+                    first_edge = atomicAdd(&T->edges[ns], e);
+                }
+            } else {
+                uint32_t incl = e;
+#pragma unroll
+                for (int o = 1; o < 32; o <<= 1) {
+                    const uint32_t y = __shfl_up_sync(0xFFFFFFFFu, incl, o);
+                    if (lane >= (unsigned)o) incl += y;
+                }
+                if (lane == 31) at = atomicAdd(&S.edges[ns], incl);
+                if (lane == 0) at = atomicAdd(&S.cnt[ns], (unsigned)__popc(m));
+                first_edge = __shfl_sync(0xFFFFFFFFu, at, 31) + incl - e;
+                at = __shfl_sync(0xFFFFFFFFu, at, 0) + __popc(m & ((1u << lane) - 1u));
+            }
+            // rows of more than kLaneRow slots that fit are written by the whole warp
+            const bool wide = got && e > kLaneRow && at < kQueueCap && first_edge + e <= Shared::kEdgeCap;
+            if (got) {
+                Shared *T = spread ? cl.map_shared_rank(&S, owner) : &S;
+                if (wide) T->qv[np][at] = w;
+                const bool fits = wide || store(T, w, b, e, at, first_edge, np);
+                if (!fits || d > g.max_d) {
+                    stop_all(ns);
+                    remote = true;
+                }
+            }
+            unsigned rows = __ballot_sync(0xFFFFFFFFu, wide);
+            while (rows) {
+                const int src = __ffs(rows) - 1;
+                rows &= rows - 1;
+                const uint64_t rb = __shfl_sync(0xFFFFFFFFu, b, src);
+                const uint32_t re = __shfl_sync(0xFFFFFFFFu, e, src), rf = __shfl_sync(0xFFFFFFFFu, first_edge, src);
+                Shared *T = cl.map_shared_rank(&S, __shfl_sync(0xFFFFFFFFu, owner, src));
+                for (uint32_t k = lane; k < re; k += 32) T->qe[np][rf + k] = (Slot)(rb + k);
+            }
+            if (remote && !spread) __threadfence();  // the relaxed barrier of such a level orders nothing
+        };
+        for (uint32_t r0 = 0; r0 < ne; r0 += kClusterThreads) {
+            const uint32_t i = r0 + threadIdx.x;
+            const Slot j = i < ne ? S.qe[p][i] : Shared::kNoEdge;
+            const bool valid = j != Shared::kNoEdge;
+            claim(valid ? g.col[j] : 0u, valid);
+        }
+        for (uint32_t h = 0; h < nh; ++h) {
+            const uint64_t b = S.hb[p][h];
+            const uint32_t d = S.hd[p][h];
+            for (uint32_t j0 = ((me + h) & (C - 1)) * kClusterThreads; j0 < d; j0 += C * kClusterThreads) {
+                const uint32_t j = j0 + threadIdx.x;
+                if ((j & ~31u) >= d) break;  // no lane of this warp has an edge
+                claim(j < d ? g.col[b + j] : 0u, j < d);
+            }
+        }
+        if (warp == kClusterThreads / 32 - 1) {  // this frontier's size, known to all blocks after the barrier
+            const Shared *R = cl.map_shared_rank(&S, lane < C ? lane : me);
+            const uint32_t t = warp_sum(lane < C ? R->cnt[cs] : 0u);
+            const unsigned long long e = warp_sum(lane < C ? (unsigned long long)R->edges[cs] : 0ull);
+            if (lane == 0) {
+                S.total[p] = t;
+                S.heavy[p] = e > g.max_e;
+            }
+        }
+        if (spread) {
+            cl.sync();
+        } else {
+            // nothing remote but claims (atomics that have returned) and fenced hub or stop marks
+            __syncthreads();
+            asm volatile("barrier.cluster.arrive.relaxed.aligned;" ::: "memory");
+            asm volatile("barrier.cluster.wait.acquire.aligned;" ::: "memory");
+        }
+        const uint32_t total = S.total[p];
+        const bool heavy = S.heavy[p] != 0;
+        if (!first) {
+            added += total;
+            visited += total;
+            if (total) top = level > top ? level : top;
+        }
+        first = false;
+        cs = ns;
+        p = np;
+        ++level;
+        if (total == 0) {  // so the next frontier is empty too
+            if (!g.whole || visited >= g.n || roots >= kMaxRoots) break;
+            // the first unvisited vertex of the working order roots the next component
+            unsigned long long best = ~0ull;
+            for (uint32_t v = me * kClusterThreads + threadIdx.x; v < g.n; v += C * kClusterThreads)
+                if (__ldcg(L + v) == kUnvisited) {  // past L1, which may still hold it unvisited
+                    const unsigned long long k = order_key(v, g.deg[v], g.order);
+                    best = k < best ? k : best;
+                }
+            best = warp_min_u64(best);
+            if (lane == 0) S.wkey[warp] = best;
+            cl.sync();
+            unsigned long long key = ~0ull;  // every warp reduces the keys of all blocks' warps
+            for (uint32_t r = 0; r < C; ++r) {
+                const unsigned long long k = cl.map_shared_rank(&S, r)->wkey[lane];
+                key = k < key ? k : key;
+            }
+            key = warp_min_u64(key);
+            cl.sync();
+            if (key == ~0ull) break;
+            const uint32_t r = (uint32_t)(key & 0xFFFFFFFFull);
+            if (me == 0 && threadIdx.x == 0) {
+                L[r] = 0;
+                push_spread(r, g.rp[r], g.deg[r], cs, p);
+                claimed += g.deg[r];
+            }
+            ++roots;
+            ++visited;
+            ++added;
+            level = 0;
+            first = true;
+            cl.sync();
+        } else if (total > g.max_f || heavy) {
+            break;
+        }
+    }
+    // what is left of the frontier (buffer p, slot cs) goes back to global memory
+    const uint32_t fc = min(S.cnt[cs], kQueueCap);
+    unsigned long long fe = 0;
+    for (uint32_t i0 = 0; i0 < fc; i0 += kClusterThreads) {
+        const uint32_t i = i0 + threadIdx.x;
+        const uint32_t v = i < fc ? S.qv[p][i] : kUnvisited;  // kUnvisited: it is in the spill list
+        const uint32_t at = warp_append(v != kUnvisited, &g.ctl->fr_count[0]);
+        if (v != kUnvisited) {
+            g.q0[at] = v;
+            fe += g.deg[v];
+        }
+    }
+    cl.sync();
+    if (me == 0) {  // and the vertices that found no place in a block's queue
+        const uint32_t spill = g.ctl->bfs_spill;
+        if (spill) {
+            if (threadIdx.x == 0) s_base = atomicAdd(&g.ctl->fr_count[0], spill);
+            __syncthreads();
+            for (uint32_t i = threadIdx.x; i < spill; i += kClusterThreads) {
+                const uint32_t v = g.spill[i];
+                g.q0[s_base + i] = v;
+                fe += g.deg[v];
+            }
+        }
+    }
+    fe = warp_sum(fe);
+    claimed = warp_sum(claimed);
+    if (lane == 0) {
+        if (fe) atomicAdd(&g.ctl->fr_edges[0], fe);
+        if (claimed) atomicAdd(&g.ctl->visited_edges, claimed);
+    }
+    __syncthreads();
+    if (me == 0 && threadIdx.x == 0) {
+        // the frontier left over was claimed here unless it is the one the kernel began with
+        const uint32_t left = atomicAdd(&g.ctl->fr_count[0], 0u);
+        if (!first && left) {
+            added += left;
+            top = level > top ? level : top;
+        }
+        g.ctl->p_level = level;
+        g.ctl->visited += added;
+        if (top > g.ctl->max_level) g.ctl->max_level = top;
+        if (g.seed && root_key != ~0ull) {  // the first root itself
+            g.ctl->visited += 1;
+            atomicAdd(&g.ctl->visited_edges, (unsigned long long)g.deg[(uint32_t)(root_key & 0xFFFFFFFFull)]);
+        }
+        g.ctl->components += roots;
     }
 }
 
@@ -468,9 +684,14 @@ unsigned grid_for(uint64_t work, unsigned threads, unsigned cap) {
     return (unsigned)b;
 }
 
-constexpr uint32_t kPersistMaxF = 32768;          // frontier vertices (whole-grid mode)
-constexpr unsigned long long kPersistMaxE = 65536;  // frontier edges
-constexpr uint32_t kPersistMaxAvg = 256;            // mean frontier degree
+// Frontiers the cluster kernel takes: 16 of 152 SMs are enough for this many
+// edges a level, and a level costs it no round trip to the host.
+constexpr uint32_t kClusterMaxF = 32768;
+constexpr uint32_t kClusterMaxE = 65536;
+constexpr uint32_t kClusterMaxD = 1024;  // one vertex's: its neighbours' edges may overflow the queues
+// Graphs it levels from the first root to the last component.
+constexpr uint32_t kWholeN = 65536;
+constexpr uint64_t kWholeSlots = 1u << 18;
 
 // Levels given by the caller: degrees, a copy of the levels, their maximum,
 // and the check that makes the count exact with them -- every edge joins
@@ -533,62 +754,95 @@ static tc_status pull_ctl(tc_ctx *ctx) {
     return TC_OK;
 }
 
+// Run the cluster kernel: from the frontier in queue `queue`, or (seed) from
+// the first vertex of the working order.  Its results are in the control block.
+static tc_status launch_cluster(tc_ctx *ctx, const PipeBufs &b, uint32_t n, uint64_t slots, bool seed, uint32_t fcount,
+                                uint32_t queue, uint32_t level) {
+    BfsArgs a{};
+    a.n = n;
+    a.q0 = b.q0;
+    a.q1 = b.q1;
+    a.spill = b.R;
+    a.rp = b.rp;
+    a.col = b.col;
+    a.deg = b.deg;
+    a.L = b.L;
+    a.ctl = ctx->d_ctl;
+    a.fcount = fcount;
+    a.queue = queue;
+    a.level = level;
+    a.seed = seed;
+    a.order = ctx->opt.order;
+    a.whole = seed && n <= kWholeN && slots <= kWholeSlots;
+    a.max_f = a.whole ? 0xFFFFFFFFu : kClusterMaxF;
+    a.max_e = a.whole ? 0xFFFFFFFFu : kClusterMaxE;
+    a.max_d = a.whole ? 0xFFFFFFFFu : kClusterMaxD;
+    cudaLaunchAttribute attr{};
+    attr.id = cudaLaunchAttributeClusterDimension;
+    cudaLaunchConfig_t cfg{};
+    cfg.blockDim = dim3(kClusterThreads);
+    const bool narrow = slots < 0xFFFFFFFFull;
+    const void *kern = narrow ? (const void *)k_bfs_cluster<uint32_t> : (const void *)k_bfs_cluster<uint64_t>;
+    cfg.dynamicSmemBytes = narrow ? sizeof(BfsShared<uint32_t>) : sizeof(BfsShared<uint64_t>);
+    cfg.stream = ctx->stream;
+    cfg.attrs = &attr;
+    cfg.numAttrs = 1;
+    uint32_t &blocks = ctx->bfs_cluster[narrow ? 0 : 1];
+    if (!blocks) {  // 16 blocks where the device allows them (more than the portable 8)
+        TC_CUDA(ctx, cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)cfg.dynamicSmemBytes));
+        int clusters = 0;
+        attr.val.clusterDim = {16, 1, 1};
+        cfg.gridDim = dim3(16);
+        if (cudaFuncSetAttribute(kern, cudaFuncAttributeNonPortableClusterSizeAllowed, 1) != cudaSuccess ||
+            cudaOccupancyMaxActiveClusters(&clusters, kern, &cfg) != cudaSuccess)
+            clusters = 0;
+        cudaGetLastError();
+        blocks = clusters > 0 ? 16 : 8;
+    }
+    attr.val.clusterDim = {blocks, 1, 1};
+    cfg.gridDim = dim3(blocks);
+    void *args[] = {&a};
+    TC_CUDA(ctx, cudaLaunchKernelExC(&cfg, kern, args));
+    note_launch(ctx);
+    return TC_OK;
+}
+
 // Level-synchronous BFS from the frontier in queue `queue`, counter slot
-// `slot` (levels 0 .. start_level already assigned).  Per level the host
-// chooses top-down (edge-balanced) or bottom-up (Beamer et al.'s edge/vertex
-// heuristics); runs of small frontiers go to the persistent kernel.
+// `slot` (levels 0 .. start_level already assigned; the control block has been
+// pulled).  Per level the host chooses top-down (edge-balanced) or bottom-up
+// (Beamer et al.'s edge/vertex heuristics); runs of small frontiers go to the
+// cluster kernel, unless it has just left this one (stuck).
 static tc_status bfs_loop(tc_ctx *ctx, const PipeBufs &b, uint32_t n, uint64_t slots, uint32_t start_level,
-                          uint32_t slot, uint32_t queue) {
+                          uint32_t slot, uint32_t queue, bool stuck) {
     cudaStream_t s = ctx->stream;
     const unsigned cap = (unsigned)ctx->num_sms * 16u;
     uint32_t level = start_level;
     bool bottom_up = false;
-    tc_status st = pull_ctl(ctx);
-    if (st != TC_OK) return st;
+    tc_status st = TC_OK;
     uint32_t fcount = ctx->h_ctl->fr_count[slot];
     unsigned long long fedges = ctx->h_ctl->fr_edges[slot];
     uint32_t prev_count = 0;
-    int persist_blocks = -1;
     while (fcount > 0) {
         const unsigned long long unexplored = slots - ctx->h_ctl->visited_edges;
         if (!bottom_up && fedges > unexplored / 14 && fcount > 64) bottom_up = true;
         else if (bottom_up && fcount < n / 24 && fcount < prev_count) bottom_up = false;
         const uint32_t nxt = slot == 2 ? 0 : slot + 1;
-        if (!bottom_up && fcount <= kPersistMaxF && fedges <= kPersistMaxE &&
-            fedges <= (unsigned long long)fcount * kPersistMaxAvg) {
-            if (persist_blocks < 0) {
-                int per_sm = 0;
-                TC_CUDA(ctx, cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k_bfs_persist, 512, 0));
-                // enough threads for the largest frontier it takes, no more: fewer
-                // blocks make the per-level grid barrier cheaper
-                persist_blocks = std::min<int>(std::max(1, std::min(per_sm, 1)) * ctx->num_sms,
-                                               (int)((kPersistMaxF + 511) / 512));
-            }
-            k_reset_next<<<1, 1, 0, s>>>(ctx->d_ctl, (int)nxt);
-            uint32_t *q0 = b.q0, *q1 = b.q1;
-            const uint64_t *rp = b.rp;
-            const uint32_t *col = b.col, *deg = b.deg;
-            uint32_t *L = b.L;
-            Ctl *ctl = ctx->d_ctl;
-            uint32_t a_slot = slot, a_queue = queue, a_level = level;
-            uint32_t a_max_f = kPersistMaxF, a_min_f = 0, a_max_avg = kPersistMaxAvg;
-            unsigned long long a_max_e = kPersistMaxE;
-            void *args[] = {&q0, &q1, &rp, &col, &deg, &L, &ctl, &a_slot, &a_queue, &a_level, &a_max_f, &a_max_e,
-                            &a_min_f, &a_max_avg};
-            TC_CUDA(ctx, cudaLaunchCooperativeKernel((const void *)k_bfs_persist, dim3(persist_blocks), dim3(512),
-                                                     args, 0, s));
-            note_launch(ctx, 2);
-            st = pull_ctl(ctx);
+        if (!bottom_up && !stuck && fcount <= kClusterMaxF && fedges <= kClusterMaxE) {
+            k_reset_next<<<1, 1, 0, s>>>(ctx->d_ctl, 0);
+            note_launch(ctx);
+            st = launch_cluster(ctx, b, n, slots, false, fcount, queue, level);
+            if (st == TC_OK) st = pull_ctl(ctx);
             if (st != TC_OK) return st;
-            if (ctx->h_ctl->error == 4) return set_error(ctx, TC_ERR_TIMEOUT, "persistent BFS barrier timed out");
-            slot = ctx->h_ctl->p_slot;
-            queue = ctx->h_ctl->p_queue;
+            stuck = ctx->h_ctl->p_level == level;  // it could not take the frontier (one block's queue overflowed)
+            slot = 0;
+            queue = 0;
             level = ctx->h_ctl->p_level;
             prev_count = fcount;
-            fcount = ctx->h_ctl->fr_count[slot];
-            fedges = ctx->h_ctl->fr_edges[slot];
-            continue;  // the frontier is empty or too large for the persistent kernel
+            fcount = ctx->h_ctl->fr_count[0];
+            fedges = ctx->h_ctl->fr_edges[0];
+            continue;  // the frontier is empty or too large for the cluster
         }
+        stuck = false;
         uint32_t *q = queue ? b.q1 : b.q0;
         uint32_t *qn = queue ? b.q0 : b.q1;
         k_reset_next<<<1, 1, 0, s>>>(ctx->d_ctl, (int)nxt);
@@ -649,10 +903,11 @@ tc_status compute_levels(tc_ctx *ctx, const PipeBufs &b, uint32_t n, uint64_t sl
     const unsigned cap = (unsigned)ctx->num_sms * 16u;
     if (n == 0) return TC_OK;
     k_init<<<grid_for(n, 256, cap), 256, 0, s>>>(n, b.rp, b.deg, b.L, ctx->d_ctl, ctx->opt.order);
-    k_seed<<<1, 1, 0, s>>>(b.deg, b.L, b.q0, ctx->d_ctl, 0);
-    note_launch(ctx, 2);
+    note_launch(ctx);
     TC_CUDA(ctx, cudaGetLastError());
-    tc_status st = bfs_loop(ctx, b, n, slots, 0, 0, 0);
+    tc_status st = launch_cluster(ctx, b, n, slots, true, 0, 0, 0);
+    if (st == TC_OK) st = pull_ctl(ctx);
+    if (st == TC_OK) st = bfs_loop(ctx, b, n, slots, ctx->h_ctl->p_level, 0, 0, true);
     if (st != TC_OK) return st;
     if (ctx->h_ctl->visited >= n) return TC_OK;
 
@@ -683,7 +938,8 @@ tc_status compute_levels(tc_ctx *ctx, const PipeBufs &b, uint32_t n, uint64_t sl
     k_count_roots<<<1, 1, 0, s>>>(ctx->d_ctl, 0);
     note_launch(ctx, 3);
     TC_CUDA(ctx, cudaGetLastError());
-    return bfs_loop(ctx, b, n, slots, 0, 0, 0);
+    st = pull_ctl(ctx);
+    return st == TC_OK ? bfs_loop(ctx, b, n, slots, 0, 0, 0, false) : st;
 }
 
 }  // namespace tc

@@ -56,7 +56,7 @@ struct Ctl {
     unsigned long long cls_inserts[4];  // table / prefilter inserts actually done (rebuilds included)
     unsigned long long fr_edges[3];  // sum of degrees per frontier slot
     unsigned long long visited_edges;
-    unsigned int fr_count[3];        // frontier sizes per slot (slots rotate in the persistent BFS)
+    unsigned int fr_count[3];        // frontier sizes per slot (slots rotate)
     unsigned int visited;            // vertices with a level
     unsigned int max_level;
     unsigned int components;         // BFS roots
@@ -67,8 +67,9 @@ struct Ctl {
     unsigned long long n_tasks[3];   // tasks per class
     unsigned int error;              // nonzero: a device-side check failed
     unsigned int max_s2;             // largest hashed row among block-class rows / max degree
-    unsigned int p_slot, p_queue, p_level;  // where the persistent BFS stopped
-    unsigned int bar_count, bar_spare;      // arrivals at the persistent BFS's grid barriers (this launch)
+    unsigned int p_level;            // level the cluster BFS stopped at
+    unsigned int bfs_spill;          // frontier vertices that found no place in its queues
+    unsigned int bar_count, bar_spare;  // arrivals at the self-test's grid barrier
     unsigned int n_big;              // rows whose A part the block sorter sorts
     unsigned int n_huge;             // rows of very high degree filled by a block each
     unsigned int n_part;             // rows whose level-spanning part k_g1_split splits
@@ -131,6 +132,7 @@ struct tc_ctx {
     uint32_t isect_flags = 0; // which intersection kernels the last count launched (1 warp, 2 block, 4 hub)
     uint32_t shard = 0, nshards = 1;  // intersection tasks of this count: share `shard` of `nshards`
     uint32_t split_R = 0;             // this count's split rank (block-class bitmap; 0: none)
+    uint32_t bfs_cluster[2] = {0, 0}; // blocks of the cluster BFS, by slot width (0: not asked yet)
     uint64_t alloc_calls = 0;         // device allocations made by this context
     uint64_t fail_alloc_at = 0;       // fault injection: fail this allocation (1-based; 0 = never)
     std::string err;
