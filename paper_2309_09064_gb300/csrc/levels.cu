@@ -266,6 +266,37 @@ __global__ void k_cc_roots(const uint32_t *__restrict__ R, uint32_t nr, const ui
     if (threadIdx.x == 0 && s_edges) atomicAdd(&ctl->fr_edges[cur], s_edges);
 }
 
+// A disjoint union's first roots: every group's first vertex in the working
+// order (its component's root too), one block per group.
+__global__ void k_group_roots(GroupSpec groups, const uint32_t *__restrict__ deg, uint32_t *__restrict__ L,
+                              uint32_t *__restrict__ q, Ctl *ctl, uint32_t order, int cur) {
+    __shared__ unsigned long long s_key[32];
+    const unsigned lane = lane_id(), warp = threadIdx.x >> 5;
+    for (uint32_t g = blockIdx.x; g < groups.n_groups; g += gridDim.x) {
+        const uint32_t lo = groups.vertex_start[g], hi = groups.vertex_start[g + 1];
+        unsigned long long best = ~0ull;
+        for (uint32_t v = lo + threadIdx.x; v < hi; v += blockDim.x) {
+            const uint32_t d = deg[v];
+            if (d == 0) continue;
+            const unsigned long long k = order_key(v, d, order);
+            best = k < best ? k : best;
+        }
+        best = warp_min_u64(best);
+        if (lane == 0) s_key[warp] = best;
+        __syncthreads();
+        if (warp == 0) {
+            best = warp_min_u64(lane < (blockDim.x >> 5) ? s_key[lane] : ~0ull);
+            if (lane == 0 && best != ~0ull) {
+                const uint32_t r = (uint32_t)(best & 0xFFFFFFFFull);
+                L[r] = 0;
+                q[atomicAdd(&ctl->fr_count[cur], 1u)] = r;
+                atomicAdd(&ctl->fr_edges[cur], (unsigned long long)deg[r]);
+            }
+        }
+        __syncthreads();
+    }
+}
+
 __global__ void k_count_roots(Ctl *ctl, int cur) {
     ctl->components += ctl->fr_count[cur];
     ctl->visited += ctl->fr_count[cur];
@@ -905,9 +936,21 @@ tc_status compute_levels(tc_ctx *ctx, const PipeBufs &b, uint32_t n, uint64_t sl
     k_init<<<grid_for(n, 256, cap), 256, 0, s>>>(n, b.rp, b.deg, b.L, ctx->d_ctl, ctx->opt.order);
     note_launch(ctx);
     TC_CUDA(ctx, cudaGetLastError());
-    tc_status st = launch_cluster(ctx, b, n, slots, true, 0, 0, 0);
+    tc_status st = TC_OK;
+    const bool grouped = b.groups.n_groups > 1;
+    if (grouped) {
+        // every graph of a union is levelled from its own first vertex at once: only the
+        // small components beside them are left to the hooking below
+        k_group_roots<<<std::min(b.groups.n_groups, cap), 256, 0, s>>>(b.groups, b.deg, b.L, b.q0, ctx->d_ctl,
+                                                                      ctx->opt.order, 0);
+        k_count_roots<<<1, 1, 0, s>>>(ctx->d_ctl, 0);
+        note_launch(ctx, 2);
+        TC_CUDA(ctx, cudaGetLastError());
+    } else {
+        st = launch_cluster(ctx, b, n, slots, true, 0, 0, 0);
+    }
     if (st == TC_OK) st = pull_ctl(ctx);
-    if (st == TC_OK) st = bfs_loop(ctx, b, n, slots, ctx->h_ctl->p_level, 0, 0, true);
+    if (st == TC_OK) st = bfs_loop(ctx, b, n, slots, grouped ? 0 : ctx->h_ctl->p_level, 0, 0, !grouped);
     if (st != TC_OK) return st;
     if (ctx->h_ctl->visited >= n) return TC_OK;
 
