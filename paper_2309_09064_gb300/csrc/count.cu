@@ -46,15 +46,17 @@ size_t pipeline_bytes(const tc_ctx *ctx, uint32_t n, uint64_t slots, uint32_t ma
     if (own_levels) bytes += r(4 * n1);            // L
     bytes += 8 * r(8 * n1);                        // fpref eoff tpref[3] lv rkeys0 rkeys1
     bytes += r(4 * (slots + 1));                   // adj2
-    bytes += r(4 * (slots / 32 + 2));              // fence
     bytes += r(16 * (slots / 2 + 1));              // probe records: one per oriented G0 edge
     bytes += r(4 * (256 * rtiles + 1)) + r(8 * (256 * rtiles + 2));  // radix digit counts and offsets
     bytes += r(8 * scan_tmp_elems(std::max<uint64_t>(n1 + 1, 256 * rtiles + 2)));  // scan tiles
-    bytes += r(8 * (slots / 2 + 1));               // task pool: at most one task per oriented G0 edge
+    // fence and task pool (at most one task per oriented G0 edge), or the wedge path's ids and plan
+    size_t own = r(4 * (slots / 32 + 2)) + r(8 * (slots / 2 + 1));
     if (plain && wedge_path(ctx, n, slots, max_deg)) {
         const WedgeSizes z = wedge_sizes(ctx, n, slots);
-        bytes += r(4 * z.counts) + r(8 * (z.counts + 1)) + r(8ull * z.tiles) + r(16ull * z.tasks) + r(8 * z.tmp);
+        own = std::max(own, r(2 * (4 * slots + 8)) + r(4 * z.counts) + r(8 * (z.counts + 1)) + r(8ull * z.tiles) +
+                                r(16ull * z.tasks) + r(8 * z.tmp));
     }
+    bytes += own;
     *hub_words = 0;
     *hub_maps = 0;
     if (max_deg > ctx->tune.block_cap) {
@@ -149,26 +151,29 @@ tc_status count_pipeline(tc_ctx *ctx, const GraphView &g, uint32_t *levels_out, 
     b.rcounts = a.take<uint32_t>(256 * rtiles + 1);
     b.roffs = a.take<uint64_t>(256 * rtiles + 2);
     b.adj2 = a.take<uint32_t>(g.slots + 1);
-    b.fence = a.take<uint32_t>(g.slots / 32 + 2);
+    const bool wedge = plain && groups.n_groups == 0 && wedge_path(ctx, n, g.slots, g.max_deg);
     b.slots = g.slots;
     b.erec_cap = g.slots / 2 + 1;
     b.erec = a.take<uint4>(b.erec_cap);
     b.scan_tmp = a.take<uint64_t>(scan_tmp_elems(std::max<uint64_t>(n1 + 1, 256 * rtiles + 2)));
     b.task_cap = g.slots / 2 + 1;
-    b.task_pool = a.take<uint2>(b.task_cap);
+    if (!wedge) {
+        b.fence = a.take<uint32_t>(g.slots / 32 + 2);
+        b.task_pool = a.take<uint2>(b.task_cap);
+        ok = ok && b.fence && b.task_pool;
+    }
     b.hub_words = hub_words;
     b.hub_sets = hub_maps > ctx->tune.hub_group ? 2u : 1u;
     if (hub_maps) b.hub_bits = a.take<uint32_t>(hub_words * hub_maps);
-    const bool wedge = plain && groups.n_groups == 0 && wedge_path(ctx, n, g.slots, g.max_deg);
     if (wedge) {
         const WedgeSizes z = wedge_sizes(ctx, n, g.slots);
-        b.wedge_ids = reinterpret_cast<uint16_t *>(b.task_pool);
+        b.wedge_ids = a.take<uint16_t>(4 * g.slots + 8);
         b.wedge_counts = a.take<uint32_t>(z.counts);
         b.wedge_offs = a.take<uint64_t>(z.counts + 1);
         b.wedge_work = a.take<unsigned long long>(z.tiles);
         b.wedge_tasks = a.take<uint4>(z.tasks);
         b.wedge_tmp = a.take<uint64_t>(z.tmp);
-        ok = ok && b.wedge_counts && b.wedge_offs && b.wedge_work && b.wedge_tasks && b.wedge_tmp;
+        ok = ok && b.wedge_ids && b.wedge_counts && b.wedge_offs && b.wedge_work && b.wedge_tasks && b.wedge_tmp;
     }
     b.groups = groups;
     if (vertex_counts) {
@@ -202,8 +207,8 @@ tc_status count_pipeline(tc_ctx *ctx, const GraphView &g, uint32_t *levels_out, 
         TC_CUDA(ctx, cudaMemsetAsync(b.hits, 0, 8 * z.tiny, s));
         TC_CUDA(ctx, cudaMemsetAsync(b.wstate, 0, 16 * z.states, s));
     }
-    ok = ok && b.fpref && b.eoff && b.lv && b.rkeys0 && b.rkeys1 && b.rcounts && b.roffs && b.adj2 && b.fence && b.erec &&
-         b.scan_tmp && b.task_pool && (!hub_maps || b.hub_bits);
+    ok = ok && b.fpref && b.eoff && b.lv && b.rkeys0 && b.rkeys1 && b.rcounts && b.roffs && b.adj2 && b.erec &&
+         b.scan_tmp && (!hub_maps || b.hub_bits);
     if (!ok) return set_error(ctx, TC_ERR_OOM, "arena carve failed");
 
     k_ctl_reset<<<1, 128, 0, s>>>(ctx->d_ctl);

@@ -86,7 +86,7 @@ struct PipeBufs {
     // wedge path (wedge.cu): the rows N(x) are kept in adj2 (keys) and wedge_ids
     // (16-bit ids), their sizes in fcnt and gcnt, their places by rank in vmeta,
     // the tile entries in erec
-    uint16_t *wedge_ids = nullptr;            // [2 S] (the task pool's memory)
+    uint16_t *wedge_ids = nullptr;            // [4 S + 8]
     uint32_t *wedge_counts = nullptr;         // entries per tile and block
     uint64_t *wedge_offs = nullptr;           // their scan
     unsigned long long *wedge_work = nullptr; // steps per tile
@@ -94,12 +94,10 @@ struct PipeBufs {
     uint64_t *wedge_tmp = nullptr;            // scan tiles
 };
 
-// Plain counts under the degree order (wedge.cu).  Vertices of degree >=
-// kWedgeTileDegree, at most kWedgeMaxU of them, are taken in tiles of 32; a
-// tile's words cover the first kWedgeMaxK ranks (16-bit ids of 15 rank bits;
+// Plain counts under the degree order (wedge.cu).  The vertices of high degree,
+// at most kWedgeMaxU of them, are taken in tiles of 32; a tile's words cover the first kWedgeMaxK ranks (16-bit ids of 15 rank bits;
 // the last rank of 15 bits stays free: it marks padding).
-constexpr uint32_t kWedgeTileDegree = 128;
-constexpr uint32_t kWedgeMaxU = 1u << 18;
+constexpr uint32_t kWedgeMaxU = 1u << 19;
 constexpr uint32_t kWedgeMaxK = 32736;
 struct WedgeSizes {
     uint32_t tiles, tasks;

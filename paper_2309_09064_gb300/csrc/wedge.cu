@@ -24,8 +24,8 @@
 // The rows are read as 16-bit ids (w < K <= 2^15, flag in the low bit).
 // k_wedge_high takes the same tiles' pairs with w >= K, k_wedge_rest those with
 // u >= U.  Measured (one GB300, whole counts, before and after): R-MAT 24
-// 130.5 -> 58.6 ms, R-MAT 20 5.39 -> 2.31, Chung-Lu 2^22 16.4 -> 7.6, uniform
-// 2^20 of mean degree 32 3.36 -> 1.87, R-MAT 16 1.32 -> 0.73.
+// 130.5 -> 45.5 ms, R-MAT 20 5.39 -> 2.23, Chung-Lu 2^22 16.4 -> 7.2, uniform
+// 2^20 of mean degree 32 3.36 -> 1.85, R-MAT 16 1.32 -> 0.64.
 #include <algorithm>
 
 #include "pipeline.cuh"
@@ -41,7 +41,8 @@ constexpr int kFillThreads = 256;
 constexpr uint32_t kAhead = 8;         // neighbours of a lane's row read ahead together
 constexpr uint16_t kPadId = 0xFFFFu;   // fills a row's last unit: rank 2^15 - 1 >= K, its word is always 0
 constexpr uint32_t kTaskSteps = 1024;  // least steps (32 ids of one entry) of a tile task
-constexpr uint32_t kTasksPerSm = 16;
+constexpr uint32_t kTasksPerSm = 8;    // (a task costs its tile's build: R-MAT 20 2.51 ms at 48, 2.31 at 16, 2.27 at 8)
+constexpr uint64_t kRangeBytes = 48u << 20;
 constexpr unsigned kGuardSort = 0x100u;
 constexpr unsigned kGuardRange = 0x800u;
 constexpr unsigned kGuardWatchdog = 0x80u;
@@ -57,12 +58,12 @@ __device__ __forceinline__ uint2 rank_level(const uint2 *__restrict__ lv, const 
     }
 }
 
-// U: the vertices of degree >= kWedgeTileDegree (the working order starts with
-// them), whole tiles, at most kWedgeMaxU; K = min(U, kWedgeMaxK).
-__global__ void k_wedge_limits(uint32_t n, const unsigned long long *__restrict__ order, uint32_t max_deg, Ctl *ctl) {
+// U: the vertices of degree >= tile_deg (the working order starts with them), whole tiles, at most kWedgeMaxU; K = min(U, kWedgeMaxK).
+__global__ void k_wedge_limits(uint32_t n, const unsigned long long *__restrict__ order, uint32_t max_deg,
+                               uint32_t tile_deg, Ctl *ctl) {
     uint32_t U = 0;
-    if (max_deg >= kWedgeTileDegree) {
-        const uint32_t last = max_deg - kWedgeTileDegree;  // largest key of a tile vertex
+    if (max_deg >= tile_deg) {
+        const uint32_t last = max_deg - tile_deg;  // largest key of a tile vertex
         uint32_t lo = 0, hi = n < kWedgeMaxU ? n : kWedgeMaxU;
         while (lo < hi) {
             const uint32_t mid = (lo + hi) >> 1;
@@ -105,15 +106,21 @@ __device__ __forceinline__ void lane_sort(uint32_t (&v)[E]) {
     }
 }
 
-// Sort buf[0..d), d <= 32 * E, in place.
+// Sort buf[0..d), d <= 32 * E, in place (descending: written back reversed).
 template <int E>
-__device__ __forceinline__ void warp_sort(uint32_t *buf, uint32_t d) {
+__device__ __forceinline__ void warp_sort(uint32_t *buf, uint32_t d, bool descending = false) {
     const unsigned lane = lane_id();
     uint32_t v[E];
 #pragma unroll
-    for (int e = 0; e < E; ++e) v[e] = e * 32 + lane < d ? buf[e * 32 + lane] : kEmpty;
+    for (int e = 0; e < E; ++e) {
+        v[e] = e * 32 + lane < d ? buf[e * 32 + lane] : kEmpty;
+        if (descending) v[e] = ~v[e];
+    }
     lane_sort<E>(v);
     __syncwarp();
+#pragma unroll
+    for (int e = 0; e < E; ++e)
+        if (descending) v[e] = ~v[e];
     if constexpr (E % 4 == 0) {
 #pragma unroll
         for (int e = 0; e < E; e += 4)
@@ -123,6 +130,72 @@ __device__ __forceinline__ void warp_sort(uint32_t *buf, uint32_t d) {
         for (int e = 0; e < E; ++e) buf[lane * E + e] = v[e];
     }
     __syncwarp();
+}
+
+// The last log2(256) steps of a bitonic merge: buf[0..256) bitonic -> sorted.
+__device__ __forceinline__ void warp_merge_256(uint32_t *buf, bool descending) {
+    constexpr int E = 8;
+    const unsigned lane = lane_id();
+    uint32_t v[E];
+#pragma unroll
+    for (int e = 0; e < E; e += 4) {
+        const uint4 q = reinterpret_cast<const uint4 *>(buf)[(lane * E + e) / 4];
+        v[e] = q.x, v[e + 1] = q.y, v[e + 2] = q.z, v[e + 3] = q.w;
+    }
+    if (descending) {
+#pragma unroll
+        for (int e = 0; e < E; ++e) v[e] = ~v[e];
+    }
+#pragma unroll
+    for (int j = 128; j > 0; j >>= 1) {
+        if (j >= E) {
+            const bool low = (lane & (j / E)) == 0;
+#pragma unroll
+            for (int e = 0; e < E; ++e) {
+                const uint32_t o = __shfl_xor_sync(0xFFFFFFFFu, v[e], j / E);
+                v[e] = low ? min(v[e], o) : max(v[e], o);
+            }
+        } else {
+#pragma unroll
+            for (int e = 0; e < E; ++e) {
+                if (e & j) continue;
+                const uint32_t x = v[e], y = v[e | j];
+                v[e] = min(x, y);
+                v[e | j] = max(x, y);
+            }
+        }
+    }
+    if (descending) {
+#pragma unroll
+        for (int e = 0; e < E; ++e) v[e] = ~v[e];
+    }
+#pragma unroll
+    for (int e = 0; e < E; e += 4)
+        reinterpret_cast<uint4 *>(buf)[(lane * E + e) / 4] = make_uint4(v[e], v[e + 1], v[e + 2], v[e + 3]);
+    __syncwarp();
+}
+
+// Sort buf[0..d), 256 < d <= P (512 or 1024, kEmpty from d on): runs of 256 in
+// registers, their merges' first steps in shared memory.  (One register sort of
+// 1024 keys is 3500 instructions; two of them beside the smaller ones miss the
+// instruction cache.)
+__device__ __forceinline__ void warp_sort_large(uint32_t *buf, uint32_t d, uint32_t P) {
+    const unsigned lane = lane_id();
+    for (uint32_t c = 0; c < P; c += 256) warp_sort<8>(buf + c, d > c ? d - c : 0u, (c & 256u) != 0);
+    for (uint32_t k = 512; k <= P; k <<= 1) {
+        for (uint32_t j = k >> 1; j >= 256; j >>= 1) {
+            for (uint32_t p = lane; p < P / 2; p += 32) {
+                const uint32_t i = ((p & ~(j - 1)) << 1) | (p & (j - 1)), l = i | j;
+                const uint32_t a = buf[i], c = buf[l];
+                if ((a > c) == ((i & k) == 0)) {
+                    buf[i] = c;
+                    buf[l] = a;
+                }
+            }
+            __syncwarp();
+        }
+        for (uint32_t c = 0; c < P; c += 256) warp_merge_256(buf + c, (c & k) != 0);
+    }
 }
 
 // What a row leaves behind besides its keys: |N(x)|, how many of them lie
@@ -139,10 +212,10 @@ __device__ __forceinline__ void row_done(const RowOut &o, uint32_t x, uint32_t r
     o.rmeta[rank] = make_uint4((uint32_t)b, (uint32_t)(b >> 32), d, nlo);
 }
 
-// First 16-bit id of the row at slot b: the row owns the 8-byte units
+// First 16-bit id of the row at slot b: the row owns the 16-byte units (8 ids)
 // [(b + 1) / 2, (b + deg + 1) / 2), at least deg / 2 of them, so a row of degree
 // >= 2 has room for its ids and their padding to whole units (kPadId).
-__device__ __forceinline__ uint16_t *ids_of(uint16_t *ids, uint64_t b) { return ids + 4 * ((b + 1) >> 1); }
+__device__ __forceinline__ uint16_t *ids_of(uint16_t *ids, uint64_t b) { return ids + 8 * ((b + 1) >> 1); }
 
 // N(x) of every vertex of degree <= kHugeRow.  Warps take chunks of 32
 // vertices; rows of degree <= 32 belong to one lane (insertion sort in its
@@ -208,7 +281,7 @@ __global__ void __launch_bounds__(kFillThreads) k_wedge_rows(uint32_t n, const u
                     ++nlo;
                 }
             }
-            for (uint32_t i = nlo; i & 3u; ++i) id[i] = kPadId;
+            for (uint32_t i = nlo; i & 7u; ++i) id[i] = kPadId;
             row_done(out, (uint32_t)x, me.x, b, d, nlo, nu);
         }
         __syncwarp();
@@ -256,8 +329,7 @@ __global__ void __launch_bounds__(kFillThreads) k_wedge_rows(uint32_t n, const u
             else if (d <= 64) warp_sort<2>(buf, d);
             else if (d <= 128) warp_sort<4>(buf, d);
             else if (d <= 256) warp_sort<8>(buf, d);
-            else if (d <= 512) warp_sort<16>(buf, d);
-            else warp_sort<32>(buf, d);
+            else warp_sort_large(buf, d, d <= 512 ? 512u : 1024u);
             uint32_t nlo = 0, nu = 0;
             uint16_t *id = ids_of(ids, bb);
             for (uint32_t i = lane; i < d; i += 32) {
@@ -271,7 +343,7 @@ __global__ void __launch_bounds__(kFillThreads) k_wedge_rows(uint32_t n, const u
             }
             nlo = warp_sum(nlo);
             nu = warp_sum(nu);
-            if (lane < ((0u - nlo) & 3u)) id[nlo + lane] = kPadId;
+            if (lane < ((0u - nlo) & 7u)) id[nlo + lane] = kPadId;
             if (lane == 0) row_done(out, bx, brx, bb, d, nlo, nu);
             __syncwarp();
         }
@@ -414,7 +486,7 @@ __global__ void __launch_bounds__(1024) k_wedge_sort(const uint32_t *__restrict_
         if (lane_id() == 0 && nlo) atomicAdd(&s_lo, nlo);
         if (lane_id() == 0 && nu) atomicAdd(&s_u, nu);
         __syncthreads();
-        if (threadIdx.x < ((0u - s_lo) & 3u)) id[s_lo + threadIdx.x] = kPadId;
+        if (threadIdx.x < ((0u - s_lo) & 7u)) id[s_lo + threadIdx.x] = kPadId;
         if (threadIdx.x == 0) row_done(out, x, rank_level<kPacked>(lv, lvp, x).x, b, d, s_lo, s_u);
         __syncthreads();
     }
@@ -423,7 +495,7 @@ __global__ void __launch_bounds__(1024) k_wedge_sort(const uint32_t *__restrict_
 // ---------------------------------------------------------------------------- entries
 
 // One entry per (vertex v, tile, kind): {first 16-bit id of v's row in units of
-// 8 bytes, mask of v's neighbours in the tile, units of the prefix | kind << 31,
+// 16 bytes, mask of v's neighbours in the tile, units of the prefix | kind << 31,
 // keys of the row below K | (slot of the row & 1) << 15 | high keys << 16}.
 // kind 1: v's edges to the mask's vertices are horizontal.  The prefix holds
 // every w of N(v) below K and not above the mask's last vertex, the high keys
@@ -533,13 +605,13 @@ __global__ void __launch_bounds__(1024) k_wedge_entries(uint32_t n, uint64_t slo
                 const uint32_t parts = (hor != 0) + (ver != 0);
                 if constexpr (kScatter) {
                     const uint32_t at = atomicAdd(&sm[tile], parts);
-                    const uint32_t id8 = (uint32_t)((br + 1) >> 1), units = (len + 3) / 4;
+                    const uint32_t unit = (uint32_t)((br + 1) >> 1), units = (len + 7) / 8;
                     const uint32_t place = lr | (uint32_t)(br & 1u) << 15 | high << 16;
                     if ((uint64_t)at + parts > cap) {
                         atomicOr(&ctl->error, kGuardRange);
                     } else {
-                        if (hor) entries[at] = make_uint4(id8, hor, units | 0x80000000u, place);
-                        if (ver) entries[at + (hor != 0)] = make_uint4(id8, ver, units, place);
+                        if (hor) entries[at] = make_uint4(unit, hor, units | 0x80000000u, place);
+                        if (ver) entries[at + (hor != 0)] = make_uint4(unit, ver, units, place);
                     }
                 } else {
                     atomicAdd(&sm[tile], parts);
@@ -564,10 +636,15 @@ __global__ void __launch_bounds__(1024) k_wedge_entries(uint32_t n, uint64_t slo
 }
 
 // Tile tasks: equal slices of a tile's entries, of about the same number of
-// steps everywhere (one block; at most task_cap of them).
+// steps everywhere (one block; at most task_cap of them).  A tile's entries are
+// in row order, so its slices are row ranges: the tasks are listed range by
+// range (`ranges` of them, each with about as many ids as L2 keeps), and the
+// blocks that run at the same time read the same rows.  Tiles from rank
+// kWedgeMaxK on, which k_wedge_high walks again, come after the others.
 __global__ void __launch_bounds__(1024) k_wedge_plan(const unsigned long long *__restrict__ offs, uint32_t nb,
                                                      const unsigned long long *__restrict__ work, uint32_t num_sms,
-                                                     uint4 *__restrict__ tasks, uint32_t task_cap, Ctl *ctl) {
+                                                     uint32_t ranges, uint4 *__restrict__ tasks, uint32_t task_cap,
+                                                     Ctl *ctl) {
     __shared__ unsigned long long s_sum[32];
     __shared__ unsigned int s_warp[32], s_base;
     const unsigned lane = lane_id(), warp = threadIdx.x >> 5;
@@ -582,36 +659,44 @@ __global__ void __launch_bounds__(1024) k_wedge_plan(const unsigned long long *_
     sum = warp_sum(s_sum[lane]);
     unsigned long long target = sum / ((unsigned long long)num_sms * kTasksPerSm) + 1;
     if (target < kTaskSteps) target = kTaskSteps;
-    for (uint32_t t0 = 0; t0 < tiles; t0 += blockDim.x) {
-        const uint32_t t = t0 + threadIdx.x;
-        unsigned long long lo = 0, ent = 0, nt = 0;
-        if (t < tiles) {
-            lo = offs[(uint64_t)t * nb];
-            ent = offs[(uint64_t)(t + 1) * nb] - lo;
-            nt = (work[t] + target - 1) / target;
-            if (nt > ent) nt = ent;
-        }
-        uint32_t incl = (uint32_t)nt;
-#pragma unroll
-        for (int o = 1; o < 32; o <<= 1) {
-            const uint32_t y = __shfl_up_sync(0xFFFFFFFFu, incl, o);
-            if (lane >= (unsigned)o) incl += y;
-        }
-        if (lane == 31) s_warp[warp] = incl;
-        __syncthreads();
-        uint32_t before = s_base + incl - (uint32_t)nt;
-        for (unsigned w = 0; w < warp; ++w) before += s_warp[w];
-        if (t == kWedgeMaxK / 32) ctl->wedge_hi_task = before;
-        for (uint32_t i = 0; i < (uint32_t)nt; ++i) {
-            if (before + i >= task_cap) {
-                atomicOr(&ctl->error, kGuardRange);
-                break;
+    const uint32_t low = tiles < kWedgeMaxK / 32 ? tiles : kWedgeMaxK / 32;
+    for (uint32_t part = 0; part < 2 * ranges; ++part) {
+        const uint32_t range = part % ranges, t_lo = part < ranges ? 0u : low, t_hi = part < ranges ? low : tiles;
+        if (part == ranges && threadIdx.x == 0) ctl->wedge_hi_task = s_base;
+        for (uint32_t t0 = t_lo; t0 < t_hi; t0 += blockDim.x) {
+            const uint32_t t = t0 + threadIdx.x;
+            unsigned long long lo = 0, ent = 0, nt = 0;
+            uint32_t i0 = 0, i1 = 0;  // the tile's slices that lie in this range
+            if (t < t_hi) {
+                lo = offs[(uint64_t)t * nb];
+                ent = offs[(uint64_t)(t + 1) * nb] - lo;
+                nt = (work[t] + target - 1) / target;
+                if (nt > ent) nt = ent;
+                i0 = (uint32_t)((nt * range + ranges - 1) / ranges);
+                i1 = (uint32_t)((nt * (range + 1) + ranges - 1) / ranges);
             }
-            tasks[before + i] = make_uint4(t, (uint32_t)(lo + ent * i / nt), (uint32_t)(lo + ent * (i + 1) / nt), 0u);
+            uint32_t incl = i1 - i0;
+#pragma unroll
+            for (int o = 1; o < 32; o <<= 1) {
+                const uint32_t y = __shfl_up_sync(0xFFFFFFFFu, incl, o);
+                if (lane >= (unsigned)o) incl += y;
+            }
+            if (lane == 31) s_warp[warp] = incl;
+            __syncthreads();
+            uint32_t before = s_base + incl - (i1 - i0);
+            for (unsigned w = 0; w < warp; ++w) before += s_warp[w];
+            for (uint32_t i = i0; i < i1; ++i) {
+                if (before + i - i0 >= task_cap) {
+                    atomicOr(&ctl->error, kGuardRange);
+                    break;
+                }
+                tasks[before + i - i0] =
+                    make_uint4(t, (uint32_t)(lo + ent * i / nt), (uint32_t)(lo + ent * (i + 1) / nt), 0u);
+            }
+            __syncthreads();
+            if (threadIdx.x == blockDim.x - 1) s_base = before + i1 - i0;
+            __syncthreads();
         }
-        __syncthreads();
-        if (threadIdx.x == blockDim.x - 1) s_base = before + (uint32_t)nt;
-        __syncthreads();
     }
     if (threadIdx.x == 0) {
         ctl->n_tasks[1] = s_base;
@@ -632,7 +717,7 @@ __device__ __forceinline__ uint32_t lds(uint32_t addr) {
     return v;
 }
 
-// The 32 entries a warp holds and the steps (`per` units each) of its walk: the
+// The 32 entries a warp holds and the steps (32 ids each) of its walk: the
 // steps of all entries are shared out evenly over the warp's eight groups of
 // four lanes, so short and long rows keep every lane busy.
 struct Walk {
@@ -660,47 +745,49 @@ __device__ __forceinline__ Walk share_steps(uint32_t steps) {
     return w;
 }
 
+// The next task of a counter, for thread 0 (x = kNoTask: none left).
+constexpr uint32_t kNoTask = 0xFFFFFFFFu;
 __device__ __forceinline__ uint4 next_tile_task(Ctl *ctl, int counter, uint32_t first, uint32_t n_tasks,
-                                                const uint4 *__restrict__ tasks, uint4 *s_task, long long t_start) {
-    __syncthreads();
-    if (threadIdx.x == 0) {
-        const uint32_t k = first + atomicAdd(&ctl->task_next[counter], 1u);
-        uint4 t = make_uint4(0xFFFFFFFFu, 0, 0, 0);
-        if (clock64() - t_start > kWatchdogCycles) atomicOr(&ctl->error, kGuardWatchdog);
-        else if (k < n_tasks) t = tasks[k];
-        *s_task = t;
-    }
-    __syncthreads();
-    return *s_task;
+                                                const uint4 *__restrict__ tasks, long long t_start) {
+    const uint32_t k = first + atomicAdd(&ctl->task_next[counter], 1u);
+    if (clock64() - t_start > kWatchdogCycles) atomicOr(&ctl->error, kGuardWatchdog);
+    else if (k < n_tasks) return tasks[k];
+    return make_uint4(kNoTask, 0, 0, 0);
 }
 
 // One block per SM; a task is a slice of one tile's entries.  Each warp takes
 // 32 entries at a time, four lanes walk a row's prefix 32 ids (64 bytes) a
 // step; the next step's ids are loaded before the current ones are looked up.
 // Units past the prefix are kPadId; ids of the prefix's last unit past the
-// mask's last vertex read words that are 0.  Bound by issue and by the bank
-// conflicts of the lookups (3.6 wavefronts per 32).
+// mask's last vertex read words that are 0.  Bound by the bank conflicts of the
+// lookups (3.5 wavefronts per 32; L1/shared data stage at 83% at R-MAT 22) and
+// by issue: R-MAT 24 (26 G lookups) 18.8 ms, with eight lanes of four ids each
+// 26.0.
 __global__ void __launch_bounds__(kTileThreads, 1) k_wedge_tiles(uint32_t n, const uint4 *__restrict__ tasks,
                                                                  const uint4 *__restrict__ entries,
                                                                  const uint16_t *__restrict__ ids,
                                                                  const uint4 *__restrict__ rmeta, Ctl *ctl) {
     extern __shared__ __align__(16) uint32_t word[];
-    __shared__ uint4 s_task;
+    __shared__ uint4 s_task[2];
     const unsigned lane = lane_id(), warp = threadIdx.x >> 5;
     const uint32_t sub = lane & 3u;
     uint4 *ent = reinterpret_cast<uint4 *>(word + kTileWords) + warp * 32;
     const uint32_t wbase = (uint32_t)__cvta_generic_to_shared(word);
     const uint32_t n_tasks = (uint32_t)ctl->n_tasks[1];
-    const uint2 *id8 = reinterpret_cast<const uint2 *>(ids);
+    const uint4 *unit = reinterpret_cast<const uint4 *>(ids);
     unsigned long long same = 0, cross = 0, inserts = 0;
     uint32_t tile = 0xFFFFFFFFu;
     const long long t_start = clock64();
     for (uint32_t i = threadIdx.x; i < kTileWords / 4; i += kTileThreads)
         reinterpret_cast<uint4 *>(word)[i] = make_uint4(0, 0, 0, 0);
     uint32_t dirty = 0;  // words [0, dirty) may be set
-    for (;;) {
-        const uint4 task = next_tile_task(ctl, 1, 0, n_tasks, tasks, &s_task, t_start);
-        if (task.x == 0xFFFFFFFFu) break;
+    if (threadIdx.x == 0) s_task[0] = next_tile_task(ctl, 1, 0, n_tasks, tasks, t_start);
+    __syncthreads();
+    for (uint32_t phase = 0;; phase ^= 1u) {
+        const uint4 task = s_task[phase];
+        if (task.x == kNoTask) break;
+        uint4 next;  // taken now, needed when this task is done
+        if (threadIdx.x == 0) next = next_tile_task(ctl, 1, 0, n_tasks, tasks, t_start);
         if (task.x != tile) {
             tile = task.x;
             for (uint32_t i = threadIdx.x; i < dirty / 4; i += kTileThreads)
@@ -710,8 +797,14 @@ __global__ void __launch_bounds__(kTileThreads, 1) k_wedge_tiles(uint32_t n, con
             const uint32_t u = 32 * tile + warp;  // one row per warp
             if (u < n) {
                 const uint4 m = rmeta[u];
-                const uint16_t *id = ids + 4 * (((((uint64_t)m.y << 32) | m.x) + 1) >> 1);
-                for (uint32_t i = lane; i < m.w; i += 32) atomicOr(&word[id[i] >> 1], 1u << warp);
+                const uint4 *id = unit + (((((uint64_t)m.y << 32) | m.x) + 1) >> 1);
+                for (uint32_t i = lane; 8 * i < m.w; i += 32) {
+                    const uint4 q = id[i];
+                    const uint32_t w[8] = {q.x, q.x >> 16, q.y, q.y >> 16, q.z, q.z >> 16, q.w, q.w >> 16};
+#pragma unroll
+                    for (uint32_t t = 0; t < 8; ++t)
+                        if (8 * i + t < m.w) atomicOr(&word[(w[t] & 0xFFFFu) >> 1], 1u << warp);
+                }
                 if (lane == 0) inserts += m.w;
             }
             __syncthreads();
@@ -723,16 +816,14 @@ __global__ void __launch_bounds__(kTileThreads, 1) k_wedge_tiles(uint32_t n, con
             __syncwarp();
             ent[lane] = en;
             __syncwarp();
-            Walk w = share_steps(((en.z & 0x7FFFFFFFu) + 7) >> 3);
+            Walk w = share_steps(((en.z & 0x7FFFFFFFu) + 3) >> 2);
             uint4 cur = ent[w.i];
-            uint32_t at = cur.x + sub + 8 * w.skip;                            // this lane's first unit
-            int rem = (int)(cur.z & 0x7FFFFFFFu) - (int)(8 * w.skip + sub);    // units from there on
-            const uint2 pad = make_uint2(0xFFFFFFFFu, 0xFFFFFFFFu);
-            uint2 a = pad, b = pad, a1, b1;
+            uint32_t at = cur.x + sub + 4 * w.skip;                            // this lane's first unit
+            int rem = (int)(cur.z & 0x7FFFFFFFu) - (int)(4 * w.skip + sub);    // units from there on
+            uint4 a, a1;
             uint32_t mv = 0, kl = 0, mv1, kl1;
-            auto fetch = [&](uint2 &x, uint2 &y, uint32_t &mm, uint32_t &kk) {
-                x = pad;
-                y = pad;
+            auto fetch = [&](uint4 &x, uint32_t &mm, uint32_t &kk) {
+                x = make_uint4(0xFFFFFFFFu, 0xFFFFFFFFu, 0xFFFFFFFFu, 0xFFFFFFFFu);
                 if (w.left) {
                     --w.left;
                     while (rem + (int)sub <= 0) {  // entries may have no units (high keys only)
@@ -741,10 +832,9 @@ __global__ void __launch_bounds__(kTileThreads, 1) k_wedge_tiles(uint32_t n, con
                         at = cur.x + sub;
                         rem = (int)(cur.z & 0x7FFFFFFFu) - (int)sub;
                     }
-                    if (rem > 0) x = __ldg(id8 + at);
-                    if (rem > 4) y = __ldg(id8 + at + 4);
-                    at += 8;
-                    rem -= 8;
+                    if (rem > 0) x = __ldg(unit + at);
+                    at += 4;
+                    rem -= 4;
                 }
                 mm = cur.y;
                 kk = cur.z >> 31;
@@ -756,21 +846,22 @@ __global__ void __launch_bounds__(kTileThreads, 1) k_wedge_tiles(uint32_t n, con
                 if (x & kk) sam += p0;
                 if (x & (kk << 16)) sam += p1;
             };
-            fetch(a, b, mv, kl);
+            fetch(a, mv, kl);
             for (uint32_t k = 0; k < w.iters; ++k) {
-                fetch(a1, b1, mv1, kl1);
+                fetch(a1, mv1, kl1);
                 look(a.x, mv, kl);
                 look(a.y, mv, kl);
-                look(b.x, mv, kl);
-                look(b.y, mv, kl);
+                look(a.z, mv, kl);
+                look(a.w, mv, kl);
                 a = a1;
-                b = b1;
                 mv = mv1;
                 kl = kl1;
             }
         }
         same += sam;
         cross += tot - sam;
+        if (threadIdx.x == 0) s_task[phase ^ 1u] = next;
+        __syncthreads();
     }
     same = warp_sum(same);
     cross = warp_sum(cross);
@@ -783,35 +874,44 @@ __global__ void __launch_bounds__(kTileThreads, 1) k_wedge_tiles(uint32_t n, con
 }
 
 // The high keys (w >= K) of the tiles from rank K on, where a tile's vertices
-// have few of them: the tile's words sit in a hash table (linear probing,
-// 8192 slots of {rank, word}, at most about half full; a tile with more high
-// keys is taken in several rounds, each with the keys of one hash class), and
-// four lanes walk the high keys of an entry's row 16 a step.
-constexpr uint32_t kHighThreads = 512;
-constexpr uint32_t kHighSlots = 8192, kHighShift = 19, kHighKeys = 4096;
-constexpr size_t kHighSmem = 8ull * kHighSlots + (kHighThreads / 32) * 32 * sizeof(uint4);
+// have few of them.  A bitmap (2^17 bits, indexed by the rank's low bits) says
+// which w the tile's vertices can have: most keys end there, with one shared
+// load.  The words of the others sit in a hash table (linear probing, {rank,
+// word}, at most three quarters full; a tile with more high keys is walked in
+// several rounds, each with the keys of one hash class).  A warp flattens the
+// high keys of 32 entries, one per lane and window.  R-MAT 24 (3.5 G keys): 7.8 ms;
+// with 4096 keys a round and no bitmap 13.5, with 2048 and a bitmap 15.5 (two
+// rounds over the entries where one now does), four lanes per entry 17.7.
+constexpr uint32_t kHighThreads = 768;
+constexpr uint32_t kHighAhead = 4;
+constexpr uint32_t kHighBits = 1u << 17;
+constexpr uint32_t kHighSlots = 8192, kHighShift = 19, kHighKeys = 6144;
+constexpr size_t kHighSmem = kHighBits / 8 + 8ull * kHighSlots + (kHighThreads / 32) * 32 * sizeof(uint4);
 constexpr unsigned kGuardInsert = 0x10u;
 
-__global__ void __launch_bounds__(kHighThreads, 3) k_wedge_high(uint32_t n, const uint4 *__restrict__ tasks,
+__global__ void __launch_bounds__(kHighThreads, 2) k_wedge_high(uint32_t n, const uint4 *__restrict__ tasks,
                                                                 const uint4 *__restrict__ entries,
                                                                 const uint32_t *__restrict__ keys,
                                                                 const uint4 *__restrict__ rmeta, Ctl *ctl) {
-    extern __shared__ __align__(16) uint32_t word[];
-    uint2 *table = reinterpret_cast<uint2 *>(word);
-    __shared__ uint4 s_task;
+    extern __shared__ __align__(16) uint32_t member[];  // kHighBits bits, the table, the warps' entries
+    uint2 *table = reinterpret_cast<uint2 *>(member + kHighBits / 32);
+    __shared__ uint4 s_task[2];
     __shared__ uint32_t s_items;
     const unsigned lane = lane_id(), warp = threadIdx.x >> 5;
-    const uint32_t sub = lane & 3u;
-    uint4 *ent = reinterpret_cast<uint4 *>(word + 2 * kHighSlots) + warp * 32;
+    uint4 *ent = reinterpret_cast<uint4 *>(table + kHighSlots) + warp * 32;
     const uint32_t n_tasks = (uint32_t)ctl->n_tasks[1];
     if (ctl->wedge_u <= kWedgeMaxK) return;
     const uint32_t first_task = ctl->wedge_hi_task;
     unsigned long long same = 0, cross = 0, inserts = 0;
-    uint32_t tile = 0xFFFFFFFFu, rounds = 1;
+    uint32_t tile = kNoTask, rounds = 1;
     const long long t_start = clock64();
-    for (;;) {
-        const uint4 task = next_tile_task(ctl, 2, first_task, n_tasks, tasks, &s_task, t_start);
-        if (task.x == 0xFFFFFFFFu) break;
+    if (threadIdx.x == 0) s_task[0] = next_tile_task(ctl, 2, first_task, n_tasks, tasks, t_start);
+    __syncthreads();
+    for (uint32_t phase = 0;; phase ^= 1u) {
+        const uint4 task = s_task[phase];
+        if (task.x == kNoTask) break;
+        uint4 next;  // taken now, needed when this task is done
+        if (threadIdx.x == 0) next = next_tile_task(ctl, 2, first_task, n_tasks, tasks, t_start);
         const bool fresh = task.x != tile || rounds > 1;
         if (fresh) {
             tile = task.x;
@@ -827,7 +927,11 @@ __global__ void __launch_bounds__(kHighThreads, 3) k_wedge_high(uint32_t n, cons
         }
         for (uint32_t round = 0; round < rounds; ++round) {
             if (fresh) {
-                for (uint32_t i = threadIdx.x; i < kHighSlots; i += kHighThreads) table[i] = make_uint2(kEmpty, 0u);
+                for (uint32_t i = threadIdx.x; i < (kHighBits / 32 + 2 * kHighSlots) / 4; i += kHighThreads) {
+                    // the bitmap to 0, the table to {kEmpty, 0}
+                    const uint32_t e = i >= kHighBits / 128 ? kEmpty : 0u;
+                    reinterpret_cast<uint4 *>(member)[i] = make_uint4(e, 0u, e, 0u);
+                }
                 __syncthreads();
                 for (uint32_t r = warp; r < 32; r += kHighThreads / 32) {
                     if (32 * tile + r >= n) break;
@@ -836,6 +940,7 @@ __global__ void __launch_bounds__(kHighThreads, 3) k_wedge_high(uint32_t n, cons
                     for (uint32_t p = m.w + lane; p < m.z; p += 32) {
                         const uint32_t w = nu[p] >> 1, h = w * 0x9E3779B1u;
                         if (rounds > 1 && (h & 0xFFFFu) % rounds != round) continue;
+                        atomicOr(&member[(w & (kHighBits - 1)) >> 5], 1u << (w & 31u));
                         uint32_t s = h >> kHighShift, tries = 0;
                         for (; tries < kHighSlots; ++tries) {
                             const uint32_t old = atomicCAS(&table[s].x, kEmpty, w);
@@ -854,30 +959,39 @@ __global__ void __launch_bounds__(kHighThreads, 3) k_wedge_high(uint32_t n, cons
             for (uint32_t base = task.y + warp * 32; base < task.z; base += kHighThreads) {
                 uint4 en = make_uint4(0, 0, 0, 0);
                 if (base + lane < task.z) en = entries[base + lane];
-                __syncwarp();
-                ent[lane] = en;
-                __syncwarp();
-                Walk w = share_steps(((en.w >> 16) + 15) >> 4);
-                while (w.left) {  // entries without high keys have no steps
-                    const uint4 cur = ent[w.i];
-                    const uint32_t cnt = cur.w >> 16;
-                    if (16 * w.skip >= cnt) {
-                        w.i = (w.i + 1) & 31u;
-                        w.skip = 0;
-                        continue;
-                    }
-                    --w.left;
-                    const uint32_t *row = keys + (2 * (uint64_t)cur.x - ((cur.w >> 15) & 1u) + (cur.w & 0x7FFFu));
-                    uint32_t key[4];
+                const uint32_t cnt = en.w >> 16;
+                uint32_t incl = cnt;
 #pragma unroll
-                    for (int t = 0; t < 4; ++t) {
-                        const uint32_t p = 16 * w.skip + sub + 4 * t;
-                        key[t] = p < cnt ? __ldg(row + p) : 0u;  // rank 0 is below K: never in the table
-                    }
-                    ++w.skip;
+                for (int o = 1; o < 32; o <<= 1) {
+                    const uint32_t y = __shfl_up_sync(0xFFFFFFFFu, incl, o);
+                    if (lane >= (unsigned)o) incl += y;
+                }
+                const uint32_t total = __shfl_sync(0xFFFFFFFFu, incl, 31), excl = incl - cnt;
+                // the entries that have high keys, packed: {first key - flat position, mask, kind}
+                const unsigned some = __ballot_sync(0xFFFFFFFFu, cnt != 0);
+                __syncwarp();
+                if (cnt)
+                    ent[__popc(some & ((1u << lane) - 1u))] =
+                        make_uint4(2 * en.x - ((en.w >> 15) & 1u) + (en.w & 0x7FFFu) - excl, en.y, en.z >> 31, 0u);
+                __syncwarp();
+                // One key per lane and window of 32 flat positions, kHighAhead windows in flight:
+                // the entry of a position is the number of entries that start up to there.
+                uint32_t before = 0;
+                for (uint32_t k = 0; k < total; k += 32 * kHighAhead) {
+                    uint32_t key[kHighAhead], at[kHighAhead];
 #pragma unroll
-                    for (int t = 0; t < 4; ++t) {
-                        const uint32_t r = key[t] >> 1;
+                    for (uint32_t t = 0; t < kHighAhead; ++t) {
+                        const uint32_t k0 = k + 32 * t;
+                        const unsigned heads =
+                            __reduce_or_sync(0xFFFFFFFFu, cnt && excl >= k0 && excl - k0 < 32 ? 1u << (excl - k0) : 0u);
+                        at[t] = (before + __popc(heads & (0xFFFFFFFFu >> (31u - lane))) - 1u) & 31u;
+                        before += __popc(heads);
+                        key[t] = k0 + lane < total ? __ldg(keys + (uint32_t)(ent[at[t]].x + k0 + lane)) : 0u;
+                    }
+#pragma unroll
+                    for (uint32_t t = 0; t < kHighAhead; ++t) {
+                        const uint32_t r = key[t] >> 1;  // (rank 0, past the end, is below K: not in the table)
+                        if (!((member[(r & (kHighBits - 1)) >> 5] >> (r & 31u)) & 1u)) continue;
                         uint32_t s = (r * 0x9E3779B1u) >> kHighShift;
                         uint2 e = table[s];
                         for (uint32_t tries = 0; e.x != r && e.x != kEmpty && tries < kHighSlots; ++tries) {
@@ -885,9 +999,9 @@ __global__ void __launch_bounds__(kHighThreads, 3) k_wedge_high(uint32_t n, cons
                             e = table[s];
                         }
                         if (e.x == r) {
-                            const uint32_t p = __popc(e.y & cur.y);
+                            const uint32_t p = __popc(e.y & ent[at[t]].y);
                             tot += p;
-                            if (key[t] & (cur.z >> 31)) sam += p;
+                            if (key[t] & ent[at[t]].z) sam += p;
                         }
                     }
                 }
@@ -897,6 +1011,8 @@ __global__ void __launch_bounds__(kHighThreads, 3) k_wedge_high(uint32_t n, cons
             cross += tot - sam;
             if (rounds > 1) __syncthreads();  // the table is cleared next
         }
+        if (threadIdx.x == 0) s_task[phase ^ 1u] = next;
+        __syncthreads();
     }
     same = warp_sum(same);
     cross = warp_sum(cross);
@@ -1043,6 +1159,16 @@ unsigned grid_for(uint64_t work, unsigned threads, unsigned cap) {
 
 uint32_t tiles_cap(uint32_t n) { return std::min(kWedgeMaxU, n) / 32 + 1; }
 
+// Least degree of a tile vertex.  A tile costs its words' build (about 5 us of
+// one SM) and saves its vertices' rows from k_wedge_rest: with 64 instead of 128
+// R-MAT 13 takes 0.38 instead of 0.43 ms and R-MAT 16 0.65 instead of 0.69 (the
+// SMs have tiles to spare), R-MAT 22 9.11 instead of 9.05 and Chung-Lu 2^22 7.65
+// instead of 7.44.
+uint32_t tile_degree(uint32_t n) { return n < (1u << 20) ? 64u : 128u; }
+// Largest degree from which a graph takes tiles at all (a uniform graph of mean
+// degree 32 would make a single tile: 2.02 instead of 1.87 ms).
+constexpr uint32_t kTilesFrom = 128;
+
 // Blocks of the entry kernels: a row range each.
 uint32_t entry_blocks(const tc_ctx *ctx, uint64_t slots) {
     return (uint32_t)std::min<uint64_t>(2ull * ctx->num_sms, slots / 4096 + 1);
@@ -1079,7 +1205,7 @@ tc_status wedge_rows(tc_ctx *ctx, const PipeBufs &b, uint32_t n, uint32_t max_de
     const RowOut out{b.fcnt, b.gcnt, b.glo, b.vmeta};
     // warps of small graphs take fewer vertices each, so that long rows spread over the GPU
     const uint32_t per_warp = n >= (1u << 20) ? 32u : n >= (1u << 18) ? 16u : 8u;
-    k_wedge_limits<<<1, 1, 0, s>>>(n, b.order, max_deg, ctx->d_ctl);
+    k_wedge_limits<<<1, 1, 0, s>>>(n, b.order, max_deg, max_deg >= kTilesFrom ? tile_degree(n) : max_deg + 1, ctx->d_ctl);
     auto rows = b.lvp ? k_wedge_rows<true> : k_wedge_rows<false>;
     rows<<<grid_for((uint64_t)n * (32 / per_warp), kFillThreads, cap), kFillThreads, 0, s>>>(
         n, b.rp, b.col, b.lv, b.lvp, b.adj2, ids, out, b.big, b.huge, per_warp, ctx->d_ctl);
@@ -1096,21 +1222,23 @@ tc_status wedge_rows(tc_ctx *ctx, const PipeBufs &b, uint32_t n, uint32_t max_de
         sort<<<(unsigned)ctx->num_sms, 1024, smem, s>>>(b.big, ctx->d_ctl, b.rp, b.lv, b.lvp, b.adj2, ids, out);
         ++launches;
     }
-    if (max_deg >= kWedgeTileDegree) {
+    if (max_deg >= kTilesFrom) {
         const uint32_t nb = entry_blocks(ctx, b.slots), tiles = tiles_cap(n);
         const uint64_t cells = (uint64_t)tiles * nb;
         TC_CUDA(ctx, cudaMemsetAsync(b.wedge_counts, 0, 4 * cells, s));
         TC_CUDA(ctx, cudaMemsetAsync(b.wedge_work, 0, 8ull * tiles, s));
         const int smem = (int)(8 * tiles);
         TC_CUDA(ctx, cudaFuncSetAttribute(k_wedge_entries<false>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem));
-        TC_CUDA(ctx, cudaFuncSetAttribute(k_wedge_entries<true>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem));
+        TC_CUDA(ctx, cudaFuncSetAttribute(k_wedge_entries<true>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem / 2));
         auto *offs = reinterpret_cast<unsigned long long *>(b.wedge_offs);
         k_wedge_entries<false><<<nb, 1024, smem, s>>>(n, b.slots, b.rp, b.adj2, b.fcnt, b.gcnt, b.wedge_counts, offs,
                                                       b.wedge_work, b.erec, b.erec_cap, tiles, ctx->d_ctl);
         launches += 3 + scan_u32_to_u64(b.wedge_counts, b.wedge_offs, cells, b.wedge_tmp, s);
-        k_wedge_entries<true><<<nb, 1024, smem, s>>>(n, b.slots, b.rp, b.adj2, b.fcnt, b.gcnt, b.wedge_counts, offs,
+        k_wedge_entries<true><<<nb, 1024, smem / 2, s>>>(n, b.slots, b.rp, b.adj2, b.fcnt, b.gcnt, b.wedge_counts, offs,
                                                      b.wedge_work, b.erec, b.erec_cap, tiles, ctx->d_ctl);
-        k_wedge_plan<<<1, 1024, 0, s>>>(offs, nb, b.wedge_work, (uint32_t)ctx->num_sms, b.wedge_tasks,
+        // row ranges of about kRangeBytes of 16-bit ids (2 bytes an edge)
+        const uint32_t ranges = (uint32_t)std::min<uint64_t>(b.slots / kRangeBytes + 1, 16);
+        k_wedge_plan<<<1, 1024, 0, s>>>(offs, nb, b.wedge_work, (uint32_t)ctx->num_sms, ranges, b.wedge_tasks,
                                         tasks_cap(ctx, n), ctx->d_ctl);
     }
     note_launch(ctx, launches);
@@ -1120,7 +1248,7 @@ tc_status wedge_rows(tc_ctx *ctx, const PipeBufs &b, uint32_t n, uint32_t max_de
 
 tc_status wedge_count(tc_ctx *ctx, const PipeBufs &b, uint32_t n, uint32_t max_deg) {
     cudaStream_t s = ctx->stream;
-    const bool tiles = max_deg >= kWedgeTileDegree;
+    const bool tiles = max_deg >= kTilesFrom;
     TC_CUDA(ctx, cudaEventRecord(ctx->ev[4], s));
     int per_sm = 0;
     TC_CUDA(ctx, cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k_wedge_rest, kRestThreads, 0));
@@ -1135,7 +1263,7 @@ tc_status wedge_count(tc_ctx *ctx, const PipeBufs &b, uint32_t n, uint32_t max_d
                                                                              b.vmeta, ctx->d_ctl);
         if (n > kWedgeMaxK) {
             TC_CUDA(ctx, cudaFuncSetAttribute(k_wedge_high, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kHighSmem));
-            k_wedge_high<<<(unsigned)ctx->num_sms * 3u, kHighThreads, kHighSmem, s>>>(n, b.wedge_tasks, b.erec, b.adj2,
+            k_wedge_high<<<(unsigned)ctx->num_sms * 2u, kHighThreads, kHighSmem, s>>>(n, b.wedge_tasks, b.erec, b.adj2,
                                                                                      b.vmeta, ctx->d_ctl);
             note_launch(ctx);
         }
