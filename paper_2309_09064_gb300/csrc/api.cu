@@ -335,7 +335,8 @@ tc_status tc_build_csr(tc_ctx *ctx, uint32_t n, uint64_t n_tuples, const uint32_
     uint32_t *col = nullptr;
     uint64_t slots = 0;
     bool pooled = false;
-    tc_status st = build_csr_device(ctx, n, n_tuples, ds, dd, &rp, &col, &slots, &pooled);
+    uint32_t max_deg = 0;
+    tc_status st = build_csr_device(ctx, n, n_tuples, ds, dd, &rp, &col, &slots, &pooled, &max_deg);
     if (tmp) {
         cudaStreamSynchronize(ctx->stream);
         cudaFree(tmp);
@@ -349,7 +350,9 @@ tc_status tc_build_csr(tc_ctx *ctx, uint32_t n, uint64_t n_tuples, const uint32_
     g->col = col;
     g->pooled = pooled;
     g->owned = true;
-    return finish_graph(ctx, g, 0, out);
+    g->max_deg = max_deg;
+    *out = g;
+    return TC_OK;
 }
 
 tc_status tc_graph_info(const tc_graph *g, uint32_t *n, uint64_t *slots, const uint64_t **d_row_ptr,

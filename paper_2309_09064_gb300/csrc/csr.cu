@@ -1,13 +1,20 @@
 // csr.cu -- building, checking and measuring the input CSR on the device.
 //
-// tc_build_csr: tuples (a, b) -> 64-bit keys (a << 32 | b) and (b << 32 | a)
-// for a != b -> stable LSD radix sort (8-bit digits, only the digits that
-// can be nonzero) -> drop repeated keys -> col = low halves, row_ptr from the
-// run boundaries of the high halves.  The result is the paper's input format:
-// symmetric, loop-free, duplicate-free, rows ascending.
+// tc_build_csr: every tuple (a, b), a != b, counts one entry for a and one for
+// b; the counts' prefix gives every vertex a row, the entries are placed in any
+// order, every row is sorted and its repeats dropped by a lane, a warp or a
+// block, and the rows left are packed.  (A radix sort of 64-bit keys over both
+// ids moves 16 bytes an entry six times for 2^21 vertices; here an entry is a
+// 4-byte id, placed once and sorted in shared memory.)  The result is the
+// paper's input format: symmetric, loop-free, duplicate-free, rows ascending.
+// Very many tuples or vertices take the radix sort: 64-bit keys (a << 32 | b)
+// and (b << 32 | a), least significant 8-bit digits first, only the digits that
+// can be nonzero; col = low halves of the distinct keys, row_ptr from the run
+// boundaries of the high halves.
 #include <algorithm>
 
 #include "pipeline.cuh"
+#include "warp_sort.cuh"
 
 namespace tc {
 namespace {
@@ -149,6 +156,333 @@ __global__ void k_empty_rowptr(uint32_t n, uint64_t *__restrict__ rp) {
     for (uint64_t v = (uint64_t)blockIdx.x * blockDim.x + threadIdx.x; v <= n; v += stride) rp[v] = 0;
 }
 
+// ---------------------------------------------------------------------------- rows by counting
+
+constexpr uint32_t kLaneRow = 32;      // entries of a row sorted by one lane
+constexpr uint32_t kWarpRow = 1024;    // by its warp
+constexpr uint32_t kBlockRow = 8192;   // by a block; longer rows go through bitmaps
+constexpr int kRowThreads = 256;
+constexpr uint32_t kMapBits = 1u << 20;  // ids a bitmap covers (128 KB of shared memory)
+constexpr uint32_t kNoPlace = 0xFFFFFFFFu;
+
+// Entries before a vertex's newest one, one atomic per distinct vertex of the
+// warp when neighbouring lanes meet on one (a hub named by most tuples).
+__device__ __forceinline__ uint32_t take_place(uint32_t *cnt, uint32_t v, bool on) {
+    const uint32_t w = on ? v : 0xFFFFFFFFu - lane_id();  // lanes without a vertex differ from all
+    const bool met = __shfl_xor_sync(0xFFFFFFFFu, w, 1) == w;
+    if (!__any_sync(0xFFFFFFFFu, met)) return on ? atomicAdd(&cnt[v], 1u) : 0u;
+    const unsigned peers = __match_any_sync(0xFFFFFFFFu, w), leader = __ffs(peers) - 1;
+    uint32_t at = 0;
+    if (on && lane_id() == leader) at = atomicAdd(&cnt[v], (unsigned)__popc(peers));
+    at = __shfl_sync(0xFFFFFFFFu, at, leader);
+    return at + __popc(peers & ((1u << lane_id()) - 1u));
+}
+
+__global__ void k_count_entries(uint64_t t, const uint32_t *__restrict__ src, const uint32_t *__restrict__ dst,
+                                uint32_t n, uint32_t *__restrict__ cnt, uint32_t *__restrict__ place_a,
+                                uint32_t *__restrict__ place_b, Ctl *ctl) {
+    const uint64_t stride = (uint64_t)gridDim.x * blockDim.x;
+    const uint64_t t_round = (t + 31) & ~uint64_t(31);
+    for (uint64_t i = (uint64_t)blockIdx.x * blockDim.x + threadIdx.x; i < t_round; i += stride) {
+        uint32_t a = 0, b = 0;
+        bool keep = false;
+        if (i < t) {
+            a = src[i];
+            b = dst[i];
+            if (a >= n || b >= n) ctl->error = 1;
+            else keep = a != b;
+        }
+        const uint32_t pa = take_place(cnt, a, keep), pb = take_place(cnt, b, keep);
+        if (i < t) {
+            place_a[i] = keep ? pa : kNoPlace;
+            place_b[i] = keep ? pb : kNoPlace;
+        }
+    }
+}
+
+__global__ void k_place_entries(uint64_t t, const uint32_t *__restrict__ src, const uint32_t *__restrict__ dst,
+                                const uint64_t *__restrict__ start, const uint32_t *__restrict__ place_a,
+                                const uint32_t *__restrict__ place_b, uint32_t *__restrict__ raw) {
+    const uint64_t stride = (uint64_t)gridDim.x * blockDim.x;
+    for (uint64_t i = (uint64_t)blockIdx.x * blockDim.x + threadIdx.x; i < t; i += stride) {
+        const uint32_t pa = place_a[i], pb = place_b[i];
+        if (pa == kNoPlace) continue;
+        const uint32_t a = src[i], b = dst[i];
+        raw[start[a] + pa] = b;
+        raw[start[b] + pb] = a;
+    }
+}
+
+// Rows of up to kWarpRow entries: sorted in place, repeats dropped; deg[v] =
+// entries left.  Longer rows are listed for a block each, or for the bitmaps.
+// Lanes own rows of up to kLaneRow entries (insertion sort in their column of
+// the warp's buffer), the warp takes the others one by one.
+__global__ void __launch_bounds__(kRowThreads) k_sort_rows(uint32_t n, const uint64_t *__restrict__ start,
+                                                           uint32_t *__restrict__ raw, uint32_t *__restrict__ deg,
+                                                           uint32_t *__restrict__ big, uint32_t *__restrict__ huge,
+                                                           uint32_t per_warp, Ctl *ctl) {
+    __shared__ __align__(16) uint32_t sbuf[kRowThreads / 32][kWarpRow];
+    const unsigned lane = lane_id(), warp = threadIdx.x >> 5;
+    const unsigned lt = (1u << lane) - 1u;
+    uint32_t *buf = sbuf[warp];
+    uint32_t top = 0;
+    const uint64_t chunks = ((uint64_t)n + per_warp - 1) / per_warp;
+    for (;;) {
+        unsigned int c = 0;
+        if (lane == 0) c = atomicAdd(&ctl->fill_next, 1u);
+        c = __shfl_sync(0xFFFFFFFFu, c, 0);
+        if (c >= chunks) break;
+        const uint64_t x = (uint64_t)c * per_warp + lane;
+        const bool valid = lane < per_warp && x < n;
+        const uint64_t b = valid ? start[x] : 0;
+        const uint64_t d64 = valid ? start[x + 1] - b : 0;
+        const uint32_t d = (uint32_t)d64;
+        if (valid && d <= kLaneRow) {
+            uint32_t k = 0;
+            for (uint32_t j0 = 0; j0 < d; j0 += 8) {
+                uint32_t y[8];
+#pragma unroll
+                for (uint32_t t = 0; t < 8; ++t) y[t] = j0 + t < d ? raw[b + j0 + t] : 0u;
+#pragma unroll
+                for (uint32_t t = 0; t < 8; ++t) {
+                    if (j0 + t >= d) break;
+                    uint32_t i = k;
+                    while (i > 0 && buf[(i - 1) * 32 + lane] > y[t]) --i;
+                    if (i > 0 && buf[(i - 1) * 32 + lane] == y[t]) continue;  // a repeat
+                    for (uint32_t m = k; m > i; --m) buf[m * 32 + lane] = buf[(m - 1) * 32 + lane];
+                    buf[i * 32 + lane] = y[t];
+                    ++k;
+                }
+            }
+            for (uint32_t i = 0; i < k; ++i) raw[b + i] = buf[i * 32 + lane];
+            deg[x] = k;
+            top = k > top ? k : top;
+        }
+        __syncwarp();
+        if (valid && d > kWarpRow) {
+            if (d <= kBlockRow) big[atomicAdd(&ctl->n_big, 1u)] = (uint32_t)x;
+            else huge[atomicAdd(&ctl->n_huge, 1u)] = (uint32_t)x;
+        }
+        unsigned pending = __ballot_sync(0xFFFFFFFFu, valid && d > kLaneRow && d <= kWarpRow);
+        while (pending) {
+            const int src = __ffs(pending) - 1;
+            pending &= pending - 1;
+            const uint32_t bd = __shfl_sync(0xFFFFFFFFu, d, src);
+            const uint64_t bb = __shfl_sync(0xFFFFFFFFu, b, src);
+            for (uint32_t j = lane; j < bd; j += 32) buf[j] = raw[bb + j];
+            __syncwarp();
+            warp_sort_any(buf, bd);
+            uint32_t k = 0;
+            for (uint32_t j0 = 0; j0 < bd; j0 += 32) {
+                const uint32_t j = j0 + lane;
+                const bool keep = j < bd && (j == 0 || buf[j] != buf[j - 1]);
+                const unsigned m = __ballot_sync(0xFFFFFFFFu, keep);
+                if (keep) raw[bb + k + __popc(m & lt)] = buf[j];
+                k += __popc(m);
+            }
+            if (lane == 0) deg[(uint64_t)c * per_warp + src] = k;
+            top = k > top ? k : top;
+            __syncwarp();
+        }
+    }
+    top = __reduce_max_sync(0xFFFFFFFFu, top);
+    if (lane == 0 && top) atomicMax(&ctl->max_s2, top);
+}
+
+// Exclusive position of this thread's flag among the block's (all threads; two barriers).
+__device__ __forceinline__ uint32_t block_rank(bool flag, uint32_t *warp_cnt, uint32_t *total) {
+    const unsigned lane = lane_id(), warp = threadIdx.x >> 5, nw = blockDim.x >> 5;
+    const unsigned m = __ballot_sync(0xFFFFFFFFu, flag);
+    if (lane == 0) warp_cnt[warp] = __popc(m);
+    __syncthreads();
+    uint32_t v = lane < nw ? warp_cnt[lane] : 0u, incl = v;
+#pragma unroll
+    for (int o = 1; o < 32; o <<= 1) {
+        const uint32_t y = __shfl_up_sync(0xFFFFFFFFu, incl, o);
+        if (lane >= (unsigned)o) incl += y;
+    }
+    const uint32_t before = __shfl_sync(0xFFFFFFFFu, incl - v, warp);
+    *total = __shfl_sync(0xFFFFFFFFu, incl, 31);
+    __syncthreads();
+    return before + __popc(m & ((1u << lane) - 1u));
+}
+
+// Rows of kWarpRow + 1 .. kBlockRow entries: a block each sorts the row in
+// shared memory and writes its distinct entries back.  Its warps sort runs of
+// 1024 in registers; a merge starts with a mirrored compare over the block (both
+// runs ascending), and its steps below 1024 are the warps' own again, so a row of
+// 8192 meets 12 barriers instead of the 91 of a plain bitonic network (R-MAT 21:
+// 1.00 -> 0.42 ms for all these rows).
+__device__ __forceinline__ void compare_swap(uint32_t *sb, uint32_t i, uint32_t l) {
+    const uint32_t u = sb[i], w = sb[l];
+    if (u > w) {
+        sb[i] = w;
+        sb[l] = u;
+    }
+}
+
+__global__ void __launch_bounds__(256) k_sort_rows_big(const uint64_t *__restrict__ start, uint32_t *__restrict__ raw,
+                                                       uint32_t *__restrict__ deg, const uint32_t *__restrict__ big,
+                                                       Ctl *ctl) {
+    __shared__ __align__(16) uint32_t sb[kBlockRow];
+    __shared__ uint32_t warp_cnt[32];
+    __shared__ unsigned int s_i;
+    const unsigned lane = lane_id(), warp = threadIdx.x >> 5;
+    uint32_t *run = sb + 1024 * warp;  // eight warps, 1024 keys each
+    const uint32_t nb = ctl->n_big;
+    for (;;) {
+        if (threadIdx.x == 0) s_i = atomicAdd(&ctl->sort_next, 1u);
+        __syncthreads();
+        const uint32_t i = s_i;
+        if (i >= nb) break;
+        const uint32_t x = big[i];
+        const uint64_t b = start[x];
+        const uint32_t d = (uint32_t)(start[x + 1] - b);
+        uint32_t P = 2048;
+        while (P < d) P <<= 1;
+        const bool mine = 1024 * warp < P;
+        const uint32_t left = d > 1024 * warp ? d - 1024 * warp : 0u;
+        if (mine) {
+            for (uint32_t t = lane; t < 1024; t += 32) run[t] = t < left ? raw[b + 1024 * warp + t] : kEmpty;
+            __syncwarp();
+            warp_sort_large(run, left < 1024 ? left : 1024u, 1024u);
+        }
+        for (uint32_t k = 2048; k <= P; k <<= 1) {
+            __syncthreads();
+            for (uint32_t p = threadIdx.x; p < P / 2; p += blockDim.x) {  // mirrored halves of every k keys
+                const uint32_t base = (p / (k / 2)) * k, o = p & (k / 2 - 1);
+                compare_swap(sb, base + o, base + k - 1 - o);
+            }
+            for (uint32_t j = k / 4; j >= 1024; j >>= 1) {
+                __syncthreads();
+                for (uint32_t p = threadIdx.x; p < P / 2; p += blockDim.x) {
+                    const uint32_t e = ((p & ~(j - 1)) << 1) | (p & (j - 1));
+                    compare_swap(sb, e, e | j);
+                }
+            }
+            __syncthreads();
+            if (mine) {
+                for (uint32_t j = 512; j >= 256; j >>= 1) {
+                    for (uint32_t p = lane; p < 512; p += 32) {
+                        const uint32_t e = ((p & ~(j - 1)) << 1) | (p & (j - 1));
+                        compare_swap(run, e, e | j);
+                    }
+                    __syncwarp();
+                }
+                for (uint32_t c = 0; c < 1024; c += 256) warp_merge_256(run + c, false);
+            }
+        }
+        __syncthreads();
+        uint32_t kept = 0;
+        for (uint32_t j0 = 0; j0 < d; j0 += blockDim.x) {
+            const uint32_t j = j0 + threadIdx.x;
+            const bool keep = j < d && (j == 0 || sb[j] != sb[j - 1]);
+            uint32_t total;
+            const uint32_t at = block_rank(keep, warp_cnt, &total);
+            if (keep) raw[b + kept + at] = sb[j];
+            kept += total;
+        }
+        if (threadIdx.x == 0) {
+            deg[x] = kept;
+            atomicMax(&ctl->max_s2, kept);
+        }
+        __syncthreads();
+    }
+}
+
+// Longer rows: one block per (row, range of kMapBits ids) marks the row's ids of
+// its range in a bitmap.  kEmit = false counts them (parts, deg); kEmit = true,
+// once the rows' places are known, writes them out in order.
+template <bool kEmit>
+__global__ void __launch_bounds__(1024) k_map_rows(uint32_t n, const uint64_t *__restrict__ start,
+                                                   const uint32_t *__restrict__ raw, const uint32_t *__restrict__ huge,
+                                                   uint32_t ranges, uint32_t *__restrict__ parts,
+                                                   uint32_t *__restrict__ deg, const uint64_t *__restrict__ rp,
+                                                   uint32_t *__restrict__ col, Ctl *ctl) {
+    extern __shared__ uint32_t map[];  // kMapBits bits
+    __shared__ uint32_t warp_cnt[32];
+    const unsigned lane = lane_id(), warp = threadIdx.x >> 5;
+    const uint64_t units = (uint64_t)ctl->n_huge * ranges;
+    for (uint64_t unit = blockIdx.x; unit < units; unit += gridDim.x) {
+        const uint32_t x = huge[unit / ranges], range = (uint32_t)(unit % ranges), lo = range * kMapBits;
+        const uint64_t b = start[x], e = start[x + 1];
+        const uint32_t words = (min(n - lo, kMapBits) + 31) / 32;
+        for (uint32_t i = threadIdx.x; i < words; i += blockDim.x) map[i] = 0;
+        __syncthreads();
+        for (uint64_t j = b + threadIdx.x; j < e; j += blockDim.x) {
+            const uint32_t y = raw[j] - lo;
+            if (y < kMapBits) atomicOr(&map[y >> 5], 1u << (y & 31u));
+        }
+        __syncthreads();
+        // every thread owns a run of words: its ids come after those of the threads before
+        const uint32_t per = (words + blockDim.x - 1) / blockDim.x, w0 = threadIdx.x * per;
+        uint32_t mine = 0;
+        for (uint32_t i = w0; i < min(w0 + per, words); ++i) mine += __popc(map[i]);
+        uint32_t incl = mine;
+#pragma unroll
+        for (int o = 1; o < 32; o <<= 1) {
+            const uint32_t y = __shfl_up_sync(0xFFFFFFFFu, incl, o);
+            if (lane >= (unsigned)o) incl += y;
+        }
+        if (lane == 31) warp_cnt[warp] = incl;
+        __syncthreads();
+        uint32_t v = warp_cnt[lane], wi = v;
+#pragma unroll
+        for (int o = 1; o < 32; o <<= 1) {
+            const uint32_t y = __shfl_up_sync(0xFFFFFFFFu, wi, o);
+            if (lane >= (unsigned)o) wi += y;
+        }
+        const uint32_t before = __shfl_sync(0xFFFFFFFFu, wi - v, warp), total = __shfl_sync(0xFFFFFFFFu, wi, 31);
+        if constexpr (kEmit) {
+            uint64_t at = rp[x] + before + incl - mine;
+            for (uint32_t r = 0; r < range; ++r) at += parts[unit - range + r];
+            for (uint32_t i = w0; i < min(w0 + per, words); ++i)
+                for (uint32_t m = map[i]; m; m &= m - 1) col[at++] = lo + 32 * i + __ffs(m) - 1;
+        } else if (threadIdx.x == 0) {
+            parts[unit] = total;
+            atomicMax(&ctl->max_s2, atomicAdd(&deg[x], total) + total);
+        }
+        __syncthreads();
+    }
+}
+
+// The sorted rows (bitmap rows aside) into their final places: a warp flattens
+// the entries of 32 rows, one per lane and step (their places are contiguous).
+__global__ void __launch_bounds__(256) k_pack_rows(uint32_t n, const uint64_t *__restrict__ start,
+                                                   const uint32_t *__restrict__ raw, const uint64_t *__restrict__ rp,
+                                                   uint32_t *__restrict__ col) {
+    const unsigned lane = lane_id();
+    const uint64_t warps = ((uint64_t)gridDim.x * blockDim.x) >> 5, groups = ((uint64_t)n + 31) / 32;
+    for (uint64_t g = ((uint64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5; g < groups; g += warps) {
+        const uint64_t x = g * 32 + lane;
+        uint64_t b = 0, to = 0;
+        uint32_t d = 0;
+        if (x < n) {
+            b = start[x];
+            to = rp[x];
+            d = (uint32_t)(rp[x + 1] - to);
+            if (start[x + 1] - b > kBlockRow) d = 0;
+        }
+        uint32_t incl = d;
+#pragma unroll
+        for (int o = 1; o < 32; o <<= 1) {
+            const uint32_t y = __shfl_up_sync(0xFFFFFFFFu, incl, o);
+            if (lane >= (unsigned)o) incl += y;
+        }
+        const uint32_t total = __shfl_sync(0xFFFFFFFFu, incl, 31);
+        const uint64_t from0 = b - (incl - d), to0 = to - (incl - d);  // minus the row's first flat position
+        for (uint32_t e0 = 0; e0 < total; e0 += 32) {
+            const uint32_t e = e0 + lane;
+            uint32_t r = 0;  // the row of flat position e: the first whose inclusive count passes it
+#pragma unroll
+            for (int o = 16; o > 0; o >>= 1)
+                if (__shfl_sync(0xFFFFFFFFu, incl, r + o - 1) <= e) r += o;
+            const uint64_t f = __shfl_sync(0xFFFFFFFFu, from0, r), w = __shfl_sync(0xFFFFFFFFu, to0, r);
+            if (e < total) col[w + e] = raw[f + e];
+        }
+    }
+}
+
 // Well-formedness: monotone row_ptr ending at `slots`, ids < n, rows strictly
 // ascending (no repeats), no self-loops, and every (v, w) has its (w, v).
 __global__ void k_validate(uint32_t n, const uint64_t *__restrict__ rp, const uint32_t *__restrict__ col,
@@ -237,8 +571,109 @@ uint32_t radix_sort_u64(unsigned long long **cur, unsigned long long **alt, uint
     return launches;
 }
 
+// Tuples and vertices the counting build takes: 32-bit places, at most 64 bitmap ranges.
+constexpr uint64_t kCountTuples = 1ull << 31;
+constexpr uint32_t kCountN = 1u << 26;
+
+static tc_status build_csr_counting(tc_ctx *ctx, uint32_t n, uint64_t t, const uint32_t *d_src, const uint32_t *d_dst,
+                                    uint64_t **rp_out, uint32_t **col_out, uint64_t *slots_out, bool *pooled_out,
+                                    uint32_t *max_deg) {
+    cudaStream_t s = ctx->stream;
+    const unsigned cap = (unsigned)ctx->num_sms * 16u;
+    const uint32_t ranges = (n + kMapBits - 1) / kMapBits;
+    const uint64_t max_huge = 2 * t / kBlockRow + 1;  // rows of more than kBlockRow entries
+    auto r = [](size_t b) { return (b + 255) & ~size_t(255); };
+    const size_t n1 = (size_t)n + 1;
+    const size_t need = 4 * r(4 * n1) + r(8 * n1) + 2 * r(4 * t) + r(8 * t) + r(4 * max_huge * ranges) +
+                        r(8 * scan_tmp_elems(n1)) + 4096;
+    tc_status st = arena_reserve(ctx, need);
+    if (st != TC_OK) return st;
+    Arena &a = ctx->arena;
+    a.reset();
+    auto *cnt = a.take<uint32_t>(n1);
+    auto *deg = a.take<uint32_t>(n1);
+    auto *big = a.take<uint32_t>(n1);
+    auto *huge = a.take<uint32_t>(n1);
+    auto *start = a.take<uint64_t>(n1);
+    auto *place_a = a.take<uint32_t>(t);
+    auto *place_b = a.take<uint32_t>(t);
+    auto *raw = a.take<uint32_t>(2 * t);
+    auto *parts = a.take<uint32_t>(max_huge * ranges);
+    auto *tmp = a.take<uint64_t>(scan_tmp_elems(n1));
+    if (!cnt || !deg || !big || !huge || !start || !place_a || !place_b || !raw || !parts || !tmp)
+        return set_error(ctx, TC_ERR_OOM, "arena carve failed (build_csr)");
+    uint64_t *rp = nullptr;
+    uint32_t *col = nullptr;
+    bool pooled = false, pooled2 = false;
+    if (graph_alloc(ctx, (void **)&rp, sizeof(uint64_t) * n1, &pooled) != cudaSuccess) {
+        cudaGetLastError();
+        return set_error(ctx, TC_ERR_OOM, "tc_build_csr: row_ptr allocation failed");
+    }
+    *pooled_out = pooled;
+    k_ctl_zero<<<1, 128, 0, s>>>(ctx->d_ctl);
+    cudaError_t e = cudaMemsetAsync(cnt, 0, 4 * n1, s);
+    if (e == cudaSuccess) e = cudaMemsetAsync(deg, 0, 4 * n1, s);
+    k_count_entries<<<grid_for(t, 256, cap), 256, 0, s>>>(t, d_src, d_dst, n, cnt, place_a, place_b, ctx->d_ctl);
+    scan_u32_to_u64(cnt, start, n, tmp, s);
+    k_place_entries<<<grid_for(t, 256, cap), 256, 0, s>>>(t, d_src, d_dst, start, place_a, place_b, raw);
+    const uint32_t per_warp = n >= (1u << 20) ? 32u : n >= (1u << 18) ? 16u : 8u;  // long rows of small graphs spread out
+    k_sort_rows<<<grid_for((uint64_t)n * (32 / per_warp), kRowThreads, cap), kRowThreads, 0, s>>>(n, start, raw, deg, big,
+                                                                                               huge, per_warp, ctx->d_ctl);
+    const bool bigs = 2 * t > kWarpRow, huges = 2 * t > kBlockRow;  // there may be some
+    const int map_smem = (int)(kMapBits / 8);
+    if (bigs) k_sort_rows_big<<<(unsigned)ctx->num_sms * 6u, 256, 0, s>>>(start, raw, deg, big, ctx->d_ctl);
+    if (huges) {
+        if (e == cudaSuccess)
+            e = cudaFuncSetAttribute(k_map_rows<false>, cudaFuncAttributeMaxDynamicSharedMemorySize, map_smem);
+        if (e == cudaSuccess)
+            e = cudaFuncSetAttribute(k_map_rows<true>, cudaFuncAttributeMaxDynamicSharedMemorySize, map_smem);
+        k_map_rows<false><<<(unsigned)ctx->num_sms, 1024, map_smem, s>>>(n, start, raw, huge, ranges, parts, deg, nullptr,
+                                                                        nullptr, ctx->d_ctl);
+    }
+    scan_u32_to_u64(deg, rp, n, tmp, s);
+    uint64_t U = 0;
+    if (e == cudaSuccess) e = cudaGetLastError();
+    if (e == cudaSuccess) e = cudaMemcpyAsync(&U, rp + n, sizeof(uint64_t), cudaMemcpyDeviceToHost, s);
+    if (e != cudaSuccess) {
+        graph_free(ctx, rp, pooled);
+        return cuda_error(ctx, e, "tc_build_csr kernels");
+    }
+    st = pull(ctx);
+    if (st == TC_OK && ctx->h_ctl->error) st = set_error(ctx, TC_ERR_INVALID, "tc_build_csr: a tuple names a vertex id >= n");
+    if (st != TC_OK) {
+        graph_free(ctx, rp, pooled);
+        return st;
+    }
+    *max_deg = ctx->h_ctl->max_s2;
+    if (graph_alloc(ctx, (void **)&col, sizeof(uint32_t) * (size_t)(U + 1), &pooled2) != cudaSuccess) {
+        cudaGetLastError();
+        graph_free(ctx, rp, pooled);
+        return set_error(ctx, TC_ERR_OOM, "tc_build_csr: col allocation failed");
+    }
+    if (U) {
+        k_pack_rows<<<grid_for(n, 256, cap), 256, 0, s>>>(n, start, raw, rp, col);
+        if (ctx->h_ctl->n_huge)
+            k_map_rows<true><<<(unsigned)ctx->num_sms, 1024, map_smem, s>>>(n, start, raw, huge, ranges, parts, deg, rp, col,
+                                                                           ctx->d_ctl);
+    }
+    e = cudaGetLastError();
+    if (e == cudaSuccess) e = cudaStreamSynchronize(s);
+    if (e != cudaSuccess) {
+        graph_free(ctx, rp, pooled);
+        graph_free(ctx, col, pooled2);
+        return cuda_error(ctx, e, "tc_build_csr kernels");
+    }
+    *rp_out = rp;
+    *col_out = col;
+    *slots_out = U;
+    return TC_OK;
+}
+
 tc_status build_csr_device(tc_ctx *ctx, uint32_t n, uint64_t t, const uint32_t *d_src, const uint32_t *d_dst,
-                           uint64_t **rp_out, uint32_t **col_out, uint64_t *slots_out, bool *pooled_out) {
+                           uint64_t **rp_out, uint32_t **col_out, uint64_t *slots_out, bool *pooled_out,
+                           uint32_t *max_deg) {
+    if (t && t < kCountTuples && n && n <= kCountN)
+        return build_csr_counting(ctx, n, t, d_src, d_dst, rp_out, col_out, slots_out, pooled_out, max_deg);
     cudaStream_t s = ctx->stream;
     const unsigned cap = (unsigned)ctx->num_sms * 16u;
     const uint64_t K = 2 * t;  // upper bound on keys
@@ -315,7 +750,7 @@ tc_status build_csr_device(tc_ctx *ctx, uint32_t n, uint64_t t, const uint32_t *
     *rp_out = rp;
     *col_out = col;
     *slots_out = U;
-    return TC_OK;
+    return max_degree_device(ctx, n, rp, max_deg);
 }
 
 tc_status validate_csr_device(tc_ctx *ctx, uint32_t n, const uint64_t *rp, const uint32_t *col, uint64_t slots,

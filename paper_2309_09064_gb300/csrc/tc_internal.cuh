@@ -208,7 +208,7 @@ size_t pipeline_bytes(const tc_ctx *ctx, uint32_t n, uint64_t slots, uint32_t ma
 // CSR construction / validation (csr.cu)
 tc_status build_csr_device(tc_ctx *ctx, uint32_t n, uint64_t t, const uint32_t *d_src,
                            const uint32_t *d_dst, uint64_t **rp_out, uint32_t **col_out,
-                           uint64_t *slots_out, bool *pooled_out);
+                           uint64_t *slots_out, bool *pooled_out, uint32_t *max_deg);
 tc_status validate_csr_device(tc_ctx *ctx, uint32_t n, const uint64_t *rp, const uint32_t *col,
                               uint64_t slots, int *ok);
 tc_status max_degree_device(tc_ctx *ctx, uint32_t n, const uint64_t *rp, uint32_t *max_deg);
