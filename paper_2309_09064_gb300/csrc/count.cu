@@ -38,7 +38,7 @@ size_t pipeline_bytes(const tc_ctx *ctx, uint32_t n, uint64_t slots, uint32_t ma
                       uint64_t *hub_words, uint32_t *hub_maps) {
     auto r = [](size_t b) { return (b + 255) & ~size_t(255); };
     const size_t n1 = (size_t)n + 1;
-    const uint64_t rtiles = radix_tiles(n1);
+    const uint64_t rtiles = radix_tiles_cap(n1);
     size_t bytes = 0;
     bytes += 21 * r(4 * n1);                       // deg q0 q1 fdeg R parent fcnt gcnt rank big huge lvp glo part rows[4] ntask[3]
     bytes += r(16 * n1);                           // vmeta
@@ -53,7 +53,7 @@ size_t pipeline_bytes(const tc_ctx *ctx, uint32_t n, uint64_t slots, uint32_t ma
     size_t own = r(4 * (slots / 32 + 2)) + r(8 * (slots / 2 + 1));
     if (plain && wedge_path(ctx, n, slots, max_deg)) {
         const WedgeSizes z = wedge_sizes(ctx, n, slots);
-        own = std::max(own, r(2 * (4 * slots + 8)) + r(4 * z.counts) + r(8 * (z.counts + 1)) + r(8ull * z.tiles) +
+        own = std::max(own, r(2 * (4 * slots + 8)) + r(8ull * z.tiles + 4 * z.counts) + r(8 * (z.counts + 1)) +
                                 r(16ull * z.tasks) + r(8 * z.tmp));
     }
     bytes += own;
@@ -147,7 +147,7 @@ tc_status count_pipeline(tc_ctx *ctx, const GraphView &g, uint32_t *levels_out, 
     b.lv = a.take<uint2>(n1);
     b.rkeys0 = a.take<unsigned long long>(n1);
     b.rkeys1 = a.take<unsigned long long>(n1);
-    const uint64_t rtiles = radix_tiles(n1);
+    const uint64_t rtiles = radix_tiles_cap(n1);
     b.rcounts = a.take<uint32_t>(256 * rtiles + 1);
     b.roffs = a.take<uint64_t>(256 * rtiles + 2);
     b.adj2 = a.take<uint32_t>(g.slots + 1);
@@ -168,12 +168,12 @@ tc_status count_pipeline(tc_ctx *ctx, const GraphView &g, uint32_t *levels_out, 
     if (wedge) {
         const WedgeSizes z = wedge_sizes(ctx, n, g.slots);
         b.wedge_ids = a.take<uint16_t>(4 * g.slots + 8);
-        b.wedge_counts = a.take<uint32_t>(z.counts);
+        b.wedge_work = reinterpret_cast<unsigned long long *>(a.take<char>(8ull * z.tiles + 4 * z.counts));
+        b.wedge_counts = reinterpret_cast<uint32_t *>(b.wedge_work + z.tiles);  // (zeroed together)
         b.wedge_offs = a.take<uint64_t>(z.counts + 1);
-        b.wedge_work = a.take<unsigned long long>(z.tiles);
         b.wedge_tasks = a.take<uint4>(z.tasks);
         b.wedge_tmp = a.take<uint64_t>(z.tmp);
-        ok = ok && b.wedge_ids && b.wedge_counts && b.wedge_offs && b.wedge_work && b.wedge_tasks && b.wedge_tmp;
+        ok = ok && b.wedge_ids && b.wedge_work && b.wedge_offs && b.wedge_tasks && b.wedge_tmp;
     }
     b.groups = groups;
     if (vertex_counts) {
@@ -219,7 +219,7 @@ tc_status count_pipeline(tc_ctx *ctx, const GraphView &g, uint32_t *levels_out, 
     TC_CUDA(ctx, cudaEventRecord(ctx->ev[1], s));
     // the packed 4-byte {rank, level} word needs ranks below 2^24 and levels below 255
     b.lvp = (n <= (1u << 24) && ctx->h_ctl->max_level < 255) ? lvp : nullptr;
-    st = compute_ranks(ctx, b, n, g.max_deg);
+    st = compute_ranks(ctx, b, n, g.max_deg, wedge ? wedge_tile_degree(n, g.max_deg) : kNoTiles);
     if (st != TC_OK) return st;
     Ctl counted{};                   // listing: the control block after phase 1
     unsigned long long list_tiny = 0;  // listing: triangles of the tiny rows

@@ -20,8 +20,13 @@ namespace tc {
 namespace {
 
 constexpr int kRsThreads = 256;
-constexpr int kRsItems = 16;
-constexpr uint64_t kRsTile = (uint64_t)kRsThreads * kRsItems;
+// Keys a thread takes: few of them for short arrays, whose tiles then fill the GPU
+// (65536 keys: a scatter takes a third of its 18 us).
+constexpr int kRsItems = 16, kRsItemsShort = 4;
+constexpr uint64_t kRsShort = 1u << 19;
+__host__ __device__ constexpr uint64_t rs_tile(uint64_t count) {
+    return (uint64_t)kRsThreads * (count <= kRsShort ? kRsItemsShort : kRsItems);
+}
 constexpr int kRsWarps = kRsThreads / 32;
 
 __global__ void k_make_keys(uint64_t t, const uint32_t *__restrict__ src, const uint32_t *__restrict__ dst, uint32_t n,
@@ -54,15 +59,16 @@ __global__ void k_make_keys(uint64_t t, const uint32_t *__restrict__ src, const 
 }
 
 // Per-tile digit histograms, digit-major: counts[d * nblocks + block].
+template <int kItems>
 __global__ void __launch_bounds__(kRsThreads) k_rs_hist(const unsigned long long *__restrict__ keys, uint64_t count,
                                                         int shift, uint32_t *__restrict__ counts, uint32_t nblocks) {
     __shared__ uint32_t h[kRsWarps][256];
     for (int i = threadIdx.x; i < kRsWarps * 256; i += kRsThreads) (&h[0][0])[i] = 0;
     __syncthreads();
     const unsigned warp = threadIdx.x >> 5;
-    const uint64_t base = (uint64_t)blockIdx.x * kRsTile;
+    const uint64_t base = (uint64_t)blockIdx.x * kRsThreads * kItems;
 #pragma unroll 4
-    for (int i = 0; i < kRsItems; ++i) {
+    for (int i = 0; i < kItems; ++i) {
         const uint64_t j = base + (uint64_t)i * kRsThreads + threadIdx.x;
         if (j < count) atomicAdd(&h[warp][(keys[j] >> shift) & 0xFF], 1u);
     }
@@ -79,6 +85,7 @@ __global__ void __launch_bounds__(kRsThreads) k_rs_hist(const unsigned long long
 // entries base + i*256 + t), so input order is (round, thread).  A key's rank
 // among equal digits = keys of that digit in earlier rounds + in earlier
 // warps of this round + in earlier lanes of its warp.
+template <int kItems>
 __global__ void __launch_bounds__(kRsThreads) k_rs_scatter(const unsigned long long *__restrict__ in,
                                                            unsigned long long *__restrict__ out, uint64_t count,
                                                            int shift, const unsigned long long *__restrict__ offs,
@@ -91,8 +98,8 @@ __global__ void __launch_bounds__(kRsThreads) k_rs_scatter(const unsigned long l
         running[d] = 0;
         start[d] = offs[(uint64_t)d * nblocks + blockIdx.x];
     }
-    const uint64_t base = (uint64_t)blockIdx.x * kRsTile;
-    for (int i = 0; i < kRsItems; ++i) {
+    const uint64_t base = (uint64_t)blockIdx.x * kRsThreads * kItems;
+    for (int i = 0; i < kItems; ++i) {
         for (int k = threadIdx.x; k < kRsWarps * 256; k += kRsThreads) (&wc[0][0])[k] = 0;
         __syncthreads();
         const uint64_t j = base + (uint64_t)i * kRsThreads + threadIdx.x;
@@ -554,13 +561,19 @@ tc_status pull(tc_ctx *ctx) {
 
 }  // namespace
 
-uint64_t radix_tiles(uint64_t count) { return (count + kRsTile - 1) / kRsTile; }
+uint64_t radix_tiles(uint64_t count) { return (count + rs_tile(count) - 1) / rs_tile(count); }
+uint64_t radix_tiles_cap(uint64_t count) {
+    return std::max(radix_tiles(count), radix_tiles(std::min<uint64_t>(count, kRsShort)));
+}
 
 uint32_t radix_sort_u64(unsigned long long **cur, unsigned long long **alt, uint64_t count, const int *shifts,
                         int nshifts, uint32_t *counts, uint64_t *coffs, uint64_t *tmp, cudaStream_t s) {
     if (count < 2) return 0;
     const uint32_t nblk = (uint32_t)radix_tiles(count);
     uint32_t launches = 0;
+    const bool few = count <= kRsShort;
+    auto k_rs_hist = few ? tc::k_rs_hist<kRsItemsShort> : tc::k_rs_hist<kRsItems>;
+    auto k_rs_scatter = few ? tc::k_rs_scatter<kRsItemsShort> : tc::k_rs_scatter<kRsItems>;
     for (int i = 0; i < nshifts; ++i) {
         k_rs_hist<<<nblk, kRsThreads, 0, s>>>(*cur, count, shifts[i], counts, nblk);
         launches += 2 + scan_u32_to_u64(counts, coffs, 256ull * nblk, tmp, s);
@@ -677,7 +690,7 @@ tc_status build_csr_device(tc_ctx *ctx, uint32_t n, uint64_t t, const uint32_t *
     cudaStream_t s = ctx->stream;
     const unsigned cap = (unsigned)ctx->num_sms * 16u;
     const uint64_t K = 2 * t;  // upper bound on keys
-    const uint64_t nblk_max = (K + kRsTile - 1) / kRsTile;
+    const uint64_t nblk_max = radix_tiles_cap(K);
     auto r = [](size_t b) { return (b + 255) & ~size_t(255); };
     const size_t need = 2 * r(8 * (K + 1)) + r(4 * (K + 1)) + r(8 * (K + 2)) + r(4 * (K + 1)) +
                         r(4 * (256 * nblk_max + 1)) + r(8 * (256 * nblk_max + 2)) +

@@ -71,6 +71,55 @@ __global__ void k_init(uint32_t n, const uint64_t *__restrict__ rp, uint32_t *__
     }
 }
 
+// Their exclusive prefix too, for a frontier one block can walk.
+constexpr uint32_t kPrefixOne = 32768;
+__global__ void __launch_bounds__(1024) k_prefix_deg(const uint32_t *__restrict__ q, uint32_t count,
+                                                     const uint32_t *__restrict__ deg,
+                                                     unsigned long long *__restrict__ out) {
+    __shared__ unsigned long long s_warp[32];
+    const unsigned lane = lane_id(), warp = threadIdx.x >> 5;
+    unsigned long long carry = 0;
+    for (uint32_t c = 0; c < count; c += 8192) {
+        uint32_t d[8];
+        unsigned long long sum = 0;
+#pragma unroll
+        for (int i = 0; i < 8; ++i) {
+            const uint32_t j = c + threadIdx.x * 8 + i;
+            d[i] = j < count ? q[j] : kUnvisited;
+        }
+#pragma unroll
+        for (int i = 0; i < 8; ++i) {
+            d[i] = d[i] != kUnvisited ? deg[d[i]] : 0u;
+            sum += d[i];
+        }
+        unsigned long long incl = sum;
+#pragma unroll
+        for (int o = 1; o < 32; o <<= 1) {
+            const unsigned long long y = __shfl_up_sync(0xFFFFFFFFu, incl, o);
+            if (lane >= (unsigned)o) incl += y;
+        }
+        if (lane == 31) s_warp[warp] = incl;
+        __syncthreads();
+        const unsigned long long w = s_warp[lane];
+        unsigned long long wi = w;
+#pragma unroll
+        for (int o = 1; o < 32; o <<= 1) {
+            const unsigned long long y = __shfl_up_sync(0xFFFFFFFFu, wi, o);
+            if (lane >= (unsigned)o) wi += y;
+        }
+        unsigned long long ex = carry + __shfl_sync(0xFFFFFFFFu, wi - w, warp) + incl - sum;
+#pragma unroll
+        for (int i = 0; i < 8; ++i) {
+            const uint32_t j = c + threadIdx.x * 8 + i;
+            if (j < count) out[j] = ex;
+            ex += d[i];
+        }
+        carry += __shfl_sync(0xFFFFFFFFu, wi, 31);
+        __syncthreads();
+    }
+    if (threadIdx.x == 0) out[count] = carry;
+}
+
 __global__ void k_gather_deg(const uint32_t *__restrict__ q, uint32_t count, const uint32_t *__restrict__ deg,
                              uint32_t *__restrict__ out) {
     const uint32_t stride = gridDim.x * blockDim.x;
@@ -297,6 +346,102 @@ __global__ void k_group_roots(GroupSpec groups, const uint32_t *__restrict__ deg
     }
 }
 
+// The components left after the first BFS, where they are small together: one
+// block hooks them, roots them and levels them (the steps of the kernels above
+// with block barriers between them, instead of ten launches and five round trips
+// to the host).  More than kResidualMax vertices, or one of degree above
+// kResidualDeg, are left to those.  Parents are read past L1: hooking changes them by atomics.
+constexpr uint32_t kResidualMax = 8192, kResidualDeg = 256;
+
+__device__ __forceinline__ uint32_t find_root_cg(const uint32_t *parent, uint32_t x, uint32_t n, Ctl *ctl) {
+    for (uint32_t it = 0; it <= n; ++it) {
+        const uint32_t p = __ldcg(parent + x);
+        if (p == x) return x;
+        x = p;
+    }
+    ctl->error = 2;
+    return x;
+}
+
+__global__ void __launch_bounds__(1024) k_residual(const uint32_t *__restrict__ R, uint32_t n,
+                                                   const uint64_t *__restrict__ rp, const uint32_t *__restrict__ col,
+                                                   const uint32_t *__restrict__ deg, uint32_t *parent, uint32_t *L,
+                                                   uint32_t *q0, uint32_t *q1, Ctl *ctl, uint32_t order) {
+    __shared__ unsigned int s_changed, s_count[2], s_roots;
+    __shared__ unsigned long long s_edges;
+    const uint32_t nr = ctl->n_residual;
+    if (nr == 0) return;
+    bool wide = nr > kResidualMax;  // a thread walks a vertex's neighbours: long rows are left too
+    for (uint32_t i = threadIdx.x; i < nr && !wide; i += blockDim.x) wide = deg[R[i]] > kResidualDeg;
+    if (__syncthreads_or(wide)) {
+        if (threadIdx.x == 0) ctl->residual_left = nr;
+        return;
+    }
+    for (uint32_t i = threadIdx.x; i < nr; i += blockDim.x) __stcg(parent + R[i], R[i]);
+    if (threadIdx.x == 0) {
+        s_count[0] = s_count[1] = s_roots = 0;
+        s_edges = 0;
+    }
+    for (int round = 0; round < 64; ++round) {
+        __syncthreads();
+        if (threadIdx.x == 0) s_changed = 0;
+        __syncthreads();
+        for (uint32_t i = threadIdx.x; i < nr; i += blockDim.x) {
+            const uint32_t v = R[i];
+            for (uint64_t j = rp[v]; j < rp[v + 1]; ++j) {
+                const uint32_t w = col[j];
+                if (w < v) continue;  // each undirected edge once
+                const uint32_t rv = find_root_cg(parent, v, n, ctl), rw = find_root_cg(parent, w, n, ctl);
+                if (rv == rw) continue;
+                const unsigned long long kv = order_key(rv, deg[rv], order), kw = order_key(rw, deg[rw], order);
+                const uint32_t hi = kv < kw ? rw : rv, lo = kv < kw ? rv : rw;
+                atomicCAS(&parent[hi], hi, lo);
+                s_changed = 1;
+            }
+        }
+        __syncthreads();
+        if (!s_changed) break;
+        for (uint32_t i = threadIdx.x; i < nr; i += blockDim.x) __stcg(parent + R[i], find_root_cg(parent, R[i], n, ctl));
+    }
+    if (s_changed && threadIdx.x == 0) ctl->error = 2;  // 64 rounds halve any path long before
+    unsigned long long edges = 0;
+    for (uint32_t i = threadIdx.x; i < nr; i += blockDim.x) {
+        const uint32_t v = R[i];
+        edges += deg[v];
+        if (__ldcg(parent + v) == v) {
+            atomicExch(&L[v], 0u);
+            __stcg(q0 + atomicAdd(&s_count[0], 1u), v);
+            atomicAdd(&s_roots, 1u);
+        }
+    }
+    if (edges) atomicAdd(&s_edges, edges);
+    uint32_t level = 0, p = 0;
+    for (;; ++level, p ^= 1u) {
+        __syncthreads();
+        const uint32_t fc = s_count[p];
+        if (fc == 0) break;
+        __syncthreads();
+        if (threadIdx.x == 0) s_count[p ^ 1u] = 0;
+        __syncthreads();
+        const uint32_t *q = p ? q1 : q0;
+        uint32_t *qn = p ? q0 : q1;
+        for (uint32_t i = threadIdx.x; i < fc; i += blockDim.x) {
+            const uint32_t v = __ldcg(q + i);
+            for (uint64_t j = rp[v]; j < rp[v + 1]; ++j) {
+                const uint32_t w = col[j];
+                if (__ldcg(L + w) == kUnvisited && atomicCAS(&L[w], kUnvisited, level + 1) == kUnvisited)
+                    __stcg(qn + atomicAdd(&s_count[p ^ 1u], 1u), w);
+            }
+        }
+    }
+    if (threadIdx.x == 0) {
+        ctl->components += s_roots;
+        ctl->visited += nr;
+        ctl->visited_edges += s_edges;
+        if (level > 0 && level - 1 > ctl->max_level) ctl->max_level = level - 1;
+    }
+}
+
 __global__ void k_count_roots(Ctl *ctl, int cur) {
     ctl->components += ctl->fr_count[cur];
     ctl->visited += ctl->fr_count[cur];
@@ -309,7 +454,11 @@ __global__ void k_reset_next(Ctl *ctl, int nxt) {
     ctl->bfs_spill = 0;
 }
 
+// Book the level just made and clear the counters of the one after it.
 __global__ void k_after_level(Ctl *ctl, int nxt, uint32_t level) {
+    const int after = nxt == 2 ? 0 : nxt + 1;
+    ctl->fr_count[after] = 0;
+    ctl->fr_edges[after] = 0;
     ctl->visited += ctl->fr_count[nxt];
     ctl->visited_edges += ctl->fr_edges[nxt];
     if (ctl->fr_count[nxt]) ctl->max_level = level + 1 > ctl->max_level ? level + 1 : ctl->max_level;
@@ -848,7 +997,7 @@ static tc_status bfs_loop(tc_ctx *ctx, const PipeBufs &b, uint32_t n, uint64_t s
     cudaStream_t s = ctx->stream;
     const unsigned cap = (unsigned)ctx->num_sms * 16u;
     uint32_t level = start_level;
-    bool bottom_up = false;
+    bool bottom_up = false, clear = false;
     tc_status st = TC_OK;
     uint32_t fcount = ctx->h_ctl->fr_count[slot];
     unsigned long long fedges = ctx->h_ctl->fr_edges[slot];
@@ -864,6 +1013,7 @@ static tc_status bfs_loop(tc_ctx *ctx, const PipeBufs &b, uint32_t n, uint64_t s
             st = launch_cluster(ctx, b, n, slots, false, fcount, queue, level);
             if (st == TC_OK) st = pull_ctl(ctx);
             if (st != TC_OK) return st;
+            clear = false;
             stuck = ctx->h_ctl->p_level == level;  // it could not take the frontier (one block's queue overflowed)
             slot = 0;
             queue = 0;
@@ -876,14 +1026,23 @@ static tc_status bfs_loop(tc_ctx *ctx, const PipeBufs &b, uint32_t n, uint64_t s
         stuck = false;
         uint32_t *q = queue ? b.q1 : b.q0;
         uint32_t *qn = queue ? b.q0 : b.q1;
-        k_reset_next<<<1, 1, 0, s>>>(ctx->d_ctl, (int)nxt);
-        note_launch(ctx, 2);  // reset + after-level bookkeeping
+        if (!clear) {  // k_after_level has done it for the later levels
+            k_reset_next<<<1, 1, 0, s>>>(ctx->d_ctl, (int)nxt);
+            note_launch(ctx);
+        }
+        clear = true;
+        note_launch(ctx);  // after-level bookkeeping
         if (bottom_up) {
             k_bu<<<grid_for(n, 256, cap), 256, 0, s>>>(n, b.rp, b.col, b.deg, b.L, qn, ctx->d_ctl, level, (int)nxt);
             note_launch(ctx);
         } else if (fedges > 0) {
-            k_gather_deg<<<grid_for(fcount, 256, cap), 256, 0, s>>>(q, fcount, b.deg, b.fdeg);
-            note_launch(ctx, 2 + scan_u32_to_u64(b.fdeg, b.fpref, fcount, b.scan_tmp, s));
+            if (fcount <= kPrefixOne) {
+                k_prefix_deg<<<1, 1024, 0, s>>>(q, fcount, b.deg, reinterpret_cast<unsigned long long *>(b.fpref));
+                note_launch(ctx, 2);
+            } else {
+                k_gather_deg<<<grid_for(fcount, 256, cap), 256, 0, s>>>(q, fcount, b.deg, b.fdeg);
+                note_launch(ctx, 2 + scan_u32_to_u64(b.fdeg, b.fpref, fcount, b.scan_tmp, s));
+            }
             k_td<<<grid_for((fedges + kTdTile - 1) / kTdTile, 1, cap), kTdThreads, 0, s>>>(
                 q, fcount, reinterpret_cast<const unsigned long long *>(b.fpref), b.rp, b.col, b.deg, b.L, qn,
                 ctx->d_ctl, level, (int)nxt);
@@ -956,10 +1115,13 @@ tc_status compute_levels(tc_ctx *ctx, const PipeBufs &b, uint32_t n, uint64_t sl
 
     // Remaining components: min-key roots by hooking, then a multi-source BFS.
     k_collect_unvisited<<<grid_for(n, 256, cap), 256, 0, s>>>(n, b.L, b.R, ctx->d_ctl);
-    note_launch(ctx);
+    k_residual<<<1, 1024, 0, s>>>(b.R, n, b.rp, b.col, b.deg, b.parent, b.L, b.q0, b.q1, ctx->d_ctl, ctx->opt.order);
+    note_launch(ctx, 2);
+    TC_CUDA(ctx, cudaGetLastError());
     st = pull_ctl(ctx);
     if (st != TC_OK) return st;
-    const uint32_t nr = ctx->h_ctl->n_residual;
+    if (ctx->h_ctl->error) return set_error(ctx, TC_ERR_INVALID, "connected-components walk did not end");
+    const uint32_t nr = ctx->h_ctl->residual_left;
     if (nr == 0) return TC_OK;
     k_cc_init<<<grid_for(nr, 256, cap), 256, 0, s>>>(b.R, nr, b.parent);
     note_launch(ctx);

@@ -143,7 +143,10 @@ tc_status compute_levels(tc_ctx *ctx, const PipeBufs &b, uint32_t n, uint64_t sl
 tc_status given_levels(tc_ctx *ctx, const PipeBufs &b, uint32_t n, const uint32_t *levels_in);
 tc_status selftest_barrier(tc_ctx *ctx, uint32_t timeout_ms);
 // rank of every vertex in the working order, packed with its level (lv)
-tc_status compute_ranks(tc_ctx *ctx, PipeBufs &b, uint32_t n, uint32_t max_deg);
+// (tile_deg: least degree of the wedge path's tile vertices, kNoTiles: none)
+constexpr uint32_t kNoTiles = 0xFFFFFFFFu;
+tc_status compute_ranks(tc_ctx *ctx, PipeBufs &b, uint32_t n, uint32_t max_deg, uint32_t tile_deg);
+uint32_t wedge_tile_degree(uint32_t n, uint32_t max_deg);
 // Listing: close the open chunks, then move the triangles written past the
 // first t_big positions into the gaps below it (list.cu).  g_end = the chunk
 // cursor after the listing pass.

@@ -98,6 +98,35 @@ __global__ void __launch_bounds__(kScanThreads) k_scan_tiles(const T *in, unsign
     if (blockIdx.x == gridDim.x - 1 && threadIdx.x == 0) out[count] = sums[blockIdx.x] + tot;
 }
 
+// The whole scan in one block (in place too), for counts where three launches
+// cost more than one block's walk over the values.
+constexpr uint64_t kOneBlock = 4 * kTile;
+template <class T>
+__global__ void __launch_bounds__(kScanThreads) k_scan_one(const T *in, unsigned long long *out, uint64_t count) {
+    unsigned long long carry = 0;
+    for (uint64_t c = 0; c < count; c += kTile) {
+        unsigned long long v[kScanItems];
+        unsigned long long s = 0;
+#pragma unroll
+        for (int i = 0; i < kScanItems; ++i) {
+            const uint64_t j = c + (uint64_t)threadIdx.x * kScanItems + i;
+            v[i] = j < count ? (unsigned long long)in[j] : 0ull;
+            s += v[i];
+        }
+        unsigned long long tot;
+        unsigned long long ex = carry + block_exclusive<T>(s, &tot);
+#pragma unroll
+        for (int i = 0; i < kScanItems; ++i) {
+            const uint64_t j = c + (uint64_t)threadIdx.x * kScanItems + i;
+            if (j < count) out[j] = ex;
+            ex += v[i];
+        }
+        carry += tot;
+        __syncthreads();
+    }
+    if (threadIdx.x == 0) out[count] = carry;
+}
+
 __global__ void k_zero_total(unsigned long long *out) { out[0] = 0ull; }
 
 template <class T>
@@ -109,6 +138,10 @@ uint32_t scan_impl(const T *in, uint64_t *out, uint64_t count, uint64_t *tmp, cu
     const uint64_t nb = (count + kTile - 1) / kTile;
     auto *sums = reinterpret_cast<unsigned long long *>(tmp);
     auto *o = reinterpret_cast<unsigned long long *>(out);
+    if (count <= kOneBlock) {
+        k_scan_one<T><<<1, kScanThreads, 0, s>>>(in, o, count);
+        return 1;
+    }
     k_tile_sums<T><<<(unsigned)nb, kScanThreads, 0, s>>>(in, count, sums);
     k_scan_sums<<<1, kScanThreads, 0, s>>>(sums, nb);
     k_scan_tiles<T><<<(unsigned)nb, kScanThreads, 0, s>>>(in, o, count, sums);

@@ -77,8 +77,10 @@ struct Ctl {
     unsigned int huge_next;          // k_row_fill_huge: next listed row a block takes
     unsigned int sort_next;          // k_sort_big: next listed row a block takes
     unsigned int split_next;         // k_g1_split: next listed row a block takes
-    unsigned int wedge_u, wedge_k;   // wedge path: vertices taken in tiles, ranks their words cover
-    unsigned int wedge_hi_task, wedge_pad;  // first task of the tiles from rank kWedgeMaxK on
+    unsigned int wedge_u;            // wedge path: vertices taken in tiles (a multiple of 32)
+    unsigned int wedge_hi_task;      // first task of the tiles from rank kWedgeMaxK on
+    unsigned int residual_left;      // vertices the one-block component step left to the host's loop
+    unsigned int pad;
     unsigned long long list_cursor;  // listing: next free chunk position
 };
 
@@ -173,8 +175,10 @@ uint32_t scan_u64(const uint64_t *in, uint64_t *out, uint64_t count, uint64_t *t
 // at shifts[0..nshifts) (least significant first); *cur holds the keys and on
 // return the sorted keys (the two buffers are swapped once per pass).  counts
 // needs 256 * radix_tiles(count) + 1 entries, coffs two more, tmp
-// scan_tmp_elems(256 * radix_tiles(count) + 1).  Returns the kernels launched.
+// scan_tmp_elems(256 * radix_tiles(count) + 1); radix_tiles_cap(count) is enough
+// for any number of keys up to count.  Returns the kernels launched.
 uint64_t radix_tiles(uint64_t count);
+uint64_t radix_tiles_cap(uint64_t count);
 uint32_t radix_sort_u64(unsigned long long **cur, unsigned long long **alt, uint64_t count, const int *shifts,
                         int nshifts, uint32_t *counts, uint64_t *coffs, uint64_t *tmp, cudaStream_t s);
 

@@ -59,22 +59,8 @@ __device__ __forceinline__ uint2 rank_level(const uint2 *__restrict__ lv, const 
     }
 }
 
-// U: the vertices of degree >= tile_deg (the working order starts with them), whole tiles, at most kWedgeMaxU; K = min(U, kWedgeMaxK).
-__global__ void k_wedge_limits(uint32_t n, const unsigned long long *__restrict__ order, uint32_t max_deg,
-                               uint32_t tile_deg, Ctl *ctl) {
-    uint32_t U = 0;
-    if (max_deg >= tile_deg) {
-        const uint32_t last = max_deg - tile_deg;  // largest key of a tile vertex
-        uint32_t lo = 0, hi = n < kWedgeMaxU ? n : kWedgeMaxU;
-        while (lo < hi) {
-            const uint32_t mid = (lo + hi) >> 1;
-            if ((uint32_t)(order[mid] >> 32) <= last) lo = mid + 1; else hi = mid;
-        }
-        U = (lo + 31u) & ~31u;
-    }
-    ctl->wedge_u = U;
-    ctl->wedge_k = U < kWedgeMaxK ? U : kWedgeMaxK;
-}
+// The first U ranks are taken in tiles (k_rank_scatter); their words cover the first K.
+__device__ __forceinline__ uint32_t words_of(uint32_t U) { return U < kWedgeMaxK ? U : kWedgeMaxK; }
 
 // What a row leaves behind besides its keys: |N(x)|, how many of them lie
 // below K and below U, and the row's place by rank.
@@ -112,7 +98,7 @@ __global__ void __launch_bounds__(kFillThreads) k_wedge_rows(uint32_t n, const u
     const unsigned lane = lane_id(), warp = threadIdx.x >> 5;
     const unsigned lt = (1u << lane) - 1u;
     uint32_t *buf = sbuf[warp];
-    const uint32_t K2 = 2 * ctl->wedge_k, U2 = 2 * ctl->wedge_u;  // a key below K2 has a rank below K
+    const uint32_t U2 = 2 * ctl->wedge_u, K2 = 2 * words_of(ctl->wedge_u);  // a key below K2 has a rank below K
     unsigned long long horizontal = 0;
     const uint64_t chunks = ((uint64_t)n + per_warp - 1) / per_warp;
     for (;;) {
@@ -309,7 +295,7 @@ __global__ void __launch_bounds__(1024) k_wedge_sort(const uint32_t *__restrict_
                                                      uint16_t *__restrict__ ids, RowOut out) {
     extern __shared__ uint32_t sb[];  // kSortCap keys
     __shared__ unsigned int s_i, s_lo, s_u;
-    const uint32_t nb = ctl->n_big, K2 = 2 * ctl->wedge_k, U2 = 2 * ctl->wedge_u;
+    const uint32_t nb = ctl->n_big, K2 = 2 * words_of(ctl->wedge_u), U2 = 2 * ctl->wedge_u;
     for (;;) {
         if (threadIdx.x == 0) {
             s_i = atomicAdd(&ctl->sort_next, 1u);
@@ -376,7 +362,7 @@ __global__ void __launch_bounds__(1024) k_wedge_sort(const uint32_t *__restrict_
 // those from K on.
 // Two launches make them tile by tile: kScatter = false counts every block's
 // entries per tile, kScatter = true writes them at the scanned offsets; a
-// block takes the same rows (a contiguous range) in both.  A warp flattens the keys of 32 rows, one per lane and step;
+// block takes the same rows (a contiguous range) in both.  A warp flattens the keys of per_warp rows, one per lane and step;
 // the last of the consecutive lanes of one row and tile makes their entries
 // (a tile that straddles two steps gets entries from both).
 template <bool kScatter>
@@ -388,7 +374,7 @@ __global__ void __launch_bounds__(1024) k_wedge_entries(uint32_t n, uint64_t slo
                                                         const unsigned long long *__restrict__ offs,
                                                         unsigned long long *__restrict__ work,
                                                         uint4 *__restrict__ entries, uint64_t cap, uint32_t tiles_cap,
-                                                        Ctl *ctl) {
+                                                        uint32_t per_warp, Ctl *ctl) {
     extern __shared__ uint32_t sm[];  // tiles_cap counts or cursors, then (counting) tiles_cap steps
     __shared__ uint32_t s_row[2], s_next;
     const unsigned lane = lane_id();
@@ -399,14 +385,19 @@ __global__ void __launch_bounds__(1024) k_wedge_entries(uint32_t n, uint64_t slo
         if (threadIdx.x == 0) atomicOr(&ctl->error, kGuardRange);
         return;
     }
-    if (threadIdx.x < 2) {  // rows are shared out by slots + rows (a long run of empty rows is spread too)
-        const uint64_t at = (slots + n) * (blockIdx.x + threadIdx.x) / nb;
-        uint32_t lo = 0, hi = n;
+    if (threadIdx.x < 64) {  // rows are shared out by slots + rows (a long run of empty rows is spread too)
+        const uint32_t end = threadIdx.x >> 5;  // one warp per end: 32 places tried at once
+        const uint64_t at = (slots + n) * (blockIdx.x + end) / nb;
+        uint32_t lo = 0, hi = n;  // the first row r with rp[r] + r >= at lies in [lo, hi]
         while (lo < hi) {
-            const uint32_t mid = lo + ((hi - lo) >> 1);
-            if (rp[mid] + mid < at) lo = mid + 1; else hi = mid;
+            const uint32_t step = (hi - lo + 31) / 32;
+            const uint64_t r = (uint64_t)lo + (uint64_t)step * lane;
+            const unsigned below = __ballot_sync(0xFFFFFFFFu, r < hi && rp[r] + r < at);
+            const uint32_t k = __popc(below);  // the places below it come first
+            hi = k == 0 ? lo : (uint32_t)min((uint64_t)hi, (uint64_t)lo + (uint64_t)step * k);
+            if (k) lo = lo + step * (k - 1) + 1;
         }
-        s_row[threadIdx.x] = blockIdx.x + threadIdx.x == nb ? n : lo;
+        if (lane == 0) s_row[end] = blockIdx.x + end == nb ? n : lo;
     }
     if (threadIdx.x == 0) s_next = 0;
     for (uint32_t t = threadIdx.x; t < tiles; t += blockDim.x) {
@@ -418,13 +409,13 @@ __global__ void __launch_bounds__(1024) k_wedge_entries(uint32_t n, uint64_t slo
     unsigned long long probes = 0;
     for (;;) {
         uint32_t g = 0;
-        if (lane == 0) g = atomicAdd(&s_next, 32u);
+        if (lane == 0) g = atomicAdd(&s_next, per_warp);
         g = __shfl_sync(0xFFFFFFFFu, g, 0);
         if (row_lo + g >= row_hi || g >= row_hi - row_lo) break;
         const uint32_t x = row_lo + g + lane;
         uint32_t d = 0, nlo = 0;
         uint64_t b = 0;
-        if (x < row_hi) {
+        if (lane < per_warp && x < row_hi) {
             d = dcnt[x];
             nlo = lcnt[x];
             if (d < 2) d = 0;
@@ -922,7 +913,8 @@ __global__ void __launch_bounds__(kRestThreads) k_wedge_rest(uint32_t n, const u
                                                              const uint32_t *__restrict__ keys,
                                                              const uint32_t *__restrict__ dcnt,
                                                              const uint32_t *__restrict__ ucnt,
-                                                             const uint4 *__restrict__ rmeta, Ctl *ctl) {
+                                                             const uint4 *__restrict__ rmeta, uint32_t per_warp,
+                                                             Ctl *ctl) {
     __shared__ uint32_t sfilter[kRestThreads / 32][kFilterBits / 32];
     const unsigned lane = lane_id(), warp = threadIdx.x >> 5;
     const uint32_t sub = lane & 7u, group = lane >> 3;
@@ -931,7 +923,7 @@ __global__ void __launch_bounds__(kRestThreads) k_wedge_rest(uint32_t n, const u
     __syncwarp();
     unsigned long long same = 0, cross = 0, probes = 0;
     uint32_t done = 0;
-    const uint64_t chunks = ((uint64_t)n + 31) / 32;
+    const uint64_t chunks = ((uint64_t)n + per_warp - 1) / per_warp;
     const long long t_start = clock64();
     for (;;) {
         unsigned int c = 0;
@@ -944,10 +936,10 @@ __global__ void __launch_bounds__(kRestThreads) k_wedge_rest(uint32_t n, const u
         }
         c = __shfl_sync(0xFFFFFFFFu, c, 0);
         if (c >= chunks) break;
-        const uint64_t x = (uint64_t)c * 32 + lane;
+        const uint64_t x = (uint64_t)c * per_warp + lane;
         uint32_t d = 0, nu = 0;  // keys, and those below U
         uint64_t b = 0;
-        if (x < n) {
+        if (lane < per_warp && x < n) {
             d = dcnt[x];
             nu = ucnt[x];
             if (d < 2 || d == nu) d = 0;
@@ -1031,7 +1023,10 @@ unsigned grid_for(uint64_t work, unsigned threads, unsigned cap) {
     return (unsigned)b;
 }
 
-uint32_t tiles_cap(uint32_t n) { return std::min(kWedgeMaxU, n) / 32 + 1; }
+// Tiles there can be (a tile vertex has degree 64 at least).
+uint32_t tiles_cap(uint32_t n, uint64_t slots) {
+    return (uint32_t)std::min<uint64_t>(std::min(kWedgeMaxU, n), slots / 64 + 32) / 32 + 1;
+}
 
 // Least degree of a tile vertex.  A tile costs its words' build (about 5 us of
 // one SM) and saves its vertices' rows from k_wedge_rest: with 64 instead of 128
@@ -1043,20 +1038,28 @@ uint32_t tile_degree(uint32_t n) { return n < (1u << 20) ? 64u : 128u; }
 // degree 32 would make a single tile: 2.02 instead of 1.87 ms).
 constexpr uint32_t kTilesFrom = 128;
 
+// Vertices a warp takes at a time: fewer in small graphs, where the rows of one
+// warp's chunk would hold up everything (R-MAT 10: k_wedge_rest 78 us at 32).
+uint32_t rows_per_warp(uint32_t n) {
+    return n >= (1u << 20) ? 32u : n >= (1u << 18) ? 16u : n >= (1u << 15) ? 8u : 2u;
+}
+
 // Blocks of the entry kernels: a row range each.
 uint32_t entry_blocks(const tc_ctx *ctx, uint64_t slots) {
     return (uint32_t)std::min<uint64_t>(2ull * ctx->num_sms, slots / 4096 + 1);
 }
 
-uint32_t tasks_cap(const tc_ctx *ctx, uint32_t n) { return tiles_cap(n) + (uint32_t)ctx->num_sms * kTasksPerSm + 1; }
+uint32_t tasks_cap(const tc_ctx *ctx, uint32_t n, uint64_t slots) { return tiles_cap(n, slots) + (uint32_t)ctx->num_sms * kTasksPerSm + 1; }
 
 }  // namespace
 
+uint32_t wedge_tile_degree(uint32_t n, uint32_t max_deg) { return max_deg >= kTilesFrom ? tile_degree(n) : kNoTiles; }
+
 WedgeSizes wedge_sizes(const tc_ctx *ctx, uint32_t n, uint64_t slots) {
     WedgeSizes z;
-    z.tiles = tiles_cap(n);
+    z.tiles = tiles_cap(n, slots);
     z.counts = (uint64_t)z.tiles * entry_blocks(ctx, slots);
-    z.tasks = tasks_cap(ctx, n);
+    z.tasks = tasks_cap(ctx, n, slots);
     z.tmp = scan_tmp_elems(z.counts + 1);
     return z;
 }
@@ -1075,11 +1078,9 @@ tc_status wedge_rows(tc_ctx *ctx, const PipeBufs &b, uint32_t n, uint32_t max_de
     cudaStream_t s = ctx->stream;
     const unsigned cap = (unsigned)ctx->num_sms * 16u;
     uint16_t *ids = b.wedge_ids;
-    uint32_t launches = 2;
+    uint32_t launches = 1;
     const RowOut out{b.fcnt, b.gcnt, b.glo, b.vmeta};
-    // warps of small graphs take fewer vertices each, so that long rows spread over the GPU
-    const uint32_t per_warp = n >= (1u << 20) ? 32u : n >= (1u << 18) ? 16u : 8u;
-    k_wedge_limits<<<1, 1, 0, s>>>(n, b.order, max_deg, max_deg >= kTilesFrom ? tile_degree(n) : max_deg + 1, ctx->d_ctl);
+    const uint32_t per_warp = rows_per_warp(n);
     auto rows = b.lvp ? k_wedge_rows<true> : k_wedge_rows<false>;
     rows<<<grid_for((uint64_t)n * (32 / per_warp), kFillThreads, cap), kFillThreads, 0, s>>>(
         n, b.rp, b.col, b.lv, b.lvp, b.adj2, ids, out, b.big, b.huge, per_warp, ctx->d_ctl);
@@ -1097,23 +1098,22 @@ tc_status wedge_rows(tc_ctx *ctx, const PipeBufs &b, uint32_t n, uint32_t max_de
         ++launches;
     }
     if (max_deg >= kTilesFrom) {
-        const uint32_t nb = entry_blocks(ctx, b.slots), tiles = tiles_cap(n);
+        const uint32_t nb = entry_blocks(ctx, b.slots), tiles = tiles_cap(n, b.slots);
         const uint64_t cells = (uint64_t)tiles * nb;
-        TC_CUDA(ctx, cudaMemsetAsync(b.wedge_counts, 0, 4 * cells, s));
-        TC_CUDA(ctx, cudaMemsetAsync(b.wedge_work, 0, 8ull * tiles, s));
+        TC_CUDA(ctx, cudaMemsetAsync(b.wedge_work, 0, 8ull * tiles + 4 * cells, s));  // work and counts
         const int smem = (int)(8 * tiles);
         TC_CUDA(ctx, cudaFuncSetAttribute(k_wedge_entries<false>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem));
         TC_CUDA(ctx, cudaFuncSetAttribute(k_wedge_entries<true>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem / 2));
         auto *offs = reinterpret_cast<unsigned long long *>(b.wedge_offs);
         k_wedge_entries<false><<<nb, 1024, smem, s>>>(n, b.slots, b.rp, b.adj2, b.fcnt, b.gcnt, b.wedge_counts, offs,
-                                                      b.wedge_work, b.erec, b.erec_cap, tiles, ctx->d_ctl);
+                                                      b.wedge_work, b.erec, b.erec_cap, tiles, per_warp, ctx->d_ctl);
         launches += 3 + scan_u32_to_u64(b.wedge_counts, b.wedge_offs, cells, b.wedge_tmp, s);
         k_wedge_entries<true><<<nb, 1024, smem / 2, s>>>(n, b.slots, b.rp, b.adj2, b.fcnt, b.gcnt, b.wedge_counts, offs,
-                                                     b.wedge_work, b.erec, b.erec_cap, tiles, ctx->d_ctl);
+                                                     b.wedge_work, b.erec, b.erec_cap, tiles, per_warp, ctx->d_ctl);
         // row ranges of about kRangeBytes of 16-bit ids (2 bytes an edge)
         const uint32_t ranges = (uint32_t)std::min<uint64_t>(b.slots / kRangeBytes + 1, 16);
         k_wedge_plan<<<1, 1024, 0, s>>>(offs, nb, b.wedge_work, (uint32_t)ctx->num_sms, ranges, b.wedge_tasks,
-                                        tasks_cap(ctx, n), ctx->d_ctl);
+                                        tasks_cap(ctx, n, b.slots), ctx->d_ctl);
     }
     note_launch(ctx, launches);
     TC_CUDA(ctx, cudaGetLastError());
@@ -1126,10 +1126,11 @@ tc_status wedge_count(tc_ctx *ctx, const PipeBufs &b, uint32_t n, uint32_t max_d
     TC_CUDA(ctx, cudaEventRecord(ctx->ev[4], s));
     int per_sm = 0;
     TC_CUDA(ctx, cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k_wedge_rest, kRestThreads, 0));
-    const uint64_t blocks = ((uint64_t)n + 32 * (kRestThreads / 32) - 1) / (32 * (kRestThreads / 32));
+    const uint32_t per_warp = rows_per_warp(n);
+    const uint64_t blocks = ((uint64_t)n + per_warp * (kRestThreads / 32) - 1) / (per_warp * (kRestThreads / 32));
     const uint64_t resident = (uint64_t)ctx->num_sms * std::max(per_sm, 1);
     k_wedge_rest<<<(unsigned)std::min(blocks, resident), kRestThreads, 0, s>>>(n, b.rp, b.adj2, b.fcnt, b.glo,
-                                                                               b.vmeta, ctx->d_ctl);
+                                                                               b.vmeta, per_warp, ctx->d_ctl);
     TC_CUDA(ctx, cudaEventRecord(ctx->ev[5], s));
     if (tiles) {
         TC_CUDA(ctx, cudaFuncSetAttribute(k_wedge_tiles, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kTileSmem));
