@@ -98,7 +98,7 @@ typedef struct tc_stats {
     float ms_mark;              /* partition, orientation, compaction, planning */
     float ms_isect;             /* intersections + reduction */
     /* intersection classes: [0] warp (shared table per warp), [1] block (shared table), [2] hub (L2
-       bitmaps + shared prefilter), [3] tiny (thread-per-row sorted merges).  Plain counts that take
+       bitmaps + shared prefilter), [3] tiny (thread-per-row sorted merges).  Counts that take
        tiles (see tc_tuning): [1] the tiles, [0] the pairs no tile takes, the others empty */
     uint64_t class_rows[4];     /* tasks (warp, block, hub) or rows (tiny) */
     uint64_t class_probes[4];   /* probed elements */
@@ -112,8 +112,8 @@ typedef struct tc_stats {
 /*
  * Launch-shape knobs of the intersection stage (Algorithm 4's hashed loop):
  * rows are classed by the size s(u) of the hashed row of the first endpoint.
- * A plain count under the degree order (tc_count, tc_count_levels,
- * tc_count_with_levels) has no such classes while warp_cap, block_cap,
+ * A count of one graph under the degree order (tc_count, tc_count_levels,
+ * tc_count_with_levels, tc_count_vertices) has no such classes while warp_cap, block_cap,
  * tiny_cap, table_kind, flat_cap and block_bits_log2 keep their defaults: it
  * finds every triangle at its latest vertex, by tiles of 32 earlier ones
  * (wedge.cu).  Any of them changed selects the classes, as do the id order,

@@ -35,7 +35,7 @@ tc_status pull(tc_ctx *ctx) {
 // Bytes of scratch for a graph with n vertices, `slots` CSR slots and the
 // given maximum degree.
 size_t pipeline_bytes(const tc_ctx *ctx, uint32_t n, uint64_t slots, uint32_t max_deg, bool own_levels, bool plain,
-                      uint64_t *hub_words, uint32_t *hub_maps) {
+                      bool wedge, uint64_t *hub_words, uint32_t *hub_maps) {
     auto r = [](size_t b) { return (b + 255) & ~size_t(255); };
     const size_t n1 = (size_t)n + 1;
     const uint64_t rtiles = radix_tiles_cap(n1);
@@ -51,10 +51,10 @@ size_t pipeline_bytes(const tc_ctx *ctx, uint32_t n, uint64_t slots, uint32_t ma
     bytes += r(8 * scan_tmp_elems(std::max<uint64_t>(n1 + 1, 256 * rtiles + 2)));  // scan tiles
     // fence and task pool (at most one task per oriented G0 edge), or the wedge path's ids and plan
     size_t own = r(4 * (slots / 32 + 2)) + r(8 * (slots / 2 + 1));
-    if (plain && wedge_path(ctx, n, slots, max_deg)) {
+    if (wedge) {
         const WedgeSizes z = wedge_sizes(ctx, n, slots);
         own = std::max(own, r(2 * (4 * slots + 8)) + r(8ull * z.tiles + 4 * z.counts) + r(8 * (z.counts + 1)) +
-                                r(16ull * z.tasks) + r(8 * z.tmp));
+                                r(16ull * z.tasks) + r(8 * z.tmp) + (plain ? 0 : r(4 * (slots / 2 + 1))));
     }
     bytes += own;
     *hub_words = 0;
@@ -101,7 +101,10 @@ tc_status count_pipeline(tc_ctx *ctx, const GraphView &g, uint32_t *levels_out, 
     uint64_t hub_words = 0;
     uint32_t hub_maps = 0;
     const bool plain = !(vertex_counts || list || alg3);
-    const size_t need = pipeline_bytes(ctx, n, g.slots, g.max_deg, levels_out == nullptr, plain, &hub_words, &hub_maps) +
+    // plain and per-vertex counts of one graph under the degree order
+    const bool wedge = !list && !alg3 && groups.n_groups == 0 && wedge_path(ctx, n, g.slots, g.max_deg);
+    const size_t need = pipeline_bytes(ctx, n, g.slots, g.max_deg, levels_out == nullptr, plain, wedge, &hub_words,
+                                       &hub_maps) +
                         (vertex_counts ? 8ull * ((size_t)n + 1) + 256 : 0) + (list ? list_bytes(ctx, n, list->capacity) : 0);
     tc_status st = arena_reserve(ctx, need);
     if (st != TC_OK) return st;
@@ -151,7 +154,6 @@ tc_status count_pipeline(tc_ctx *ctx, const GraphView &g, uint32_t *levels_out, 
     b.rcounts = a.take<uint32_t>(256 * rtiles + 1);
     b.roffs = a.take<uint64_t>(256 * rtiles + 2);
     b.adj2 = a.take<uint32_t>(g.slots + 1);
-    const bool wedge = plain && groups.n_groups == 0 && wedge_path(ctx, n, g.slots, g.max_deg);
     b.slots = g.slots;
     b.erec_cap = g.slots / 2 + 1;
     b.erec = a.take<uint4>(b.erec_cap);
@@ -173,7 +175,8 @@ tc_status count_pipeline(tc_ctx *ctx, const GraphView &g, uint32_t *levels_out, 
         b.wedge_offs = a.take<uint64_t>(z.counts + 1);
         b.wedge_tasks = a.take<uint4>(z.tasks);
         b.wedge_tmp = a.take<uint64_t>(z.tmp);
-        ok = ok && b.wedge_ids && b.wedge_work && b.wedge_offs && b.wedge_tasks && b.wedge_tmp;
+        if (!plain) b.wedge_v = a.take<uint32_t>(b.erec_cap);
+        ok = ok && b.wedge_ids && b.wedge_work && b.wedge_offs && b.wedge_tasks && b.wedge_tmp && (plain || b.wedge_v);
     }
     b.groups = groups;
     if (vertex_counts) {

@@ -92,6 +92,7 @@ struct PipeBufs {
     unsigned long long *wedge_work = nullptr; // steps per tile
     uint4 *wedge_tasks = nullptr;             // {tile, first entry, last entry}
     uint64_t *wedge_tmp = nullptr;            // scan tiles
+    uint32_t *wedge_v = nullptr;              // [S/2] rank of every entry's vertex (per-vertex counts only)
 };
 
 // Plain counts under the degree order (wedge.cu).  The vertices of high degree,

@@ -100,7 +100,7 @@ __global__ void __launch_bounds__(kScanThreads) k_scan_tiles(const T *in, unsign
 
 // The whole scan in one block (in place too), for counts where three launches
 // cost more than one block's walk over the values.
-constexpr uint64_t kOneBlock = 4 * kTile;
+constexpr uint64_t kOneBlock = kTile;
 template <class T>
 __global__ void __launch_bounds__(kScanThreads) k_scan_one(const T *in, unsigned long long *out, uint64_t count) {
     unsigned long long carry = 0;

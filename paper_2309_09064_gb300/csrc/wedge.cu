@@ -374,7 +374,8 @@ __global__ void __launch_bounds__(1024) k_wedge_entries(uint32_t n, uint64_t slo
                                                         const unsigned long long *__restrict__ offs,
                                                         unsigned long long *__restrict__ work,
                                                         uint4 *__restrict__ entries, uint64_t cap, uint32_t tiles_cap,
-                                                        uint32_t per_warp, Ctl *ctl) {
+                                                        uint32_t per_warp, const uint2 *__restrict__ lv,
+                                                        uint32_t *__restrict__ entry_v, Ctl *ctl) {
     extern __shared__ uint32_t sm[];  // tiles_cap counts or cursors, then (counting) tiles_cap steps
     __shared__ uint32_t s_row[2], s_next;
     const unsigned lane = lane_id();
@@ -413,13 +414,14 @@ __global__ void __launch_bounds__(1024) k_wedge_entries(uint32_t n, uint64_t slo
         g = __shfl_sync(0xFFFFFFFFu, g, 0);
         if (row_lo + g >= row_hi || g >= row_hi - row_lo) break;
         const uint32_t x = row_lo + g + lane;
-        uint32_t d = 0, nlo = 0;
+        uint32_t d = 0, nlo = 0, vrank = 0;
         uint64_t b = 0;
         if (lane < per_warp && x < row_hi) {
             d = dcnt[x];
             nlo = lcnt[x];
             if (d < 2) d = 0;
             else b = rp[x];
+            if (kScatter && entry_v) vrank = lv[x].x;
         }
         uint32_t incl = d;
 #pragma unroll
@@ -439,6 +441,7 @@ __global__ void __launch_bounds__(1024) k_wedge_entries(uint32_t n, uint64_t slo
             const uint32_t pos = e - (__shfl_sync(0xFFFFFFFFu, incl, r) - dr);
             const uint64_t br = __shfl_sync(0xFFFFFFFFu, b, r);
             const uint32_t lr = __shfl_sync(0xFFFFFFFFu, nlo, r);
+            const uint32_t vr = kScatter ? __shfl_sync(0xFFFFFFFFu, vrank, r) : 0u;
             uint32_t rank = 0xFFFFFFFFu, kind = 0;
             if (e < total) {
                 const uint32_t key = keys[br + pos];
@@ -477,6 +480,8 @@ __global__ void __launch_bounds__(1024) k_wedge_entries(uint32_t n, uint64_t slo
                     } else {
                         if (hor) entries[at] = make_uint4(unit, hor, units | 0x80000000u, place);
                         if (ver) entries[at + (hor != 0)] = make_uint4(unit, ver, units, place);
+                        if (entry_v)
+                            for (uint32_t k = 0; k < parts; ++k) entry_v[at + k] = vr;
                     }
                 } else {
                     atomicAdd(&sm[tile], parts);
@@ -575,6 +580,10 @@ __global__ void __launch_bounds__(1024) k_wedge_plan(const unsigned long long *_
 constexpr uint32_t kTileThreads = 1024;
 constexpr uint32_t kTileWords = 32768;
 constexpr size_t kTileSmem = 4ull * kTileWords + (kTileThreads / 32) * 32 * sizeof(uint4);
+// Per-vertex counts (kM = 1) add: block-private counts of the first kPrivRanks
+// ranks (the w that close most triangles) and each warp's of the tile's vertices.
+constexpr uint32_t kPrivRanks = 1024;
+constexpr size_t kCreditSmem = 4ull * kPrivRanks + (kTileThreads / 32) * 32 * 4ull;
 
 __device__ __forceinline__ uint32_t lds(uint32_t addr) {
     uint32_t v;
@@ -628,14 +637,33 @@ __device__ __forceinline__ uint4 next_tile_task(Ctl *ctl, int counter, uint32_t 
 // lookups (3.5 wavefronts per 32; L1/shared data stage at 83% at R-MAT 22) and
 // by issue: R-MAT 24 (26 G lookups) 18.8 ms, with eight lanes of four ids each
 // 26.0.
+// With kM = 1 every triangle adds one to each of its vertices in `credit` (by
+// rank): v once per run of steps on its entry, w once per lookup that hits, u
+// once per triangle in the warp's own counters of the tile.
+template <int kM>
 __global__ void __launch_bounds__(kTileThreads, 1) k_wedge_tiles(uint32_t n, const uint4 *__restrict__ tasks,
                                                                  const uint4 *__restrict__ entries,
                                                                  const uint16_t *__restrict__ ids,
-                                                                 const uint4 *__restrict__ rmeta, Ctl *ctl) {
+                                                                 const uint4 *__restrict__ rmeta, Ctl *ctl,
+                                                                 const uint32_t *__restrict__ entry_v,
+                                                                 unsigned long long *__restrict__ credit) {
     extern __shared__ __align__(16) uint32_t word[];
     __shared__ uint4 s_task[2];
     const unsigned lane = lane_id(), warp = threadIdx.x >> 5;
     const uint32_t sub = lane & 3u;
+    uint32_t *priv = word + kTileWords + (kTileThreads / 32) * 32 * 4;  // kM = 1: kPrivRanks counts
+    uint32_t *ucnt = priv + kPrivRanks + 32 * warp;                     // and this warp's of the tile
+    // add the block's private counts to `credit` (all threads; the tile's vertices start at u0)
+    auto flush = [&](uint32_t u0) {
+        __syncthreads();
+        for (uint32_t i = threadIdx.x; i < kPrivRanks; i += kTileThreads) {
+            if (priv[i]) atomicAdd(credit + i, (unsigned long long)priv[i]);
+            priv[i] = 0;
+        }
+        if (ucnt[lane]) atomicAdd(credit + u0 + lane, (unsigned long long)ucnt[lane]);
+        ucnt[lane] = 0;
+        __syncthreads();
+    };
     uint4 *ent = reinterpret_cast<uint4 *>(word + kTileWords) + warp * 32;
     const uint32_t wbase = (uint32_t)__cvta_generic_to_shared(word);
     const uint32_t n_tasks = (uint32_t)ctl->n_tasks[1];
@@ -646,6 +674,10 @@ __global__ void __launch_bounds__(kTileThreads, 1) k_wedge_tiles(uint32_t n, con
     for (uint32_t i = threadIdx.x; i < kTileWords / 4; i += kTileThreads)
         reinterpret_cast<uint4 *>(word)[i] = make_uint4(0, 0, 0, 0);
     uint32_t dirty = 0;  // words [0, dirty) may be set
+    if constexpr (kM == 1) {
+        for (uint32_t i = threadIdx.x; i < kPrivRanks; i += kTileThreads) priv[i] = 0;
+        ucnt[lane] = 0;
+    }
     if (threadIdx.x == 0) s_task[0] = next_tile_task(ctl, 1, 0, n_tasks, tasks, t_start);
     __syncthreads();
     for (uint32_t phase = 0;; phase ^= 1u) {
@@ -677,7 +709,10 @@ __global__ void __launch_bounds__(kTileThreads, 1) k_wedge_tiles(uint32_t n, con
         uint32_t tot = 0, sam = 0;
         for (uint32_t base = task.y + warp * 32; base < task.z; base += kTileThreads) {
             uint4 en = make_uint4(0, 0, 0, 0);
-            if (base + lane < task.z) en = entries[base + lane];
+            if (base + lane < task.z) {
+                en = entries[base + lane];
+                if constexpr (kM == 1) en.w = entry_v[base + lane];
+            }
             __syncwarp();
             ent[lane] = en;
             __syncwarp();
@@ -687,7 +722,8 @@ __global__ void __launch_bounds__(kTileThreads, 1) k_wedge_tiles(uint32_t n, con
             int rem = (int)(cur.z & 0x7FFFFFFFu) - (int)(4 * w.skip + sub);    // units from there on
             uint4 a, a1;
             uint32_t mv = 0, kl = 0, mv1, kl1;
-            auto fetch = [&](uint4 &x, uint32_t &mm, uint32_t &kk) {
+            uint32_t vr = 0, vr1 = 0, vlast = kNoTask, vsum = 0;  // kM = 1: v, and its triangles not yet credited
+            auto fetch = [&](uint4 &x, uint32_t &mm, uint32_t &kk, uint32_t &vv) {
                 x = make_uint4(0xFFFFFFFFu, 0xFFFFFFFFu, 0xFFFFFFFFu, 0xFFFFFFFFu);
                 if (w.left) {
                     --w.left;
@@ -703,6 +739,13 @@ __global__ void __launch_bounds__(kTileThreads, 1) k_wedge_tiles(uint32_t n, con
                 }
                 mm = cur.y;
                 kk = cur.z >> 31;
+                if constexpr (kM == 1) vv = cur.w;
+            };
+            auto hit = [&](uint32_t rank, uint32_t h, uint32_t p) {
+                vsum += p;
+                if (rank < kPrivRanks) atomicAdd(priv + rank, p);
+                else atomicAdd(credit + rank, (unsigned long long)p);
+                for (; h; h &= h - 1) atomicAdd(ucnt + __ffs(h) - 1, 1u);
             };
             auto look = [&](uint32_t x, uint32_t mm, uint32_t kk) {
                 const uint32_t w0 = lds(wbase + ((x << 1) & 0x1FFFCu)), w1 = lds(wbase + ((x >> 15) & 0x1FFFCu));
@@ -710,10 +753,21 @@ __global__ void __launch_bounds__(kTileThreads, 1) k_wedge_tiles(uint32_t n, con
                 tot += p0 + p1;
                 if (x & kk) sam += p0;
                 if (x & (kk << 16)) sam += p1;
+                if constexpr (kM == 1) {
+                    if (p0) hit((x >> 1) & 0x7FFFu, w0 & mm, p0);
+                    if (p1) hit(x >> 17, w1 & mm, p1);
+                }
             };
-            fetch(a, mv, kl);
+            fetch(a, mv, kl, vr);
             for (uint32_t k = 0; k < w.iters; ++k) {
-                fetch(a1, mv1, kl1);
+                fetch(a1, mv1, kl1, vr1);
+                if constexpr (kM == 1) {
+                    if (vr != vlast) {
+                        if (vsum) atomicAdd(credit + vlast, (unsigned long long)vsum);
+                        vsum = 0;
+                        vlast = vr;
+                    }
+                }
                 look(a.x, mv, kl);
                 look(a.y, mv, kl);
                 look(a.z, mv, kl);
@@ -721,10 +775,14 @@ __global__ void __launch_bounds__(kTileThreads, 1) k_wedge_tiles(uint32_t n, con
                 a = a1;
                 mv = mv1;
                 kl = kl1;
+                vr = vr1;
             }
+            if constexpr (kM == 1)
+                if (vsum) atomicAdd(credit + vlast, (unsigned long long)vsum);
         }
         same += sam;
         cross += tot - sam;
+        if constexpr (kM == 1) flush(32 * tile);
         if (threadIdx.x == 0) s_task[phase ^ 1u] = next;
         __syncthreads();
     }
@@ -754,10 +812,13 @@ constexpr uint32_t kHighSlots = 8192, kHighShift = 19, kHighKeys = 6144;
 constexpr size_t kHighSmem = kHighBits / 8 + 8ull * kHighSlots + (kHighThreads / 32) * 32 * sizeof(uint4);
 constexpr unsigned kGuardInsert = 0x10u;
 
+template <int kM>
 __global__ void __launch_bounds__(kHighThreads, 2) k_wedge_high(uint32_t n, const uint4 *__restrict__ tasks,
                                                                 const uint4 *__restrict__ entries,
                                                                 const uint32_t *__restrict__ keys,
-                                                                const uint4 *__restrict__ rmeta, Ctl *ctl) {
+                                                                const uint4 *__restrict__ rmeta, Ctl *ctl,
+                                                                const uint32_t *__restrict__ entry_v,
+                                                                unsigned long long *__restrict__ credit) {
     extern __shared__ __align__(16) uint32_t member[];  // kHighBits bits, the table, the warps' entries
     uint2 *table = reinterpret_cast<uint2 *>(member + kHighBits / 32);
     __shared__ uint4 s_task[2];
@@ -832,12 +893,13 @@ __global__ void __launch_bounds__(kHighThreads, 2) k_wedge_high(uint32_t n, cons
                     if (lane >= (unsigned)o) incl += y;
                 }
                 const uint32_t total = __shfl_sync(0xFFFFFFFFu, incl, 31), excl = incl - cnt;
-                // the entries that have high keys, packed: {first key - flat position, mask, kind}
+                // the entries that have high keys, packed: {first key - flat position, mask, kind, v}
                 const unsigned some = __ballot_sync(0xFFFFFFFFu, cnt != 0);
                 __syncwarp();
                 if (cnt)
                     ent[__popc(some & ((1u << lane) - 1u))] =
-                        make_uint4(2 * en.x - ((en.w >> 15) & 1u) + (en.w & 0x7FFFu) - excl, en.y, en.z >> 31, 0u);
+                        make_uint4(2 * en.x - ((en.w >> 15) & 1u) + (en.w & 0x7FFFu) - excl, en.y, en.z >> 31,
+                                   kM == 1 ? entry_v[base + lane] : 0u);
                 __syncwarp();
                 // One key per lane and window of 32 flat positions, kHighAhead windows in flight:
                 // the entry of a position is the number of entries that start up to there.
@@ -864,9 +926,17 @@ __global__ void __launch_bounds__(kHighThreads, 2) k_wedge_high(uint32_t n, cons
                             e = table[s];
                         }
                         if (e.x == r) {
-                            const uint32_t p = __popc(e.y & ent[at[t]].y);
+                            uint32_t h = e.y & ent[at[t]].y;
+                            const uint32_t p = __popc(h);
                             tot += p;
                             if (key[t] & ent[at[t]].z) sam += p;
+                            if constexpr (kM == 1) {
+                                if (p) {
+                                    atomicAdd(credit + ent[at[t]].w, (unsigned long long)p);
+                                    atomicAdd(credit + r, (unsigned long long)p);
+                                    for (; h; h &= h - 1) atomicAdd(credit + 32 * tile + __ffs(h) - 1, 1ull);
+                                }
+                            }
                         }
                     }
                 }
@@ -909,12 +979,14 @@ __device__ __forceinline__ uint32_t find_key(const uint32_t *__restrict__ a, uin
 // kRestTiny keys: one lane tries its pairs, each by a search of w in N(u).  A
 // longer one: its warp sets a filter bit per key of N(v), eight lanes a time
 // walk N(u) and search N(v) for the keys that pass the filter.
+template <int kM>
 __global__ void __launch_bounds__(kRestThreads) k_wedge_rest(uint32_t n, const uint64_t *__restrict__ rp,
                                                              const uint32_t *__restrict__ keys,
                                                              const uint32_t *__restrict__ dcnt,
                                                              const uint32_t *__restrict__ ucnt,
                                                              const uint4 *__restrict__ rmeta, uint32_t per_warp,
-                                                             Ctl *ctl) {
+                                                             Ctl *ctl, const uint2 *__restrict__ lv,
+                                                             unsigned long long *__restrict__ credit) {
     __shared__ uint32_t sfilter[kRestThreads / 32][kFilterBits / 32];
     const unsigned lane = lane_id(), warp = threadIdx.x >> 5;
     const uint32_t sub = lane & 7u, group = lane >> 3;
@@ -937,14 +1009,24 @@ __global__ void __launch_bounds__(kRestThreads) k_wedge_rest(uint32_t n, const u
         c = __shfl_sync(0xFFFFFFFFu, c, 0);
         if (c >= chunks) break;
         const uint64_t x = (uint64_t)c * per_warp + lane;
-        uint32_t d = 0, nu = 0;  // keys, and those below U
+        uint32_t d = 0, nu = 0, vr = 0;  // keys, and those below U; its rank (kM = 1)
         uint64_t b = 0;
         if (lane < per_warp && x < n) {
             d = dcnt[x];
             nu = ucnt[x];
             if (d < 2 || d == nu) d = 0;
             else b = rp[x];
+            if (kM == 1 && d) vr = lv[x].x;
         }
+        // one triangle: w < u < v with these keys of w and u in v's row
+        auto found = [&](uint32_t ku, uint32_t kw, uint32_t v) {
+            if (ku & kw & 1u) ++same; else ++cross;
+            if constexpr (kM == 1) {
+                atomicAdd(credit + v, 1ull);
+                atomicAdd(credit + (ku >> 1), 1ull);
+                atomicAdd(credit + (kw >> 1), 1ull);
+            }
+        };
         if (d && d <= kRestTiny) {
             const uint32_t *row = keys + b;
             for (uint32_t j = nu > 1 ? nu : 1; j < d; ++j) {
@@ -954,9 +1036,7 @@ __global__ void __launch_bounds__(kRestThreads) k_wedge_rest(uint32_t n, const u
                 const uint32_t *nb = keys + (((uint64_t)m.y << 32) | m.x);
                 for (uint32_t i = 0; i < j; ++i) {
                     const uint32_t kw = row[i];
-                    if (find_key(nb, 0, m.z, kw >> 1) != kEmpty) {
-                        if (ku & kw & 1u) ++same; else ++cross;
-                    }
+                    if (find_key(nb, 0, m.z, kw >> 1) != kEmpty) found(ku, kw, vr);
                 }
                 probes += j;
             }
@@ -968,6 +1048,7 @@ __global__ void __launch_bounds__(kRestThreads) k_wedge_rest(uint32_t n, const u
             pending &= pending - 1;
             const uint32_t vd = __shfl_sync(0xFFFFFFFFu, d, src), vu = __shfl_sync(0xFFFFFFFFu, nu, src);
             const uint64_t vb = __shfl_sync(0xFFFFFFFFu, b, src);
+            const uint32_t vrank = kM == 1 ? __shfl_sync(0xFFFFFFFFu, vr, src) : 0u;
             const uint32_t *row = keys + vb;
             for (uint32_t i = lane; i < vd; i += 32) {
                 const uint32_t h = (row[i] >> 1) & (kFilterBits - 1);
@@ -988,9 +1069,7 @@ __global__ void __launch_bounds__(kRestThreads) k_wedge_rest(uint32_t n, const u
                         const uint32_t h = w[t] & (kFilterBits - 1);
                         if (w[t] != kEmpty && ((filter[h >> 5] >> (h & 31u)) & 1u)) {
                             const uint32_t kw = find_key(row, 0, j, w[t]);
-                            if (kw != kEmpty) {
-                                if (ku & kw & 1u) ++same; else ++cross;
-                            }
+                            if (kw != kEmpty) found(ku, kw, vrank);
                         }
                     }
                 }
@@ -1106,10 +1185,10 @@ tc_status wedge_rows(tc_ctx *ctx, const PipeBufs &b, uint32_t n, uint32_t max_de
         TC_CUDA(ctx, cudaFuncSetAttribute(k_wedge_entries<true>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem / 2));
         auto *offs = reinterpret_cast<unsigned long long *>(b.wedge_offs);
         k_wedge_entries<false><<<nb, 1024, smem, s>>>(n, b.slots, b.rp, b.adj2, b.fcnt, b.gcnt, b.wedge_counts, offs,
-                                                      b.wedge_work, b.erec, b.erec_cap, tiles, per_warp, ctx->d_ctl);
+                                                      b.wedge_work, b.erec, b.erec_cap, tiles, per_warp, b.lv, b.wedge_v, ctx->d_ctl);
         launches += 3 + scan_u32_to_u64(b.wedge_counts, b.wedge_offs, cells, b.wedge_tmp, s);
         k_wedge_entries<true><<<nb, 1024, smem / 2, s>>>(n, b.slots, b.rp, b.adj2, b.fcnt, b.gcnt, b.wedge_counts, offs,
-                                                     b.wedge_work, b.erec, b.erec_cap, tiles, per_warp, ctx->d_ctl);
+                                                     b.wedge_work, b.erec, b.erec_cap, tiles, per_warp, b.lv, b.wedge_v, ctx->d_ctl);
         // row ranges of about kRangeBytes of 16-bit ids (2 bytes an edge)
         const uint32_t ranges = (uint32_t)std::min<uint64_t>(b.slots / kRangeBytes + 1, 16);
         k_wedge_plan<<<1, 1024, 0, s>>>(offs, nb, b.wedge_work, (uint32_t)ctx->num_sms, ranges, b.wedge_tasks,
@@ -1122,24 +1201,28 @@ tc_status wedge_rows(tc_ctx *ctx, const PipeBufs &b, uint32_t n, uint32_t max_de
 
 tc_status wedge_count(tc_ctx *ctx, const PipeBufs &b, uint32_t n, uint32_t max_deg) {
     cudaStream_t s = ctx->stream;
-    const bool tiles = max_deg >= kTilesFrom;
+    const bool tiles = max_deg >= kTilesFrom, credit = b.vcount != nullptr;
     TC_CUDA(ctx, cudaEventRecord(ctx->ev[4], s));
     int per_sm = 0;
-    TC_CUDA(ctx, cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k_wedge_rest, kRestThreads, 0));
+    auto rest = credit ? k_wedge_rest<1> : k_wedge_rest<0>;
+    TC_CUDA(ctx, cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, rest, kRestThreads, 0));
     const uint32_t per_warp = rows_per_warp(n);
     const uint64_t blocks = ((uint64_t)n + per_warp * (kRestThreads / 32) - 1) / (per_warp * (kRestThreads / 32));
     const uint64_t resident = (uint64_t)ctx->num_sms * std::max(per_sm, 1);
-    k_wedge_rest<<<(unsigned)std::min(blocks, resident), kRestThreads, 0, s>>>(n, b.rp, b.adj2, b.fcnt, b.glo,
-                                                                               b.vmeta, per_warp, ctx->d_ctl);
+    rest<<<(unsigned)std::min(blocks, resident), kRestThreads, 0, s>>>(n, b.rp, b.adj2, b.fcnt, b.glo, b.vmeta, per_warp,
+                                                                       ctx->d_ctl, b.lv, b.vcount_rank);
     TC_CUDA(ctx, cudaEventRecord(ctx->ev[5], s));
     if (tiles) {
-        TC_CUDA(ctx, cudaFuncSetAttribute(k_wedge_tiles, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kTileSmem));
-        k_wedge_tiles<<<(unsigned)ctx->num_sms, kTileThreads, kTileSmem, s>>>(n, b.wedge_tasks, b.erec, b.wedge_ids,
-                                                                             b.vmeta, ctx->d_ctl);
+        auto tile = credit ? k_wedge_tiles<1> : k_wedge_tiles<0>;
+        const size_t smem = kTileSmem + (credit ? kCreditSmem : 0);
+        TC_CUDA(ctx, cudaFuncSetAttribute(tile, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
+        tile<<<(unsigned)ctx->num_sms, kTileThreads, smem, s>>>(n, b.wedge_tasks, b.erec, b.wedge_ids, b.vmeta, ctx->d_ctl,
+                                                                b.wedge_v, b.vcount_rank);
         if (n > kWedgeMaxK) {
-            TC_CUDA(ctx, cudaFuncSetAttribute(k_wedge_high, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kHighSmem));
-            k_wedge_high<<<(unsigned)ctx->num_sms * 2u, kHighThreads, kHighSmem, s>>>(n, b.wedge_tasks, b.erec, b.adj2,
-                                                                                     b.vmeta, ctx->d_ctl);
+            auto high = credit ? k_wedge_high<1> : k_wedge_high<0>;
+            TC_CUDA(ctx, cudaFuncSetAttribute(high, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kHighSmem));
+            high<<<(unsigned)ctx->num_sms * 2u, kHighThreads, kHighSmem, s>>>(n, b.wedge_tasks, b.erec, b.adj2, b.vmeta,
+                                                                             ctx->d_ctl, b.wedge_v, b.vcount_rank);
             note_launch(ctx);
         }
     }

@@ -11,6 +11,7 @@ import pytest
 import graphgen as gg
 import oracle
 
+torch = pytest.importorskip("torch")
 pytestmark = pytest.mark.gpu
 
 
@@ -69,6 +70,23 @@ def test_wedge_counts(tc, name):
                 tc.tc_set_tuning(c, **knobs)
             T, st = tc.tc_count(c, g)
             assert (T, st["t_same"], st["t_cross"], st["horizontal_edges"], st["levels"]) == want
+        tc.tc_graph_free(g)
+    finally:
+        tc.tc_destroy(c)
+
+
+@pytest.mark.parametrize("name", sorted(GRAPHS))
+def test_wedge_vertex_counts(tc, name):
+    """Per-vertex counts by tiles: every vertex's triangles, element by element."""
+    n, s, d = GRAPHS[name]()
+    rp, col = oracle.build_csr(n, s, d)
+    _, want = oracle.vertex_counts(rp, col)
+    c = tc.tc_create(0)
+    try:
+        g = tc.tc_graph_from_csr(c, rp, col)
+        out = torch.full((n,), -1, dtype=torch.int64, device="cuda")
+        T, _ = tc.tc_count_vertices(c, g, out)
+        assert np.array_equal(out.cpu().numpy().astype(np.uint64), want) and 3 * T == int(want.sum())
         tc.tc_graph_free(g)
     finally:
         tc.tc_destroy(c)
