@@ -99,7 +99,8 @@ typedef struct tc_stats {
     float ms_isect;             /* intersections + reduction */
     /* intersection classes: [0] warp (shared table per warp), [1] block (shared table), [2] hub (L2
        bitmaps + shared prefilter), [3] tiny (thread-per-row sorted merges).  Counts that take
-       tiles (see tc_tuning): [1] the tiles, [0] the pairs no tile takes, the others empty */
+       tiles (see tc_tuning): [1] the tiles, [0] the pairs no tile takes, the others empty.  Plain counts
+       of graphs of up to 2^15 vertices and a mean degree of up to 64: [0] all */
     uint64_t class_rows[4];     /* tasks (warp, block, hub) or rows (tiny) */
     uint64_t class_probes[4];   /* probed elements */
     uint64_t class_bytes[4];    /* algorithmic bytes: hashed rows once + probed rows */
@@ -116,7 +117,9 @@ typedef struct tc_stats {
  * tc_count_with_levels, tc_count_vertices) has no such classes while warp_cap, block_cap,
  * tiny_cap, table_kind, flat_cap and block_bits_log2 keep their defaults: it
  * finds every triangle at its latest vertex, by tiles of 32 earlier ones
- * (wedge.cu).  Any of them changed selects the classes, as do the id order,
+ * (wedge.cu) or, of up to 2^15 vertices, by a bitmap of the latest's neighbours
+ * (small.cu; tc_count_batch too, when no graph of the union has more than 65536
+ * vertices and the mean degree is at most 64).  Any of them changed selects the classes, as do the id order,
  * more than 2^30 CSR slots, and every other mode.
  */
 typedef struct tc_tuning {
@@ -191,7 +194,7 @@ tc_status tc_arena_bytes(const tc_ctx *ctx, uint64_t *bytes);
 
 /*
  * No counterpart in the paper (failure handling of this library).
- * Self-test of the bounded device-wide wait used by the persistent BFS: one
+ * Self-test of the bounded device-wide wait: one
  * launch waits at a grid barrier that can never complete (one arrival is
  * missing), gives up after timeout_ms (1..10000) and reports it.  Returns
  * TC_ERR_TIMEOUT when the wait ended as designed; the context stays usable.

@@ -81,7 +81,7 @@ tc_status count_batch(tc_ctx *ctx, uint32_t G, const tc_graph *const *graphs, ui
     std::vector<uint32_t> vstart(GL + 1);
     std::vector<unsigned long long> sstart(GL + 1);
     uint64_t N = 0, S = 0;
-    uint32_t max_deg = 0;
+    uint32_t max_deg = 0, max_n = 0;
     for (uint32_t k = 0; k < GL; ++k) {
         const tc_graph *g = graphs[large[k]];
         vstart[k] = (uint32_t)N;
@@ -90,6 +90,7 @@ tc_status count_batch(tc_ctx *ctx, uint32_t G, const tc_graph *const *graphs, ui
         N += g->n;
         S += g->slots;
         max_deg = g->max_deg > max_deg ? g->max_deg : max_deg;
+        max_n = std::max(max_n, g->n);
         if (N >= 0xFFFFFFFFull) return set_error(ctx, TC_ERR_INVALID, "batch has 2^32 - 1 or more vertices in total");
     }
     vstart[GL] = (uint32_t)N;
@@ -149,6 +150,7 @@ tc_status count_batch(tc_ctx *ctx, uint32_t G, const tc_graph *const *graphs, ui
         grp.vertex_start = d_vstart;
         grp.n_groups = GL;
         grp.counts = d_counts;
+        grp.max_n = max_n;
         uint64_t total = 0;
         st = count_pipeline(ctx, v, nullptr, grp, &total, nullptr);
         if (st != TC_OK) return st;

@@ -102,7 +102,8 @@ tc_status count_pipeline(tc_ctx *ctx, const GraphView &g, uint32_t *levels_out, 
     uint32_t hub_maps = 0;
     const bool plain = !(vertex_counts || list || alg3);
     // plain and per-vertex counts of one graph under the degree order
-    const bool wedge = !list && !alg3 && groups.n_groups == 0 && wedge_path(ctx, n, g.slots, g.max_deg);
+    const bool small = plain && small_path(ctx, n, g.slots, g.max_deg, groups);
+    const bool wedge = !small && !list && !alg3 && groups.n_groups == 0 && wedge_path(ctx, n, g.slots, g.max_deg);
     const size_t need = pipeline_bytes(ctx, n, g.slots, g.max_deg, levels_out == nullptr, plain, wedge, &hub_words,
                                        &hub_maps) +
                         (vertex_counts ? 8ull * ((size_t)n + 1) + 256 : 0) + (list ? list_bytes(ctx, n, list->capacity) : 0);
@@ -222,7 +223,7 @@ tc_status count_pipeline(tc_ctx *ctx, const GraphView &g, uint32_t *levels_out, 
     TC_CUDA(ctx, cudaEventRecord(ctx->ev[1], s));
     // the packed 4-byte {rank, level} word needs ranks below 2^24 and levels below 255
     b.lvp = (n <= (1u << 24) && ctx->h_ctl->max_level < 255) ? lvp : nullptr;
-    st = compute_ranks(ctx, b, n, g.max_deg, wedge ? wedge_tile_degree(n, g.max_deg) : kNoTiles);
+    if (!small) st = compute_ranks(ctx, b, n, g.max_deg, wedge ? wedge_tile_degree(n, g.max_deg) : kNoTiles);
     if (st != TC_OK) return st;
     Ctl counted{};                   // listing: the control block after phase 1
     unsigned long long list_tiny = 0;  // listing: triangles of the tiny rows
@@ -231,6 +232,9 @@ tc_status count_pipeline(tc_ctx *ctx, const GraphView &g, uint32_t *levels_out, 
         st = intersect_alg3(ctx, b, n, g.slots);
         if (st != TC_OK) return st;
         ctx->isect_flags = 0;
+    } else if (small) {
+        st = small_count(ctx, b, n, g.max_deg);
+        if (st != TC_OK) return st;
     } else if (wedge) {
         st = wedge_rows(ctx, b, n, g.max_deg);
         if (st != TC_OK) return st;
@@ -346,7 +350,8 @@ tc_status count_pipeline(tc_ctx *ctx, const GraphView &g, uint32_t *levels_out, 
             stats->class_rows[c] = h.cls_rows[c];
             stats->class_probes[c] = h.cls_probes[c];
             // wedge path: tiles read 16-byte entries and 16-bit ids, the other pairs 4-byte keys
-            stats->class_bytes[c] = wedge && c == 1 ? 16ull * h.cls_build[1] + 2ull * (h.cls_probes[1] + h.cls_inserts[1])
+            stats->class_bytes[c] = small ? 2ull * h.cls_probes[c]  // 16-bit ids
+                                    : wedge && c == 1 ? 16ull * h.cls_build[1] + 2ull * (h.cls_probes[1] + h.cls_inserts[1])
                                                     : 4ull * (h.cls_build[c] + h.cls_probes[c]);
             stats->class_inserts[c] = h.cls_inserts[c];
             is += stats->class_bytes[c];

@@ -95,9 +95,10 @@ struct PipeBufs {
     uint32_t *wedge_v = nullptr;              // [S/2] rank of every entry's vertex (per-vertex counts only)
 };
 
-// Plain counts under the degree order (wedge.cu).  The vertices of high degree,
-// at most kWedgeMaxU of them, are taken in tiles of 32; a tile's words cover the first kWedgeMaxK ranks (16-bit ids of 15 rank bits;
-// the last rank of 15 bits stays free: it marks padding).
+// Plain and per-vertex counts under the degree order (wedge.cu).  The vertices of
+// high degree, at most kWedgeMaxU of them, are taken in tiles of 32; a tile's words
+// cover the first kWedgeMaxK ranks (16-bit ids of 15 rank bits; the last rank of 15
+// bits stays free: it marks padding).
 constexpr uint32_t kWedgeMaxU = 1u << 19;
 constexpr uint32_t kWedgeMaxK = 32736;
 struct WedgeSizes {
@@ -165,6 +166,12 @@ tc_status emit_tasks(tc_ctx *ctx, PipeBufs &b);
 // a count split into shards: the probe records of this shard's tasks only
 tc_status records_for_shard(tc_ctx *ctx, const PipeBufs &b);
 tc_status intersect(tc_ctx *ctx, PipeBufs &b, uint32_t n);
+// graphs of up to 65536 vertices (small.cu): rows and count, no ranks
+// (a single graph up to 2^15: R-MAT 15 of edge factors 4 / 16 / 30 takes 685 / 339 / 407 us against 786 / 436 / 482
+// by tiles, R-MAT 16 365 / 535 / 806 against 471 / 522 / 591)
+constexpr uint32_t kSmallOne = 32768;
+bool small_path(const tc_ctx *ctx, uint32_t n, uint64_t slots, uint32_t max_deg, const GroupSpec &groups);
+tc_status small_count(tc_ctx *ctx, const PipeBufs &b, uint32_t n, uint32_t max_deg);
 // the wedge path: rows, entries and tasks, then the two counting kernels
 tc_status wedge_rows(tc_ctx *ctx, const PipeBufs &b, uint32_t n, uint32_t max_deg);
 tc_status wedge_count(tc_ctx *ctx, const PipeBufs &b, uint32_t n, uint32_t max_deg);

@@ -190,6 +190,7 @@ struct GroupSpec {
     const uint32_t *vertex_start = nullptr;
     uint32_t n_groups = 0;
     unsigned long long *counts = nullptr;
+    uint32_t max_n = 0;  // vertices of the largest group
 };
 struct GraphView {
     uint32_t n = 0;

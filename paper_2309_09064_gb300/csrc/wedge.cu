@@ -24,11 +24,13 @@
 // The rows are read as 16-bit ids (w < K <= 2^15, flag in the low bit).
 // k_wedge_high takes the same tiles' pairs with w >= K, k_wedge_rest those with
 // u >= U.  Measured (one GB300, whole counts, before and after): R-MAT 24
-// 130.5 -> 45.5 ms, R-MAT 20 5.39 -> 2.23, Chung-Lu 2^22 16.4 -> 7.2, uniform
-// 2^20 of mean degree 32 3.36 -> 1.85, R-MAT 16 1.32 -> 0.64.
+// 130.8 -> 45.7 ms, R-MAT 20 5.36 -> 2.03, Chung-Lu 2^22 16.4 -> 7.3, uniform
+// 2^20 of mean degree 32 3.33 -> 1.78, R-MAT 16 1.28 -> 0.52; per-vertex counts
+// of R-MAT 19 4.35 -> 2.03.
 #include <algorithm>
 
 #include "pipeline.cuh"
+#include "walk.cuh"
 #include "warp_sort.cuh"
 
 namespace tc {
@@ -589,34 +591,6 @@ __device__ __forceinline__ uint32_t lds(uint32_t addr) {
     uint32_t v;
     asm volatile("ld.shared.u32 %0, [%1];" : "=r"(v) : "r"(addr));
     return v;
-}
-
-// The 32 entries a warp holds and the steps (32 ids each) of its walk: the
-// steps of all entries are shared out evenly over the warp's eight groups of
-// four lanes, so short and long rows keep every lane busy.
-struct Walk {
-    uint32_t i, left, iters;  // the group's entry, its steps, the steps of the longest group
-    uint32_t skip;            // steps of entry i that belong to the groups before
-};
-__device__ __forceinline__ Walk share_steps(uint32_t steps) {
-    const unsigned lane = lane_id();
-    uint32_t incl = steps;
-#pragma unroll
-    for (int o = 1; o < 32; o <<= 1) {
-        const uint32_t y = __shfl_up_sync(0xFFFFFFFFu, incl, o);
-        if (lane >= (unsigned)o) incl += y;
-    }
-    const uint32_t total = __shfl_sync(0xFFFFFFFFu, incl, 31);
-    Walk w;
-    w.iters = (total + 7) / 8;
-    const uint32_t c = min((lane >> 2) * w.iters, total);
-    w.left = min(w.iters, total - c);
-    w.i = 0;  // the entry of step c: the first whose inclusive count passes it
-#pragma unroll
-    for (int o = 16; o > 0; o >>= 1)
-        if (__shfl_sync(0xFFFFFFFFu, incl, w.i + o - 1) <= c) w.i += o;
-    w.skip = c - __shfl_sync(0xFFFFFFFFu, incl - steps, w.i);
-    return w;
 }
 
 // The next task of a counter, for thread 0 (x = kNoTask: none left).

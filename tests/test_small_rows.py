@@ -1,0 +1,71 @@
+"""Graphs of up to 65536 vertices (csrc/small.cu): alone (the same / cross split)
+and in a union, with rows at the lane, warp and block limits, rows walked in
+slices, ids at the ends of the 16-bit range, and a graph one vertex too large.
+Counts are whole numbers: no tolerance."""
+import numpy as np
+import pytest
+
+import graphgen as gg
+import oracle
+
+torch = pytest.importorskip("torch")
+pytestmark = pytest.mark.gpu
+
+
+def at_end(n, graph):
+    """The graph's vertices as the last of n."""
+    k, s, d = graph[:3]
+    return n, s + np.uint32(n - k), d + np.uint32(n - k)
+
+
+GRAPHS = {
+    "empty": lambda: (3, np.zeros(0, np.uint32), np.zeros(0, np.uint32)),
+    "edge": lambda: gg.path(2),
+    "k9": lambda: gg.complete(9),
+    "k33": lambda: gg.complete(33),       # degree 32: the last lane row
+    "k34": lambda: gg.complete(34),       # degree 33: a warp's
+    "k66": lambda: at_end(99, gg.complete(66)),  # |N| to 65: one row in slices
+    "k300": lambda: at_end(2000, gg.complete(300)),
+    "wheel": lambda: gg.wheel(2051),      # degree above 2048: a block's row
+    "bipartite": lambda: gg.complete_bipartite(5, 2049),
+    "rmat12": lambda: gg.rmat(12, 20, seed=5)[:3],
+    "k70_at_end": lambda: at_end(65536, gg.complete(70)),
+    "rmat14": lambda: gg.rmat(14, 30, seed=2)[:3],
+}
+
+
+@pytest.mark.parametrize("name", sorted(GRAPHS))
+def test_one_graph(name):
+    import paper_2309_09064_gb300 as tc
+    rp, col = oracle.build_csr(*GRAPHS[name]())
+    ref = oracle.alg4(rp, col, True)
+    c = tc.tc_create(0)
+    try:
+        g = tc.tc_graph_from_csr(c, rp, col)
+        T, st = tc.tc_count(c, g)
+        assert (T, st["t_same"], st["t_cross"], st["horizontal_edges"]) == (
+            ref["T"], ref["T_same"], ref["T_cross"], ref["E0"])
+        tc.tc_graph_free(g)
+    finally:
+        tc.tc_destroy(c)
+
+
+@pytest.mark.parametrize("extra", [None, 65537])
+def test_union(extra):
+    """All of them in one batch, in two orders; a larger graph takes the union to the classes."""
+    import paper_2309_09064_gb300 as tc
+    graphs = [GRAPHS[k]() for k in sorted(GRAPHS)]
+    if extra:
+        graphs.append(at_end(extra, gg.complete(12)))
+    csr = [oracle.build_csr(*g) for g in graphs]
+    ref = [oracle.alg4(*x, True)["T"] for x in csr]
+    c = tc.tc_create(0)
+    try:
+        tc.tc_set_tuning(c, batch_small_slots=0)
+        gs = [tc.tc_graph_from_csr(c, *x) for x in csr]
+        assert list(tc.tc_count_batch(c, gs)) == ref
+        assert list(tc.tc_count_batch(c, gs[::-1])) == ref[::-1]
+        for g in gs:
+            tc.tc_graph_free(g)
+    finally:
+        tc.tc_destroy(c)
