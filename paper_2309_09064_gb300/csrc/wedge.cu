@@ -1155,8 +1155,10 @@ tc_status wedge_rows(tc_ctx *ctx, const PipeBufs &b, uint32_t n, uint32_t max_de
         const uint64_t cells = (uint64_t)tiles * nb;
         TC_CUDA(ctx, cudaMemsetAsync(b.wedge_work, 0, 8ull * tiles + 4 * cells, s));  // work and counts
         const int smem = (int)(8 * tiles);
-        TC_CUDA(ctx, cudaFuncSetAttribute(k_wedge_entries<false>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem));
-        TC_CUDA(ctx, cudaFuncSetAttribute(k_wedge_entries<true>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem / 2));
+        // (the limit is the process's, not the call's: one value for every thread's launches)
+        const int most = (int)(8 * (kWedgeMaxU / 32 + 1));  // tiles_cap at its largest
+        TC_CUDA(ctx, cudaFuncSetAttribute(k_wedge_entries<false>, cudaFuncAttributeMaxDynamicSharedMemorySize, most));
+        TC_CUDA(ctx, cudaFuncSetAttribute(k_wedge_entries<true>, cudaFuncAttributeMaxDynamicSharedMemorySize, most / 2));
         auto *offs = reinterpret_cast<unsigned long long *>(b.wedge_offs);
         k_wedge_entries<false><<<nb, 1024, smem, s>>>(n, b.slots, b.rp, b.adj2, b.fcnt, b.gcnt, b.wedge_counts, offs,
                                                       b.wedge_work, b.erec, b.erec_cap, tiles, per_warp, b.lv, b.wedge_v, ctx->d_ctl);

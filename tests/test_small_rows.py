@@ -69,3 +69,36 @@ def test_union(extra):
             tc.tc_graph_free(g)
     finally:
         tc.tc_destroy(c)
+
+
+@pytest.mark.parametrize("form", ["count", "batch"])
+def test_threads_with_graphs_of_different_sizes(form):
+    """Two contexts count small and large graphs at once: what a launch may use is set for all of them."""
+    import threading
+    import paper_2309_09064_gb300 as tc
+    sizes = [gg.rmat(7, 8, seed=1)[:3], gg.rmat(15, 8, seed=1)[:3]] if form == "batch" else [
+        gg.rmat(16, 8, seed=1)[:3], gg.rmat(19, 8, seed=1)[:3]]
+    errors = []
+
+    def work(graph):
+        c = tc.tc_create(0)
+        try:
+            rp, col = oracle.build_csr(*graph)
+            want = oracle.alg4(rp, col, True)["T"]
+            g = tc.tc_graph_from_csr(c, rp, col)
+            for _ in range(150):
+                got = list(tc.tc_count_batch(c, [g, g])) if form == "batch" else [tc.tc_count(c, g)[0]]
+                if set(got) != {want}:
+                    errors.append((got, want))
+            tc.tc_graph_free(g)
+        except Exception as e:  # noqa: BLE001 -- reported by the test's thread
+            errors.append(e)
+        finally:
+            tc.tc_destroy(c)
+
+    threads = [threading.Thread(target=work, args=(x,)) for x in sizes for _ in range(2)]
+    for t in threads:
+        t.start()
+    for t in threads:
+        t.join()
+    assert not errors
