@@ -103,11 +103,18 @@ tc_status count_pipeline(tc_ctx *ctx, const GraphView &g, uint32_t *levels_out, 
     const bool plain = !(vertex_counts || list || alg3);
     // plain and per-vertex counts of one graph under the degree order
     const bool small = plain && small_path(ctx, n, g.slots, g.max_deg, groups);
-    const bool wedge = !small && !list && !alg3 && groups.n_groups == 0 && wedge_path(ctx, n, g.slots, g.max_deg);
-    const size_t need = pipeline_bytes(ctx, n, g.slots, g.max_deg, levels_out == nullptr, plain, wedge, &hub_words,
-                                       &hub_maps) +
-                        (vertex_counts ? 8ull * ((size_t)n + 1) + 256 : 0) + (list ? list_bytes(ctx, n, list->capacity) : 0);
-    tc_status st = arena_reserve(ctx, need);
+    bool wedge = !small && !list && !alg3 && groups.n_groups == 0 && wedge_path(ctx, n, g.slots, g.max_deg);
+    auto reserve = [&] {
+        return arena_reserve(ctx, pipeline_bytes(ctx, n, g.slots, g.max_deg, levels_out == nullptr, plain, wedge, &hub_words,
+                                                 &hub_maps) +
+                                      (vertex_counts ? 8ull * ((size_t)n + 1) + 256 : 0) +
+                                      (list ? list_bytes(ctx, n, list->capacity) : 0));
+    };
+    tc_status st = reserve();
+    if (st == TC_ERR_OOM && wedge) {  // the tiles' scratch (20 bytes a slot) does not fit: the classes need 16
+        wedge = false;
+        st = reserve();
+    }
     if (st != TC_OK) return st;
     Arena &a = ctx->arena;
     a.reset();

@@ -71,6 +71,49 @@ def test_union(extra):
         tc.tc_destroy(c)
 
 
+def test_classes_when_the_tiles_scratch_does_not_fit():
+    """Device memory for the classes' scratch but not for the tiles': the count takes the classes."""
+    import paper_2309_09064_gb300 as tc
+    rp, col = oracle.build_csr(*gg.rmat(18, 16, seed=3)[:3])
+    want = oracle.alg4(rp, col, True)
+
+    def count(tuned, c):
+        if tuned:
+            tc.tc_set_tuning(c, flat_cap=96)
+        g = tc.tc_graph_from_csr(c, rp, col)
+        T, st = tc.tc_count(c, g)
+        held = tc.tc_arena_bytes(c)
+        tc.tc_graph_free(g)
+        assert (T, st["t_same"]) == (want["T"], want["T_same"])
+        return held, sum(st["class_rows"][2:]) > 0
+
+    def fresh(tuned):
+        c = tc.tc_create(0)
+        try:
+            return count(tuned, c)
+        finally:
+            tc.tc_destroy(c)
+
+    (tiles, no), (classes, yes) = fresh(False), fresh(True)  # (an arena holds 9/8 of what a count asks for)
+    assert not no and yes and tiles > classes + (16 << 20)
+    c = tc.tc_create(0)
+    try:
+        g = tc.tc_graph_from_csr(c, rp, col)  # (its memory comes before the rest is taken)
+        torch.cuda.empty_cache()
+        room = (tiles + classes) // 2 * 8 // 9
+        fill = torch.empty(torch.cuda.mem_get_info()[0] - room, dtype=torch.uint8, device="cuda")
+        try:
+            T, st = tc.tc_count(c, g)
+        finally:
+            del fill
+            torch.cuda.empty_cache()
+        assert (T, st["t_same"]) == (want["T"], want["T_same"])
+        assert sum(st["class_rows"][2:]) > 0
+        tc.tc_graph_free(g)
+    finally:
+        tc.tc_destroy(c)
+
+
 @pytest.mark.parametrize("form", ["count", "batch"])
 def test_threads_with_graphs_of_different_sizes(form):
     """Two contexts count small and large graphs at once: what a launch may use is set for all of them."""
