@@ -45,13 +45,13 @@ WORKLOADS = {
     "grid4096": dict(kind="grid", rows=4096, cols=4096, p=0.3, seed=4),
 }
 CPU_SAMPLE = dict(kind="rmat", scale=18, edge_factor=16, seed=1)
-# DRAM bytes (read + write) of one launch of the dominant kernel, from a one-pass
+# DRAM bytes (read + write) of the dominant kernels in one count, from a one-pass
 # ncu capture of this bench's default command (plain count, default tuning),
 # with the digest of the kernel sources it was taken on (kernel_sources_digest):
 # once those sources change the figure no longer describes the kernel, and the
 # line reports traffic as null until it is captured again.
-MEASURED_TRAFFIC = {("rmat24", "k_isect_block"): (183.95e9, "151078ba95cca03e")}
-KERNEL_SOURCES = ["isect.cu", "rows.cu", "pipeline.cuh", "tc_internal.cuh"]
+MEASURED_TRAFFIC = {}
+KERNEL_SOURCES = ["wedge.cu", "walk.cuh", "pipeline.cuh", "tc_internal.cuh"]
 
 
 def kernel_sources_digest():
@@ -512,6 +512,9 @@ def main():
         "k_isect_hub": (mean("ms_class", 2), mean("class_bytes", 2)),
         "k_isect_tiny": (mean("ms_class", 3), mean("class_bytes", 3)),
     }
+    if not any(stats[-1]["class_rows"][2:]):  # no hub or tiny rows: the tiles (or, of a small graph, the bitmaps) counted
+        kernels = {"k_wedge_tiles + k_wedge_high": kernels["k_isect_block"],
+                   "k_wedge_rest" if n_ > 32768 else "k_small_count": kernels["k_isect_warp"]}
     if args.alg3:  # one kernel: its time is the intersection stage's
         kernels = {"k_alg3": (mean("ms_isect"), mean("class_bytes", 0))}
     dom = max(kernels, key=lambda k: kernels[k][0])
@@ -575,6 +578,7 @@ def main():
         "triangles": T0, "t_same": last["t_same"], "t_cross": last["t_cross"],
         "horizontal_edges": last["horizontal_edges"], "levels": last["levels"],
         "stage_ms": {"levels": mean("ms_levels"), "rows": mean("ms_mark"), "intersect": mean("ms_isect"),
+                     # (counts without classes: warp = k_wedge_rest or k_small_count, block = the tiles)
                      "isect_warp": mean("ms_class", 0), "isect_block": mean("ms_class", 1),
                      "isect_hub": mean("ms_class", 2), "isect_tiny": mean("ms_class", 3)},
         "roofline": roofline, "gpu_launches": int(sum(st["launches"] for st in stats)),
