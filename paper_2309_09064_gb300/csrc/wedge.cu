@@ -774,8 +774,9 @@ __global__ void __launch_bounds__(kTileThreads, 1) k_wedge_tiles(uint32_t n, con
 // have few of them.  A bitmap (2^17 bits, indexed by the rank's low bits) says
 // which w the tile's vertices can have: most keys end there, with one shared
 // load.  The words of the others sit in a hash table (linear probing, {rank,
-// word}, at most three quarters full; a tile with more high keys is walked in
-// several rounds, each with the keys of one hash class).  A warp flattens the
+// word}, at most three quarters full: a tile with more high keys is walked in
+// several rounds, each with the next kHighKeys of them in row order, so that
+// every key of a row is in one round's table).  A warp flattens the
 // high keys of 32 entries, one per lane and window.  R-MAT 24 (3.5 G keys): 7.8 ms;
 // with 4096 keys a round and no bitmap 13.5, with 2048 and a bitmap 15.5 (two
 // rounds over the entries where one now does), four lanes per entry 17.7.
@@ -796,7 +797,7 @@ __global__ void __launch_bounds__(kHighThreads, 2) k_wedge_high(uint32_t n, cons
     extern __shared__ __align__(16) uint32_t member[];  // kHighBits bits, the table, the warps' entries
     uint2 *table = reinterpret_cast<uint2 *>(member + kHighBits / 32);
     __shared__ uint4 s_task[2];
-    __shared__ uint32_t s_items;
+    __shared__ uint32_t s_first[33];  // high keys of the tile's vertices before each of them
     const unsigned lane = lane_id(), warp = threadIdx.x >> 5;
     uint4 *ent = reinterpret_cast<uint4 *>(table + kHighSlots) + warp * 32;
     const uint32_t n_tasks = (uint32_t)ctl->n_tasks[1];
@@ -815,15 +816,23 @@ __global__ void __launch_bounds__(kHighThreads, 2) k_wedge_high(uint32_t n, cons
         const bool fresh = task.x != tile || rounds > 1;
         if (fresh) {
             tile = task.x;
-            if (threadIdx.x == 0) s_items = 0;
-            __syncthreads();
-            if (threadIdx.x < 32 && 32 * tile + lane < n) {
-                const uint4 m = rmeta[32 * tile + lane];
-                if (m.z > m.w) atomicAdd(&s_items, m.z - m.w);
+            if (warp == 0) {
+                uint32_t incl = 0;
+                if (32 * tile + lane < n) {
+                    const uint4 m = rmeta[32 * tile + lane];
+                    incl = m.z - m.w;
+                }
+#pragma unroll
+                for (int o = 1; o < 32; o <<= 1) {
+                    const uint32_t y = __shfl_up_sync(0xFFFFFFFFu, incl, o);
+                    if (lane >= (unsigned)o) incl += y;
+                }
+                s_first[lane + 1] = incl;
+                if (lane == 0) s_first[0] = 0;
             }
             __syncthreads();
-            rounds = (s_items + kHighKeys - 1) / kHighKeys;
-            if (threadIdx.x == 0) inserts += s_items;
+            rounds = (s_first[32] + kHighKeys - 1) / kHighKeys;
+            if (threadIdx.x == 0) inserts += s_first[32];
         }
         for (uint32_t round = 0; round < rounds; ++round) {
             if (fresh) {
@@ -834,12 +843,14 @@ __global__ void __launch_bounds__(kHighThreads, 2) k_wedge_high(uint32_t n, cons
                 }
                 __syncthreads();
                 for (uint32_t r = warp; r < 32; r += kHighThreads / 32) {
-                    if (32 * tile + r >= n) break;
+                    // the row's high keys that are this round's
+                    const uint32_t first = s_first[r], lo = max(first, round * kHighKeys);
+                    const uint32_t hi = min(s_first[r + 1], (round + 1) * kHighKeys);
+                    if (lo >= hi) continue;
                     const uint4 m = rmeta[32 * tile + r];
-                    const uint32_t *nu = keys + (((uint64_t)m.y << 32) | m.x);
-                    for (uint32_t p = m.w + lane; p < m.z; p += 32) {
+                    const uint32_t *nu = keys + (((uint64_t)m.y << 32) | m.x) + m.w;
+                    for (uint32_t p = lo - first + lane; p < hi - first; p += 32) {
                         const uint32_t w = nu[p] >> 1, h = w * 0x9E3779B1u;
-                        if (rounds > 1 && (h & 0xFFFFu) % rounds != round) continue;
                         atomicOr(&member[(w & (kHighBits - 1)) >> 5], 1u << (w & 31u));
                         uint32_t s = h >> kHighShift, tries = 0;
                         for (; tries < kHighSlots; ++tries) {
