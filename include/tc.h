@@ -120,7 +120,8 @@ typedef struct tc_stats {
  * (wedge.cu) or, of up to 2^15 vertices, by a bitmap of the latest's neighbours
  * (small.cu; tc_count_batch too, when no graph of the union has more than 65536
  * vertices and the mean degree is at most 64).  Any of them changed selects the classes, as do the id order,
- * more than 2^30 CSR slots, and every other mode.
+ * more than 2^30 CSR slots, every other mode, and an estimate that they are
+ * faster (many vertices of high and much the same degree, wedge.cu).
  */
 typedef struct tc_tuning {
     uint32_t warp_cap;         /* s(u) <= warp_cap: one warp per task, per-warp shared table (1..4096) */

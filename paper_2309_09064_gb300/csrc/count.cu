@@ -167,25 +167,9 @@ tc_status count_pipeline(tc_ctx *ctx, const GraphView &g, uint32_t *levels_out, 
     b.erec = a.take<uint4>(b.erec_cap);
     b.scan_tmp = a.take<uint64_t>(scan_tmp_elems(std::max<uint64_t>(n1 + 1, 256 * rtiles + 2)));
     b.task_cap = g.slots / 2 + 1;
-    if (!wedge) {
-        b.fence = a.take<uint32_t>(g.slots / 32 + 2);
-        b.task_pool = a.take<uint2>(b.task_cap);
-        ok = ok && b.fence && b.task_pool;
-    }
     b.hub_words = hub_words;
     b.hub_sets = hub_maps > ctx->tune.hub_group ? 2u : 1u;
     if (hub_maps) b.hub_bits = a.take<uint32_t>(hub_words * hub_maps);
-    if (wedge) {
-        const WedgeSizes z = wedge_sizes(ctx, n, g.slots);
-        b.wedge_ids = a.take<uint16_t>(4 * g.slots + 8);
-        b.wedge_work = reinterpret_cast<unsigned long long *>(a.take<char>(8ull * z.tiles + 4 * z.counts));
-        b.wedge_counts = reinterpret_cast<uint32_t *>(b.wedge_work + z.tiles);  // (zeroed together)
-        b.wedge_offs = a.take<uint64_t>(z.counts + 1);
-        b.wedge_tasks = a.take<uint4>(z.tasks);
-        b.wedge_tmp = a.take<uint64_t>(z.tmp);
-        if (!plain) b.wedge_v = a.take<uint32_t>(b.erec_cap);
-        ok = ok && b.wedge_ids && b.wedge_work && b.wedge_offs && b.wedge_tasks && b.wedge_tmp && (plain || b.wedge_v);
-    }
     b.groups = groups;
     if (vertex_counts) {
         b.vcount = reinterpret_cast<unsigned long long *>(vertex_counts);
@@ -218,6 +202,26 @@ tc_status count_pipeline(tc_ctx *ctx, const GraphView &g, uint32_t *levels_out, 
         TC_CUDA(ctx, cudaMemsetAsync(b.hits, 0, 8 * z.tiny, s));
         TC_CUDA(ctx, cudaMemsetAsync(b.wstate, 0, 16 * z.states, s));
     }
+    // last, so that a count that turns from the tiles to the classes takes these again in the same place
+    const size_t own = a.off;
+    auto take_own = [&] {
+        a.off = own;
+        if (!wedge) {
+            b.fence = a.take<uint32_t>(g.slots / 32 + 2);
+            b.task_pool = a.take<uint2>(b.task_cap);
+            return b.fence && b.task_pool;
+        }
+        const WedgeSizes z = wedge_sizes(ctx, n, g.slots);
+        b.wedge_ids = a.take<uint16_t>(4 * g.slots + 8);
+        b.wedge_work = reinterpret_cast<unsigned long long *>(a.take<char>(8ull * z.tiles + 4 * z.counts));
+        b.wedge_counts = reinterpret_cast<uint32_t *>(b.wedge_work + z.tiles);  // (zeroed together)
+        b.wedge_offs = a.take<uint64_t>(z.counts + 1);
+        b.wedge_tasks = a.take<uint4>(z.tasks);
+        b.wedge_tmp = a.take<uint64_t>(z.tmp);
+        if (!plain) b.wedge_v = a.take<uint32_t>(b.erec_cap);
+        return b.wedge_ids && b.wedge_work && b.wedge_offs && b.wedge_tasks && b.wedge_tmp && (plain || b.wedge_v);
+    };
+    ok = take_own() && ok;
     ok = ok && b.fpref && b.eoff && b.lv && b.rkeys0 && b.rkeys1 && b.rcounts && b.roffs && b.adj2 && b.erec &&
          b.scan_tmp && (!hub_maps || b.hub_bits);
     if (!ok) return set_error(ctx, TC_ERR_OOM, "arena carve failed");
@@ -232,6 +236,15 @@ tc_status count_pipeline(tc_ctx *ctx, const GraphView &g, uint32_t *levels_out, 
     b.lvp = (n <= (1u << 24) && ctx->h_ctl->max_level < 255) ? lvp : nullptr;
     if (!small) st = compute_ranks(ctx, b, n, g.max_deg, wedge ? wedge_tile_degree(n, g.max_deg) : kNoTiles);
     if (st != TC_OK) return st;
+    if (wedge && ctx->h_ctl->n_dense > kWedgeDense) {
+        bool classes = false;
+        st = wedge_estimate(ctx, b, n, &classes);
+        if (st != TC_OK) return st;
+        if (classes) {
+            wedge = false;
+            if (!take_own()) return set_error(ctx, TC_ERR_OOM, "arena carve failed");
+        }
+    }
     Ctl counted{};                   // listing: the control block after phase 1
     unsigned long long list_tiny = 0;  // listing: triangles of the tiny rows
     if (alg3) {  // the comparison kernel: full neighbourhoods, no rows

@@ -33,19 +33,20 @@ __device__ __forceinline__ unsigned long long warp_min_u64(unsigned long long v)
 
 __global__ void k_init(uint32_t n, const uint64_t *__restrict__ rp, uint32_t *__restrict__ deg,
                        uint32_t *__restrict__ L, Ctl *ctl, uint32_t order) {
-    __shared__ unsigned int s_iso;
+    __shared__ unsigned int s_iso, s_dense;
     __shared__ unsigned long long s_key;
     if (threadIdx.x == 0) {
-        s_iso = 0;
+        s_iso = s_dense = 0;
         s_key = ~0ull;
     }
     __syncthreads();
     unsigned long long best = ~0ull;
-    unsigned iso = 0;
+    unsigned iso = 0, dense = 0;
     const uint64_t stride = (uint64_t)gridDim.x * blockDim.x;
     for (uint64_t v = (uint64_t)blockIdx.x * blockDim.x + threadIdx.x; v < n; v += stride) {
         uint32_t d = (uint32_t)(rp[v + 1] - rp[v]);
         deg[v] = d;
+        dense += d >= kDenseDeg;
         if (d == 0) {
             L[v] = 0;
             ++iso;
@@ -57,13 +58,16 @@ __global__ void k_init(uint32_t n, const uint64_t *__restrict__ rp, uint32_t *__
     }
     best = warp_min_u64(best);
     iso = warp_sum(iso);
+    dense = warp_sum(dense);
     if (lane_id() == 0) {
         atomicMin(&s_key, best);
         atomicAdd(&s_iso, iso);
+        if (dense) atomicAdd(&s_dense, dense);
     }
     __syncthreads();
     if (threadIdx.x == 0) {
         if (s_key != ~0ull) atomicMin(&ctl->root_key, s_key);
+        if (s_dense) atomicAdd(&ctl->n_dense, s_dense);
         if (s_iso) {
             atomicAdd(&ctl->visited, s_iso);
             atomicAdd(&ctl->components, s_iso);
@@ -875,7 +879,7 @@ __global__ void k_given_levels(uint32_t n, const uint64_t *__restrict__ rp, cons
     const unsigned lane = lane_id();
     const uint64_t stride = (uint64_t)gridDim.x * blockDim.x;
     const uint64_t n_round = ((uint64_t)n + 31) & ~uint64_t(31);
-    unsigned bad = 0, top = 0;
+    unsigned bad = 0, top = 0, dense = 0;
     for (uint64_t x = (uint64_t)blockIdx.x * blockDim.x + threadIdx.x; x < n_round; x += stride) {
         const bool valid = x < n;
         const uint64_t b = valid ? rp[x] : 0;
@@ -885,6 +889,7 @@ __global__ void k_given_levels(uint32_t n, const uint64_t *__restrict__ rp, cons
             deg[x] = d;
             L[x] = lx;
             top = lx > top ? lx : top;
+            dense += d >= kDenseDeg;
         }
         if (valid && d <= 32)
             for (uint32_t j = 0; j < d; ++j) {
@@ -905,6 +910,7 @@ __global__ void k_given_levels(uint32_t n, const uint64_t *__restrict__ rp, cons
         }
     }
     bad = __any_sync(0xFFFFFFFFu, bad);
+    dense = warp_sum(dense);
 #pragma unroll
     for (int o = 16; o > 0; o >>= 1) {
         const unsigned y = __shfl_xor_sync(0xFFFFFFFFu, top, o);
@@ -913,6 +919,7 @@ __global__ void k_given_levels(uint32_t n, const uint64_t *__restrict__ rp, cons
     if (lane == 0) {
         if (bad) atomicOr(&ctl->error, 0x200u);
         if (top) atomicMax(&ctl->max_level, top);
+        if (dense) atomicAdd(&ctl->n_dense, dense);
     }
 }
 

@@ -101,6 +101,7 @@ struct PipeBufs {
 // bits stays free: it marks padding).
 constexpr uint32_t kWedgeMaxU = 1u << 19;
 constexpr uint32_t kWedgeMaxK = 32736;
+constexpr uint32_t kWedgeDense = kWedgeMaxK / 2 * 3;  // with more vertices of high degree wedge_estimate chooses
 struct WedgeSizes {
     uint32_t tiles, tasks;
     uint64_t counts, tmp;
@@ -175,5 +176,7 @@ tc_status small_count(tc_ctx *ctx, const PipeBufs &b, uint32_t n, uint32_t max_d
 // the wedge path: rows, entries and tasks, then the two counting kernels
 tc_status wedge_rows(tc_ctx *ctx, const PipeBufs &b, uint32_t n, uint32_t max_deg);
 tc_status wedge_count(tc_ctx *ctx, const PipeBufs &b, uint32_t n, uint32_t max_deg);
+// after compute_ranks, for graphs of many vertices of high degree: whether the classes are the faster path
+tc_status wedge_estimate(tc_ctx *ctx, const PipeBufs &b, uint32_t n, bool *classes);
 
 }  // namespace tc

@@ -42,6 +42,9 @@ struct Tuning {
     uint32_t batch_small_slots = 0;  // batches: graphs this small counted a block each in one launch (0: off)
 };
 
+// Degree from which vertices count towards Ctl::n_dense.
+constexpr uint32_t kDenseDeg = 256;
+
 // Control block in device memory: counters the kernels update and the host
 // reads back between launches.
 struct Ctl {
@@ -80,7 +83,8 @@ struct Ctl {
     unsigned int wedge_u;            // wedge path: vertices taken in tiles (a multiple of 32)
     unsigned int wedge_hi_task;      // first task of the tiles from rank kWedgeMaxK on
     unsigned int residual_left;      // vertices the one-block component step left to the host's loop
-    unsigned int pad;
+    unsigned int n_dense;            // vertices of degree >= kDenseDeg
+    unsigned long long est_wedge, est_classes;  // estimated times of the two counting paths (k_wedge_estimate)
     unsigned long long list_cursor;  // listing: next free chunk position
 };
 

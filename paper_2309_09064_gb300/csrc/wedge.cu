@@ -1080,6 +1080,110 @@ __global__ void __launch_bounds__(kRestThreads) k_wedge_rest(uint32_t n, const u
     }
 }
 
+// ---------------------------------------------------------------------------- tiles or classes
+
+// Where more vertices than a tile's words cover have a high and much the same
+// degree, a tile holds one or two neighbours of any row: a lookup serves one pair
+// instead of 32, and k_wedge_high walks its entries once per kHighKeys keys.  The
+// classes of isect.cu are the faster path there (uniform graphs, tiles / classes:
+// 2^18 vertices of mean degree 512 / 1024 / 2048 32.7 / 201 / 1404 against 18.9 /
+// 69 / 196 ms; at 256 7.05 against 7.27; R-MAT 20 of edge factor 300 59 against 161).
+// So a count with more than kWedgeDense vertices of degree >= kDenseDeg (with half as
+// many ranks past the words as in them, 4% of the pairs are high ones) samples
+// kSamples slots, and for the vertex v of each takes the lookups that its row would
+// cost: every tile with a neighbour of v walks the keys of N(v) up to it, the rest
+// walks N(u), and the classes compare v's horizontal neighbours pairwise and probe its
+// level-spanning ones once per horizontal edge.  Picoseconds, from uniform graphs of
+// 2^16 to 2^21 vertices and mean degree 256 to 4096: high keys 3.7 (times the rounds of
+// v's tiles), 16-bit ids 0.7, rest 2.9; classes 1 a probe (0.7 at degree 2048, 0.5 at
+// 4096), 70 a horizontal edge, and 33 a slot for the larger row stage.  The ratio of the
+// two estimates is within 1.2 of the measured one, and the classes are taken from there
+// on.  One block a sample: about 40 us and a readback.
+constexpr uint32_t kSamples = 1024;
+constexpr uint32_t kSampleDeg = 32768;  // longer rows are not looked at (their vertex has few earlier ones)
+
+__global__ void __launch_bounds__(256) k_wedge_estimate(uint32_t n, uint64_t slots, const uint64_t *__restrict__ rp,
+                                                        const uint32_t *__restrict__ col,
+                                                        const uint32_t *__restrict__ deg,
+                                                        const uint2 *__restrict__ lv, Ctl *ctl) {
+    __shared__ uint32_t seen[kWedgeMaxU / 1024];  // tiles with a neighbour
+    __shared__ unsigned int s_low, s_high, s_hor, s_span, s_tl, s_th;
+    __shared__ unsigned long long s_rest;
+    const uint32_t U = ctl->wedge_u, K = words_of(U);
+    for (uint32_t i = blockIdx.x; i < kSamples; i += gridDim.x) {
+        const uint64_t at = slots * i / kSamples;
+        uint32_t v = 0, hi = n;  // the last row that starts at or before slot `at`
+        while (hi - v > 1) {
+            const uint32_t mid = v + (hi - v) / 2;
+            if (rp[mid] <= at) v = mid; else hi = mid;
+        }
+        const uint64_t b = rp[v];
+        const uint32_t d = deg[v];
+        const uint2 me = lv[v];
+        if (d > kSampleDeg || me.x == 0) continue;
+        for (uint32_t t = threadIdx.x; t < kWedgeMaxU / 1024; t += 256) seen[t] = 0;
+        if (threadIdx.x == 0) {
+            s_low = s_high = s_hor = s_span = s_tl = s_th = 0;
+            s_rest = 0;
+        }
+        __syncthreads();
+        uint32_t low = 0, high = 0, hor = 0, span = 0;
+        unsigned long long rest = 0;
+        for (uint32_t j0 = threadIdx.x; j0 < d; j0 += 1024) {
+            uint32_t y[4];
+            uint2 q[4];
+#pragma unroll
+            for (uint32_t t = 0; t < 4; ++t) y[t] = j0 + 256 * t < d ? col[b + j0 + 256 * t] : v;
+#pragma unroll
+            for (uint32_t t = 0; t < 4; ++t) q[t] = lv[y[t]];
+#pragma unroll
+            for (uint32_t t = 0; t < 4; ++t) {
+                span += q[t].y != me.y;
+                if (q[t].x >= me.x) continue;
+                hor += q[t].y == me.y;
+                if (q[t].x < U) {
+                    atomicOr(&seen[q[t].x >> 10], 1u << ((q[t].x >> 5) & 31u));
+                    if (q[t].x < K) ++low; else ++high;
+                } else {
+                    rest += deg[y[t]] / 2;  // about |N(u)|
+                }
+            }
+        }
+        low = warp_sum(low);
+        high = warp_sum(high);
+        hor = warp_sum(hor);
+        span = warp_sum(span);
+        rest = warp_sum(rest);
+        if (lane_id() == 0) {
+            atomicAdd(&s_low, low);
+            atomicAdd(&s_high, high);
+            atomicAdd(&s_hor, hor);
+            atomicAdd(&s_span, span);
+            atomicAdd(&s_rest, rest);
+        }
+        __syncthreads();
+        for (uint32_t t = threadIdx.x; t < kWedgeMaxU / 1024; t += 256) {
+            const uint32_t first = 32 * t, end = K / 32;  // tiles of this word, tiles below K
+            const uint32_t below = end <= first ? 0u : end - first >= 32 ? 0xFFFFFFFFu : (1u << (end - first)) - 1u;
+            if (seen[t] & below) atomicAdd(&s_tl, (unsigned)__popc(seen[t] & below));
+            if (seen[t] & ~below) atomicAdd(&s_th, (unsigned)__popc(seen[t] & ~below));
+        }
+        __syncthreads();
+        if (threadIdx.x == 0) {
+            const float rounds = fmaxf(1.f, 32.f * (2.f / 3.f) * s_high / kHighKeys);
+            const float keys = 0.5f * s_th * s_high * rounds, ids = 0.5f * s_tl * s_low + (float)s_th * s_low;
+            const float tiles_ps = 3.7f * keys + 0.7f * ids + 2.9f * s_rest;
+            const float probe_ps = sqrtf(1024.f / fmaxf(1024.f, d));
+            const float classes_ps = (probe_ps * (0.5f * s_hor + s_span) + 70.f) * s_hor + 33.f * d;
+            // a slot stands for slots / kSamples, and v is met once per slot of its row (whole numbers: the
+            // sums do not depend on the order)
+            atomicAdd(&ctl->est_wedge, (unsigned long long)(1024.f * tiles_ps / d));
+            atomicAdd(&ctl->est_classes, (unsigned long long)(1024.f * classes_ps / d));
+        }
+        __syncthreads();
+    }
+}
+
 unsigned grid_for(uint64_t work, unsigned threads, unsigned cap) {
     uint64_t b = (work + threads - 1) / threads;
     if (b < 1) b = 1;
@@ -1136,6 +1240,17 @@ bool wedge_path(const tc_ctx *ctx, uint32_t n, uint64_t slots, uint32_t max_deg)
                          t.block_bits_log2 != def.block_bits_log2;
     return !classes && ctx->opt.order == TC_ORDER_DEGREE && ctx->nshards == 1 && max_deg > 0 && n < (1u << 31) &&
            slots <= (uint64_t)kSortCap * kSortCap;
+}
+
+tc_status wedge_estimate(tc_ctx *ctx, const PipeBufs &b, uint32_t n, bool *classes) {
+    k_wedge_estimate<<<std::min<unsigned>(kSamples, (unsigned)ctx->num_sms * 8u), 256, 0, ctx->stream>>>(
+        n, b.slots, b.rp, b.col, b.deg, b.lv, ctx->d_ctl);
+    note_launch(ctx);
+    TC_CUDA(ctx, cudaGetLastError());
+    TC_CUDA(ctx, cudaMemcpyAsync(ctx->h_ctl, ctx->d_ctl, sizeof(Ctl), cudaMemcpyDeviceToHost, ctx->stream));
+    TC_CUDA(ctx, cudaStreamSynchronize(ctx->stream));
+    *classes = 5 * (double)ctx->h_ctl->est_wedge > 6 * (double)ctx->h_ctl->est_classes;
+    return TC_OK;
 }
 
 tc_status wedge_rows(tc_ctx *ctx, const PipeBufs &b, uint32_t n, uint32_t max_deg) {
