@@ -228,6 +228,7 @@ __global__ void __launch_bounds__(512) k_small_count(uint32_t n, const uint16_t 
                                                      const uint2 *__restrict__ slices, GroupSpec groups,
                                                      uint32_t words, uint32_t per_warp, Ctl *ctl) {
     extern __shared__ __align__(16) uint32_t smem[];
+    if (ctl->e0 == 0) return;  // (every triangle has a horizontal edge)
     constexpr uint32_t kW = kSplit ? 2 : 1;
     const unsigned lane = lane_id(), warp = threadIdx.x >> 5;
     const uint32_t sub = lane & 3u;

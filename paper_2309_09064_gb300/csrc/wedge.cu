@@ -367,6 +367,9 @@ __global__ void __launch_bounds__(1024) k_wedge_sort(const uint32_t *__restrict_
 // block takes the same rows (a contiguous range) in both.  A warp flattens the keys of per_warp rows, one per lane and step;
 // the last of the consecutive lanes of one row and tile makes their entries
 // (a tile that straddles two steps gets entries from both).
+// Without horizontal edges (bipartite graphs) there are no entries, and so no tasks,
+// and the other kernels return as well: R-MAT 22 made bipartite 8.58 -> 2.76 ms, a uniform
+// bipartite graph of 2^20 vertices and mean degree 32 1.75 -> 0.94 (the classes 4.35 and 1.16).
 template <bool kScatter>
 __global__ void __launch_bounds__(1024) k_wedge_entries(uint32_t n, uint64_t slots, const uint64_t *__restrict__ rp,
                                                         const uint32_t *__restrict__ keys,
@@ -383,7 +386,7 @@ __global__ void __launch_bounds__(1024) k_wedge_entries(uint32_t n, uint64_t slo
     const unsigned lane = lane_id();
     const uint32_t U = ctl->wedge_u;
     const uint32_t tiles = U >> 5, nb = gridDim.x;
-    if (tiles == 0) return;
+    if (tiles == 0 || ctl->e0 == 0) return;  // (every triangle has a horizontal edge)
     if (tiles > tiles_cap) {
         if (threadIdx.x == 0) atomicOr(&ctl->error, kGuardRange);
         return;
@@ -973,6 +976,7 @@ __global__ void __launch_bounds__(kRestThreads) k_wedge_rest(uint32_t n, const u
                                                              Ctl *ctl, const uint2 *__restrict__ lv,
                                                              unsigned long long *__restrict__ credit) {
     __shared__ uint32_t sfilter[kRestThreads / 32][kFilterBits / 32];
+    if (ctl->e0 == 0) return;  // (every triangle has a horizontal edge)
     const unsigned lane = lane_id(), warp = threadIdx.x >> 5;
     const uint32_t sub = lane & 7u, group = lane >> 3;
     uint32_t *filter = sfilter[warp];
