@@ -104,16 +104,25 @@ tc_status count_pipeline(tc_ctx *ctx, const GraphView &g, uint32_t *levels_out, 
     // plain and per-vertex counts of one graph under the degree order
     const bool small = plain && small_path(ctx, n, g.slots, g.max_deg, groups);
     bool wedge = !small && !list && !alg3 && groups.n_groups == 0 && wedge_path(ctx, n, g.slots, g.max_deg);
-    auto reserve = [&] {
-        return arena_reserve(ctx, pipeline_bytes(ctx, n, g.slots, g.max_deg, levels_out == nullptr, plain, wedge, &hub_words,
-                                                 &hub_maps) +
-                                      (vertex_counts ? 8ull * ((size_t)n + 1) + 256 : 0) +
-                                      (list ? list_bytes(ctx, n, list->capacity) : 0));
+    auto bytes = [&] {
+        return pipeline_bytes(ctx, n, g.slots, g.max_deg, levels_out == nullptr, plain, wedge, &hub_words, &hub_maps) +
+               (vertex_counts ? 8ull * ((size_t)n + 1) + 256 : 0) + (list ? list_bytes(ctx, n, list->capacity) : 0);
     };
-    tc_status st = reserve();
-    if (st == TC_ERR_OOM && wedge) {  // the tiles' scratch (20 bytes a slot) does not fit: the classes need 16
+    // Where the tiles' scratch (20 bytes a slot) does not fit, the classes count (16 bytes).  A size that did not
+    // is asked for again only once the device has room for it: trying gives the arena back first.
+    size_t need = bytes();
+    if (wedge && need > ctx->arena.cap && need >= ctx->wedge_oom) {
+        size_t free_b = 0, total_b = 0;
+        if (cudaMemGetInfo(&free_b, &total_b) != cudaSuccess) cudaGetLastError();
+        wedge = free_b + ctx->arena.cap >= need + need / 8;
+        need = bytes();
+    }
+    tc_status st = arena_reserve(ctx, need);
+    if (wedge && st == TC_OK) ctx->wedge_oom = std::max(ctx->wedge_oom, need + 1);
+    if (wedge && st == TC_ERR_OOM) {
+        ctx->wedge_oom = std::min(ctx->wedge_oom, need);
         wedge = false;
-        st = reserve();
+        st = arena_reserve(ctx, bytes());
     }
     if (st != TC_OK) return st;
     Arena &a = ctx->arena;

@@ -139,6 +139,7 @@ struct tc_ctx {
     uint32_t shard = 0, nshards = 1;  // intersection tasks of this count: share `shard` of `nshards`
     uint32_t split_R = 0;             // this count's split rank (block-class bitmap; 0: none)
     uint32_t bfs_cluster[2] = {0, 0}; // blocks of the cluster BFS, by slot width (0: not asked yet)
+    size_t wedge_oom = ~size_t(0);    // arena sizes of the tiles from this on did not fit (count.cu)
     uint64_t alloc_calls = 0;         // device allocations made by this context
     uint64_t fail_alloc_at = 0;       // fault injection: fail this allocation (1-based; 0 = never)
     std::string err;
