@@ -355,9 +355,13 @@ __global__ void k_group_roots(GroupSpec groups, const uint32_t *__restrict__ deg
 // The components left after the first BFS, where they are small together: one
 // block hooks them, roots them and levels them (the steps of the kernels above
 // with block barriers between them, instead of ten launches and five round trips
-// to the host).  More than kResidualMax vertices, or one of degree above
-// kResidualDeg, are left to those.  Parents are read past L1: hooking changes them by atomics.
-constexpr uint32_t kResidualMax = 8192, kResidualDeg = 256;
+// to the host).  More than kResidualMax vertices, kResidualSlots CSR slots (trees and
+// cycles, two slots a vertex, may have more), or a vertex of degree above kResidualDeg are
+// left to those.  All levels of R-MAT 17 beside a uniform component, in one block / by the
+// kernels above: 2000 vertices of mean degree 8 0.44 / 0.31 ms, 8000 of 4 0.64 / 0.36, 1000 of
+// 30 0.57 / 0.36, 1000 of 8 0.32 / 0.32; R-MAT 18 beside a path of 8000 11.2 / 18.8.
+// Parents are read past L1: hooking changes them by atomics.
+constexpr uint32_t kResidualMax = 8192, kResidualSlots = 4096, kResidualDeg = 256;
 
 __device__ __forceinline__ uint32_t find_root_cg(const uint32_t *parent, uint32_t x, uint32_t n, Ctl *ctl) {
     for (uint32_t it = 0; it <= n; ++it) {
@@ -373,13 +377,22 @@ __global__ void __launch_bounds__(1024) k_residual(const uint32_t *__restrict__ 
                                                    const uint64_t *__restrict__ rp, const uint32_t *__restrict__ col,
                                                    const uint32_t *__restrict__ deg, uint32_t *parent, uint32_t *L,
                                                    uint32_t *q0, uint32_t *q1, Ctl *ctl, uint32_t order) {
-    __shared__ unsigned int s_changed, s_count[2], s_roots;
+    __shared__ unsigned int s_changed, s_count[2], s_roots, s_slots;
     __shared__ unsigned long long s_edges;
     const uint32_t nr = ctl->n_residual;
     if (nr == 0) return;
     bool wide = nr > kResidualMax;  // a thread walks a vertex's neighbours: long rows are left too
-    for (uint32_t i = threadIdx.x; i < nr && !wide; i += blockDim.x) wide = deg[R[i]] > kResidualDeg;
-    if (__syncthreads_or(wide)) {
+    if (threadIdx.x == 0) s_slots = 0;
+    __syncthreads();
+    uint32_t slots = 0;
+    for (uint32_t i = threadIdx.x; i < nr && !wide; i += blockDim.x) {
+        const uint32_t d = deg[R[i]];
+        wide = d > kResidualDeg;
+        slots += d;
+    }
+    slots = warp_sum(slots);
+    if (lane_id() == 0) atomicAdd(&s_slots, slots);
+    if (__syncthreads_or(wide) || s_slots > max(kResidualSlots, 2 * nr)) {
         if (threadIdx.x == 0) ctl->residual_left = nr;
         return;
     }
@@ -518,7 +531,10 @@ __device__ __forceinline__ bool grid_barrier(Ctl *ctl, unsigned nblocks, unsigne
 // block before the barrier, so that all leave at the same level) when a vertex
 // of degree above max_d is claimed or a queue overflows; the frontier left is
 // written back to q0.  With `whole` it goes on with the first vertex of the next
-// component, up to kMaxRoots of them.
+// component, up to kMaxRoots of them: a root costs a walk over all vertices and three
+// barriers, 13 us, and k_residual takes small components together (500 triangles 0.55
+// ms with up to 32 roots, 0.11 with 2; R-MAT 13 beside 1 / 3 / 20 triangles 0.10 / 0.16 /
+// 0.37 against 0.11 / 0.11 / 0.12).
 // Where ids follow the geometry (grids, road networks) the lines ahead of and
 // behind a claimed vertex's are the next levels': they are asked into L2.
 constexpr uint32_t kClusterThreads = 1024;  // 32 warps: wkey below counts on it
@@ -526,7 +542,7 @@ constexpr uint32_t kQueueCap = 4096;   // frontier vertices a block keeps (past 
 constexpr uint32_t kEdgeBytes = 48 * 1024;  // room for the edge slots of one frontier
 constexpr uint32_t kHubDeg = 256;
 constexpr uint32_t kHubCap = 256;      // hubs per level expanded by the whole cluster
-constexpr uint32_t kMaxRoots = 32;
+constexpr uint32_t kMaxRoots = 2;
 constexpr uint32_t kSpreadFirst = 3;
 constexpr uint32_t kLaneRow = 8;
 
