@@ -523,8 +523,11 @@ __device__ __forceinline__ bool grid_barrier(Ctl *ctl, unsigned nblocks, unsigne
 // read beside it) -> queue -> barrier; a 4096 x 4096 grid (4746 levels of about
 // 3500 vertices) took 5.7 us a level with a grid-wide barrier over 64 blocks and
 // a queue in global memory, 4.8 with queues of vertices here.
-// Claimed vertices stay with their block, except in the first levels and every
-// 16th one, when they are spread over the cluster by their ids.
+// Claimed vertices stay with their block, except those of degree above kFarRow, and all in
+// the first levels and every 16th one: these are spread over the cluster by their ids.  (One
+// block claims all of a few long rows' ends, whose edges are then too many for its queue: a
+// ring of 2^17 vertices of degree 200 takes 23 us a level without kFarRow, 8.1 with it;
+// a chain of cliques of 200 vertices 20 and 6.2.)
 // A vertex of degree above kHubDeg is expanded by the whole cluster (its edges
 // strided over all blocks).  The kernel ends when a frontier was empty or had
 // more than max_f vertices or max_e edges, or (the `stop` flag, set in every
@@ -545,6 +548,7 @@ constexpr uint32_t kHubCap = 256;      // hubs per level expanded by the whole c
 constexpr uint32_t kMaxRoots = 2;
 constexpr uint32_t kSpreadFirst = 3;
 constexpr uint32_t kLaneRow = 8;
+constexpr uint32_t kFarRow = 32;
 
 // Slot: an edge's place in col (32 bits where they are enough).
 template <class Slot>
@@ -620,7 +624,7 @@ __global__ void __launch_bounds__(kClusterThreads, 1) k_bfs_cluster(const BfsArg
     auto push_spread = [&](uint32_t v, uint64_t b, uint32_t d, uint32_t s, uint32_t p) {
         const uint32_t e = d > kHubDeg && push_hub(b, d, s, p) ? 0u : d;
         Shared *T = cl.map_shared_rank(&S, (v * 0x9E3779B1u) >> hshift);
-        const uint32_t at = atomicAdd(&T->cnt[s], 1u), first = atomicAdd(&T->edges[s], e);
+        const uint32_t at = atomicAdd(&T->cnt[s], 1u), first = atomicAdd(&T->edges[s], min(e, Shared::kEdgeCap + 1));
         if (!store(T, v, b, e, at, first, p) || d > g.max_d) stop_all(s);
     };
     // Ask L2 for the lines of L, rp, deg and col 32 vertices either side of v (a DRAM
@@ -699,29 +703,35 @@ __global__ void __launch_bounds__(kClusterThreads, 1) k_bfs_cluster(const BfsArg
             if (e > kHubDeg && push_hub(b, d, ns, np)) e = 0;
             // places in the queues: the claiming block's, or the one the id hashes to
             uint32_t owner = me, at = 0, first_edge = 0;
-            if (spread) {
+            const bool far = got && (spread || e > kFarRow);
+            if (far) {
                 owner = (w * 0x9E3779B1u) >> hshift;
-                if (got) {
-                    Shared *T = cl.map_shared_rank(&S, owner);
-                    at = atomicAdd(&T->cnt[ns], 1u);
-                    first_edge = atomicAdd(&T->edges[ns], e);
-                }
-            } else {
-                uint32_t incl = e;
+                Shared *T = cl.map_shared_rank(&S, owner);
+                at = atomicAdd(&T->cnt[ns], 1u);
+                first_edge = atomicAdd(&T->edges[ns], min(e, Shared::kEdgeCap + 1));  // (more does not fit either)
+            }
+            if (!spread) {
+                const bool near = got && !far;
+                const unsigned nm = __ballot_sync(0xFFFFFFFFu, near);
+                const uint32_t ne = near ? e : 0u;
+                uint32_t incl = ne, place = 0;
 #pragma unroll
                 for (int o = 1; o < 32; o <<= 1) {
                     const uint32_t y = __shfl_up_sync(0xFFFFFFFFu, incl, o);
                     if (lane >= (unsigned)o) incl += y;
                 }
-                if (lane == 31) at = atomicAdd(&S.edges[ns], incl);
-                if (lane == 0) at = atomicAdd(&S.cnt[ns], (unsigned)__popc(m));
-                first_edge = __shfl_sync(0xFFFFFFFFu, at, 31) + incl - e;
-                at = __shfl_sync(0xFFFFFFFFu, at, 0) + __popc(m & ((1u << lane) - 1u));
+                if (lane == 31) place = atomicAdd(&S.edges[ns], incl);
+                if (lane == 0) place = atomicAdd(&S.cnt[ns], (unsigned)__popc(nm));
+                const uint32_t e0 = __shfl_sync(0xFFFFFFFFu, place, 31), v0 = __shfl_sync(0xFFFFFFFFu, place, 0);
+                if (near) {
+                    first_edge = e0 + incl - ne;
+                    at = v0 + __popc(nm & ((1u << lane) - 1u));
+                }
             }
             // rows of more than kLaneRow slots that fit are written by the whole warp
             const bool wide = got && e > kLaneRow && at < kQueueCap && first_edge + e <= Shared::kEdgeCap;
             if (got) {
-                Shared *T = spread ? cl.map_shared_rank(&S, owner) : &S;
+                Shared *T = far ? cl.map_shared_rank(&S, owner) : &S;
                 if (wide) T->qv[np][at] = w;
                 const bool fits = wide || store(T, w, b, e, at, first_edge, np);
                 if (!fits || d > g.max_d) stop_all(ns);
@@ -879,7 +889,11 @@ unsigned grid_for(uint64_t work, unsigned threads, unsigned cap) {
 // edges a level, and a level costs it no round trip to the host.
 constexpr uint32_t kClusterMaxF = 32768;
 constexpr uint32_t kClusterMaxE = 65536;
-constexpr uint32_t kClusterMaxD = 1024;  // one vertex's: its neighbours' edges may overflow the queues
+// One vertex's degree: its neighbours' edges may overflow the queues.  The first vertex is
+// the one of the highest degree, and its neighbours have more edges than later ones do: a
+// path of vertices with 1100 leaves each takes 74 us a level at 1024 later on too, 3.9 at 4096;
+// a power law of 2^18 vertices whose first has degree 2048 takes 0.20 ms at 1024 there, 0.23 at 4096.
+constexpr uint32_t kClusterMaxD = 4096, kClusterSeedD = 1024;
 // Graphs it levels from the first root to the last component.
 constexpr uint32_t kWholeN = 65536;
 constexpr uint64_t kWholeSlots = 1u << 18;
@@ -970,7 +984,7 @@ static tc_status launch_cluster(tc_ctx *ctx, const PipeBufs &b, uint32_t n, uint
     a.whole = seed && n <= kWholeN && slots <= kWholeSlots;
     a.max_f = a.whole ? 0xFFFFFFFFu : kClusterMaxF;
     a.max_e = a.whole ? 0xFFFFFFFFu : kClusterMaxE;
-    a.max_d = a.whole ? 0xFFFFFFFFu : kClusterMaxD;
+    a.max_d = a.whole ? 0xFFFFFFFFu : seed ? kClusterSeedD : kClusterMaxD;
     cudaLaunchAttribute attr{};
     attr.id = cudaLaunchAttributeClusterDimension;
     cudaLaunchConfig_t cfg{};
