@@ -170,6 +170,8 @@ constexpr uint32_t kWarpRow = 1024;    // by its warp
 constexpr uint32_t kBlockRow = 8192;   // by a block; longer rows go through bitmaps
 constexpr int kRowThreads = 256;
 constexpr uint32_t kMapBits = 1u << 20;  // ids a bitmap covers (128 KB of shared memory)
+// Rows whose bitmap lies in global memory: least entries, and how many (more of them keep every SM busy as it is).
+constexpr uint32_t kGiantRow = 1u << 17, kGiants = 64;
 constexpr uint32_t kNoPlace = 0xFFFFFFFFu;
 
 // Entries before a vertex's newest one, one atomic per distinct vertex of the
@@ -221,13 +223,15 @@ __global__ void k_place_entries(uint64_t t, const uint32_t *__restrict__ src, co
 }
 
 // Rows of up to kWarpRow entries: sorted in place, repeats dropped; deg[v] =
-// entries left.  Longer rows are listed for a block each, or for the bitmaps.
+// entries left.  Longer rows are listed for a block each, or for the bitmaps (from
+// `giant` entries on in global memory).
 // Lanes own rows of up to kLaneRow entries (insertion sort in their column of
 // the warp's buffer), the warp takes the others one by one.
 __global__ void __launch_bounds__(kRowThreads) k_sort_rows(uint32_t n, const uint64_t *__restrict__ start,
                                                            uint32_t *__restrict__ raw, uint32_t *__restrict__ deg,
                                                            uint32_t *__restrict__ big, uint32_t *__restrict__ huge,
-                                                           uint32_t per_warp, Ctl *ctl) {
+                                                           uint32_t *__restrict__ giants, uint32_t per_warp,
+                                                           uint32_t giant, Ctl *ctl) {
     __shared__ __align__(16) uint32_t sbuf[kRowThreads / 32][kWarpRow];
     const unsigned lane = lane_id(), warp = threadIdx.x >> 5;
     const unsigned lt = (1u << lane) - 1u;
@@ -268,7 +272,14 @@ __global__ void __launch_bounds__(kRowThreads) k_sort_rows(uint32_t n, const uin
         __syncwarp();
         if (valid && d > kWarpRow) {
             if (d <= kBlockRow) big[atomicAdd(&ctl->n_big, 1u)] = (uint32_t)x;
-            else huge[atomicAdd(&ctl->n_huge, 1u)] = (uint32_t)x;
+            else {
+                const uint32_t at = atomicAdd(&ctl->n_huge, 1u);
+                huge[at] = (uint32_t)x;
+                const uint32_t g = d >= giant ? atomicAdd(&ctl->n_giant, 1u) : kGiants;
+                if (g < kGiants) giants[g] = (uint32_t)x;
+                // the number of its bitmap (the list of big rows ends before: a row is in one of the two)
+                big[n - 1 - at] = g < kGiants ? g : kNoPlace;
+            }
         }
         unsigned pending = __ballot_sync(0xFFFFFFFFu, valid && d > kLaneRow && d <= kWarpRow);
         while (pending) {
@@ -330,13 +341,16 @@ __device__ __forceinline__ void compare_swap(uint32_t *sb, uint32_t i, uint32_t 
 
 __global__ void __launch_bounds__(256) k_sort_rows_big(const uint64_t *__restrict__ start, uint32_t *__restrict__ raw,
                                                        uint32_t *__restrict__ deg, const uint32_t *__restrict__ big,
-                                                       Ctl *ctl) {
+                                                       uint32_t *__restrict__ maps, uint32_t giant_words, Ctl *ctl) {
     __shared__ __align__(16) uint32_t sb[kBlockRow];
     __shared__ uint32_t warp_cnt[32];
     __shared__ unsigned int s_i;
     const unsigned lane = lane_id(), warp = threadIdx.x >> 5;
     uint32_t *run = sb + 1024 * warp;  // eight warps, 1024 keys each
     const uint32_t nb = ctl->n_big;
+    const uint64_t words = (uint64_t)min(ctl->n_giant, kGiants) * giant_words;
+    for (uint64_t i = (uint64_t)blockIdx.x * blockDim.x + threadIdx.x; i < words; i += (uint64_t)gridDim.x * blockDim.x)
+        maps[i] = 0;  // (for k_mark_giant)
     for (;;) {
         if (threadIdx.x == 0) s_i = atomicAdd(&ctl->sort_next, 1u);
         __syncthreads();
@@ -397,13 +411,47 @@ __global__ void __launch_bounds__(256) k_sort_rows_big(const uint64_t *__restric
     }
 }
 
+// The ids of the giant rows, marked in bitmaps in global memory (L2) by the whole grid: a
+// block of k_map_rows reads 2.3 entries a clock, so a vertex named by most tuples kept a
+// few blocks busy and the others idle (2^24 tuples of 2^22 vertices, one of them in every
+// tuple: 17.4 -> 1.9 ms; the radix sort 3.1).  A warp takes 1024 entries; set bits are not set again.
+__global__ void __launch_bounds__(256) k_mark_giant(const uint64_t *__restrict__ start,
+                                                    const uint32_t *__restrict__ raw,
+                                                    const uint32_t *__restrict__ giants, uint32_t *maps,
+                                                    uint32_t giant_words, const Ctl *ctl) {
+    const uint32_t ng = min(ctl->n_giant, kGiants);
+    const uint64_t warps = ((uint64_t)gridDim.x * blockDim.x) >> 5;
+    const uint64_t w0 = ((uint64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5;
+    for (uint32_t g = 0; g < ng; ++g) {
+        uint32_t *map = maps + (uint64_t)g * giant_words;
+        const uint64_t b = start[giants[g]], e = start[giants[g] + 1];
+        for (uint64_t j0 = b + 1024 * w0; j0 < e; j0 += 1024 * warps) {
+#pragma unroll
+            for (uint32_t k = 0; k < 1024; k += 256) {
+                uint32_t y[8], m[8];
+#pragma unroll
+                for (uint32_t t = 0; t < 8; ++t) {
+                    const uint64_t j = j0 + k + 32 * t + lane_id();
+                    y[t] = raw[j < e ? j : b];
+                }
+#pragma unroll
+                for (uint32_t t = 0; t < 8; ++t) m[t] = __ldcg(map + (y[t] >> 5));
+#pragma unroll
+                for (uint32_t t = 0; t < 8; ++t)
+                    if (!((m[t] >> (y[t] & 31u)) & 1u)) atomicOr(map + (y[t] >> 5), 1u << (y[t] & 31u));
+            }
+        }
+    }
+}
+
 // Longer rows: one block per (row, range of kMapBits ids) marks the row's ids of
-// its range in a bitmap.  kEmit = false counts them (parts, deg); kEmit = true,
+// its range in a bitmap (a giant row's are marked already).  kEmit = false counts them (parts, deg); kEmit = true,
 // once the rows' places are known, writes them out in order.
 template <bool kEmit>
 __global__ void __launch_bounds__(1024) k_map_rows(uint32_t n, const uint64_t *__restrict__ start,
                                                    const uint32_t *__restrict__ raw, const uint32_t *__restrict__ huge,
-                                                   uint32_t ranges, uint32_t *__restrict__ parts,
+                                                   const uint32_t *__restrict__ big, const uint32_t *__restrict__ maps,
+                                                   uint32_t giant_words, uint32_t ranges, uint32_t *__restrict__ parts,
                                                    uint32_t *__restrict__ deg, const uint64_t *__restrict__ rp,
                                                    uint32_t *__restrict__ col, Ctl *ctl) {
     extern __shared__ uint32_t map[];  // kMapBits bits
@@ -414,11 +462,25 @@ __global__ void __launch_bounds__(1024) k_map_rows(uint32_t n, const uint64_t *_
         const uint32_t x = huge[unit / ranges], range = (uint32_t)(unit % ranges), lo = range * kMapBits;
         const uint64_t b = start[x], e = start[x + 1];
         const uint32_t words = (min(n - lo, kMapBits) + 31) / 32;
-        for (uint32_t i = threadIdx.x; i < words; i += blockDim.x) map[i] = 0;
-        __syncthreads();
-        for (uint64_t j = b + threadIdx.x; j < e; j += blockDim.x) {
-            const uint32_t y = raw[j] - lo;
-            if (y < kMapBits) atomicOr(&map[y >> 5], 1u << (y & 31u));
+        const uint32_t giant = big[n - 1 - (uint32_t)(unit / ranges)];
+        if (giant != kNoPlace) {
+            const uint32_t *m = maps + (uint64_t)giant * giant_words + lo / 32;
+            for (uint32_t i = threadIdx.x; i < words; i += blockDim.x) map[i] = m[i];
+        } else {
+            for (uint32_t i = threadIdx.x; i < words; i += blockDim.x) map[i] = 0;
+            __syncthreads();
+            for (uint64_t j0 = b + threadIdx.x; j0 < e; j0 += 16 * blockDim.x) {  // sixteen in flight (one: half the rate)
+                uint32_t y[16];
+#pragma unroll
+                for (uint32_t t = 0; t < 16; ++t) {
+                    const uint64_t j = j0 + t * blockDim.x;
+                    y[t] = j < e ? raw[j] - lo : kMapBits;
+                }
+#pragma unroll
+                for (uint32_t t = 0; t < 16; ++t)
+                    if (y[t] < kMapBits && !((map[y[t] >> 5] >> (y[t] & 31u)) & 1u))
+                        atomicOr(&map[y[t] >> 5], 1u << (y[t] & 31u));
+            }
         }
         __syncthreads();
         // every thread owns a run of words: its ids come after those of the threads before
@@ -595,9 +657,12 @@ static tc_status build_csr_counting(tc_ctx *ctx, uint32_t n, uint64_t t, const u
     const unsigned cap = (unsigned)ctx->num_sms * 16u;
     const uint32_t ranges = (n + kMapBits - 1) / kMapBits;
     const uint64_t max_huge = 2 * t / kBlockRow + 1;  // rows of more than kBlockRow entries
+    // rows of at least n / 16 entries: at most 32 t / n bitmaps of n / 8 bytes, which the places' 8 t bytes hold
+    // once the entries are placed
+    const uint32_t giant = std::max(kGiantRow, n / 16), giant_words = (n + 31) / 32;
     auto r = [](size_t b) { return (b + 255) & ~size_t(255); };
     const size_t n1 = (size_t)n + 1;
-    const size_t need = 4 * r(4 * n1) + r(8 * n1) + 2 * r(4 * t) + r(8 * t) + r(4 * max_huge * ranges) +
+    const size_t need = 4 * r(4 * n1) + r(8 * n1) + 2 * r(8 * t) + r(4 * max_huge * ranges) +
                         r(8 * scan_tmp_elems(n1)) + 4096;
     tc_status st = arena_reserve(ctx, need);
     if (st != TC_OK) return st;
@@ -608,12 +673,12 @@ static tc_status build_csr_counting(tc_ctx *ctx, uint32_t n, uint64_t t, const u
     auto *big = a.take<uint32_t>(n1);
     auto *huge = a.take<uint32_t>(n1);
     auto *start = a.take<uint64_t>(n1);
-    auto *place_a = a.take<uint32_t>(t);
-    auto *place_b = a.take<uint32_t>(t);
+    auto *place_a = a.take<uint32_t>(2 * t);
+    uint32_t *place_b = place_a + t, *maps = place_a;
     auto *raw = a.take<uint32_t>(2 * t);
     auto *parts = a.take<uint32_t>(max_huge * ranges);
     auto *tmp = a.take<uint64_t>(scan_tmp_elems(n1));
-    if (!cnt || !deg || !big || !huge || !start || !place_a || !place_b || !raw || !parts || !tmp)
+    if (!cnt || !deg || !big || !huge || !start || !place_a || !raw || !parts || !tmp)
         return set_error(ctx, TC_ERR_OOM, "arena carve failed (build_csr)");
     uint64_t *rp = nullptr;
     uint32_t *col = nullptr;
@@ -631,17 +696,19 @@ static tc_status build_csr_counting(tc_ctx *ctx, uint32_t n, uint64_t t, const u
     k_place_entries<<<grid_for(t, 256, cap), 256, 0, s>>>(t, d_src, d_dst, start, place_a, place_b, raw);
     const uint32_t per_warp = n >= (1u << 20) ? 32u : n >= (1u << 18) ? 16u : 8u;  // long rows of small graphs spread out
     k_sort_rows<<<grid_for((uint64_t)n * (32 / per_warp), kRowThreads, cap), kRowThreads, 0, s>>>(n, start, raw, deg, big,
-                                                                                               huge, per_warp, ctx->d_ctl);
+                                                                                               huge, cnt, per_warp, giant, ctx->d_ctl);
     const bool bigs = 2 * t > kWarpRow, huges = 2 * t > kBlockRow;  // there may be some
     const int map_smem = (int)(kMapBits / 8);
-    if (bigs) k_sort_rows_big<<<(unsigned)ctx->num_sms * 6u, 256, 0, s>>>(start, raw, deg, big, ctx->d_ctl);
+    if (bigs) k_sort_rows_big<<<(unsigned)ctx->num_sms * 6u, 256, 0, s>>>(start, raw, deg, big, maps, giant_words, ctx->d_ctl);
+    if (2 * t >= giant)
+        k_mark_giant<<<cap / 2, 256, 0, s>>>(start, raw, cnt, maps, giant_words, ctx->d_ctl);
     if (huges) {
         if (e == cudaSuccess)
             e = cudaFuncSetAttribute(k_map_rows<false>, cudaFuncAttributeMaxDynamicSharedMemorySize, map_smem);
         if (e == cudaSuccess)
             e = cudaFuncSetAttribute(k_map_rows<true>, cudaFuncAttributeMaxDynamicSharedMemorySize, map_smem);
-        k_map_rows<false><<<(unsigned)ctx->num_sms, 1024, map_smem, s>>>(n, start, raw, huge, ranges, parts, deg, nullptr,
-                                                                        nullptr, ctx->d_ctl);
+        k_map_rows<false><<<(unsigned)ctx->num_sms, 1024, map_smem, s>>>(n, start, raw, huge, big, maps, giant_words, ranges,
+                                                                        parts, deg, nullptr, nullptr, ctx->d_ctl);
     }
     scan_u32_to_u64(deg, rp, n, tmp, s);
     uint64_t U = 0;
@@ -666,8 +733,8 @@ static tc_status build_csr_counting(tc_ctx *ctx, uint32_t n, uint64_t t, const u
     if (U) {
         k_pack_rows<<<grid_for(n, 256, cap), 256, 0, s>>>(n, start, raw, rp, col);
         if (ctx->h_ctl->n_huge)
-            k_map_rows<true><<<(unsigned)ctx->num_sms, 1024, map_smem, s>>>(n, start, raw, huge, ranges, parts, deg, rp, col,
-                                                                           ctx->d_ctl);
+            k_map_rows<true><<<(unsigned)ctx->num_sms, 1024, map_smem, s>>>(n, start, raw, huge, big, maps, giant_words, ranges,
+                                                                           parts, deg, rp, col, ctx->d_ctl);
     }
     e = cudaGetLastError();
     if (e == cudaSuccess) e = cudaStreamSynchronize(s);

@@ -84,6 +84,7 @@ struct Ctl {
     unsigned int wedge_hi_task;      // first task of the tiles from rank kWedgeMaxK on
     unsigned int residual_left;      // vertices the one-block component step left to the host's loop
     unsigned int n_dense;            // vertices of degree >= kDenseDeg
+    unsigned int n_giant, pad;       // CSR build: rows marked by the whole grid
     unsigned long long est_wedge, est_classes;  // estimated times of the two counting paths (k_wedge_estimate)
     unsigned long long list_cursor;  // listing: next free chunk position
 };
