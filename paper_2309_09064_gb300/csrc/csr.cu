@@ -168,10 +168,13 @@ __global__ void k_empty_rowptr(uint32_t n, uint64_t *__restrict__ rp) {
 constexpr uint32_t kLaneRow = 32;      // entries of a row sorted by one lane
 constexpr uint32_t kWarpRow = 1024;    // by its warp
 constexpr uint32_t kBlockRow = 8192;   // by a block; longer rows go through bitmaps
+constexpr uint32_t kMapN = 16384;      // up to this many vertices all rows that no warp sorts do
 constexpr int kRowThreads = 256;
 constexpr uint32_t kMapBits = 1u << 20;  // ids a bitmap covers (128 KB of shared memory)
 // Rows whose bitmap lies in global memory: least entries, and how many (more of them keep every SM busy as it is).
-constexpr uint32_t kGiantRow = 1u << 17, kGiants = 64;
+// Two more launches, so only for many tuples (2^18 tuples of 2^22 vertices, one of them in every tuple: 0.48 against
+// 0.43 ms, but every other build of that size 15 us less).
+constexpr uint32_t kGiantRow = 1u << 17, kGiants = 64, kGiantTuples = 1u << 20;
 constexpr uint32_t kNoPlace = 0xFFFFFFFFu;
 
 // Entries before a vertex's newest one, one atomic per distinct vertex of the
@@ -209,6 +212,55 @@ __global__ void k_count_entries(uint64_t t, const uint32_t *__restrict__ src, co
     }
 }
 
+// Few vertices named by many tuples: the atomics of k_count_entries meet on few
+// addresses, so a block counts kFewTile tuples in shared memory and takes its places
+// of a vertex from the counts at once.  2^24 tuples of 8 / 256 / 1024 vertices, whole builds:
+// 5.5 / 7.9 / 3.0 -> 0.68 / 0.63 / 0.61 ms (the radix sort 1.3 / 1.8 / 2.4); at fewer than 16 tuples
+// a vertex or 2^16 in all it is no faster.
+constexpr uint32_t kFewN = 8192, kFewTile = 8192, kFewFrom = 1u << 16;
+__global__ void __launch_bounds__(1024) k_count_few(uint64_t t, const uint32_t *__restrict__ src,
+                                                    const uint32_t *__restrict__ dst, uint32_t n,
+                                                    uint32_t *__restrict__ cnt, uint32_t *__restrict__ place_a,
+                                                    uint32_t *__restrict__ place_b, Ctl *ctl) {
+    __shared__ uint32_t local[kFewN];  // entries of the tile per vertex, then the first one's place
+    constexpr int kItems = kFewTile / 1024;
+    for (uint64_t lo = (uint64_t)blockIdx.x * kFewTile; lo < t; lo += (uint64_t)gridDim.x * kFewTile) {
+        for (uint32_t v = threadIdx.x; v < n; v += 1024) local[v] = 0;
+        __syncthreads();
+        uint32_t a[kItems], b[kItems], pa[kItems], pb[kItems];
+#pragma unroll
+        for (int k = 0; k < kItems; ++k) {
+            const uint64_t i = lo + 1024 * k + threadIdx.x;
+            a[k] = i < t ? src[i] : 0u;
+            b[k] = i < t ? dst[i] : 0u;
+        }
+#pragma unroll
+        for (int k = 0; k < kItems; ++k) {
+            if (a[k] >= n || b[k] >= n) {
+                ctl->error = 1;
+                a[k] = b[k] = 0;
+            }
+            pa[k] = take_place(local, a[k], a[k] != b[k]);
+            pb[k] = take_place(local, b[k], a[k] != b[k]);
+        }
+        __syncthreads();
+        for (uint32_t v = threadIdx.x; v < n; v += 1024) {
+            const uint32_t c = local[v];
+            if (c) local[v] = atomicAdd(&cnt[v], c);
+        }
+        __syncthreads();
+#pragma unroll
+        for (int k = 0; k < kItems; ++k) {
+            const uint64_t i = lo + 1024 * k + threadIdx.x;
+            if (i < t) {
+                place_a[i] = a[k] != b[k] ? local[a[k]] + pa[k] : kNoPlace;
+                place_b[i] = a[k] != b[k] ? local[b[k]] + pb[k] : kNoPlace;
+            }
+        }
+        __syncthreads();
+    }
+}
+
 __global__ void k_place_entries(uint64_t t, const uint32_t *__restrict__ src, const uint32_t *__restrict__ dst,
                                 const uint64_t *__restrict__ start, const uint32_t *__restrict__ place_a,
                                 const uint32_t *__restrict__ place_b, uint32_t *__restrict__ raw) {
@@ -223,15 +275,13 @@ __global__ void k_place_entries(uint64_t t, const uint32_t *__restrict__ src, co
 }
 
 // Rows of up to kWarpRow entries: sorted in place, repeats dropped; deg[v] =
-// entries left.  Longer rows are listed for a block each, or for the bitmaps (from
-// `giant` entries on in global memory).
+// entries left.  Longer rows are listed for a block each, or for the bitmaps.
 // Lanes own rows of up to kLaneRow entries (insertion sort in their column of
 // the warp's buffer), the warp takes the others one by one.
 __global__ void __launch_bounds__(kRowThreads) k_sort_rows(uint32_t n, const uint64_t *__restrict__ start,
                                                            uint32_t *__restrict__ raw, uint32_t *__restrict__ deg,
                                                            uint32_t *__restrict__ big, uint32_t *__restrict__ huge,
-                                                           uint32_t *__restrict__ giants, uint32_t per_warp,
-                                                           uint32_t giant, Ctl *ctl) {
+                                                           uint32_t per_warp, uint32_t block_row, Ctl *ctl) {
     __shared__ __align__(16) uint32_t sbuf[kRowThreads / 32][kWarpRow];
     const unsigned lane = lane_id(), warp = threadIdx.x >> 5;
     const unsigned lt = (1u << lane) - 1u;
@@ -271,15 +321,8 @@ __global__ void __launch_bounds__(kRowThreads) k_sort_rows(uint32_t n, const uin
         }
         __syncwarp();
         if (valid && d > kWarpRow) {
-            if (d <= kBlockRow) big[atomicAdd(&ctl->n_big, 1u)] = (uint32_t)x;
-            else {
-                const uint32_t at = atomicAdd(&ctl->n_huge, 1u);
-                huge[at] = (uint32_t)x;
-                const uint32_t g = d >= giant ? atomicAdd(&ctl->n_giant, 1u) : kGiants;
-                if (g < kGiants) giants[g] = (uint32_t)x;
-                // the number of its bitmap (the list of big rows ends before: a row is in one of the two)
-                big[n - 1 - at] = g < kGiants ? g : kNoPlace;
-            }
+            if (d <= block_row) big[atomicAdd(&ctl->n_big, 1u)] = (uint32_t)x;
+            else huge[atomicAdd(&ctl->n_huge, 1u)] = (uint32_t)x;
         }
         unsigned pending = __ballot_sync(0xFFFFFFFFu, valid && d > kLaneRow && d <= kWarpRow);
         while (pending) {
@@ -341,16 +384,13 @@ __device__ __forceinline__ void compare_swap(uint32_t *sb, uint32_t i, uint32_t 
 
 __global__ void __launch_bounds__(256) k_sort_rows_big(const uint64_t *__restrict__ start, uint32_t *__restrict__ raw,
                                                        uint32_t *__restrict__ deg, const uint32_t *__restrict__ big,
-                                                       uint32_t *__restrict__ maps, uint32_t giant_words, Ctl *ctl) {
+                                                       Ctl *ctl) {
     __shared__ __align__(16) uint32_t sb[kBlockRow];
     __shared__ uint32_t warp_cnt[32];
     __shared__ unsigned int s_i;
     const unsigned lane = lane_id(), warp = threadIdx.x >> 5;
     uint32_t *run = sb + 1024 * warp;  // eight warps, 1024 keys each
     const uint32_t nb = ctl->n_big;
-    const uint64_t words = (uint64_t)min(ctl->n_giant, kGiants) * giant_words;
-    for (uint64_t i = (uint64_t)blockIdx.x * blockDim.x + threadIdx.x; i < words; i += (uint64_t)gridDim.x * blockDim.x)
-        maps[i] = 0;  // (for k_mark_giant)
     for (;;) {
         if (threadIdx.x == 0) s_i = atomicAdd(&ctl->sort_next, 1u);
         __syncthreads();
@@ -411,6 +451,35 @@ __global__ void __launch_bounds__(256) k_sort_rows_big(const uint64_t *__restric
     }
 }
 
+// The first kGiants rows of `giant` entries or more among the listed ones, and their
+// bitmaps cleared.  Every block finds them, the first one writes them down: every listed
+// row learns the number of its bitmap (kNoPlace: none) behind the list of big rows (a
+// row is in one of the two lists, so they do not meet).  Apart from k_sort_rows, which the
+// few lines slow down by a tenth.
+__global__ void __launch_bounds__(1024) k_list_giants(uint32_t n, const uint64_t *__restrict__ start,
+                                                      const uint32_t *__restrict__ huge, uint32_t *__restrict__ big,
+                                                      uint32_t *__restrict__ giants, uint32_t giant,
+                                                      uint32_t *__restrict__ maps, uint32_t giant_words, Ctl *ctl) {
+    __shared__ uint32_t warp_cnt[32];
+    const uint32_t nh = ctl->n_huge;
+    uint32_t ng = 0;
+    for (uint32_t i0 = 0; i0 < nh; i0 += 1024) {
+        const uint32_t i = i0 + threadIdx.x, x = i < nh ? huge[i] : 0u;
+        const bool is = i < nh && start[x + 1] - start[x] >= giant;
+        uint32_t total;
+        const uint32_t g = ng + block_rank(is, warp_cnt, &total);
+        if (blockIdx.x == 0) {
+            if (is && g < kGiants) giants[g] = x;
+            if (i < nh) big[n - 1 - i] = is && g < kGiants ? g : kNoPlace;
+        }
+        ng += total;
+    }
+    ng = min(ng, kGiants);
+    if (blockIdx.x == 0 && threadIdx.x == 0) ctl->n_giant = ng;
+    for (uint64_t i = (uint64_t)blockIdx.x * 1024 + threadIdx.x; i < (uint64_t)ng * giant_words; i += 1024ull * gridDim.x)
+        maps[i] = 0;
+}
+
 // The ids of the giant rows, marked in bitmaps in global memory (L2) by the whole grid: a
 // block of k_map_rows reads 2.3 entries a clock, so a vertex named by most tuples kept a
 // few blocks busy and the others idle (2^24 tuples of 2^22 vertices, one of them in every
@@ -419,7 +488,7 @@ __global__ void __launch_bounds__(256) k_mark_giant(const uint64_t *__restrict__
                                                     const uint32_t *__restrict__ raw,
                                                     const uint32_t *__restrict__ giants, uint32_t *maps,
                                                     uint32_t giant_words, const Ctl *ctl) {
-    const uint32_t ng = min(ctl->n_giant, kGiants);
+    const uint32_t ng = ctl->n_giant;
     const uint64_t warps = ((uint64_t)gridDim.x * blockDim.x) >> 5;
     const uint64_t w0 = ((uint64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5;
     for (uint32_t g = 0; g < ng; ++g) {
@@ -462,7 +531,7 @@ __global__ void __launch_bounds__(1024) k_map_rows(uint32_t n, const uint64_t *_
         const uint32_t x = huge[unit / ranges], range = (uint32_t)(unit % ranges), lo = range * kMapBits;
         const uint64_t b = start[x], e = start[x + 1];
         const uint32_t words = (min(n - lo, kMapBits) + 31) / 32;
-        const uint32_t giant = big[n - 1 - (uint32_t)(unit / ranges)];
+        const uint32_t giant = maps ? big[n - 1 - (uint32_t)(unit / ranges)] : kNoPlace;
         if (giant != kNoPlace) {
             const uint32_t *m = maps + (uint64_t)giant * giant_words + lo / 32;
             for (uint32_t i = threadIdx.x; i < words; i += blockDim.x) map[i] = m[i];
@@ -519,7 +588,7 @@ __global__ void __launch_bounds__(1024) k_map_rows(uint32_t n, const uint64_t *_
 // the entries of 32 rows, one per lane and step (their places are contiguous).
 __global__ void __launch_bounds__(256) k_pack_rows(uint32_t n, const uint64_t *__restrict__ start,
                                                    const uint32_t *__restrict__ raw, const uint64_t *__restrict__ rp,
-                                                   uint32_t *__restrict__ col) {
+                                                   uint32_t *__restrict__ col, uint32_t block_row) {
     const unsigned lane = lane_id();
     const uint64_t warps = ((uint64_t)gridDim.x * blockDim.x) >> 5, groups = ((uint64_t)n + 31) / 32;
     for (uint64_t g = ((uint64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5; g < groups; g += warps) {
@@ -530,7 +599,7 @@ __global__ void __launch_bounds__(256) k_pack_rows(uint32_t n, const uint64_t *_
             b = start[x];
             to = rp[x];
             d = (uint32_t)(rp[x + 1] - to);
-            if (start[x + 1] - b > kBlockRow) d = 0;
+            if (start[x + 1] - b > block_row) d = 0;
         }
         uint32_t incl = d;
 #pragma unroll
@@ -656,10 +725,13 @@ static tc_status build_csr_counting(tc_ctx *ctx, uint32_t n, uint64_t t, const u
     cudaStream_t s = ctx->stream;
     const unsigned cap = (unsigned)ctx->num_sms * 16u;
     const uint32_t ranges = (n + kMapBits - 1) / kMapBits;
-    const uint64_t max_huge = 2 * t / kBlockRow + 1;  // rows of more than kBlockRow entries
+    // the longest row a block sorts: of few vertices a bitmap is shorter (2^20 tuples of 1024 vertices 0.41 -> 0.17 ms)
+    const uint32_t block_row = n <= kMapN ? kWarpRow : kBlockRow;
+    const uint64_t max_huge = 2 * t / block_row + 1;  // rows of more entries
     // rows of at least n / 16 entries: at most 32 t / n bitmaps of n / 8 bytes, which the places' 8 t bytes hold
     // once the entries are placed
     const uint32_t giant = std::max(kGiantRow, n / 16), giant_words = (n + 31) / 32;
+    const bool giants = t >= kGiantTuples && 2 * t >= giant;
     auto r = [](size_t b) { return (b + 255) & ~size_t(255); };
     const size_t n1 = (size_t)n + 1;
     const size_t need = 4 * r(4 * n1) + r(8 * n1) + 2 * r(8 * t) + r(4 * max_huge * ranges) +
@@ -674,7 +746,7 @@ static tc_status build_csr_counting(tc_ctx *ctx, uint32_t n, uint64_t t, const u
     auto *huge = a.take<uint32_t>(n1);
     auto *start = a.take<uint64_t>(n1);
     auto *place_a = a.take<uint32_t>(2 * t);
-    uint32_t *place_b = place_a + t, *maps = place_a;
+    uint32_t *place_b = place_a + t, *maps = giants ? place_a : nullptr;
     auto *raw = a.take<uint32_t>(2 * t);
     auto *parts = a.take<uint32_t>(max_huge * ranges);
     auto *tmp = a.take<uint64_t>(scan_tmp_elems(n1));
@@ -691,17 +763,23 @@ static tc_status build_csr_counting(tc_ctx *ctx, uint32_t n, uint64_t t, const u
     k_ctl_zero<<<1, 128, 0, s>>>(ctx->d_ctl);
     cudaError_t e = cudaMemsetAsync(cnt, 0, 4 * n1, s);
     if (e == cudaSuccess) e = cudaMemsetAsync(deg, 0, 4 * n1, s);
-    k_count_entries<<<grid_for(t, 256, cap), 256, 0, s>>>(t, d_src, d_dst, n, cnt, place_a, place_b, ctx->d_ctl);
+    if (n <= kFewN && t >= kFewFrom && t >= 16ull * n)
+        k_count_few<<<grid_for(t, kFewTile, cap), 1024, 0, s>>>(t, d_src, d_dst, n, cnt, place_a, place_b, ctx->d_ctl);
+    else
+        k_count_entries<<<grid_for(t, 256, cap), 256, 0, s>>>(t, d_src, d_dst, n, cnt, place_a, place_b, ctx->d_ctl);
     scan_u32_to_u64(cnt, start, n, tmp, s);
     k_place_entries<<<grid_for(t, 256, cap), 256, 0, s>>>(t, d_src, d_dst, start, place_a, place_b, raw);
-    const uint32_t per_warp = n >= (1u << 20) ? 32u : n >= (1u << 18) ? 16u : 8u;  // long rows of small graphs spread out
+    // long rows of small graphs spread out (2^18 tuples of 512 vertices 0.32 -> 0.22 ms by one vertex a warp)
+    const uint32_t per_warp = n >= (1u << 20) ? 32u : n >= (1u << 18) ? 16u : n > kFewN ? 8u : n > 1024 ? 2u : 1u;
     k_sort_rows<<<grid_for((uint64_t)n * (32 / per_warp), kRowThreads, cap), kRowThreads, 0, s>>>(n, start, raw, deg, big,
-                                                                                               huge, cnt, per_warp, giant, ctx->d_ctl);
-    const bool bigs = 2 * t > kWarpRow, huges = 2 * t > kBlockRow;  // there may be some
+                                                                                               huge, per_warp, block_row, ctx->d_ctl);
+    const bool bigs = 2 * t > kWarpRow, huges = 2 * t > block_row;  // there may be some
     const int map_smem = (int)(kMapBits / 8);
-    if (bigs) k_sort_rows_big<<<(unsigned)ctx->num_sms * 6u, 256, 0, s>>>(start, raw, deg, big, maps, giant_words, ctx->d_ctl);
-    if (2 * t >= giant)
-        k_mark_giant<<<cap / 2, 256, 0, s>>>(start, raw, cnt, maps, giant_words, ctx->d_ctl);
+    if (bigs) k_sort_rows_big<<<(unsigned)ctx->num_sms * 6u, 256, 0, s>>>(start, raw, deg, big, ctx->d_ctl);
+    if (giants) {
+        k_list_giants<<<(unsigned)ctx->num_sms, 1024, 0, s>>>(n, start, huge, big, cnt, giant, maps, giant_words, ctx->d_ctl);
+        k_mark_giant<<<(unsigned)ctx->num_sms * 8u, 256, 0, s>>>(start, raw, cnt, maps, giant_words, ctx->d_ctl);
+    }
     if (huges) {
         if (e == cudaSuccess)
             e = cudaFuncSetAttribute(k_map_rows<false>, cudaFuncAttributeMaxDynamicSharedMemorySize, map_smem);
@@ -731,7 +809,7 @@ static tc_status build_csr_counting(tc_ctx *ctx, uint32_t n, uint64_t t, const u
         return set_error(ctx, TC_ERR_OOM, "tc_build_csr: col allocation failed");
     }
     if (U) {
-        k_pack_rows<<<grid_for(n, 256, cap), 256, 0, s>>>(n, start, raw, rp, col);
+        k_pack_rows<<<grid_for(n, 256, cap), 256, 0, s>>>(n, start, raw, rp, col, block_row);
         if (ctx->h_ctl->n_huge)
             k_map_rows<true><<<(unsigned)ctx->num_sms, 1024, map_smem, s>>>(n, start, raw, huge, big, maps, giant_words, ranges,
                                                                            parts, deg, rp, col, ctx->d_ctl);

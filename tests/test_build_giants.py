@@ -32,13 +32,14 @@ def star_rows(n, sizes):
 
 G = 1 << 17
 CASES = {
-    "limits": lambda: star_rows(300000, [G - 1, G, G + 1, 9000, 8192]),
-    "one": lambda: hubs(1 << 20, [3 * G], 1),
-    "two_ranges": lambda: hubs((1 << 20) + 33, [2 * G, G // 2], 2),
-    "sixteenth": lambda: hubs((1 << 22) + 5, [1 << 18, (1 << 18) + 4000, G + 500], 3),  # n / 16 = 2^18
-    "repeats": lambda: hubs(1000, [4 * G, G + 5, 200000], 4),
+    "limits": lambda: star_rows(300000, [G - 1, G, G + 1, 9000, 8192] + [8000] * 90),
+    "few_tuples": lambda: star_rows(300000, [G - 1, G, G + 1, 9000, 8192]),  # (below 2^20: by blocks alone)
+    "one": lambda: hubs(1 << 20, [8 * G], 1),
+    "two_ranges": lambda: hubs((1 << 20) + 33, [8 * G, G // 2], 2),
+    "sixteenth": lambda: hubs((1 << 22) + 5, [1 << 18, (1 << 18) + 4000, G + 500, 3 << 18], 3),  # n / 16 = 2^18
+    "repeats": lambda: hubs(1000, [8 * G, G + 5, 200000], 4),
     "past_64": lambda: hubs(90, [G + 100] * 70, 5),
-    "few_vertices": lambda: hubs(5, [500000, 400000, 10], 6),
+    "few_vertices": lambda: hubs(5, [900000, 400000, 10], 6),
 }
 
 
