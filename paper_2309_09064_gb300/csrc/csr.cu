@@ -281,17 +281,21 @@ __global__ void k_place_entries(uint64_t t, const uint32_t *__restrict__ src, co
 __global__ void __launch_bounds__(kRowThreads) k_sort_rows(uint32_t n, const uint64_t *__restrict__ start,
                                                            uint32_t *__restrict__ raw, uint32_t *__restrict__ deg,
                                                            uint32_t *__restrict__ big, uint32_t *__restrict__ huge,
-                                                           uint32_t per_warp, uint32_t block_row, Ctl *ctl) {
+                                                           uint32_t per_warp, uint32_t grab, uint32_t block_row, Ctl *ctl) {
     __shared__ __align__(16) uint32_t sbuf[kRowThreads / 32][kWarpRow];
     const unsigned lane = lane_id(), warp = threadIdx.x >> 5;
     const unsigned lt = (1u << lane) - 1u;
     uint32_t *buf = sbuf[warp];
     uint32_t top = 0;
     const uint64_t chunks = ((uint64_t)n + per_warp - 1) / per_warp;
-    for (;;) {
-        unsigned int c = 0;
-        if (lane == 0) c = atomicAdd(&ctl->fill_next, 1u);
-        c = __shfl_sync(0xFFFFFFFFu, c, 0);
+    uint32_t c = 0, left = 0;
+    for (;; ++c) {
+        if (left == 0) {  // the next `grab` chunks (one by one, the atomics of 2^21 chunks take 1.6 ms)
+            if (lane == 0) c = atomicAdd(&ctl->fill_next, grab);
+            c = __shfl_sync(0xFFFFFFFFu, c, 0);
+            left = grab;
+        }
+        --left;
         if (c >= chunks) break;
         const uint64_t x = (uint64_t)c * per_warp + lane;
         const bool valid = lane < per_warp && x < n;
@@ -719,9 +723,16 @@ uint32_t radix_sort_u64(unsigned long long **cur, unsigned long long **alt, uint
 constexpr uint64_t kCountTuples = 1ull << 31;
 constexpr uint32_t kCountN = 1u << 26;
 
+// Few tuples over very many vertices: the counting build passes over the vertices eight
+// times, the sort once.  Radix sort / counting: 2^24 vertices, 2^17 / 2^20 / 2^21 tuples 0.51 / 0.58 /
+// 0.74 against 0.59 / 0.66 / 0.72 ms, 2^26 and 2^14 / 2^20 / 2^22 / 2^24 1.0 / 1.1 / 1.8 / 4.8 against 1.5 / 1.8 /
+// 2.2 / 4.6 (2^22 vertices 0.42 against 0.30 at 2^16 tuples); with 2^10 tuples its row_ptr has runs
+// that one thread each fills: 5.9 against 1.5.
+static bool sparse_tuples(uint32_t n, uint64_t t) { return n >= (1u << 24) && t <= n / 16 && t > n / 8192; }
+
 static tc_status build_csr_counting(tc_ctx *ctx, uint32_t n, uint64_t t, const uint32_t *d_src, const uint32_t *d_dst,
                                     uint64_t **rp_out, uint32_t **col_out, uint64_t *slots_out, bool *pooled_out,
-                                    uint32_t *max_deg) {
+                                    uint32_t *max_deg, bool *no_room) {
     cudaStream_t s = ctx->stream;
     const unsigned cap = (unsigned)ctx->num_sms * 16u;
     const uint32_t ranges = (n + kMapBits - 1) / kMapBits;
@@ -737,6 +748,7 @@ static tc_status build_csr_counting(tc_ctx *ctx, uint32_t n, uint64_t t, const u
     const size_t need = 4 * r(4 * n1) + r(8 * n1) + 2 * r(8 * t) + r(4 * max_huge * ranges) +
                         r(8 * scan_tmp_elems(n1)) + 4096;
     tc_status st = arena_reserve(ctx, need);
+    *no_room = st == TC_ERR_OOM;
     if (st != TC_OK) return st;
     Arena &a = ctx->arena;
     a.reset();
@@ -771,8 +783,10 @@ static tc_status build_csr_counting(tc_ctx *ctx, uint32_t n, uint64_t t, const u
     k_place_entries<<<grid_for(t, 256, cap), 256, 0, s>>>(t, d_src, d_dst, start, place_a, place_b, raw);
     // long rows of small graphs spread out (2^18 tuples of 512 vertices 0.32 -> 0.22 ms by one vertex a warp)
     const uint32_t per_warp = n >= (1u << 20) ? 32u : n >= (1u << 18) ? 16u : n > kFewN ? 8u : n > 1024 ? 2u : 1u;
+    // an eighth of a warp's share of the chunks
+    const uint32_t grab = std::max(1u, std::min(16u, n / (32u * 8u * (kRowThreads / 32) * cap)));
     k_sort_rows<<<grid_for((uint64_t)n * (32 / per_warp), kRowThreads, cap), kRowThreads, 0, s>>>(n, start, raw, deg, big,
-                                                                                               huge, per_warp, block_row, ctx->d_ctl);
+                                                                                               huge, per_warp, grab, block_row, ctx->d_ctl);
     const bool bigs = 2 * t > kWarpRow, huges = 2 * t > block_row;  // there may be some
     const int map_smem = (int)(kMapBits / 8);
     if (bigs) k_sort_rows_big<<<(unsigned)ctx->num_sms * 6u, 256, 0, s>>>(start, raw, deg, big, ctx->d_ctl);
@@ -830,8 +844,12 @@ static tc_status build_csr_counting(tc_ctx *ctx, uint32_t n, uint64_t t, const u
 tc_status build_csr_device(tc_ctx *ctx, uint32_t n, uint64_t t, const uint32_t *d_src, const uint32_t *d_dst,
                            uint64_t **rp_out, uint32_t **col_out, uint64_t *slots_out, bool *pooled_out,
                            uint32_t *max_deg) {
-    if (t && t < kCountTuples && n && n <= kCountN)
-        return build_csr_counting(ctx, n, t, d_src, d_dst, rp_out, col_out, slots_out, pooled_out, max_deg);
+    if (t && t < kCountTuples && n && n <= kCountN && !sparse_tuples(n, t)) {
+        bool no_room = false;
+        const tc_status st =
+            build_csr_counting(ctx, n, t, d_src, d_dst, rp_out, col_out, slots_out, pooled_out, max_deg, &no_room);
+        if (!no_room) return st;  // (its scratch grows with the vertices, the sort's does not)
+    }
     cudaStream_t s = ctx->stream;
     const unsigned cap = (unsigned)ctx->num_sms * 16u;
     const uint64_t K = 2 * t;  // upper bound on keys
