@@ -71,6 +71,14 @@ static tc_status reserve_in(tc_ctx *ctx, Arena &a, size_t bytes) {
     return TC_OK;
 }
 
+cudaError_t allow_dynamic_smem(const void *kern) {
+    cudaFuncAttributes at{};
+    const cudaError_t e = cudaFuncGetAttributes(&at, kern);
+    if (e != cudaSuccess) return e;
+    return cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                (int)(kSmemLimitBytes - at.sharedSizeBytes));
+}
+
 tc_status arena_reserve(tc_ctx *ctx, size_t bytes) { return reserve_in(ctx, ctx->arena, bytes); }
 tc_status batch_arena_reserve(tc_ctx *ctx, size_t bytes) { return reserve_in(ctx, ctx->batch_arena, bytes); }
 

@@ -367,7 +367,7 @@ tc_status count_small_graphs(tc_ctx *ctx, const tc_graph *const *graphs, const s
     TC_CUDA(ctx, cudaMemsetAsync(d_next, 0, 8, s));
     const uint32_t bm_words = (nmax + 31) / 32;
     const size_t smem = 4ull * kGWarps * bm_words;
-    TC_CUDA(ctx, cudaFuncSetAttribute(k_count_graphs, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
+    TC_CUDA(ctx, allow_dynamic_smem((const void *)k_count_graphs));
     k_count_graphs<<<blocks, kGThreads, smem, s>>>(d_gs, d_order, G, d_next, d_scr, words, nmax, bm_words,
                                                    ctx->opt.order, d_counts, d_next + 1);
     note_launch(ctx);

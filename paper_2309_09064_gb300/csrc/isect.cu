@@ -1785,7 +1785,7 @@ tc_status intersect(tc_ctx *ctx, PipeBufs &b, uint32_t n) {
         const int tmode = b.list_phase == 1 ? 0 : mode;
         const size_t smem = 4ull * tu.tiny_cap * 256 + priv;
         auto tiny = tmode == 0 ? k_isect_tiny<0> : tmode == 1 ? k_isect_tiny<1> : k_isect_tiny<2>;
-        TC_CUDA(ctx, cudaFuncSetAttribute(tiny, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
+        TC_CUDA(ctx, allow_dynamic_smem((const void *)tiny));
         const uint32_t grid = std::min<uint32_t>((hi3 - lo3 + 255) / 256, (uint32_t)ctx->num_sms * 8u);
         VertexOut vt = vo;
         if (b.list_phase == 1) vt.task_hits = b.hits;
@@ -1820,7 +1820,7 @@ tc_status intersect(tc_ctx *ctx, PipeBufs &b, uint32_t n) {
                         ? (mode == 0 ? k_isect_warp<true, 0> : mode == 1 ? k_isect_warp<true, 1> : k_isect_warp<true, 2>)
                         : (mode == 0 ? k_isect_warp<false, 0>
                                      : mode == 1 ? k_isect_warp<false, 1> : k_isect_warp<false, 2>);
-        TC_CUDA(ctx, cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
+        TC_CUDA(ctx, allow_dynamic_smem((const void *)kern));
         int per_sm = 0;
         TC_CUDA(ctx, cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kern, 32 * tu.warps_per_block, smem));
         if (per_sm < 1) per_sm = 1;
@@ -1850,7 +1850,7 @@ tc_status intersect(tc_ctx *ctx, PipeBufs &b, uint32_t n) {
                                       : (mode == 0   ? k_isect_block<0, 0>
                                           : mode == 1 ? k_isect_block<0, 1>
                                                       : k_isect_block<0, 2>);
-        TC_CUDA(ctx, cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
+        TC_CUDA(ctx, allow_dynamic_smem((const void *)kern));
         int per_sm = 0;
         TC_CUDA(ctx, cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kern, tu.block_threads, smem));
         if (per_sm < 1) per_sm = 1;
@@ -1884,7 +1884,7 @@ tc_status intersect(tc_ctx *ctx, PipeBufs &b, uint32_t n) {
         if (smem > kSmemLimit) return set_error(ctx, TC_ERR_INVALID, "tuning leaves no shared memory for this mode");
         auto hub = split_R ? k_isect_hub<0, true>
                            : mode == 0 ? k_isect_hub<0> : mode == 1 ? k_isect_hub<1> : k_isect_hub<2>;
-        TC_CUDA(ctx, cudaFuncSetAttribute(hub, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
+        TC_CUDA(ctx, allow_dynamic_smem((const void *)hub));
         int per_sm = 0;
         TC_CUDA(ctx, cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, hub, tu.hub_threads, smem));
         if (per_sm < 1) per_sm = 1;

@@ -121,7 +121,6 @@ constexpr uint32_t kNoSplit = 0xFFFFFFFFu;  // glo[x]: G1(x) was not split
 // holds the low-rank bitmap, so its tasks take at most 1024 records to leave
 // room for a larger prefilter (the planner and the kernel use the same value).
 inline uint32_t hub_max_v(const Tuning &tu, uint32_t R) { return (R && tu.max_v > 1024) ? 1024u : tu.max_v; }
-constexpr size_t kSmemLimitBytes = 227 * 1024;  // shared memory one block may opt into on sm_103a
 // Cuckoo slots per table of the block class and the most ranks at or above
 // R one block-class set may hold (R = 0: no split, the whole set).
 uint32_t block_units_for(const Tuning &tu, uint32_t R);

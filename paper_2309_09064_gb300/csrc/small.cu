@@ -421,8 +421,7 @@ tc_status small_count(tc_ctx *ctx, const PipeBufs &b, uint32_t n, uint32_t max_d
     const uint32_t warps = (uint32_t)std::min<size_t>(8, kSmemLimitBytes / per);
     const size_t smem = per * warps;
     auto kern = grouped ? k_small_count<false> : k_small_count<true>;
-    // (the limit is the process's, not the call's: one value for every thread's launches)
-    TC_CUDA(ctx, cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kSmemLimitBytes));
+    TC_CUDA(ctx, allow_dynamic_smem((const void *)kern));
     int per_sm = 0;
     TC_CUDA(ctx, cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kern, 32 * warps, smem));
     const uint64_t blocks = ((uint64_t)n + per_warp * warps - 1) / (per_warp * warps);

@@ -227,6 +227,12 @@ tc_status max_degree_device(tc_ctx *ctx, uint32_t n, const uint64_t *rp, uint32_
 // Batched counting of G graphs as one disjoint union (batch.cu).
 tc_status count_batch(tc_ctx *ctx, uint32_t G, const tc_graph *const *graphs, uint64_t *counts);
 
+constexpr size_t kSmemLimitBytes = 227 * 1024;  // shared memory one block may opt into on sm_103a
+// Let launches of `kern` ask for all the dynamic shared memory that its static one leaves.  The
+// limit is the process's, not the call's: set to a call's own size it fails the launch of
+// another thread that needs more.
+cudaError_t allow_dynamic_smem(const void *kern);
+
 // Shared-memory bytes of the intersection kernels under a tuning (isect.cu)
 size_t warp_kernel_smem(const Tuning &tu);
 size_t block_kernel_smem(const Tuning &tu);
