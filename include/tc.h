@@ -100,7 +100,8 @@ typedef struct tc_stats {
     /* intersection classes: [0] warp (shared table per warp), [1] block (shared table), [2] hub (L2
        bitmaps + shared prefilter), [3] tiny (thread-per-row sorted merges).  Counts that take
        tiles (see tc_tuning): [1] the tiles, [0] the pairs no tile takes, the others empty.  Plain counts
-       of graphs of up to 2^15 vertices and a mean degree of up to 64: [0] all */
+       of graphs of up to 2^15 vertices and a mean degree of up to 64: [0] all
+       (a row of more than 64 earlier neighbours is a task per 64, and its row counts once for each) */
     uint64_t class_rows[4];     /* tasks (warp, block, hub) or rows (tiny) */
     uint64_t class_probes[4];   /* probed elements */
     uint64_t class_bytes[4];    /* algorithmic bytes: hashed rows once + probed rows */

@@ -379,7 +379,7 @@ tc_status count_pipeline(tc_ctx *ctx, const GraphView &g, uint32_t *levels_out, 
             stats->class_rows[c] = h.cls_rows[c];
             stats->class_probes[c] = h.cls_probes[c];
             // wedge path: tiles read 16-byte entries and 16-bit ids, the other pairs 4-byte keys
-            stats->class_bytes[c] = small ? 2ull * h.cls_probes[c]  // 16-bit ids
+            stats->class_bytes[c] = small ? 2ull * (h.cls_build[c] + h.cls_probes[c])  // 16-bit ids
                                     : wedge && c == 1 ? 16ull * h.cls_build[1] + 2ull * (h.cls_probes[1] + h.cls_inserts[1])
                                                     : 4ull * (h.cls_build[c] + h.cls_probes[c]);
             stats->class_inserts[c] = h.cls_inserts[c];

@@ -238,6 +238,8 @@ __global__ void __launch_bounds__(512) k_small_count(uint32_t n, const uint16_t 
     for (uint32_t i = lane; i < kW * words; i += 32) map[i] = 0;
     __syncwarp();
     unsigned long long same = 0, cross = 0, probes = 0, group_sum = 0;
+    unsigned long long marked = 0;  // ids put into the bitmap by this lane
+    uint32_t walks = 0;
     uint32_t group = 0, base = 0, group_end = groups.n_groups ? 0u : 0xFFFFFFFFu;  // group_end 0: none yet
     const long long t_start = clock64();
     // pairs of v with u among the keys [lo, hi) of its row
@@ -253,7 +255,9 @@ __global__ void __launch_bounds__(512) k_small_count(uint32_t n, const uint16_t 
         const uint2 mv = meta[v];
         const uint32_t d = mv.y & 0xFFFFu, level = mv.y >> 16;
         const uint16_t *row = ids + 8ull * mv.x;
+        ++walks;
         for (uint32_t i = lane; i < d; i += 32) {
+            ++marked;
             const uint32_t e = row[i], bit = 1u << (e & 31u);
             atomicOr(&map[kW * (e >> 5)], bit);
             if (kSplit && meta[base + e].y >> 16 == level) atomicOr(&map[kW * (e >> 5) + 1], bit);
@@ -373,12 +377,18 @@ __global__ void __launch_bounds__(512) k_small_count(uint32_t n, const uint16_t 
     same = warp_sum(same);
     cross = warp_sum(cross);
     probes = warp_sum(probes);
+    marked = warp_sum(marked);
     if (lane == 0) {
         if (same) atomicAdd(&ctl->t_same, same);
         if (cross) atomicAdd(&ctl->t_cross, cross);
         if (probes) {
             atomicAdd(&ctl->probes, probes);
             atomicAdd(&ctl->cls_probes[0], probes);
+        }
+        if (walks) {
+            atomicAdd(&ctl->cls_rows[0], (unsigned long long)walks);
+            atomicAdd(&ctl->cls_build[0], marked);
+            atomicAdd(&ctl->cls_inserts[0], marked);
         }
     }
 }
