@@ -785,13 +785,14 @@ static tc_status build_csr_counting(tc_ctx *ctx, uint32_t n, uint64_t t, const u
     const uint32_t per_warp = n >= (1u << 20) ? 32u : n >= (1u << 18) ? 16u : n > kFewN ? 8u : n > 1024 ? 2u : 1u;
     // an eighth of a warp's share of the chunks
     const uint32_t grab = std::max(1u, std::min(16u, n / (32u * 8u * (kRowThreads / 32) * cap)));
-    k_sort_rows<<<grid_for((uint64_t)n * (32 / per_warp), kRowThreads, cap), kRowThreads, 0, s>>>(n, start, raw, deg, big,
-                                                                                               huge, per_warp, grab, block_row, ctx->d_ctl);
+    k_sort_rows<<<grid_for((uint64_t)n * (32 / per_warp), kRowThreads, cap), kRowThreads, 0, s>>>(
+        n, start, raw, deg, big, huge, per_warp, grab, block_row, ctx->d_ctl);
     const bool bigs = 2 * t > kWarpRow, huges = 2 * t > block_row;  // there may be some
     const int map_smem = (int)(kMapBits / 8);
     if (bigs) k_sort_rows_big<<<(unsigned)ctx->num_sms * 6u, 256, 0, s>>>(start, raw, deg, big, ctx->d_ctl);
     if (giants) {
-        k_list_giants<<<(unsigned)ctx->num_sms, 1024, 0, s>>>(n, start, huge, big, cnt, giant, maps, giant_words, ctx->d_ctl);
+        k_list_giants<<<(unsigned)ctx->num_sms, 1024, 0, s>>>(n, start, huge, big, cnt, giant, maps, giant_words,
+                                                              ctx->d_ctl);
         k_mark_giant<<<(unsigned)ctx->num_sms * 8u, 256, 0, s>>>(start, raw, cnt, maps, giant_words, ctx->d_ctl);
     }
     if (huges) {
@@ -799,8 +800,8 @@ static tc_status build_csr_counting(tc_ctx *ctx, uint32_t n, uint64_t t, const u
             e = cudaFuncSetAttribute(k_map_rows<false>, cudaFuncAttributeMaxDynamicSharedMemorySize, map_smem);
         if (e == cudaSuccess)
             e = cudaFuncSetAttribute(k_map_rows<true>, cudaFuncAttributeMaxDynamicSharedMemorySize, map_smem);
-        k_map_rows<false><<<(unsigned)ctx->num_sms, 1024, map_smem, s>>>(n, start, raw, huge, big, maps, giant_words, ranges,
-                                                                        parts, deg, nullptr, nullptr, ctx->d_ctl);
+        k_map_rows<false><<<(unsigned)ctx->num_sms, 1024, map_smem, s>>>(
+            n, start, raw, huge, big, maps, giant_words, ranges, parts, deg, nullptr, nullptr, ctx->d_ctl);
     }
     scan_u32_to_u64(deg, rp, n, tmp, s);
     uint64_t U = 0;
@@ -825,8 +826,8 @@ static tc_status build_csr_counting(tc_ctx *ctx, uint32_t n, uint64_t t, const u
     if (U) {
         k_pack_rows<<<grid_for(n, 256, cap), 256, 0, s>>>(n, start, raw, rp, col, block_row);
         if (ctx->h_ctl->n_huge)
-            k_map_rows<true><<<(unsigned)ctx->num_sms, 1024, map_smem, s>>>(n, start, raw, huge, big, maps, giant_words, ranges,
-                                                                           parts, deg, rp, col, ctx->d_ctl);
+            k_map_rows<true><<<(unsigned)ctx->num_sms, 1024, map_smem, s>>>(
+                n, start, raw, huge, big, maps, giant_words, ranges, parts, deg, rp, col, ctx->d_ctl);
     }
     e = cudaGetLastError();
     if (e == cudaSuccess) e = cudaStreamSynchronize(s);

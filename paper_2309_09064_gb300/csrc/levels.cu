@@ -483,37 +483,6 @@ __global__ void k_after_level(Ctl *ctl, int nxt, uint32_t level) {
     if (ctl->fr_count[nxt]) ctl->max_level = level + 1 > ctl->max_level ? level + 1 : ctl->max_level;
 }
 
-// Grid-wide barrier with a bounded wait (all blocks are co-resident: the
-// kernel is launched cooperatively); tc_selftest_barrier drives it.  Barrier k
-// of a launch is passed once the arrival counter, zero before the launch,
-// reaches (k + 1) x nblocks.  A wait gives up after `timeout_cycles` of clock
-// time, raises the error flag and returns false, so the kernel ends and the
-// host reads TC_ERR_TIMEOUT.
-__device__ __forceinline__ bool grid_barrier(Ctl *ctl, unsigned nblocks, unsigned k, long long timeout_cycles) {
-    __shared__ int s_ok;
-    __syncthreads();
-    if (threadIdx.x == 0) {
-        volatile unsigned *count = &ctl->bar_count;
-        const unsigned target = (k + 1) * nblocks;
-        __threadfence();  // this block's frontier writes before its arrival
-        atomicAdd(&ctl->bar_count, 1u);
-        int ok = 1;
-        const long long t0 = clock64();
-        while (*count < target) {
-            if (clock64() - t0 > timeout_cycles) {
-                ctl->error = 4;
-                ok = 0;
-                break;
-            }
-            __nanosleep(32);
-        }
-        __threadfence();
-        s_ok = ok;
-    }
-    __syncthreads();
-    return s_ok != 0;
-}
-
 // Levels of small frontiers (high-diameter graphs, and whole small graphs): one
 // thread-block cluster runs level after level with a hardware cluster barrier
 // each.  The frontier lives in shared memory as a queue of edge slots: a
@@ -872,10 +841,24 @@ __global__ void __launch_bounds__(kClusterThreads, 1) k_bfs_cluster(const BfsArg
     }
 }
 
-// Self-test of the bounded wait: the barrier expects one more block than the
-// grid has, so no generation change ever comes and every block times out.
+// A grid-wide wait that is bounded (all blocks are co-resident: the kernel is launched
+// cooperatively), for tc_selftest_barrier: every block arrives and waits for one arrival more
+// than the grid has.  A wait gives up after `timeout_cycles` of clock time and raises the
+// error flag, so the kernel ends and the host reads TC_ERR_TIMEOUT.
 __global__ void k_barrier_selftest(Ctl *ctl, long long timeout_cycles) {
-    grid_barrier(ctl, gridDim.x + 1, 0, timeout_cycles);
+    if (threadIdx.x != 0) return;
+    volatile unsigned *count = &ctl->bar_count;
+    const unsigned target = gridDim.x + 1;
+    __threadfence();
+    atomicAdd(&ctl->bar_count, 1u);
+    const long long t0 = clock64();
+    while (*count < target) {
+        if (clock64() - t0 > timeout_cycles) {
+            ctl->error = 4;
+            break;
+        }
+        __nanosleep(32);
+    }
 }
 
 unsigned grid_for(uint64_t work, unsigned threads, unsigned cap) {

@@ -98,33 +98,26 @@ __global__ void __launch_bounds__(kScanThreads) k_scan_tiles(const T *in, unsign
     if (blockIdx.x == gridDim.x - 1 && threadIdx.x == 0) out[count] = sums[blockIdx.x] + tot;
 }
 
-// The whole scan in one block (in place too), for counts where three launches
-// cost more than one block's walk over the values.
-constexpr uint64_t kOneBlock = kTile;
+// One tile (in place too): one launch instead of three.
 template <class T>
 __global__ void __launch_bounds__(kScanThreads) k_scan_one(const T *in, unsigned long long *out, uint64_t count) {
-    unsigned long long carry = 0;
-    for (uint64_t c = 0; c < count; c += kTile) {
-        unsigned long long v[kScanItems];
-        unsigned long long s = 0;
+    unsigned long long v[kScanItems];
+    unsigned long long s = 0;
 #pragma unroll
-        for (int i = 0; i < kScanItems; ++i) {
-            const uint64_t j = c + (uint64_t)threadIdx.x * kScanItems + i;
-            v[i] = j < count ? (unsigned long long)in[j] : 0ull;
-            s += v[i];
-        }
-        unsigned long long tot;
-        unsigned long long ex = carry + block_exclusive<T>(s, &tot);
-#pragma unroll
-        for (int i = 0; i < kScanItems; ++i) {
-            const uint64_t j = c + (uint64_t)threadIdx.x * kScanItems + i;
-            if (j < count) out[j] = ex;
-            ex += v[i];
-        }
-        carry += tot;
-        __syncthreads();
+    for (int i = 0; i < kScanItems; ++i) {
+        const uint64_t j = (uint64_t)threadIdx.x * kScanItems + i;
+        v[i] = j < count ? (unsigned long long)in[j] : 0ull;
+        s += v[i];
     }
-    if (threadIdx.x == 0) out[count] = carry;
+    unsigned long long tot;
+    unsigned long long ex = block_exclusive<T>(s, &tot);
+#pragma unroll
+    for (int i = 0; i < kScanItems; ++i) {
+        const uint64_t j = (uint64_t)threadIdx.x * kScanItems + i;
+        if (j < count) out[j] = ex;
+        ex += v[i];
+    }
+    if (threadIdx.x == 0) out[count] = tot;
 }
 
 __global__ void k_zero_total(unsigned long long *out) { out[0] = 0ull; }
@@ -138,7 +131,7 @@ uint32_t scan_impl(const T *in, uint64_t *out, uint64_t count, uint64_t *tmp, cu
     const uint64_t nb = (count + kTile - 1) / kTile;
     auto *sums = reinterpret_cast<unsigned long long *>(tmp);
     auto *o = reinterpret_cast<unsigned long long *>(out);
-    if (count <= kOneBlock) {
+    if (count <= kTile) {
         k_scan_one<T><<<1, kScanThreads, 0, s>>>(in, o, count);
         return 1;
     }

@@ -71,7 +71,7 @@ __device__ __forceinline__ void small_row_done(const SmallRows &o, uint32_t x, u
 __global__ void __launch_bounds__(kRowThreads) k_small_rows(uint32_t n, const uint64_t *__restrict__ rp,
                                                             const uint32_t *__restrict__ col,
                                                             const uint32_t *__restrict__ dl, GroupSpec groups,
- SmallRows out,
+                                                            SmallRows out,
                                                             uint32_t per_warp, Ctl *ctl) {
     const unsigned lane = lane_id();
     const unsigned lt = (1u << lane) - 1u;
@@ -151,7 +151,7 @@ __global__ void __launch_bounds__(kRowThreads) k_small_rows(uint32_t n, const ui
 __global__ void __launch_bounds__(1024) k_small_rows_huge(const uint64_t *__restrict__ rp,
                                                           const uint32_t *__restrict__ col,
                                                           const uint32_t *__restrict__ dl, GroupSpec groups,
- SmallRows out, Ctl *ctl) {
+                                                          SmallRows out, Ctl *ctl) {
     __shared__ unsigned int wcnt[32];
     __shared__ unsigned int s_i;
     const unsigned lane = lane_id(), warp = threadIdx.x >> 5;

@@ -72,7 +72,7 @@ struct Ctl {
     unsigned int max_s2;             // largest hashed row among block-class rows / max degree
     unsigned int p_level;            // level the cluster BFS stopped at
     unsigned int bfs_spill;          // frontier vertices that found no place in its queues
-    unsigned int bar_count, bar_spare;  // arrivals at the self-test's grid barrier
+    unsigned int bar_count, bar_spare;  // arrivals at the self-test's wait
     unsigned int n_big;              // rows whose A part the block sorter sorts
     unsigned int n_huge;             // rows of very high degree filled by a block each
     unsigned int n_part;             // rows whose level-spanning part k_g1_split splits

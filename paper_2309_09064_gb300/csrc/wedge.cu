@@ -364,7 +364,8 @@ __global__ void __launch_bounds__(1024) k_wedge_sort(const uint32_t *__restrict_
 // those from K on.
 // Two launches make them tile by tile: kScatter = false counts every block's
 // entries per tile, kScatter = true writes them at the scanned offsets; a
-// block takes the same rows (a contiguous range) in both.  A warp flattens the keys of per_warp rows, one per lane and step;
+// block takes the same rows (a contiguous range) in both.  A warp flattens the keys
+// of per_warp rows, one per lane and step;
 // the last of the consecutive lanes of one row and tile makes their entries
 // (a tile that straddles two steps gets entries from both).
 // Without horizontal edges (bipartite graphs) there are no entries, and so no tasks,
@@ -1084,7 +1085,8 @@ __global__ void __launch_bounds__(kRestThreads) k_wedge_rest(uint32_t n, const u
                     return k - 1;
                 });
                 __syncwarp();
-                for (uint32_t i = lane; i < kRestSlots / 4; i += 32) reinterpret_cast<uint4 *>(table)[i] = make_uint4(0, 0, 0, 0);
+                for (uint32_t i = lane; i < kRestSlots / 4; i += 32)
+                    reinterpret_cast<uint4 *>(table)[i] = make_uint4(0, 0, 0, 0);
             } else {
                 for (uint32_t i = lane; i < vd; i += 32) {
                     const uint32_t h = (row[i] >> 1) & (kFilterBits - 1);
@@ -1255,7 +1257,9 @@ uint32_t entry_blocks(const tc_ctx *ctx, uint64_t slots) {
     return (uint32_t)std::min<uint64_t>(2ull * ctx->num_sms, slots / 4096 + 1);
 }
 
-uint32_t tasks_cap(const tc_ctx *ctx, uint32_t n, uint64_t slots) { return tiles_cap(n, slots) + (uint32_t)ctx->num_sms * kTasksPerSm + 1; }
+uint32_t tasks_cap(const tc_ctx *ctx, uint32_t n, uint64_t slots) {
+    return tiles_cap(n, slots) + (uint32_t)ctx->num_sms * kTasksPerSm + 1;
+}
 
 }  // namespace
 
@@ -1325,10 +1329,12 @@ tc_status wedge_rows(tc_ctx *ctx, const PipeBufs &b, uint32_t n, uint32_t max_de
         TC_CUDA(ctx, cudaFuncSetAttribute(k_wedge_entries<true>, cudaFuncAttributeMaxDynamicSharedMemorySize, most / 2));
         auto *offs = reinterpret_cast<unsigned long long *>(b.wedge_offs);
         k_wedge_entries<false><<<nb, 1024, smem, s>>>(n, b.slots, b.rp, b.adj2, b.fcnt, b.gcnt, b.wedge_counts, offs,
-                                                      b.wedge_work, b.erec, b.erec_cap, tiles, per_warp, b.lv, b.wedge_v, ctx->d_ctl);
+                                                      b.wedge_work, b.erec, b.erec_cap, tiles, per_warp, b.lv, b.wedge_v,
+                                                      ctx->d_ctl);
         launches += 3 + scan_u32_to_u64(b.wedge_counts, b.wedge_offs, cells, b.wedge_tmp, s);
         k_wedge_entries<true><<<nb, 1024, smem / 2, s>>>(n, b.slots, b.rp, b.adj2, b.fcnt, b.gcnt, b.wedge_counts, offs,
-                                                     b.wedge_work, b.erec, b.erec_cap, tiles, per_warp, b.lv, b.wedge_v, ctx->d_ctl);
+                                                     b.wedge_work, b.erec, b.erec_cap, tiles, per_warp, b.lv, b.wedge_v,
+                                                     ctx->d_ctl);
         // row ranges of about kRangeBytes of 16-bit ids (2 bytes an edge)
         const uint32_t ranges = (uint32_t)std::min<uint64_t>(b.slots / kRangeBytes + 1, 16);
         k_wedge_plan<<<1, 1024, 0, s>>>(offs, nb, b.wedge_work, (uint32_t)ctx->num_sms, ranges, b.wedge_tasks,
