@@ -339,7 +339,11 @@ tc_status count_pipeline(tc_ctx *ctx, const GraphView &g, uint32_t *levels_out, 
         *ctx->h_ctl = counted;  // statistics of the listing pass
         ctx->h_ctl->error = err;
     }
-    const Ctl &h = *ctx->h_ctl;
+    Ctl &h = *ctx->h_ctl;
+    if (small) {  // one class, whose ids are marked once each
+        h.probes = h.cls_probes[0];
+        h.cls_inserts[0] = h.cls_build[0];
+    }
     if (h.error) {
         char msg[96];
         std::snprintf(msg, sizeof msg, "device-side check failed during the count (code 0x%x)", h.error);

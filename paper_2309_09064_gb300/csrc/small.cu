@@ -27,6 +27,8 @@ constexpr uint32_t kLaneRow = 32;        // rows of degree <= 32: one lane each
 constexpr uint32_t kBlockRow = 2048;     // rows of higher degree: a block each
 constexpr uint32_t kSlice = 64;          // a row of more than this many u is walked by several warps
 constexpr int kRowThreads = 256;
+constexpr uint32_t kCountWarps = 8;      // of a block that walks rows
+constexpr uint32_t kDirectBlocks = 128;  // grids of up to so many: every warp adds its sums itself
 constexpr unsigned kGuardWatchdog = 0x80u;
 constexpr long long kWatchdogCycles = 20000000000ll;  // about 10 s of SM clock
 
@@ -228,7 +230,13 @@ __global__ void __launch_bounds__(512) k_small_count(uint32_t n, const uint16_t 
                                                      const uint2 *__restrict__ slices, GroupSpec groups,
                                                      uint32_t words, uint32_t per_warp, Ctl *ctl) {
     extern __shared__ __align__(16) uint32_t smem[];
+    __shared__ volatile unsigned long long s_sum[kCountWarps][5];  // {same, cross, probes, marked, walks}
+    __shared__ unsigned int s_done;
     if (ctl->e0 == 0) return;  // (every triangle has a horizontal edge)
+    if (gridDim.x > kDirectBlocks) {
+        if (threadIdx.x == 0) s_done = 0;
+        __syncthreads();
+    }
     constexpr uint32_t kW = kSplit ? 2 : 1;
     const unsigned lane = lane_id(), warp = threadIdx.x >> 5;
     const uint32_t sub = lane & 3u;
@@ -378,19 +386,28 @@ __global__ void __launch_bounds__(512) k_small_count(uint32_t n, const uint16_t 
     cross = warp_sum(cross);
     probes = warp_sum(probes);
     marked = warp_sum(marked);
-    if (lane == 0) {
-        if (same) atomicAdd(&ctl->t_same, same);
-        if (cross) atomicAdd(&ctl->t_cross, cross);
-        if (probes) {
-            atomicAdd(&ctl->probes, probes);
-            atomicAdd(&ctl->cls_probes[0], probes);
+    unsigned long long *const to = lane == 0   ? &ctl->t_same
+                                   : lane == 1 ? &ctl->t_cross
+                                   : lane == 2 ? &ctl->cls_probes[0]
+                                   : lane == 3 ? &ctl->cls_build[0]
+                                               : &ctl->cls_rows[0];
+    unsigned long long sum = lane == 0 ? same : lane == 1 ? cross : lane == 2 ? probes : lane == 3 ? marked : walks;
+    // In larger grids the block's last warp adds its warps' sums up: the warps' own atomics, on the same few
+    // addresses, take 10 us of a graph of 20000 vertices.  (At 1024 vertices the reduction takes 1 us more.)
+    if (gridDim.x > kDirectBlocks) {
+        bool last = false;
+        if (lane < 5) s_sum[warp][lane] = sum;
+        __syncwarp();
+        if (lane == 0) {
+            __threadfence_block();
+            last = atomicAdd(&s_done, 1u) + 1 == blockDim.x / 32;
         }
-        if (walks) {
-            atomicAdd(&ctl->cls_rows[0], (unsigned long long)walks);
-            atomicAdd(&ctl->cls_build[0], marked);
-            atomicAdd(&ctl->cls_inserts[0], marked);
-        }
+        if (!__shfl_sync(0xFFFFFFFFu, last, 0)) return;
+        __threadfence_block();
+        sum = 0;
+        for (uint32_t w = 0; lane < 5 && w < blockDim.x / 32; ++w) sum += s_sum[w][lane];
     }
+    if (lane < 5 && sum) atomicAdd(to, sum);
 }
 
 unsigned grid_for(uint64_t work, unsigned threads, unsigned cap) {
@@ -428,7 +445,7 @@ tc_status small_count(tc_ctx *ctx, const PipeBufs &b, uint32_t n, uint32_t max_d
     TC_CUDA(ctx, cudaEventRecord(ctx->ev[4], s));
     const uint32_t words = ((grouped ? b.groups.max_n : n) + 127) / 128 * 4;  // whole 16-byte pieces
     const size_t per = 4ull * ((grouped ? 1 : 2) * words + 128);
-    const uint32_t warps = (uint32_t)std::min<size_t>(8, kSmemLimitBytes / per);
+    const uint32_t warps = (uint32_t)std::min<size_t>(kCountWarps, kSmemLimitBytes / per);
     const size_t smem = per * warps;
     auto kern = grouped ? k_small_count<false> : k_small_count<true>;
     TC_CUDA(ctx, allow_dynamic_smem((const void *)kern));
