@@ -7,7 +7,8 @@
 // ids moves 16 bytes an entry six times for 2^21 vertices; here an entry is a
 // 4-byte id, placed once and sorted in shared memory.)  The result is the
 // paper's input format: symmetric, loop-free, duplicate-free, rows ascending.
-// Very many tuples or vertices take the radix sort: 64-bit keys (a << 32 | b)
+// Very many tuples or vertices, few tuples over many vertices, and a device without
+// room for the counts take the radix sort: 64-bit keys (a << 32 | b)
 // and (b << 32 | a), least significant 8-bit digits first, only the digits that
 // can be nonzero; col = low halves of the distinct keys, row_ptr from the run
 // boundaries of the high halves.
